@@ -66,7 +66,7 @@ struct Plan {
     int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG;
     size_t carry_bytes_per_table = 0;
     // sweep kernel
-    int n_pairs = 0, sweep_ptiles = 0, chunk_len = 0;
+    int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
     size_t off_pair_m = 0, off_pair_chunk = 0, off_pair_row = 0, off_pair_base = 0;
     int tables_per_batch = 0;
     size_t scratch_bytes = 0;
@@ -351,7 +351,10 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
         pl.off_pair_chunk = append_aligned(blob, pc);
         pl.off_pair_row = append_aligned(blob, pr);
         pl.off_pair_base = append_aligned(blob, pair_base);
-        pl.sweep_ptiles = (n_P + kThreads * kSweepR - 1) / (kThreads * kSweepR);
+        const int p_tiles = (n_P + 32 * kSweepR - 1) / (32 * kSweepR);
+        pl.sweep_wp = kWarps;
+        while (pl.sweep_wp > 1 && pl.sweep_wp / 2 >= p_tiles) pl.sweep_wp >>= 1;
+        pl.sweep_ptiles = (p_tiles + pl.sweep_wp - 1) / pl.sweep_wp;
     }
 
     if (blob.size() > h->grid_cap) {
@@ -487,10 +490,11 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sp.pair_m = reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_m);
             sp.pair_chunk = reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_chunk);
             sp.pair_row = reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_row);
-            sp.n_pairs = pl.n_pairs; sp.n_ptiles = pl.sweep_ptiles; sp.chunk_len = pl.chunk_len;
+            sp.n_pairs = pl.n_pairs; sp.n_ptiles = pl.sweep_ptiles; sp.chunk_len = pl.chunk_len; sp.wp = pl.sweep_wp;
             sp.part_time = part_time; sp.part_idx = part_idx; sp.n_seg = pl.n_seg; sp.table0 = t0;
-            { LaunchTimer lt(h, PLOGP_KERNEL_SWEEP, st); CK(launch_sweep(sp, nt, st)); }
-            g_launches += 1;
+            int n_launches = 0;
+            { LaunchTimer lt(h, PLOGP_KERNEL_SWEEP, st); CK(launch_sweep(sp, nt, &n_launches, st)); }
+            g_launches += unsigned(n_launches);
         }
         if (need_carry) {
             S1Params s{};

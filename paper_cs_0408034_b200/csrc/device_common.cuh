@@ -66,6 +66,30 @@ __device__ __forceinline__ uint32_t segments(uint32_t m, uint32_t s, int k_mode)
     return q + ((k_mode == 0 && q * s != m) ? 1u : 0u);
 }
 
+// Lower bounds in FP32: two fused multiply-adds at a time, rounded towards minus infinity.  With operands that are
+// rounded down themselves and non-negative, a result is never above the FP64 value of the same expression.
+using f32x2 = unsigned long long;
+struct __align__(16) f32x2x2 { f32x2 x, y; };
+__device__ __forceinline__ f32x2 splat2(float a)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2_down(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// the smallest of a and the two values of t (one three-input minimum)
+__device__ __forceinline__ float min_with2(float a, f32x2 t)
+{
+    float r;
+    asm("{.reg .f32 lo, hi;\n\tmov.b64 {lo, hi}, %2;\n\tmin.f32 %0, %1, lo, hi;}" : "=f"(r) : "f"(a), "l"(t));
+    return r;
+}
+
 // Interval search alone: largest i with key[i] <= x (0 when x is below the table).
 __device__ __forceinline__ int interval_of(const double *s_tab, int npad, double x)
 {

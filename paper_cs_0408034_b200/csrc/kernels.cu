@@ -6,7 +6,8 @@
 //   sweep_kernel   lane <-> process count P.  One CTA owns one message size m, a tile of P values
 //                  and a chunk of the candidate segment sizes; the per-(m, s) line coefficients are
 //                  computed once per CTA into shared memory and broadcast to all lanes, so a model
-//                  cell costs one DFMA and one integer compare.  Used when the candidate list is long.
+//                  cell costs half a packed FP32 multiply-add and half a minimum; what the FP32 bounds leave
+//                  open is decided in FP64.  Used when the candidate list is long.
 //   fused_kernel   lane <-> message size m (32 consecutive m per warp, so every output row is
 //                  written as full, aligned segments).  Evaluates all enabled strategies, runs short
 //                  candidate lists inline or reduces the sweep kernel's partial minima, keeps the
@@ -30,18 +31,41 @@ namespace plogp {
 //   id 5: (P-1) (g(s)+L) + g(s)(k-1)          = fma(P-1, B, C)   B = g(s)+L, C = g(s)(k-1)
 //   id 2: (P-1) (g(s) k) + L                  = fma(P-1, Q, L)   Q = g(s) k
 //   id 9: floor(log2 P) g(s) k + ceil(log2 P) L = fma(lf, Q, lc L)
-// so the CTA computes (B, C, Q) once per candidate and every lane spends one DFMA and one
-// compare per cell.
+// so the CTA computes (B, C, Q) once per candidate and every lane spends one multiply-add per cell.
+//
+// Every cell is first evaluated as a lower bound: coefficients and process count rounded down to FP32, the packed
+// fused multiply-add rounded down as well.  All terms are non-negative, so the bound is never above the FP64 time.
+// The smallest bound of a batch of candidates, per process count, is compared with an upper bound of the best time
+// known there; only where it is not above does the batch come back, group by group, to the exact FP64 comparison.
+// The results are those of the exhaustive FP64 search, bit for bit.  The upper bounds start from a few log-spaced
+// candidates of the whole list (rounded up in FP32), so a chunk far from the optimum never leaves the fast loop.
+// The best times themselves are touched by the exact pass alone and live in shared memory.
+//
+// What bounds it: issue.  Two cells cost one packed multiply-add and one three-input minimum, 2.1 cycles of a scheduler
+// per 32 cells by themselves (an FP64 multiply-add with an integer compare of the high words, as the loop had it before:
+// 4.6); with list building, barriers and exact passes (2 %) 2.5.  P = 2..4096, 128 message sizes, 1.25e11 cells of
+// ids 2 and 5: 15.05 -> 8.5 ms.  Scalar multiply-adds, 16 process counts per lane, lanes <-> candidates and packing
+// along P run at the same 2.0 - 2.5 cycles.
+//
+// A warp owns 256 consecutive process counts (lane + 32 r).  The CTA's 8 warps cover p.wp such tiles side by side and
+// split the candidates of a sub-chunk 8 / p.wp ways, so that a short range of process counts leaves no warp idle.
 
-template <int SEGMASK>
+template <bool HAS2, bool HAS5, bool IS9>
 __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
 {
-    constexpr bool HAS2 = (SEGMASK & 1) != 0, HAS5 = (SEGMASK & 2) != 0, HAS9 = (SEGMASK & 4) != 0;
+    static_assert(!IS9 || !(HAS2 || HAS5), "id 9 has lines of its own");
+    constexpr bool QL = HAS2 || IS9;  // lists of Q
     constexpr int R = kSweepR;
+    constexpr unsigned kFull = 0xffffffffu;
+    constexpr int kNid = (HAS2 ? 1 : 0) + (HAS5 ? 1 : 0) + (IS9 ? 1 : 0);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *s_tab = reinterpret_cast<double *>(smem_raw);
     double2 *s_bc = reinterpret_cast<double2 *>(s_tab + 3 * p.T.npad);  // [2][kSweepSub]
     double *s_q = reinterpret_cast<double *>(s_bc + 2 * kSweepSub);     // [2][kSweepSub]
+    double *s_best = s_q + 2 * kSweepSub;                               // [kNid][kWarps][R][32]
+    float *s_bf = reinterpret_cast<float *>(s_best + kNid * kWarps * R * 32);  // [2][kSweepSub]
+    float *s_cf = s_bf + 2 * kSweepSub, *s_qf = s_cf + 2 * kSweepSub;
+    uint32_t *s_idx = reinterpret_cast<uint32_t *>(s_qf + 2 * kSweepSub);      // [kNid][kWarps][R][32]
 
     const int tid = threadIdx.x;
     const int pi = blockIdx.x / p.n_ptiles;
@@ -60,117 +84,185 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     stage_table(s_tab, p.T, table);
     const double L = p.T.lat[table];
 
-    // A warp owns 256 consecutive process counts (lane + 32 r), so neighbouring cells see similar optima
-    // and the stores below stay coalesced.
     const int lane = tid & 31, warp = tid >> 5;
-    const int p_first = ptile * (kThreads * R) + warp * (32 * R) + lane;
-    double pm1[R], best2[R], best5[R], best9[R], lf[R], lcL[R];
-    uint32_t idx2[R], idx5[R], idx9[R];
+    const int wp = p.wp, wc = kWarps / wp, my_p = warp & (wp - 1), my_c = warp / wp;
+    const int c_len = kSweepSub / wc, batch = min(c_len, kSweepBatch);  // this warp's candidates of a sub-chunk
+    const int p_first = (ptile * wp + my_p) * (32 * R) + lane;
+    // a process count past the last one repeats the last one
+    auto P_of = [&](int r) { return P_at(p.G, min(p_first + 32 * r, p.G.n_P - 1)); };
+    auto x_exact = [&](int P) { return IS9 ? static_cast<double>(31 - __clz(P)) : static_cast<double>(P - 1); };
+    auto c_exact = [&](int P) { return IS9 ? static_cast<double>(32 - __clz(P - 1)) * L : L; };
+
+    f32x2 x2[R], c2[IS9 ? R : 1];  // multiplier and, where the offset is not a candidate's, offset, rounded down, twice each
+    float T2[HAS2 || IS9 ? R : 1], T5[HAS5 ? R : 1];  // upper bounds of the best times
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int pidx = min(p_first + 32 * r, p.G.n_P - 1);
-        const int P = P_at(p.G, pidx);
-        pm1[r] = static_cast<double>(P - 1);
-        lf[r] = static_cast<double>(31 - __clz(P));
-        lcL[r] = static_cast<double>(32 - __clz(P - 1)) * L;
-        best2[r] = best5[r] = best9[r] = CUDART_INF;
-        idx2[r] = idx5[r] = idx9[r] = 0xFFFFFFFFu;
+        const int P = P_of(r);
+        x2[r] = splat2(IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_rd(P - 1));
+        if (IS9) c2[r] = splat2(__double2float_rd(c_exact(P)));
+        if (QL) T2[r] = CUDART_INF_F;
+        if (HAS5) T5[r] = CUDART_INF_F;
     }
+    if (!IS9) c2[0] = splat2(__double2float_rd(L));
+    double *best = s_best + warp * R * 32 + lane;  // + id slot * kWarps * R * 32 + r * 32
+    uint32_t *bidx = s_idx + warp * R * 32 + lane;
+    constexpr int kIdStep = kWarps * R * 32;
+#pragma unroll
+    for (int q = 0; q < kNid; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) { best[q * kIdStep + r * 32] = CUDART_INF; bidx[q * kIdStep + r * 32] = 0xFFFFFFFFu; }
     __syncthreads();
 
-    auto fill = [&](int sub, int buf) {
-        const int si = s_begin + sub * kSweepSub + tid;
-        double B = CUDART_INF, C = CUDART_INF, Q = CUDART_INF;  // padding never wins a strict '<'
-        if (si < s_end) {
-            const uint32_t s = s_at(p.G, si);
-            const double gs = gap_at(s_tab, p.T.npad, static_cast<double>(s));
-            const double k = static_cast<double>(segments(m_u, s, p.G.k_mode));
-            B = gs + L;
-            C = gs * (k - 1.0);
-            Q = gs * k;
-        }
-        s_bc[buf * kSweepSub + tid] = make_double2(B, C);
-        s_q[buf * kSweepSub + tid] = Q;
+    auto coefficients = [&](int si, double &B, double &C, double &Q) {
+        const uint32_t s = s_at(p.G, si);
+        const double gs = gap_at(s_tab, p.T.npad, static_cast<double>(s));
+        const double k = static_cast<double>(segments(m_u, s, p.G.k_mode));
+        B = gs + L;
+        C = gs * (k - 1.0);
+        Q = gs * k;
     };
+    auto fill = [&](int sub, int buf) {
+        const int si = s_begin + sub * kSweepSub + tid, o = buf * kSweepSub + tid;
+        double B = 0.0, C = CUDART_INF, Q = CUDART_INF;  // padding: the bound is +inf
+        if (si < s_end) coefficients(si, B, C, Q);
+        if (HAS5) {
+            s_bc[o] = make_double2(B, C);
+            s_bf[o] = __double2float_rd(B);
+            s_cf[o] = __double2float_rd(C);
+        }
+        if (QL) {
+            s_q[o] = Q;
+            s_qf[o] = __double2float_rd(Q);
+        }
+    };
+
+    // ---- upper bounds from log-spaced candidates of the whole list ----
+    const int n_seed = min(kSweepSeeds, ns);
+    if (tid < kSweepSeeds) {
+        float B = 0.f, C = CUDART_INF_F, Q = CUDART_INF_F;
+        if (tid < n_seed) {
+            int si = min(ns - 1, static_cast<int>(exp2f(log2f(static_cast<float>(ns)) * (static_cast<float>(tid + 1) / n_seed))) - 1);
+            if (!p.G.s_list) {  // the smallest candidate with the same number of segments is the better one
+                const uint32_t s = s_at(p.G, si), k = max(segments(m_u, s, p.G.k_mode), 1u);
+                const uint32_t t = p.G.k_mode == 0 ? (m_u + k - 1) / k : m_u / (k + 1) + 1;
+                si = t <= p.G.s_lo ? 0 : min(si, static_cast<int>((t - p.G.s_lo + p.G.s_step - 1) / p.G.s_step));
+            }
+            double Bd, Cd, Qd;
+            coefficients(max(si, 0), Bd, Cd, Qd);
+            B = __double2float_ru(Bd); C = __double2float_ru(Cd); Q = __double2float_ru(Qd);
+        }
+        s_bf[tid] = B; s_cf[tid] = C; s_qf[tid] = Q;
+    }
+    __syncthreads();
+    {
+        float xu[R], cu[IS9 ? R : 1];  // rounded up
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int P = P_of(r);
+            xu[r] = IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_ru(P - 1);
+            if (IS9) cu[r] = __double2float_ru(c_exact(P));
+        }
+        if (!IS9) cu[0] = __double2float_ru(L);
+#pragma unroll 1
+        for (int i = 0; i < n_seed; ++i) {
+            const float B = s_bf[i], C = s_cf[i], Q = s_qf[i];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (HAS5) T5[r] = fminf(T5[r], __fmaf_ru(xu[r], B, C));
+                if (QL) T2[r] = fminf(T2[r], __fmaf_ru(xu[r], Q, cu[IS9 ? r : 0]));
+            }
+        }
+    }
+    __syncthreads();
 
     fill(0, 0);
     __syncthreads();
     for (int sub = 0; sub < n_sub; ++sub) {
         const int buf = sub & 1;
         if (sub + 1 < n_sub) fill(sub + 1, buf ^ 1);
-        const double2 *bc = s_bc + buf * kSweepSub;
-        const double *qq = s_q + buf * kSweepSub;
         const uint32_t base = static_cast<uint32_t>(s_begin + sub * kSweepSub);
 #pragma unroll 1
-        for (int i = 0; i < kSweepSub; i += kSweepU) {
-            // Hot path: every cell is evaluated (one DFMA); the comparison with the running minimum is
-            // first taken on the high words only, in the integer pipe.  Times are non-negative, so the
-            // high word of a smaller double is never larger: a cell can only improve if that test holds.
-            // (one flag per register cell: a single flag would chain all the integer compares of the
-            // chunk through one predicate, and that dependent chain, not a pipe, then sets the pace)
-            bool f5[R], f2[R], f9[R];
+        for (int j0 = my_c * c_len; j0 < (my_c + 1) * c_len; j0 += batch) {
+            const float *bf = s_bf + buf * kSweepSub + j0, *cf = s_cf + buf * kSweepSub + j0, *qf = s_qf + buf * kSweepSub + j0;
+            float mn5[HAS5 ? R : 1], mn2[QL ? R : 1];
 #pragma unroll
-            for (int r = 0; r < R; ++r) f5[r] = f2[r] = f9[r] = false;
-#pragma unroll
-            for (int u = 0; u < kSweepU; ++u) {
-                if (HAS5) {
-                    const double2 c = bc[i + u];
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        f5[r] |= __double2hiint(fma(pm1[r], c.x, c.y)) <= __double2hiint(best5[r]);
-                }
-                if (HAS2 || HAS9) {
-                    const double q = qq[i + u];
-                    if (HAS2) {
-#pragma unroll
-                        for (int r = 0; r < R; ++r)
-                            f2[r] |= __double2hiint(fma(pm1[r], q, L)) <= __double2hiint(best2[r]);
-                    }
-                    if (HAS9) {
-#pragma unroll
-                        for (int r = 0; r < R; ++r)
-                            f9[r] |= __double2hiint(fma(lf[r], q, lcL[r])) <= __double2hiint(best9[r]);
-                    }
-                }
+            for (int r = 0; r < R; ++r) {
+                if (HAS5) mn5[r] = CUDART_INF_F;
+                if (QL) mn2[r] = CUDART_INF_F;
             }
-            bool any5 = false, any2 = false, any9 = false;
-#pragma unroll
-            for (int r = 0; r < R; r += 2) {
-                any5 |= f5[r] | f5[r + 1];
-                any2 |= f2[r] | f2[r + 1];
-                any9 |= f9[r] | f9[r + 1];
-            }
-            // Exact passes over the same candidates, in ascending order, strict '<' (smallest s on ties).
-            if (HAS5 && any5) {
 #pragma unroll 1
-                for (int u = 0; u < kSweepU; ++u) {
-                    const double2 c = bc[i + u];
+            for (int i = 0; i < batch; i += kSweepU) {
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double t = fma(pm1[r], c.x, c.y);
-                        if (t < best5[r]) { best5[r] = t; idx5[r] = base + i + u; }
+                for (int u = 0; u < kSweepU; u += 4) {
+                    if (HAS5) {
+                        const f32x2x2 bb = *reinterpret_cast<const f32x2x2 *>(bf + i + u), cc = *reinterpret_cast<const f32x2x2 *>(cf + i + u);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) mn5[r] = min_with2(mn5[r], fma2_down(x2[r], bb.x, cc.x));
+#pragma unroll
+                        for (int r = 0; r < R; ++r) mn5[r] = min_with2(mn5[r], fma2_down(x2[r], bb.y, cc.y));
+                    }
+                    if (QL) {
+                        const f32x2x2 qq = *reinterpret_cast<const f32x2x2 *>(qf + i + u);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) mn2[r] = min_with2(mn2[r], fma2_down(x2[r], qq.x, c2[IS9 ? r : 0]));
+#pragma unroll
+                        for (int r = 0; r < R; ++r) mn2[r] = min_with2(mn2[r], fma2_down(x2[r], qq.y, c2[IS9 ? r : 0]));
                     }
                 }
             }
-            if (HAS2 && any2) {
-#pragma unroll 1
-                for (int u = 0; u < kSweepU; ++u) {
-                    const double q = qq[i + u];
+            unsigned hit = 0;  // bit r: id 2 or 9, bit 16 + r: id 5
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double t = fma(pm1[r], q, L);
-                        if (t < best2[r]) { best2[r] = t; idx2[r] = base + i + u; }
-                    }
-                }
+            for (int r = 0; r < R; ++r) {
+                if (QL && mn2[r] <= T2[r]) hit |= 1u << r;
+                if (HAS5 && mn5[r] <= T5[r]) hit |= 0x10000u << r;
             }
-            if (HAS9 && any9) {
+            if (__any_sync(kFull, hit != 0)) {
+                // Exact pass over the batch for the flagged rows: candidates in ascending order, strict '<' (smallest s on
+                // ties).  The bounds in T only ever shrink towards the best time, so nothing that could win is passed over.
 #pragma unroll 1
-                for (int u = 0; u < kSweepU; ++u) {
-                    const double q = qq[i + u];
+                for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
+                    const int bit = __ffs(rows) - 1, r = bit & 15;
+                    const bool five = HAS5 && (bit >> 4);
+                    const int P = P_of(r);
+                    const double x = x_exact(P), c = c_exact(P);
+                    const float xf = IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_rd(P - 1), cfl = __double2float_rd(c);
+                    const int o = (five && HAS2 ? kIdStep : 0) + r * 32;
+                    double bt = best[o];
+                    uint32_t bi = bidx[o];
+                    float T = CUDART_INF_F;
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double t = fma(lf[r], q, lcL[r]);
-                        if (t < best9[r]) { best9[r] = t; idx9[r] = base + i + u; }
+                    for (int q = 0; q < R; ++q) {
+                        if (HAS5 && five && q == r) T = T5[q];
+                        if (QL && !five && q == r) T = T2[q];
+                    }
+#pragma unroll 1
+                    for (int i = 0; i < batch; i += 4) {
+                        float t[4];
+                        if (HAS5 && five) {
+                            const float4 b4 = *reinterpret_cast<const float4 *>(bf + i), c4 = *reinterpret_cast<const float4 *>(cf + i);
+                            t[0] = __fmaf_rd(xf, b4.x, c4.x); t[1] = __fmaf_rd(xf, b4.y, c4.y);
+                            t[2] = __fmaf_rd(xf, b4.z, c4.z); t[3] = __fmaf_rd(xf, b4.w, c4.w);
+                        } else {
+                            const float4 q4 = *reinterpret_cast<const float4 *>(qf + i);
+                            t[0] = __fmaf_rd(xf, q4.x, cfl); t[1] = __fmaf_rd(xf, q4.y, cfl);
+                            t[2] = __fmaf_rd(xf, q4.z, cfl); t[3] = __fmaf_rd(xf, q4.w, cfl);
+                        }
+                        if (__any_sync(kFull, fminf(fminf(t[0], t[1]), fminf(t[2], t[3])) <= T)) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const int e = buf * kSweepSub + j0 + i + u;
+                                const double tt = five ? fma(x, s_bc[e].x, s_bc[e].y) : fma(x, s_q[e], c);
+                                if (tt < bt) { bt = tt; bi = base + j0 + i + u; }
+                            }
+                            T = fminf(T, __double2float_ru(bt));
+                        }
+                    }
+                    best[o] = bt;
+                    bidx[o] = bi;
+#pragma unroll
+                    for (int q = 0; q < R; ++q) {
+                        if (HAS5 && five && q == r) T5[q] = T;
+                        if (QL && !five && q == r) T2[q] = T;
                     }
                 }
             }
@@ -178,23 +270,26 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
         __syncthreads();
     }
 
-    // partial results, one row per (table, strategy slot, (m, chunk) pair), P contiguous
-    int slot = 0;
-    auto store = [&](const double *best, const uint32_t *idx) {
-        const size_t rbase = (static_cast<size_t>(trel) * p.n_seg + slot) * p.n_pairs + row;
+    // partial results, one row per (table, strategy slot, (m, chunk) pair), P contiguous; the warps that shared a tile of
+    // process counts hand over the smallest (time, s) of theirs
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int pidx = p_first + 32 * r;
-            if (pidx < p.G.n_P) {
-                p.part_time[rbase * p.G.n_P + pidx] = best[r];
-                p.part_idx[rbase * p.G.n_P + pidx] = idx[r];
+    for (int q = 0; q < kNid; ++q) {
+        const int slot = IS9 ? p.n_seg - 1 : q;
+        const size_t rbase = (static_cast<size_t>(trel) * p.n_seg + slot) * p.n_pairs + row;
+        for (int i = tid; i < wp * 32 * R; i += kThreads) {
+            const int pidx = ptile * wp * 32 * R + i;
+            if (pidx >= p.G.n_P) break;
+            double bt = s_best[q * kIdStep + i];
+            uint32_t bi = s_idx[q * kIdStep + i];
+            for (int w = 1; w < wc; ++w) {
+                const double t = s_best[q * kIdStep + w * wp * 32 * R + i];
+                const uint32_t e = s_idx[q * kIdStep + w * wp * 32 * R + i];
+                if (t < bt || (t == bt && e < bi)) { bt = t; bi = e; }
             }
+            p.part_time[rbase * p.G.n_P + pidx] = bt;
+            p.part_idx[rbase * p.G.n_P + pidx] = bi;
         }
-        ++slot;
-    };
-    if (HAS2) store(best2, idx2);
-    if (HAS5) store(best5, idx5);
-    if (HAS9) store(best9, idx9);
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -612,34 +707,39 @@ cudaError_t launch_fused(const FusedParams &p, bool predict, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <int SEGMASK>
+template <bool HAS2, bool HAS5, bool IS9>
 static cudaError_t launch_sweep_t(const SweepParams &p, int n_tables_launch, cudaStream_t st)
 {
+    constexpr int n_id = (HAS2 ? 1 : 0) + (HAS5 ? 1 : 0) + (IS9 ? 1 : 0);
     const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double) +
-                        2 * kSweepSub * (sizeof(double2) + sizeof(double));
-    cudaError_t e = set_smem(sweep_kernel<SEGMASK>, smem);
+                        2 * kSweepSub * (sizeof(double2) + sizeof(double) + 3 * sizeof(float)) +
+                        static_cast<size_t>(n_id) * kWarps * kSweepR * 32 * (sizeof(double) + sizeof(uint32_t));
+    cudaError_t e = set_smem(sweep_kernel<HAS2, HAS5, IS9>, smem);
     if (e != cudaSuccess) return e;
     const long long bx = static_cast<long long>(p.n_pairs) * p.n_ptiles;
     if (bx <= 0 || bx > 0x7FFFFFFFLL || n_tables_launch > 65535) return cudaErrorInvalidConfiguration;
     dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(n_tables_launch));
-    sweep_kernel<SEGMASK><<<grid, kThreads, smem, st>>>(p);
+    sweep_kernel<HAS2, HAS5, IS9><<<grid, kThreads, smem, st>>>(p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, cudaStream_t st)
+// Ids 2 and 5 share a launch (one set of coefficients, lines in P); id 9, whose lines are in floor(log2 P), has its own.
+cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st)
 {
-    const uint32_t m = p.G.mask;
-    const int segmask = ((m >> 2) & 1) | (((m >> 5) & 1) << 1) | (((m >> 9) & 1) << 2);
-    switch (segmask) {
-    case 1: return launch_sweep_t<1>(p, n_tables_launch, st);
-    case 2: return launch_sweep_t<2>(p, n_tables_launch, st);
-    case 3: return launch_sweep_t<3>(p, n_tables_launch, st);
-    case 4: return launch_sweep_t<4>(p, n_tables_launch, st);
-    case 5: return launch_sweep_t<5>(p, n_tables_launch, st);
-    case 6: return launch_sweep_t<6>(p, n_tables_launch, st);
-    case 7: return launch_sweep_t<7>(p, n_tables_launch, st);
-    default: return cudaSuccess;
+    const bool has2 = (p.G.mask >> 2) & 1, has5 = (p.G.mask >> 5) & 1, has9 = (p.G.mask >> 9) & 1;
+    cudaError_t e = cudaSuccess;
+    *launches = 0;
+    if (has2 || has5) {
+        e = has2 && has5 ? launch_sweep_t<true, true, false>(p, n_tables_launch, st)
+                         : (has2 ? launch_sweep_t<true, false, false>(p, n_tables_launch, st) : launch_sweep_t<false, true, false>(p, n_tables_launch, st));
+        if (e != cudaSuccess) return e;
+        ++*launches;
     }
+    if (has9) {
+        e = launch_sweep_t<false, false, true>(p, n_tables_launch, st);
+        if (e == cudaSuccess) ++*launches;
+    }
+    return e;
 }
 
 cudaError_t launch_s1_tiles(const S1Params &p, cudaStream_t st)

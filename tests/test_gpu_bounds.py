@@ -1,0 +1,57 @@
+"""GPU parity where the FP32 lower bounds of the segment search decide what is looked at in FP64: tilings of the process
+counts and candidates at their edges, and tables whose times lie far outside FP32's range."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+from paper_cs_0408034_b200 import workloads as wl
+from parity import check_decision, check_prediction, oracle_tables
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def plogp():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_cs_0408034_b200 import plogp as mod
+    return mod
+
+
+def both(plogp, w):
+    """Decision table and predictions of every cell against the oracle (times to 1e-12, picks exact: tests/parity.py)."""
+    import torch
+    ot = oracle_tables(w)
+    with plogp.Tables.from_workload(w) as tabs:
+        dec = plogp.select_best(tabs, w)
+        pred = plogp.predict(tabs, w)
+        torch.cuda.synchronize()
+        assert check_decision(w, ot, dec) + check_prediction(w, ot, pred) > 0
+
+
+@pytest.mark.parametrize("n_P,ids,k_mode", [(1, (2, 5, 9), 0), (31, (5,), 1), (256, (2, 5), 0), (257, (9,), 0), (700, (2, 9), 1),
+                                            (1100, (2, 5, 9), 0), (2049, (0, 2, 5, 7), 0)])
+def test_long_lists_at_the_edges_of_the_process_count_tiles(plogp, n_P, ids, k_mode):
+    """1, 2, 4 and 8 tiles of 256 process counts per CTA (the warps then split the candidates 8, 4, 2 and 1 ways), and a
+    candidate list that ends inside a sub-chunk of 256."""
+    base = wl.config4(n_tables=2, P_hi=n_P + 1, n_m=5, seed_offset=70 + n_P)
+    both(plogp, replace(base, s_list=None, s_lo=4, s_hi=4 * 700, s_step=4, strategy_mask=sum(1 << i for i in ids), k_mode=k_mode))
+
+
+def test_long_list_over_several_chunks(plogp):
+    """A list of 2300 sizes: two chunks of candidates per message size, the optimum in either."""
+    base = wl.config4(n_tables=2, P_hi=90, n_m=4, seed_offset=5)
+    both(plogp, replace(base, m=np.array([4, 3000, 9000, 400000], dtype=np.uint64), s_list=None, s_lo=4, s_hi=9200, s_step=4))
+
+
+@pytest.mark.parametrize("scale", [1e-60, 1e-42, 1e36, 1e60])
+@pytest.mark.parametrize("long_list", [False, True])
+def test_times_outside_the_range_of_fp32(plogp, scale, long_list):
+    """Below FP32's smallest number every bound is 0, above its largest every upper bound is infinite: all cells are
+    then compared in FP64, and the results are the oracle's."""
+    base = wl.config4(n_tables=2, P_hi=300, n_m=6, n_s=24, seed_offset=8)
+    w = replace(base, gaps=base.gaps * scale, latency=base.latency * scale)
+    if long_list:
+        w = replace(w, P_hi=70, s_list=None, s_lo=4, s_hi=4 * 300, s_step=4)
+    both(plogp, w)
