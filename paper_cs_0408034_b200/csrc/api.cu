@@ -46,6 +46,9 @@ int ceil_log2(int64_t P)
     return e;
 }
 
+// 2 floor(log2 P) + (P is no power of two): numbers the (floor, ceil) pairs in the order of P
+int log2_pair(int64_t P) { return 2 * ceil_log2(P) - ((P & (P - 1)) ? 1 : 0); }
+
 // Everything derived from a grid that the launches need; cached on the handle while the same
 // grid keeps being passed.
 struct Plan {
@@ -63,7 +66,7 @@ struct Plan {
     // and an unsplit range needs no tile sums, i.e. one launch less)
     int sc_ptiles = 1, sc_passes_per_tile = 1;
     // decision kernel tiling (short candidate lists)
-    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG;
+    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_pairs = 1;
     size_t carry_bytes_per_table = 0;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
@@ -290,6 +293,11 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
     while (pl.dec_mg > kDecWarps && (long long)((n_m + pl.dec_mg - 1) / pl.dec_mg) * pl.dec_ptiles * h->T.n_tables < (long long)h->sm_count * 4)
         pl.dec_mg >>= 1;
     pl.dec_mgroups = (n_m + pl.dec_mg - 1) / pl.dec_mg;
+    for (int t = 0; t < pl.dec_ptiles; ++t) {
+        const int first = t * kDecTileP, last = std::min(n_P, first + kDecTileP) - 1;
+        const int64_t P0 = g->P ? g->P[first] : int64_t(g->P_lo) + first, P1 = g->P ? g->P[last] : int64_t(g->P_lo) + last;
+        pl.dec_pairs = std::max(pl.dec_pairs, log2_pair(P1) - log2_pair(P0) + 1);
+    }
 
     // ---- device arrays ----
     std::vector<unsigned char> blob;
@@ -527,7 +535,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             DecideParams dp{};
             dp.T = h->T; dp.G = pl.G;
             dp.G.mask &= 0x3FFu;
-            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg;
+            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.n_pairs = pl.dec_pairs;
             dp.table0 = t0; dp.n_tables_launch = nt; dp.out_table0 = out.out_table0; dp.om = out.om;
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
             dp.envelope = pl.envelope_short ? 1 : 0;

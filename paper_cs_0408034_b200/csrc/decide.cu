@@ -7,27 +7,27 @@
 // sizes, so a warp runs on its own from the candidate lists to the staged result and only the
 // write-out needs the whole CTA.
 //
-// Every model of Table 1 is, for a fixed message size (and segment size), a line in P or in
-// floor(log2 P):
-//     ids 0 1 2 3 4 5:  t = fma(P-1, a, c)           "P list", entries (a, c)
-//     ids 7 9:          t = fma(floor(log2 P), a, ceil(log2 P) L)   "log list", entries a
-//     ids 6 8:          one cell each, evaluated on their own
+// Every model of Table 1 is, for a fixed message size (and segment size), a line in P or a function of
+// floor(log2 P) and ceil(log2 P) alone:
+//     ids 0 1 2 3 4 5:  t = fma(P-1, a, c)
+//     ids 6 7 8 9:      constant while (floor, ceil) stays, i.e. between a power of two and the next
 // The decision is the lexicographic minimum of (t, id, s) over all cells of all enabled strategies
-// (the minimum over s inside a strategy and then over strategies, smallest s and lowest id on
-// ties), so one running minimum per process count serves the whole search.  A warp builds the two
-// lists of a message size in shared memory (lanes <-> candidates), guesses the winner at the
-// process count in the middle of its range (the pilot), starts the running minimum from the
-// pilot's cells and takes the pilot out of its list.  Then every cell is evaluated with one DFMA
-// and compared with the running minimum on the high 32 bits only, in the integer pipe (times are
-// non-negative, so a smaller double never has a larger high word); a group of four list entries in
-// which some cell can reach the minimum is re-evaluated with the exact FP64 comparison, for the
-// eight-cell rows that need it.  With a good pilot that is rare.
+// (the minimum over s inside a strategy and then over strategies, smallest s and lowest id on ties).
+// A warp numbers the cells of a message size in exactly that order: "slots" [lines of ids 0, 1, 2, 3, 4, 5]
+// [one per (floor, ceil) pair of the tile], each with its coefficients (a, c) in shared memory (a pair's slot is
+// (0, its smallest time)), so that a decision is a slot number and equal times go to the smaller one.
 //
-// Once started, the running minima (time and winner code) live in shared memory as [m][P], which is
-// also the staging layout of the write-out: the loops keep only minus their high words in registers,
-// the exact pass reads and writes the minima themselves.  The codes carry the strategy ids as the
-// caller names them (OutMap::id_of keeps their order), so the write-out, rows of consecutive m per
-// process count, only has to split a code into its id and its segment size.
+// Per message size:
+//   1. lanes <-> candidates: the lines' coefficients, in FP64 and rounded down to FP32; the pilot, the line that is
+//      best at the tile's middle process count.
+//   2. lanes <-> (floor, ceil) pairs: the best of ids 6 to 9 in FP64, one candidate after another.
+//   3. per process count the better of the pilot and its pair: the running minimum's start.
+//   4. every cell of every other line as a lower bound: FP32 coefficients, process count and fused multiply-add all
+//      rounded down, two lines per instruction; the smallest bound per process count is compared with the running
+//      minimum rounded up.  All terms are non-negative, so the bound is never above the FP64 time.
+//   5. only rows of 32 process counts in which some bound is not above (1.4 of 8 on average) are searched exactly.
+// Results are those of the exhaustive FP64 search, bit for bit.  Staged as slot numbers [m][P] (1 byte); the write-out,
+// rows of consecutive m per process count, evaluates the winner's line again (the same fma, the same double).
 #include "device_common.cuh"
 
 #include <algorithm>
@@ -36,73 +36,67 @@ namespace plogp {
 
 namespace {
 
-constexpr int R = kDecR, U = kDecU;
+constexpr int R = kDecR;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kStageStride = kDecTileP + 1;  // doubles per staged row: the transposed reads stay conflict-free
-constexpr int kCodeStride = kDecTileP + 2;   // 16-bit codes per staged row, for the same reason
-
+constexpr int kPosStride = kDecTileP + 4;    // bytes per staged row
 constexpr uint32_t kCandNone = 255;   // winner is an unsegmented strategy
 constexpr uint32_t kCandWhole = 254;  // segmented winner with no fitting candidate: the whole message
-constexpr uint32_t kCodeNever = 0xFFFFu;
 constexpr unsigned kNoPilot = 0x1FFu;
 constexpr int kIntMax = 0x7FFFFFFF;
+constexpr int kPairBlock = 16;  // (floor, ceil) pairs per pass: half a warp, the halves split the candidates
 
 struct DecSmem {
-    double *tab, *gs, *gm, *lf, *lc, *pm1, *l2, *st_time;
-    double2 *l1;
+    double *tab, *gs, *gm, *pm1;
+    double2 *line;    // [kDecMG][slots]: coefficients by slot
+    float *fa, *fc;   // [kDecWarps][cap]: the lines' coefficients rounded down, for the warp's current message size
+    double *q;        // [kDecWarps][n_s]: g(s) k, for the warp's current message size
     uint32_t *sval;   // [256]: segment sizes by candidate index; [kCandNone] = 0
-    uint16_t *c1, *c2, *st_code;
-    int cap1, cap2;
+    uint16_t *code;   // [kDecMG][slots]: id << 8 | candidate index
+    uint8_t *pair, *pos;  // [kDecTileP]: pair of a process count; [kDecMG][kPosStride]: winners
+    int cap, slots;
 };
 
 __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
-// Shared-memory layout.  cap1 / cap2: entries of one warp's P list / log list (multiples of U).
-__host__ __device__ inline size_t dec_layout(int npad, int n_s, unsigned char *base, DecSmem *o)
+// Shared-memory layout.  cap: lines of one message size (a multiple of 4); n_pairs: (floor, ceil) pairs of a tile at most.
+// A slot number fits a byte: at most 4 + 2 * 64 lines and 61 pairs.
+__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap1 = round_up(2 * nsv + 4, U), cap2 = round_up(nsv + 1, U);
+    const int cap = round_up(2 * nsv + 4, 4), slots = cap + n_pairs;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
-    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_sv = take(256 * 4),
-                 o_gm = take(kDecMG * 8), o_lf = take(kDecTileP * 8), o_lc = take(kDecTileP * 8), o_pm = take(kDecTileP * 8),
-                 o_l1 = take(size_t(kDecWarps) * cap1 * 16), o_l2 = take(size_t(kDecWarps) * cap2 * 8),
-                 o_c1 = take(size_t(kDecWarps) * cap1 * 2), o_c2 = take(size_t(kDecWarps) * cap2 * 2),
-                 o_t = take(size_t(kDecMG) * kStageStride * 8), o_c = take(size_t(kDecMG) * kCodeStride * 2);
+    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(kDecTileP * 8),
+                 o_line = take(size_t(kDecMG) * slots * 16), o_fa = take(size_t(kDecWarps) * cap * 4), o_fc = take(size_t(kDecWarps) * cap * 4),
+                 o_q = take(size_t(kDecWarps) * nsv * 8), o_sv = take(256 * 4), o_code = take(size_t(kDecMG) * slots * 2),
+                 o_pair = take(kDecTileP), o_pos = take(size_t(kDecMG) * kPosStride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
-        o->sval = reinterpret_cast<uint32_t *>(base + o_sv); o->gm = reinterpret_cast<double *>(base + o_gm);
-        o->lf = reinterpret_cast<double *>(base + o_lf); o->lc = reinterpret_cast<double *>(base + o_lc);
-        o->pm1 = reinterpret_cast<double *>(base + o_pm);
-        o->l1 = reinterpret_cast<double2 *>(base + o_l1); o->l2 = reinterpret_cast<double *>(base + o_l2);
-        o->c1 = reinterpret_cast<uint16_t *>(base + o_c1); o->c2 = reinterpret_cast<uint16_t *>(base + o_c2);
-        o->st_time = reinterpret_cast<double *>(base + o_t); o->st_code = reinterpret_cast<uint16_t *>(base + o_c);
-        o->cap1 = cap1; o->cap2 = cap2;
+        o->gm = reinterpret_cast<double *>(base + o_gm); o->pm1 = reinterpret_cast<double *>(base + o_pm);
+        o->line = reinterpret_cast<double2 *>(base + o_line);
+        o->fa = reinterpret_cast<float *>(base + o_fa); o->fc = reinterpret_cast<float *>(base + o_fc);
+        o->q = reinterpret_cast<double *>(base + o_q); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
+        o->code = reinterpret_cast<uint16_t *>(base + o_code); o->pair = base + o_pair; o->pos = base + o_pos;
+        o->cap = cap; o->slots = slots;
     }
     return off;
 }
 
 __device__ __forceinline__ int hi32(double x) { return __double2hiint(x); }
 
-// Exact comparison of one cell with the running minimum: (time, code) in lexicographic order, where the code
-// orders strategy id first and candidate index (= segment size order) second.
-__device__ __forceinline__ void offer(double &bt, uint32_t &bcode, double t, uint32_t code)
-{
-    if (t <= bt) {
-        if (t < bt || code < bcode) { bt = t; bcode = code; }
-    }
-}
+// (floor, ceil) of log2 P as one number that grows with P: 2 floor + (P is no power of two)
+__device__ __forceinline__ int pair_of(int P) { return 2 * (31 - __clz(P)) + ((P & (P - 1)) != 0 ? 1 : 0); }
 
 }  // namespace
 
 // ENV: lower-envelope search (DecideParams::envelope), compiled apart so that the exhaustive kernel carries none of it.
 template <bool ENV>
-__global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecideParams p)
+__global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecideParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
     DecSmem sm;
-    dec_layout(npad, p.G.n_s, smem_raw, &sm);
+    dec_layout(npad, p.G.n_s, p.n_pairs, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
 
     int b = blockIdx.x;
@@ -116,16 +110,15 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
     const int n_mi = min(p.mg, p.G.n_m - m0);
     const int tile0 = ptile * kDecTileP;
     const int n_valid = min(kDecTileP, p.G.n_P - tile0);
+    const int pair0 = pair_of(P_at(p.G, tile0)), n_pairs = pair_of(P_at(p.G, tile0 + n_valid - 1)) - pair0 + 1;
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
     if (!grow) stage_table(sm.tab, p.T, table);
-    // floor(log2 P) and ceil(log2 P) of the tile's process counts, as doubles
     for (int i = tid; i < kDecTileP; i += kDecThreads) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
-        sm.lf[i] = static_cast<double>(31 - __clz(P));
-        sm.lc[i] = static_cast<double>(32 - __clz(P - 1));
         sm.pm1[i] = static_cast<double>(P - 1);
+        sm.pair[i] = static_cast<uint8_t>(min(pair_of(P) - pair0, n_pairs - 1));
     }
     __syncthreads();
     const double L = p.T.lat[table];
@@ -143,33 +136,28 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
     const double rdv = 2.0 * g1 + 3.0 * L;  // rendezvous handshake: 2 g(1) + 3 L
     __syncthreads();
 
-    // this thread's cells: process counts at tile offset 32 r + lane; P-1, floor(log2 P) and ceil(log2 P) are read
-    // from shared memory where a loop needs them, so that only one of the sets is live at a time
     // the pilot's process count: middle of the tile's valid range
-    const int P_mid = P_at(p.G, tile0 + n_valid / 2);
-    const double x1_mid = static_cast<double>(P_mid - 1);
-    const double x2_mid = static_cast<double>(31 - __clz(P_mid));
-    const double c2_mid = static_cast<double>(32 - __clz(P_mid - 1)) * L;
+    const double x_mid = sm.pm1[n_valid / 2];
+    f32x2 x2[R];  // this lane's process counts less one, rounded down, twice each
+#pragma unroll
+    for (int r = 0; r < R; ++r) x2[r] = splat2(__double2float_rd(sm.pm1[32 * r + lane]));
 
-    // the codes carry the strategy ids as the caller names them (the relabelling keeps their order)
+    // the codes carry the strategy ids as the caller names them
     auto idc = [&](int id) { return static_cast<uint32_t>(p.om.id_of[id]) << 8; };
     const uint32_t code2 = idc(2), code5 = idc(5), code9 = idc(9);
-    const uint32_t un = mask & 0x1Bu;  // unsegmented members of the P list: ids 0, 1, 3, 4
-    const int n_un = __popc(un);
     const bool has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has6 = (mask >> 6) & 1u, has7 = (mask >> 7) & 1u,
                has8 = (mask >> 8) & 1u, has9 = (mask >> 9) & 1u;
-    // The unsegmented members of the lists do not depend on the message size beyond g(m): lanes 0..3 hold ids 0, 1, 3, 4
-    // (Flat Tree (P-1) g + L, its rendezvous form (P-1) g + rdv; Chain (P-1)(g + L), rendezvous (P-1)(g + rdv)) as
-    // P-list entries (g(m) + fa, fc), lane 4 the Binomial Tree's log-list entry g(m).
-    const int fid = lane < 4 ? lane + (lane >> 1) : 7;
-    const bool f_on = lane < 5 && ((mask >> fid) & 1u);
-    const int fpos = __popc(un & ((1u << fid) - 1u));
+    const bool any_log = mask & 0x3C0u;
+    // The unsegmented lines do not depend on the message size beyond g(m): lanes 0..3 hold ids 0, 1, 3, 4
+    // (Flat Tree (P-1) g + L, its rendezvous form (P-1) g + rdv; Chain (P-1)(g + L), rendezvous (P-1)(g + rdv)) as (g(m) + fa, fc).
+    const int n01 = __popc(mask & 3u), n34 = __popc(mask & 0x18u);
+    const int fid = lane < 4 ? lane + (lane >> 1) : 0;
+    const bool f_on = lane < 4 && ((mask >> fid) & 1u);
     const double fa = fid == 3 ? L : (fid == 4 ? rdv : 0.0);
     const double fc = fid == 0 ? L : (fid == 1 ? rdv : 0.0);
     const uint16_t fcode = static_cast<uint16_t>(idc(fid) | kCandNone);
-    double2 *l1 = sm.l1 + warp * sm.cap1;
-    double *l2 = sm.l2 + warp * sm.cap2;
-    uint16_t *c1 = sm.c1 + warp * sm.cap1, *c2 = sm.c2 + warp * sm.cap2;
+    float *const la = sm.fa + warp * sm.cap, *const lc = sm.fc + warp * sm.cap;
+    double *const lq = sm.q + warp * max(p.G.n_s, 1);
 
     for (int mi = warp; mi < n_mi; mi += kDecWarps) {
         const int midx = m0 + mi;
@@ -177,6 +165,8 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
         const double gm = sm.gm[mi];
         const double *krow = p.G.k_list + static_cast<size_t>(midx) * p.G.n_s;
+        double2 *const line = sm.line + mi * sm.slots;
+        uint16_t *const code = sm.code + mi * sm.slots;
         // Lower-envelope search (p.envelope, tables whose gaps never decrease): ids 2 and 9 keep only the candidate
         // with the smallest g(s) k (their minimum over s for every P at once, a rounded fused multiply-add being
         // monotone in it), id 5 only the candidates between its winners at the tile's last and first process
@@ -204,35 +194,25 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
             n5 = min(max(ef, el) + 1, ns - 1) - lo5 + 1;
         }
         const int nq = env ? 1 : nsv;  // entries of ids 2 and 9
-        const int o2 = n_un, o5 = o2 + (has2 ? nq : 0), n1 = o5 + (has5 ? n5 : 0);
-        const int o9 = has7 ? 1 : 0, n2 = o9 + (has9 ? nq : 0);
-        const int n1p = round_up(n1, U), n2p = round_up(n2, U);
+        const int o2 = n01, o3 = o2 + (has2 ? nq : 0), o5 = o3 + n34, n1 = o5 + (has5 ? n5 : 0);
+        const int n1p = round_up(n1, 4);
 
-        // ---- the two lists of this message size, and each lane's best entry at the pilot's process count ----
-        __syncwarp();  // the previous message size's loops have finished reading the lists
+        // ---- the lines of this message size, and each lane's best one at the pilot's process count ----
+        __syncwarp();  // the previous message size's loops have finished reading the warp's lists
         double tb = CUDART_INF;
-        unsigned pb = kNoPilot;  // P-list position, or 256 + log-list position
-        auto pilot_offer = [&](double t, unsigned pos) {
-            if (t < tb) { tb = t; pb = pos; }
+        unsigned pb = kNoPilot;
+        auto put = [&](int slot, double a, double c, uint32_t cd) {
+            line[slot] = make_double2(a, c);
+            la[slot] = __double2float_rd(a);
+            lc[slot] = __double2float_rd(c);
+            code[slot] = static_cast<uint16_t>(cd);
+            const double t = fma(x_mid, a, c);
+            if (t < tb || pb == kNoPilot) { tb = t; pb = static_cast<unsigned>(slot); }
         };
-        if (f_on) {  // this lane's unsegmented strategy
-            if (lane < 4) {
-                l1[fpos] = make_double2(gm + fa, fc);
-                c1[fpos] = fcode;
-                pilot_offer(fma(x1_mid, gm + fa, fc), fpos);
-            } else {
-                l2[0] = gm;
-                c2[0] = fcode;
-                pilot_offer(fma(x2_mid, gm, c2_mid), 256u);
-            }
-        }
-        for (int i = n1 + lane; i < n1p; i += 32) {  // padding never reaches the minimum
-            l1[i] = make_double2(CUDART_INF, CUDART_INF);
-            c1[i] = static_cast<uint16_t>(kCodeNever);
-        }
-        for (int i = n2 + lane; i < n2p; i += 32) {
-            l2[i] = CUDART_INF;
-            c2[i] = static_cast<uint16_t>(kCodeNever);
+        if (f_on) put((fid < 3 ? 0 : o3 - n01) + __popc(mask & 0x1Bu & ((1u << fid) - 1u)), gm + fa, fc, fcode);
+        if (lane >= 28 && n1 + lane - 28 < n1p) {  // padding: the bound is +inf
+            la[n1 + lane - 28] = 0.0f;
+            lc[n1 + lane - 28] = CUDART_INF_F;
         }
         for (int c = lane; c < nsv; c += 32) {
             // Section 2's k and the line coefficients of Table 1's segmented rows
@@ -244,222 +224,182 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
                 cand = static_cast<uint32_t>(c);
             }
             const double Q = gsv * k;
-            const bool in_q = !env || c == q_c, in_5 = !env || (c >= lo5 && c < lo5 + n5);
-            const int pq = env ? 0 : c, p5 = env ? c - lo5 : c;  // positions inside the strategies' parts of the lists
-            if (has2 && in_q) {  // (P-1) (g(s) k) + L
-                l1[o2 + pq] = make_double2(Q, L);
-                c1[o2 + pq] = static_cast<uint16_t>(code2 | cand);
-                pilot_offer(fma(x1_mid, Q, L), o2 + pq);
-            }
-            if (has5 && in_5) {  // (P-1) (g(s) + L) + g(s) (k-1)
-                const double B = gsv + L, C = gsv * (k - 1.0);
-                l1[o5 + p5] = make_double2(B, C);
-                c1[o5 + p5] = static_cast<uint16_t>(code5 | cand);
-                pilot_offer(fma(x1_mid, B, C), o5 + p5);
-            }
-            if (has9 && in_q) {  // floor(log2 P) g(s) k + ceil(log2 P) L
-                l2[o9 + pq] = Q;
-                c2[o9 + pq] = static_cast<uint16_t>(code9 | cand);
-                pilot_offer(fma(x2_mid, Q, c2_mid), 256u + o9 + pq);
-            }
+            lq[c] = Q;
+            if (has2 && (!env || c == q_c)) put(o2 + (env ? 0 : c), Q, L, code2 | cand);  // (P-1) (g(s) k) + L
+            if (has5 && (!env || (c >= lo5 && c < lo5 + n5)))                             // (P-1) (g(s) + L) + g(s) (k-1)
+                put(o5 + (env ? c - lo5 : c), gsv + L, gsv * (k - 1.0), code5 | cand);
         }
-        // warp-wide pilot: smallest time (high word first, then low word with the position in its last 9 bits)
+        // warp-wide pilot: smallest time (high word first, then low word with the slot in its last 9 bits)
         const int hmin = __reduce_min_sync(kFull, hi32(tb));
         const unsigned k2 = hi32(tb) == hmin ? ((static_cast<unsigned>(__double2loint(tb)) & ~0x1FFu) | pb) : 0xFFFFFFFFu;
         const unsigned pilot = __reduce_min_sync(kFull, k2) & 0x1FFu;
         __syncwarp();
 
-        double lf[R], lcL[R];  // floor(log2 P); ceil(log2 P), later ceil(log2 P) L
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            lf[r] = sm.lf[32 * r + lane];
-            lcL[r] = sm.lc[32 * r + lane];
+        // ---- the best of ids 6 to 9 per (floor, ceil) pair ----
+        if (any_log)
+        for (int b0 = 0; b0 < n_pairs; b0 += kPairBlock) {
+            const int pr = b0 + (lane & (kPairBlock - 1)), half = lane / kPairBlock;
+            const int li = pair0 + pr;
+            const double lf = static_cast<double>(li >> 1), lcd = static_cast<double>((li >> 1) + (li & 1)), lcL = lcd * L;
+            double t = CUDART_INF;
+            uint32_t cd = 0;
+            if (has9) {  // floor(log2 P) g(s) k + ceil(log2 P) L; the half-warps take every other candidate
+                double tc = CUDART_INF;
+                int cb = 0x1000;
+                if (env) {
+                    tc = fma(lf, lq[q_c], lcL);
+                    cb = q_c;
+                } else {
+#pragma unroll 4
+                    for (int c = half; c < nsv; c += 2) {
+                        const double v = fma(lf, lq[c], lcL);
+                        if (v < tc) { tc = v; cb = c; }
+                    }
+                    const double t2 = __shfl_xor_sync(kFull, tc, kPairBlock);
+                    const int cb2 = __shfl_xor_sync(kFull, cb, kPairBlock);
+                    if (t2 < tc || (t2 == tc && cb2 < cb)) { tc = t2; cb = cb2; }
+                }
+                t = tc;
+                cd = code9 | (ns > 0 ? static_cast<uint32_t>(min(cb, ns - 1)) : kCandWhole);
+            }
+            // lower ids win ties: in descending order, '<='
+            if (has8) {  // Binomial Tree Rendezvous: floor(log2 P) g(m) + ceil(log2 P) rdv
+                const double v = fma(lf, gm, lcd * rdv);
+                if (v <= t) { t = v; cd = idc(8) | kCandNone; }
+            }
+            if (has7) {  // Binomial Tree: floor(log2 P) g(m) + ceil(log2 P) L
+                const double v = fma(lf, gm, lcL);
+                if (v <= t) { t = v; cd = idc(7) | kCandNone; }
+            }
+            if (has6) {  // Binary Tree (the printed bound): ceil(log2 P) (2 g(m) + L)
+                const double v = lcd * fma(2.0, gm, L);
+                if (v <= t) { t = v; cd = idc(6) | kCandNone; }
+            }
+            if (half == 0 && pr < n_pairs) {
+                line[sm.cap + pr] = make_double2(0.0, t);
+                code[sm.cap + pr] = static_cast<uint16_t>(cd);
+            }
         }
 
-        // ---- running minimum per process count, started from the pilot's cells ----
-        double bt[R];
-        uint32_t bcode[R];  // strategy id << 8 | candidate index (or kCandNone / kCandWhole)
-        if (pilot == kNoPilot) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) { bt[r] = CUDART_INF; bcode[r] = kCodeNever; }
-        } else if (pilot < 256u) {
-            const double2 e = l1[pilot];
-            const uint32_t code = c1[pilot];
-            __syncwarp();
-            if (lane == 0) l1[pilot] = make_double2(CUDART_INF, CUDART_INF);
-#pragma unroll
-            for (int r = 0; r < R; ++r) { bt[r] = fma(sm.pm1[32 * r + lane], e.x, e.y); bcode[r] = code; }
-        } else {
-            const double a = l2[pilot - 256u];
-            const uint32_t code = c2[pilot - 256u];
-            __syncwarp();
-            if (lane == 0) l2[pilot - 256u] = CUDART_INF;
-#pragma unroll
-            for (int r = 0; r < R; ++r) { bt[r] = fma(lf[r], a, lcL[r] * L); bcode[r] = code; }
+        // ---- start of the running minima: the pilot or the pair ----
+        double2 e = make_double2(0.0, CUDART_INF);
+        if (pilot != kNoPilot) {
+            e = line[pilot];
+            if (lane == 0) { la[pilot] = 0.0f; lc[pilot] = CUDART_INF_F; }  // its own bounds would always pass
         }
         __syncwarp();
-
-        // one cell per process count (ids 6 and 8): high-word test, exact comparison where it holds
-        auto single = [&](uint32_t code, const double *t) {
-            int acc = kIntMax;
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc = min(acc, hi32(t[r]) - hi32(bt[r]));
-            if (acc <= 0) {
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-                    if (t[r] < bt[r] || (t[r] == bt[r] && code < bcode[r])) { bt[r] = t[r]; bcode[r] = code; }
-            }
-        };
-        if (has6) {  // Binary Tree (the printed bound): ceil(log2 P) (2 g(m) + L)
-            const double w = fma(2.0, gm, L);
-            double t[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) t[r] = lcL[r] * w;
-            single(idc(6) | kCandNone, t);
-        }
-        if (has8) {  // Binomial Tree Rendezvous: floor(log2 P) g(m) + ceil(log2 P) rdv
-            double t[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) t[r] = fma(lf[r], gm, lcL[r] * rdv);
-            single(idc(8) | kCandNone, t);
-        }
-        // from here on the running minima live in shared memory (the staging area of the write-out): the loops only need
-        // minus their high words, and only the exact pass touches the minima themselves.  (The plain add-then-min form
-        // below is left to the compiler on purpose: it splits the work between two pipes and measured faster than the
-        // fused add-min instruction.)
-        double *st = sm.st_time + mi * kStageStride + lane;
-        uint16_t *sc = sm.st_code + mi * kCodeStride + lane;
-        int nhb[R];
+        uint8_t *const pos = sm.pos + mi * kPosStride + lane;
+        float T[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            lcL[r] *= L;
-            nhb[r] = -hi32(bt[r]);
-            st[32 * r] = bt[r];
-            sc[32 * r] = static_cast<uint16_t>(bcode[r]);
+            double t = fma(sm.pm1[32 * r + lane], e.x, e.y);
+            unsigned at = pilot;
+            if (any_log) {
+                const unsigned slot = sm.cap + sm.pair[32 * r + lane];
+                const double tl = line[slot].y;
+                if (tl < t || pilot == kNoPilot) { t = tl; at = slot; }  // lines have the lower ids
+            }
+            T[r] = __double2float_ru(t);
+            pos[32 * r] = static_cast<uint8_t>(at);
         }
 
-        // The filter of a group of U list entries: every cell is evaluated (one DFMA each); per process
-        // count the smallest high word of the U times minus the high word of the running minimum says
-        // whether a cell can reach it (<= 0), and the differences of all R process counts are folded into
-        // one minimum, so the test costs integer min / add instructions only (no predicates, no branches)
-        // and a single vote decides whether the group needs the exact pass.  The exact pass, (time, id,
-        // candidate) in lexicographic order, runs for the rows r that some lane flagged.
+        // ---- lower bounds of all other lines ----
+        float mn[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) mn[r] = CUDART_INF_F;
+#pragma unroll 2
+        for (int j = 0; j < n1p; j += 4) {
+            const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
+#pragma unroll
+            for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], aa.x, cc.x));
+#pragma unroll
+            for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], aa.y, cc.y));
+        }
+        unsigned hit = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (mn[r] <= T[r] && mn[r] < CUDART_INF_F) hit |= 1u << r;
 
-        // ---- log list: t = fma(floor(log2 P), a, ceil(log2 P) L) ----
+        // ---- exact search of the rows in which some bound is not above the running minimum ----
 #pragma unroll 1
-        for (int j = 0; j < n2p; j += U) {
-            const double2 q01 = *reinterpret_cast<const double2 *>(l2 + j), q23 = *reinterpret_cast<const double2 *>(l2 + j + 2);
-            int acc = kIntMax;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int h0 = hi32(fma(lf[r], q01.x, lcL[r])), h1 = hi32(fma(lf[r], q01.y, lcL[r]));
-                const int h2 = hi32(fma(lf[r], q23.x, lcL[r])), h3 = hi32(fma(lf[r], q23.y, lcL[r]));
-                acc = min(acc, min(min(h0, h1), min(h2, h3)) + nhb[r]);
-            }
-            if (__any_sync(kFull, acc <= 0)) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int h0 = hi32(fma(lf[r], q01.x, lcL[r])), h1 = hi32(fma(lf[r], q01.y, lcL[r]));
-                    const int h2 = hi32(fma(lf[r], q23.x, lcL[r])), h3 = hi32(fma(lf[r], q23.y, lcL[r]));
-                    if (__any_sync(kFull, min(min(h0, h1), min(h2, h3)) + nhb[r] <= 0)) {
-                        double b = st[32 * r];
-                        uint32_t code = sc[32 * r];
+        for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
+            const int r = __ffs(rows) - 1;
+            const double x = sm.pm1[32 * r + lane];
+            const f32x2 xx = splat2(__double2float_rd(x));
+            unsigned at = pos[32 * r];
+            const double2 w = line[at];
+            double t = fma(x, w.x, w.y);
+            float Tr = __double2float_ru(t);
 #pragma unroll 1
-                        for (int u = 0; u < U; ++u) offer(b, code, fma(lf[r], l2[j + u], lcL[r]), c2[j + u]);
-                        st[32 * r] = b;
-                        sc[32 * r] = static_cast<uint16_t>(code);
-                        nhb[r] = -hi32(b);
+            for (int j = 0; j < n1p; j += 4) {
+                const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
+                const float low = min_with2(min_with2(CUDART_INF_F, fma2_down(xx, aa.x, cc.x)), fma2_down(xx, aa.y, cc.y));
+                if (__any_sync(kFull, low <= Tr)) {
+#pragma unroll 1
+                    for (int u = j; u < min(j + 4, n1); ++u) {
+                        const double2 v = line[u];
+                        const double tt = fma(x, v.x, v.y);
+                        if (tt <= t && (tt < t || static_cast<unsigned>(u) < at)) { t = tt; at = static_cast<unsigned>(u); }
                     }
+                    Tr = __double2float_ru(t);
                 }
             }
+            pos[32 * r] = static_cast<uint8_t>(at);
         }
-
-        // ---- P list: t = fma(P-1, a, c) ----
-        double pm1[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) pm1[r] = sm.pm1[32 * r + lane];
-#pragma unroll 1
-        for (int j = 0; j < n1p; j += U) {
-            const double2 e0 = l1[j], e1 = l1[j + 1], e2 = l1[j + 2], e3 = l1[j + 3];
-            int acc = kIntMax;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int h0 = hi32(fma(pm1[r], e0.x, e0.y)), h1 = hi32(fma(pm1[r], e1.x, e1.y));
-                const int h2 = hi32(fma(pm1[r], e2.x, e2.y)), h3 = hi32(fma(pm1[r], e3.x, e3.y));
-                acc = min(acc, min(min(h0, h1), min(h2, h3)) + nhb[r]);
-            }
-            if (__any_sync(kFull, acc <= 0)) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const int h0 = hi32(fma(pm1[r], e0.x, e0.y)), h1 = hi32(fma(pm1[r], e1.x, e1.y));
-                    const int h2 = hi32(fma(pm1[r], e2.x, e2.y)), h3 = hi32(fma(pm1[r], e3.x, e3.y));
-                    if (__any_sync(kFull, min(min(h0, h1), min(h2, h3)) + nhb[r] <= 0)) {
-                        double b = st[32 * r];
-                        uint32_t code = sc[32 * r];
-#pragma unroll 1
-                        for (int u = 0; u < U; ++u) {
-                            const double2 e = l1[j + u];
-                            offer(b, code, fma(pm1[r], e.x, e.y), c1[j + u]);
-                        }
-                        st[32 * r] = b;
-                        sc[32 * r] = static_cast<uint16_t>(code);
-                        nhb[r] = -hi32(b);
-                    }
-                }
-            }
-        }
-
     }
     __syncthreads();
 
     // transposed write-out of the staged group: rows of p.mg consecutive m per process count, running pointers
+    const size_t plane = static_cast<size_t>(p.G.n_P) * p.G.n_m;
+    const size_t base = (static_cast<size_t>(table - p.out_table0) * p.om.planes + p.om.plane_bcast) * plane + static_cast<size_t>(tile0) * p.G.n_m + m0;
     if (p.vec_out) {
         // two message sizes per lane: 16-byte, 8-byte and 2-byte stores (the host has checked the alignment)
         const int half = p.mg >> 1;
         const int mi = 2 * (lane & (half - 1)), rows = 32 / half, pr0 = warp * rows + lane / half, prs = kDecWarps * rows;
         if (mi < n_mi) {
             const uint32_t m_u0 = p.G.m_list[m0 + mi], m_u1 = p.G.m_list[m0 + mi + 1];
-            const size_t plane = static_cast<size_t>(p.G.n_P) * p.G.n_m;
-            const size_t o = (static_cast<size_t>(table - p.out_table0) * p.om.planes + p.om.plane_bcast) * plane +
-                             static_cast<size_t>(tile0 + pr0) * p.G.n_m + static_cast<size_t>(m0 + mi);
+            const size_t o = base + static_cast<size_t>(pr0) * p.G.n_m + mi;
             const size_t step = static_cast<size_t>(prs) * p.G.n_m;
             double *out_t = p.d_time + o;
             uint32_t *out_s = p.d_sbytes + o;
             uint8_t *out_id = p.d_strategy + o;
-            const double *st0 = sm.st_time + mi * kStageStride + pr0, *st1 = st0 + kStageStride;
-            const uint16_t *sc0 = sm.st_code + mi * kCodeStride + pr0, *sc1 = sc0 + kCodeStride;
+            const double2 *l0 = sm.line + mi * sm.slots, *l1 = l0 + sm.slots;
+            const uint16_t *c0 = sm.code + mi * sm.slots, *c1 = c0 + sm.slots;
+            const uint8_t *p0 = sm.pos + mi * kPosStride + pr0, *p1 = p0 + kPosStride;
+            const double *px = sm.pm1 + pr0;
             for (int pr = pr0; pr < n_valid; pr += prs) {
-                const uint32_t code0 = *sc0, code1 = *sc1;
+                const unsigned at0 = *p0, at1 = *p1;
+                const double x = *px;
+                const double2 e0 = l0[at0], e1 = l1[at1];
+                const uint32_t code0 = c0[at0], code1 = c1[at1];
                 const uint32_t cand0 = code0 & 255u, cand1 = code1 & 255u;
                 uint32_t s0 = sm.sval[cand0], s1 = sm.sval[cand1];
                 if (cand0 == kCandWhole) s0 = m_u0;
                 if (cand1 == kCandWhole) s1 = m_u1;
-                *reinterpret_cast<double2 *>(out_t) = make_double2(*st0, *st1);
+                *reinterpret_cast<double2 *>(out_t) = make_double2(fma(x, e0.x, e0.y), fma(x, e1.x, e1.y));
                 *reinterpret_cast<uint2 *>(out_s) = make_uint2(s0, s1);
                 *reinterpret_cast<uint16_t *>(out_id) = static_cast<uint16_t>(__byte_perm(code0, code1, 0x0051));
                 out_t += step; out_s += step; out_id += step;
-                st0 += prs; st1 += prs; sc0 += prs; sc1 += prs;
+                p0 += prs; p1 += prs; px += prs;
             }
         }
     } else {
         const int mi = lane & (p.mg - 1), prow = lane / p.mg, rows = 32 / p.mg;
         if (mi < n_mi) {
             const uint32_t m_u = p.G.m_list[m0 + mi];
-            const size_t plane = static_cast<size_t>(p.G.n_P) * p.G.n_m;
-            const size_t base = (static_cast<size_t>(table - p.out_table0) * p.om.planes + p.om.plane_bcast) * plane + static_cast<size_t>(m0 + mi);
             for (int pr = warp * rows + prow; pr < n_valid; pr += kDecWarps * rows) {
-                const size_t o = base + static_cast<size_t>(tile0 + pr) * p.G.n_m;
-                const uint32_t code = sm.st_code[mi * kCodeStride + pr];
+                const size_t o = base + static_cast<size_t>(pr) * p.G.n_m + mi;
+                const unsigned at = sm.pos[mi * kPosStride + pr];
+                const double2 e = sm.line[mi * sm.slots + at];
+                const uint32_t code = sm.code[mi * sm.slots + at];
                 const uint32_t cand = code & 255u;
-                p.d_time[o] = sm.st_time[mi * kStageStride + pr];
+                p.d_time[o] = fma(sm.pm1[pr], e.x, e.y);
                 p.d_strategy[o] = static_cast<uint8_t>(code >> 8);
                 p.d_sbytes[o] = cand == kCandWhole ? m_u : sm.sval[cand];
             }
         }
     }
 }
-
-size_t decide_smem_bytes(const TableDev &T, const GridDev &G) { return dec_layout(T.npad, G.n_s, nullptr, nullptr); }
 
 template <bool ENV>
 static cudaError_t launch_decide_t(const DecideParams &p, size_t smem, unsigned blocks, cudaStream_t st)
@@ -474,7 +414,7 @@ static cudaError_t launch_decide_t(const DecideParams &p, size_t smem, unsigned 
 
 cudaError_t launch_decide(const DecideParams &p, cudaStream_t st)
 {
-    const size_t smem = decide_smem_bytes(p.T, p.G);
+    const size_t smem = dec_layout(p.T.npad, p.G.n_s, p.n_pairs, nullptr, nullptr);
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
     return p.envelope ? launch_decide_t<true>(p, smem, static_cast<unsigned>(blocks), st)

@@ -134,6 +134,7 @@ struct DecideParams {
     int gaps_stride;
     int n_mgroups, n_ptiles;
     int mg;  // message sizes per CTA, 1..kDecMG
+    int n_pairs;  // distinct (floor, ceil) pairs of log2 P in a tile of process counts, at most
     int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cu)
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16 / 8 / 2-byte aligned bases)
     int table0, n_tables_launch;
@@ -149,7 +150,6 @@ constexpr int kDecWarps = kDecThreads / 32;
 constexpr int kDecR = 8;                               // process counts per thread
 constexpr int kDecTileP = 32 * kDecR;                  // 256 process counts per CTA, shared by its warps
 constexpr int kDecMG = 16;                             // message sizes per CTA (at most), split over the warps
-constexpr int kDecU = 4;                               // list entries per filter test
 
 // segmin_kernel (segmented minima of plogp_predict on short candidate lists, lanes <-> P): see segmin.cu
 struct SegminParams {
@@ -184,7 +184,6 @@ cudaError_t launch_fused(const FusedParams &p, bool predict, cudaStream_t st);
 cudaError_t launch_scatter(const FusedParams &p, cudaStream_t st);  // decision table, Scatter strategies only
 cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st);
 cudaError_t launch_s1_tiles(const S1Params &p, cudaStream_t st);
-size_t decide_smem_bytes(const TableDev &T, const GridDev &G);
 cudaError_t launch_decide(const DecideParams &p, cudaStream_t st);
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st);
 size_t segmin_smem_bytes(const TableDev &T, const GridDev &G);
