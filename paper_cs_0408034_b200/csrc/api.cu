@@ -66,7 +66,7 @@ struct Plan {
     // and an unsplit range needs no tile sums, i.e. one launch less)
     int sc_ptiles = 1, sc_passes_per_tile = 1;
     // decision kernel tiling (short candidate lists)
-    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_pairs = 1;
+    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_tiles = 1, dec_pairs = 1;
     size_t carry_bytes_per_table = 0;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
@@ -293,8 +293,14 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
     while (pl.dec_mg > kDecWarps && (long long)((n_m + pl.dec_mg - 1) / pl.dec_mg) * pl.dec_ptiles * h->T.n_tables < (long long)h->sm_count * 4)
         pl.dec_mg >>= 1;
     pl.dec_mgroups = (n_m + pl.dec_mg - 1) / pl.dec_mg;
+    // two tiles per CTA share the candidate lists, where that leaves enough CTAs
+    if (pl.dec_ptiles % 2 == 0 && (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables >= (long long)h->sm_count * 40) {
+        pl.dec_tiles = 2;
+        pl.dec_ptiles /= 2;
+    }
+    const int dec_p = pl.dec_tiles * kDecTileP;
     for (int t = 0; t < pl.dec_ptiles; ++t) {
-        const int first = t * kDecTileP, last = std::min(n_P, first + kDecTileP) - 1;
+        const int first = t * dec_p, last = std::min(n_P, first + dec_p) - 1;
         const int64_t P0 = g->P ? g->P[first] : int64_t(g->P_lo) + first, P1 = g->P ? g->P[last] : int64_t(g->P_lo) + last;
         pl.dec_pairs = std::max(pl.dec_pairs, log2_pair(P1) - log2_pair(P0) + 1);
     }
@@ -535,7 +541,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             DecideParams dp{};
             dp.T = h->T; dp.G = pl.G;
             dp.G.mask &= 0x3FFu;
-            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.n_pairs = pl.dec_pairs;
+            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs;
             dp.table0 = t0; dp.n_tables_launch = nt; dp.out_table0 = out.out_table0; dp.om = out.om;
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
             dp.envelope = pl.envelope_short ? 1 : 0;

@@ -38,38 +38,37 @@ namespace {
 
 constexpr int R = kDecR;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kPosStride = kDecTileP + 4;    // bytes per staged row
 constexpr uint32_t kCandNone = 255;   // winner is an unsegmented strategy
 constexpr uint32_t kCandWhole = 254;  // segmented winner with no fitting candidate: the whole message
-constexpr unsigned kNoPilot = 0x1FFu;
+constexpr int kPilots = 4;
 constexpr int kIntMax = 0x7FFFFFFF;
-constexpr int kPairBlock = 16;  // (floor, ceil) pairs per pass: half a warp, the halves split the candidates
 
 struct DecSmem {
     double *tab, *gs, *gm, *pm1;
     double2 *line;    // [kDecMG][slots]: coefficients by slot
+    float *x;         // [n_p]: P-1 rounded down
     float *fa, *fc;   // [kDecWarps][cap]: the lines' coefficients rounded down, for the warp's current message size
     double *q;        // [kDecWarps][n_s]: g(s) k, for the warp's current message size
     uint32_t *sval;   // [256]: segment sizes by candidate index; [kCandNone] = 0
     uint16_t *code;   // [kDecMG][slots]: id << 8 | candidate index
-    uint8_t *pair, *pos;  // [kDecTileP]: pair of a process count; [kDecMG][kPosStride]: winners
-    int cap, slots;
+    uint8_t *pair, *pos;  // [n_p]: pair of a process count; [kDecMG][pos_stride]: winners
+    int cap, slots, pos_stride;
 };
 
 __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
-// Shared-memory layout.  cap: lines of one message size (a multiple of 4); n_pairs: (floor, ceil) pairs of a tile at most.
+// Shared-memory layout.  cap: lines of one message size (a multiple of 4); n_pairs: (floor, ceil) pairs of a CTA at most.
 // A slot number fits a byte: at most 4 + 2 * 64 lines and 61 pairs.
-__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, unsigned char *base, DecSmem *o)
+__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int tiles, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(2 * nsv + 4, 4), slots = cap + n_pairs;
+    const int cap = round_up(2 * nsv + 4, 4), slots = cap + n_pairs, n_p = tiles * kDecTileP, pos_stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
-    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(kDecTileP * 8),
+    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
                  o_line = take(size_t(kDecMG) * slots * 16), o_fa = take(size_t(kDecWarps) * cap * 4), o_fc = take(size_t(kDecWarps) * cap * 4),
                  o_q = take(size_t(kDecWarps) * nsv * 8), o_sv = take(256 * 4), o_code = take(size_t(kDecMG) * slots * 2),
-                 o_pair = take(kDecTileP), o_pos = take(size_t(kDecMG) * kPosStride);
+                 o_pair = take(n_p), o_pos = take(size_t(kDecMG) * pos_stride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
         o->gm = reinterpret_cast<double *>(base + o_gm); o->pm1 = reinterpret_cast<double *>(base + o_pm);
@@ -77,7 +76,8 @@ __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, uns
         o->fa = reinterpret_cast<float *>(base + o_fa); o->fc = reinterpret_cast<float *>(base + o_fc);
         o->q = reinterpret_cast<double *>(base + o_q); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
         o->code = reinterpret_cast<uint16_t *>(base + o_code); o->pair = base + o_pair; o->pos = base + o_pos;
-        o->cap = cap; o->slots = slots;
+        o->x = reinterpret_cast<float *>(base + o_x);
+        o->cap = cap; o->slots = slots; o->pos_stride = pos_stride;
     }
     return off;
 }
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
     DecSmem sm;
-    dec_layout(npad, p.G.n_s, p.n_pairs, smem_raw, &sm);
+    dec_layout(npad, p.G.n_s, p.n_pairs, p.tiles, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
 
     int b = blockIdx.x;
@@ -108,16 +108,17 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = mgroup * p.mg;  // p.mg <= kDecMG message sizes per CTA (fewer on small grids, for more CTAs)
     const int n_mi = min(p.mg, p.G.n_m - m0);
-    const int tile0 = ptile * kDecTileP;
-    const int n_valid = min(kDecTileP, p.G.n_P - tile0);
+    const int n_p = p.tiles * kDecTileP, tile0 = ptile * n_p;
+    const int n_valid = min(n_p, p.G.n_P - tile0);
     const int pair0 = pair_of(P_at(p.G, tile0)), n_pairs = pair_of(P_at(p.G, tile0 + n_valid - 1)) - pair0 + 1;
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
     if (!grow) stage_table(sm.tab, p.T, table);
-    for (int i = tid; i < kDecTileP; i += kDecThreads) {
+    for (int i = tid; i < n_p; i += kDecThreads) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
         sm.pm1[i] = static_cast<double>(P - 1);
+        sm.x[i] = __int2float_rd(P - 1);
         sm.pair[i] = static_cast<uint8_t>(min(pair_of(P) - pair0, n_pairs - 1));
     }
     __syncthreads();
@@ -136,16 +137,20 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     const double rdv = 2.0 * g1 + 3.0 * L;  // rendezvous handshake: 2 g(1) + 3 L
     __syncthreads();
 
-    // the pilot's process count: middle of the tile's valid range
-    const double x_mid = sm.pm1[n_valid / 2];
-    f32x2 x2[R];  // this lane's process counts less one, rounded down, twice each
+    // the pilots' process counts: the winner changes more often where P is small
+    float x_pilot[kPilots];
+    {
+        const int at[kPilots] = {n_valid >> 5, n_valid * 5 >> 5, n_valid * 15 >> 5, n_valid - 1};
 #pragma unroll
-    for (int r = 0; r < R; ++r) x2[r] = splat2(__double2float_rd(sm.pm1[32 * r + lane]));
+        for (int i = 0; i < kPilots; ++i) x_pilot[i] = sm.x[at[i]];
+    }
+    // At P = 2 a segmented flat tree and a segmented chain cost the same for every s, which no bound can tell apart.
+    const bool two = sm.pm1[0] == 1.0;
 
     // the codes carry the strategy ids as the caller names them
     auto idc = [&](int id) { return static_cast<uint32_t>(p.om.id_of[id]) << 8; };
     const uint32_t code2 = idc(2), code5 = idc(5), code9 = idc(9);
-    const bool has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has6 = (mask >> 6) & 1u, has7 = (mask >> 7) & 1u,
+    const bool has0 = mask & 1u, has3 = (mask >> 3) & 1u, has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has6 = (mask >> 6) & 1u, has7 = (mask >> 7) & 1u,
                has8 = (mask >> 8) & 1u, has9 = (mask >> 9) & 1u;
     const bool any_log = mask & 0x3C0u;
     // The unsegmented lines do not depend on the message size beyond g(m): lanes 0..3 hold ids 0, 1, 3, 4
@@ -156,6 +161,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     const double fa = fid == 3 ? L : (fid == 4 ? rdv : 0.0);
     const double fc = fid == 0 ? L : (fid == 1 ? rdv : 0.0);
     const uint16_t fcode = static_cast<uint16_t>(idc(fid) | kCandNone);
+    const int pair_w = n_pairs <= 16 ? 16 : 32;
     float *const la = sm.fa + warp * sm.cap, *const lc = sm.fc + warp * sm.cap;
     double *const lq = sm.q + warp * max(p.G.n_s, 1);
 
@@ -164,6 +170,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
         const int ns = p.G.ns_of_m[midx];
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
         const double gm = sm.gm[mi];
+        const uint32_t m_u = p.G.m_list[midx];
         const double *krow = p.G.k_list + static_cast<size_t>(midx) * p.G.n_s;
         double2 *const line = sm.line + mi * sm.slots;
         uint16_t *const code = sm.code + mi * sm.slots;
@@ -197,19 +204,22 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
         const int o2 = n01, o3 = o2 + (has2 ? nq : 0), o5 = o3 + n34, n1 = o5 + (has5 ? n5 : 0);
         const int n1p = round_up(n1, 4);
 
-        // ---- the lines of this message size, and each lane's best one at the pilot's process count ----
+        // ---- the lines of this message size, and each lane's best ones at the pilots' process counts ----
         __syncwarp();  // the previous message size's loops have finished reading the warp's lists
-        double tb = CUDART_INF;
-        unsigned pb = kNoPilot;
-        auto put = [&](int slot, double a, double c, uint32_t cd) {
+        unsigned pilot[kPilots];  // bound (without its last 8 bits) and slot in one number
+#pragma unroll
+        for (int i = 0; i < kPilots; ++i) pilot[i] = 0xFFFFFFFFu;
+        auto put = [&](int slot, double a, double c, uint32_t cd, bool twin) {
+            const float af = __double2float_rd(a), cf = __double2float_rd(c);
             line[slot] = make_double2(a, c);
-            la[slot] = __double2float_rd(a);
-            lc[slot] = __double2float_rd(c);
+            la[slot] = af;
+            lc[slot] = twin ? CUDART_INF_F : cf;
             code[slot] = static_cast<uint16_t>(cd);
-            const double t = fma(x_mid, a, c);
-            if (t < tb || pb == kNoPilot) { tb = t; pb = static_cast<unsigned>(slot); }
+#pragma unroll
+            for (int i = 0; i < kPilots; ++i)
+                pilot[i] = min(pilot[i], (__float_as_uint(__fmaf_rd(x_pilot[i], af, cf)) & ~0xFFu) | static_cast<unsigned>(slot));
         };
-        if (f_on) put((fid < 3 ? 0 : o3 - n01) + __popc(mask & 0x1Bu & ((1u << fid) - 1u)), gm + fa, fc, fcode);
+        if (f_on) put((fid < 3 ? 0 : o3 - n01) + __popc(mask & 0x1Bu & ((1u << fid) - 1u)), gm + fa, fc, fcode, false);
         if (lane >= 28 && n1 + lane - 28 < n1p) {  // padding: the bound is +inf
             la[n1 + lane - 28] = 0.0f;
             lc[n1 + lane - 28] = CUDART_INF_F;
@@ -218,27 +228,27 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
             // Section 2's k and the line coefficients of Table 1's segmented rows
             double gsv = gm, k = 1.0;
             uint32_t cand = kCandWhole;
+            bool whole = true;  // one segment: the line of the unsegmented sibling, whose lower id wins the tie
             if (ns > 0) {
                 gsv = sm.gs[c];
                 k = krow[c];  // Section 2's k, from the host's table
                 cand = static_cast<uint32_t>(c);
+                whole = sm.sval[c] == m_u;
             }
             const double Q = gsv * k;
             lq[c] = Q;
-            if (has2 && (!env || c == q_c)) put(o2 + (env ? 0 : c), Q, L, code2 | cand);  // (P-1) (g(s) k) + L
-            if (has5 && (!env || (c >= lo5 && c < lo5 + n5)))                             // (P-1) (g(s) + L) + g(s) (k-1)
-                put(o5 + (env ? c - lo5 : c), gsv + L, gsv * (k - 1.0), code5 | cand);
+            if (has2 && (!env || c == q_c)) put(o2 + (env ? 0 : c), Q, L, code2 | cand, whole && has0);  // (P-1) (g(s) k) + L
+            if (has5 && (!env || (c >= lo5 && c < lo5 + n5)))                                            // (P-1) (g(s) + L) + g(s) (k-1)
+                put(o5 + (env ? c - lo5 : c), gsv + L, gsv * (k - 1.0), code5 | cand, whole && has3);
         }
-        // warp-wide pilot: smallest time (high word first, then low word with the slot in its last 9 bits)
-        const int hmin = __reduce_min_sync(kFull, hi32(tb));
-        const unsigned k2 = hi32(tb) == hmin ? ((static_cast<unsigned>(__double2loint(tb)) & ~0x1FFu) | pb) : 0xFFFFFFFFu;
-        const unsigned pilot = __reduce_min_sync(kFull, k2) & 0x1FFu;
+#pragma unroll
+        for (int i = 0; i < kPilots; ++i) pilot[i] = __reduce_min_sync(kFull, pilot[i]) & 0xFFu;
         __syncwarp();
 
-        // ---- the best of ids 6 to 9 per (floor, ceil) pair ----
+        // ---- the best of ids 6 to 9 per (floor, ceil) pair: half a warp where it is enough, the halves split the candidates ----
         if (any_log)
-        for (int b0 = 0; b0 < n_pairs; b0 += kPairBlock) {
-            const int pr = b0 + (lane & (kPairBlock - 1)), half = lane / kPairBlock;
+        for (int b0 = 0; b0 < n_pairs; b0 += pair_w) {
+            const int pr = b0 + (lane & (pair_w - 1)), half = lane / pair_w;
             const int li = pair0 + pr;
             const double lf = static_cast<double>(li >> 1), lcd = static_cast<double>((li >> 1) + (li & 1)), lcL = lcd * L;
             double t = CUDART_INF;
@@ -251,13 +261,15 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
                     cb = q_c;
                 } else {
 #pragma unroll 4
-                    for (int c = half; c < nsv; c += 2) {
+                    for (int c = half; c < nsv; c += 32 / pair_w) {
                         const double v = fma(lf, lq[c], lcL);
                         if (v < tc) { tc = v; cb = c; }
                     }
-                    const double t2 = __shfl_xor_sync(kFull, tc, kPairBlock);
-                    const int cb2 = __shfl_xor_sync(kFull, cb, kPairBlock);
-                    if (t2 < tc || (t2 == tc && cb2 < cb)) { tc = t2; cb = cb2; }
+                    if (pair_w == 16) {
+                        const double t2 = __shfl_xor_sync(kFull, tc, 16);
+                        const int cb2 = __shfl_xor_sync(kFull, cb, 16);
+                        if (t2 < tc || (t2 == tc && cb2 < cb)) { tc = t2; cb = cb2; }
+                    }
                 }
                 t = tc;
                 cd = code9 | (ns > 0 ? static_cast<uint32_t>(min(cb, ns - 1)) : kCandWhole);
@@ -281,70 +293,121 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
             }
         }
 
-        // ---- start of the running minima: the pilot or the pair ----
-        double2 e = make_double2(0.0, CUDART_INF);
-        if (pilot != kNoPilot) {
-            e = line[pilot];
-            if (lane == 0) { la[pilot] = 0.0f; lc[pilot] = CUDART_INF_F; }  // its own bounds would always pass
+        // ---- the pilots leave the lists: their own bounds would always pass ----
+        double t_two = CUDART_INF;
+        unsigned at_two = 0xFFu;
+        if (two && n1 > 0) {  // P = 2: the best line, exactly, lanes <-> lines
+            for (int u = lane; u < n1; u += 32) {
+                const double2 v = line[u];
+                const double t = fma(1.0, v.x, v.y);
+                if (t < t_two || at_two == 0xFFu) { t_two = t; at_two = static_cast<unsigned>(u); }
+            }
+            const int h = __reduce_min_sync(kFull, at_two == 0xFFu ? kIntMax : hi32(t_two));
+            const bool on_h = at_two != 0xFFu && hi32(t_two) == h;
+            const unsigned l = __reduce_min_sync(kFull, on_h ? static_cast<unsigned>(__double2loint(t_two)) : 0xFFFFFFFFu);
+            at_two = __reduce_min_sync(kFull, on_h && static_cast<unsigned>(__double2loint(t_two)) == l ? at_two : 0xFFu);
+            t_two = __hiloint2double(h, static_cast<int>(l));
+        }
+        if (n1 > 0 && lane < kPilots) {
+            unsigned mine = pilot[0];
+#pragma unroll
+            for (int i = 1; i < kPilots; ++i) mine = lane == i ? pilot[i] : mine;
+            la[mine] = 0.0f;
+            lc[mine] = CUDART_INF_F;
         }
         __syncwarp();
-        uint8_t *const pos = sm.pos + mi * kPosStride + lane;
-        float T[R];
+
+        for (int tile = 0; tile < p.tiles; ++tile) {
+            if (tile * kDecTileP >= n_valid) break;
+            const double *const xd = sm.pm1 + tile * kDecTileP + lane;
+            uint8_t *const pos = sm.pos + mi * sm.pos_stride + tile * kDecTileP + lane;
+            float T[R];
+            // ---- start of the running minima: the best of the pilots and the pair ----
+            {
+                double t[R];
+                unsigned at[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            double t = fma(sm.pm1[32 * r + lane], e.x, e.y);
-            unsigned at = pilot;
-            if (any_log) {
-                const unsigned slot = sm.cap + sm.pair[32 * r + lane];
-                const double tl = line[slot].y;
-                if (tl < t || pilot == kNoPilot) { t = tl; at = slot; }  // lines have the lower ids
+                for (int r = 0; r < R; ++r) { t[r] = CUDART_INF; at[r] = 0xFFu; }
+                if (n1 > 0) {
+                    const double2 e = line[pilot[0]];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) { t[r] = fma(xd[32 * r], e.x, e.y); at[r] = pilot[0]; }
+#pragma unroll
+                    for (int i = 1; i < kPilots; ++i) {
+                        if (pilot[i] == pilot[i - 1]) continue;
+                        const double2 v = line[pilot[i]];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const double tt = fma(xd[32 * r], v.x, v.y);
+                            if (tt < t[r] || (tt == t[r] && pilot[i] < at[r])) { t[r] = tt; at[r] = pilot[i]; }
+                        }
+                    }
+                    if (two && tile == 0 && lane == 0) { t[0] = t_two; at[0] = at_two; }
+                }
+                if (any_log) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const unsigned slot = sm.cap + sm.pair[tile * kDecTileP + 32 * r + lane];
+                        const double tl = line[slot].y;
+                        if (tl < t[r] || n1 == 0) { t[r] = tl; at[r] = slot; }  // lines have the lower ids
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    T[r] = __double2float_ru(t[r]);
+                    pos[32 * r] = static_cast<uint8_t>(at[r]);
+                }
+                if (two && tile == 0 && lane == 0) T[0] = -1.0f;  // settled
             }
-            T[r] = __double2float_ru(t);
-            pos[32 * r] = static_cast<uint8_t>(at);
-        }
 
-        // ---- lower bounds of all other lines ----
-        float mn[R];
+            // ---- lower bounds of all other lines ----
+            float mn[R];
+            f32x2 x2[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) mn[r] = CUDART_INF_F;
+            for (int r = 0; r < R; ++r) { mn[r] = CUDART_INF_F; x2[r] = splat2(sm.x[tile * kDecTileP + 32 * r + lane]); }
 #pragma unroll 2
-        for (int j = 0; j < n1p; j += 4) {
-            const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
-#pragma unroll
-            for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], aa.x, cc.x));
-#pragma unroll
-            for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], aa.y, cc.y));
-        }
-        unsigned hit = 0;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (mn[r] <= T[r] && mn[r] < CUDART_INF_F) hit |= 1u << r;
-
-        // ---- exact search of the rows in which some bound is not above the running minimum ----
-#pragma unroll 1
-        for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
-            const int r = __ffs(rows) - 1;
-            const double x = sm.pm1[32 * r + lane];
-            const f32x2 xx = splat2(__double2float_rd(x));
-            unsigned at = pos[32 * r];
-            const double2 w = line[at];
-            double t = fma(x, w.x, w.y);
-            float Tr = __double2float_ru(t);
-#pragma unroll 1
             for (int j = 0; j < n1p; j += 4) {
                 const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
-                const float low = min_with2(min_with2(CUDART_INF_F, fma2_down(xx, aa.x, cc.x)), fma2_down(xx, aa.y, cc.y));
-                if (__any_sync(kFull, low <= Tr)) {
-#pragma unroll 1
-                    for (int u = j; u < min(j + 4, n1); ++u) {
-                        const double2 v = line[u];
-                        const double tt = fma(x, v.x, v.y);
-                        if (tt <= t && (tt < t || static_cast<unsigned>(u) < at)) { t = tt; at = static_cast<unsigned>(u); }
-                    }
-                    Tr = __double2float_ru(t);
-                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], aa.x, cc.x));
+#pragma unroll
+                for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], aa.y, cc.y));
             }
-            pos[32 * r] = static_cast<uint8_t>(at);
+            bool any = false;
+#pragma unroll
+            for (int r = 0; r < R; ++r) any |= mn[r] <= T[r];
+            if (!__any_sync(kFull, any)) continue;
+
+            // ---- exact search of the rows in which some bound is not above the running minimum ----
+            unsigned hit = 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (mn[r] <= T[r]) hit |= 1u << r;
+#pragma unroll 1
+            for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
+                const int r = __ffs(rows) - 1;
+                const double x = xd[32 * r];
+                const f32x2 xx = splat2(__double2float_rd(x));
+                unsigned at = pos[32 * r];
+                const double2 w = line[at];
+                double t = fma(x, w.x, w.y);
+                float Tr = (hit >> r) & 1u ? __double2float_ru(t) : -1.0f;
+#pragma unroll 1
+                for (int j = 0; j < n1p; j += 4) {
+                    const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
+                    const float low = min_with2(min_with2(CUDART_INF_F, fma2_down(xx, aa.x, cc.x)), fma2_down(xx, aa.y, cc.y));
+                    if (__any_sync(kFull, low <= Tr)) {
+#pragma unroll 1
+                        for (int u = j; u < min(j + 4, n1); ++u) {
+                            const double2 v = line[u];
+                            const double tt = fma(x, v.x, v.y);
+                            if (tt <= t && (tt < t || static_cast<unsigned>(u) < at)) { t = tt; at = static_cast<unsigned>(u); }
+                        }
+                        if (Tr >= 0.0f) Tr = __double2float_ru(t);
+                    }
+                }
+                pos[32 * r] = static_cast<uint8_t>(at);
+            }
         }
     }
     __syncthreads();
@@ -365,7 +428,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
             uint8_t *out_id = p.d_strategy + o;
             const double2 *l0 = sm.line + mi * sm.slots, *l1 = l0 + sm.slots;
             const uint16_t *c0 = sm.code + mi * sm.slots, *c1 = c0 + sm.slots;
-            const uint8_t *p0 = sm.pos + mi * kPosStride + pr0, *p1 = p0 + kPosStride;
+            const uint8_t *p0 = sm.pos + mi * sm.pos_stride + pr0, *p1 = p0 + sm.pos_stride;
             const double *px = sm.pm1 + pr0;
             for (int pr = pr0; pr < n_valid; pr += prs) {
                 const unsigned at0 = *p0, at1 = *p1;
@@ -389,7 +452,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
             const uint32_t m_u = p.G.m_list[m0 + mi];
             for (int pr = warp * rows + prow; pr < n_valid; pr += kDecWarps * rows) {
                 const size_t o = base + static_cast<size_t>(pr) * p.G.n_m + mi;
-                const unsigned at = sm.pos[mi * kPosStride + pr];
+                const unsigned at = sm.pos[mi * sm.pos_stride + pr];
                 const double2 e = sm.line[mi * sm.slots + at];
                 const uint32_t code = sm.code[mi * sm.slots + at];
                 const uint32_t cand = code & 255u;
@@ -414,7 +477,7 @@ static cudaError_t launch_decide_t(const DecideParams &p, size_t smem, unsigned 
 
 cudaError_t launch_decide(const DecideParams &p, cudaStream_t st)
 {
-    const size_t smem = dec_layout(p.T.npad, p.G.n_s, p.n_pairs, nullptr, nullptr);
+    const size_t smem = dec_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles, nullptr, nullptr);
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
     return p.envelope ? launch_decide_t<true>(p, smem, static_cast<unsigned>(blocks), st)

@@ -134,7 +134,8 @@ struct DecideParams {
     int gaps_stride;
     int n_mgroups, n_ptiles;
     int mg;  // message sizes per CTA, 1..kDecMG
-    int n_pairs;  // distinct (floor, ceil) pairs of log2 P in a tile of process counts, at most
+    int tiles;    // tiles of kDecTileP process counts per CTA
+    int n_pairs;  // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most
     int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cu)
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16 / 8 / 2-byte aligned bases)
     int table0, n_tables_launch;
