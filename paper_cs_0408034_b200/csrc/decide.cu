@@ -41,6 +41,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr uint32_t kCandNone = 255;   // winner is an unsegmented strategy
 constexpr uint32_t kCandWhole = 254;  // segmented winner with no fitting candidate: the whole message
 constexpr int kPilots = 4;
+constexpr int kStep = 16;  // lines per vote of the exact search
 constexpr int kIntMax = 0x7FFFFFFF;
 
 struct DecSmem {
@@ -57,12 +58,12 @@ struct DecSmem {
 
 __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
-// Shared-memory layout.  cap: lines of one message size (a multiple of 4); n_pairs: (floor, ceil) pairs of a CTA at most.
-// A slot number fits a byte: at most 4 + 2 * 64 lines and 61 pairs.
+// Shared-memory layout.  cap: lines of one message size (a multiple of kStep); n_pairs: (floor, ceil) pairs of a CTA at most.
+// A slot number fits a byte: at most 144 lines and 61 pairs.
 __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int tiles, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(2 * nsv + 4, 4), slots = cap + n_pairs, n_p = tiles * kDecTileP, pos_stride = n_p + 4;
+    const int cap = round_up(2 * nsv + 4, kStep), slots = cap + n_pairs, n_p = tiles * kDecTileP, pos_stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     const double fa = fid == 3 ? L : (fid == 4 ? rdv : 0.0);
     const double fc = fid == 0 ? L : (fid == 1 ? rdv : 0.0);
     const uint16_t fcode = static_cast<uint16_t>(idc(fid) | kCandNone);
-    const int pair_w = n_pairs <= 16 ? 16 : 32;
+    const int pair_w = n_pairs <= 16 ? 16 : 32, pair_step = n_pairs <= 16 ? 2 : 1;
     float *const la = sm.fa + warp * sm.cap, *const lc = sm.fc + warp * sm.cap;
     double *const lq = sm.q + warp * max(p.G.n_s, 1);
 
@@ -220,9 +221,9 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
                 pilot[i] = min(pilot[i], (__float_as_uint(__fmaf_rd(x_pilot[i], af, cf)) & ~0xFFu) | static_cast<unsigned>(slot));
         };
         if (f_on) put((fid < 3 ? 0 : o3 - n01) + __popc(mask & 0x1Bu & ((1u << fid) - 1u)), gm + fa, fc, fcode, false);
-        if (lane >= 28 && n1 + lane - 28 < n1p) {  // padding: the bound is +inf
-            la[n1 + lane - 28] = 0.0f;
-            lc[n1 + lane - 28] = CUDART_INF_F;
+        if (lane >= 16 && n1 + lane - 16 < round_up(n1, kStep)) {  // padding: the bound is +inf
+            la[n1 + lane - 16] = 0.0f;
+            lc[n1 + lane - 16] = CUDART_INF_F;
         }
         for (int c = lane; c < nsv; c += 32) {
             // Section 2's k and the line coefficients of Table 1's segmented rows
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
         // ---- the best of ids 6 to 9 per (floor, ceil) pair: half a warp where it is enough, the halves split the candidates ----
         if (any_log)
         for (int b0 = 0; b0 < n_pairs; b0 += pair_w) {
-            const int pr = b0 + (lane & (pair_w - 1)), half = lane / pair_w;
+            const int pr = b0 + (lane & (pair_w - 1)), half = pair_w == 16 ? lane >> 4 : 0;
             const int li = pair0 + pr;
             const double lf = static_cast<double>(li >> 1), lcd = static_cast<double>((li >> 1) + (li & 1)), lcL = lcd * L;
             double t = CUDART_INF;
@@ -261,7 +262,7 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
                     cb = q_c;
                 } else {
 #pragma unroll 4
-                    for (int c = half; c < nsv; c += 32 / pair_w) {
+                    for (int c = half; c < nsv; c += pair_step) {
                         const double v = fma(lf, lq[c], lcL);
                         if (v < tc) { tc = v; cb = c; }
                     }
@@ -393,12 +394,21 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
                 double t = fma(x, w.x, w.y);
                 float Tr = (hit >> r) & 1u ? __double2float_ru(t) : -1.0f;
 #pragma unroll 1
-                for (int j = 0; j < n1p; j += 4) {
-                    const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
-                    const float low = min_with2(min_with2(CUDART_INF_F, fma2_down(xx, aa.x, cc.x)), fma2_down(xx, aa.y, cc.y));
-                    if (__any_sync(kFull, low <= Tr)) {
-#pragma unroll 1
-                        for (int u = j; u < min(j + 4, n1); ++u) {
+                for (int j = 0; j < n1; j += kStep) {
+                    float low[kStep / 4];
+#pragma unroll
+                    for (int q = 0; q < kStep / 4; ++q) {
+                        const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j + 4 * q), cc = *reinterpret_cast<const f32x2x2 *>(lc + j + 4 * q);
+                        low[q] = min_with2(min_with2(CUDART_INF_F, fma2_down(xx, aa.x, cc.x)), fma2_down(xx, aa.y, cc.y));
+                    }
+                    if (!__any_sync(kFull, fminf(fminf(low[0], low[1]), fminf(low[2], low[3])) <= Tr)) continue;
+#pragma unroll
+                    for (int q = 0; q < kStep / 4; ++q) {
+                        if (!__any_sync(kFull, low[q] <= Tr)) continue;
+                        const int u0 = j + 4 * q;
+#pragma unroll
+                        for (int u = u0; u < u0 + 4; ++u) {
+                            if (u >= n1) break;
                             const double2 v = line[u];
                             const double tt = fma(x, v.x, v.y);
                             if (tt <= t && (tt < t || static_cast<unsigned>(u) < at)) { t = tt; at = static_cast<unsigned>(u); }
