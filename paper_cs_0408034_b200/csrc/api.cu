@@ -62,12 +62,10 @@ struct Plan {
     int env_threads = 256, env_rep_cap = 0, env_coarse = 64, env_max_coarse = 0;
     // fused kernel tiling
     int n_mtiles = 0, n_ptiles = 1, passes_per_tile = 1;
-    // Scatter decision kernel: its own split of P (one CTA run covers a short P range in a few microseconds,
-    // and an unsplit range needs no tile sums, i.e. one launch less)
-    int sc_ptiles = 1, sc_passes_per_tile = 1;
+    // Scatter decision kernel: its own split of P (vec = 2: two message sizes per lane, where the outputs allow it)
+    int sc_vec = 1, sc_ptiles = 1, sc_run = 1;
     // decision kernel tiling (short candidate lists)
     int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_tiles = 1, dec_pairs = 1;
-    size_t carry_bytes_per_table = 0;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
     size_t off_pair_m = 0, off_pair_chunk = 0, off_pair_row = 0, off_pair_base = 0;
@@ -283,8 +281,17 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
     n_ptiles = std::min(n_ptiles, 256);
     pl.passes_per_tile = (total_passes + n_ptiles - 1) / n_ptiles;
     pl.n_ptiles = (total_passes + pl.passes_per_tile - 1) / pl.passes_per_tile;
-    if (n_P <= 512) { pl.sc_ptiles = 1; pl.sc_passes_per_tile = total_passes; }
-    else { pl.sc_ptiles = pl.n_ptiles; pl.sc_passes_per_tile = pl.passes_per_tile; }
+    // Two message sizes per lane halve the stores and the address arithmetic per cell: taken where the message sizes alone
+    // give four CTAs per SM (4096 tables, P = 2..512, 128 m: 0.55 ms against 0.58) and leave no warp half empty.  Smaller
+    // grids take one per lane (one table, P = 2..65536, 64 m: 17 us against 24, P = 2..1024, 256 m: 5.7 against 8.1) and
+    // split the process counts over CTAs, 8 runs of at least 4 each, until four CTAs per SM are there.
+    {
+        const long long base = (long long)pl.n_mtiles * h->T.n_tables, want = (long long)h->sm_count * 4;
+        pl.sc_vec = n_m % 2 == 0 && (n_m + 63) / 64 * 2 == pl.n_mtiles && base / 2 >= want ? 2 : 1;
+        const long long split = std::max<long long>(1, (want + base - 1) / base);
+        pl.sc_run = int(std::max<long long>(4, (n_P + kWarps * split - 1) / (kWarps * split)));
+        pl.sc_ptiles = (n_P + kWarps * pl.sc_run - 1) / (kWarps * pl.sc_run);
+    }
 
     pl.dec_ptiles = (n_P + kDecTileP - 1) / kDecTileP;
     // 16 message sizes per CTA give the widest output rows; small grids trade that for more CTAs
@@ -398,12 +405,9 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
     G.k_mode = g->k_mode;
     G.lc_max = std::max(1, ceil_log2(P_hi));
 
-    // ---- scratch: sweep partials (per table batch) and Scatter Chain tile prefixes ----
-    const bool s1_on = (g->strategy_mask >> 11) & 1u;
+    // ---- scratch: sweep partials (per table batch), gap rows ----
     size_t per_table = 0;
     if (!pl.inline_sweep) per_table += size_t(pl.n_seg) * pl.n_pairs * n_P * (sizeof(double) + sizeof(uint32_t)) + 512;
-    if (s1_on && pl.n_ptiles > 1) pl.carry_bytes_per_table = size_t(pl.n_ptiles) * (kWarps + 1) * n_m * sizeof(double);
-    per_table += pl.carry_bytes_per_table;
     // The gap pre-pass costs a launch: taken where the lane <-> P kernels run many CTAs per table and fill the GPU several times over
     if (pl.inline_sweep && pl.n_seg > 0) {
         const long long ctas_per_table = (long long)pl.dec_mgroups * pl.dec_ptiles;
@@ -452,15 +456,11 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
     if (rc != PLOGP_OK) { h->plan = Plan(); return rc; }
     const Plan &pl = h->plan;
     if (pl.empty) return PLOGP_OK;
-    const bool s1 = (pl.G.mask >> 11) & 1u;
     // Short candidate lists with segmented strategies: the lane<->P decision kernel; everything else
     // (predictions, long lists reduced by the sweep kernel, Scatter-only grids) goes through fused_kernel.
     const bool use_decide = !predict && pl.inline_sweep && pl.n_seg > 0;
     // the kernel that follows the (optional) Broadcast decision kernel: Scatter strategies only => scatter_kernel
     const bool use_scatter = !predict && ((use_decide ? pl.G.mask & 0x1C00u : pl.G.mask) & 0x3FFu) == 0;
-    const int n_ptiles = use_scatter ? pl.sc_ptiles : pl.n_ptiles;
-    const int passes_per_tile = use_scatter ? pl.sc_passes_per_tile : pl.passes_per_tile;
-    const bool need_carry = s1 && n_ptiles > 1;
 
     if (t_end < 0) t_end = h->T.n_tables;
     for (int t0 = t_begin; t0 < t_end; t0 += pl.tables_per_batch) {
@@ -468,17 +468,12 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         unsigned char *ws = h->d_ws;
         double *part_time = nullptr;
         uint32_t *part_idx = nullptr;
-        double *tile_sum = nullptr;
         if (!pl.inline_sweep) {
             const size_t cells = size_t(nt) * pl.n_seg * pl.n_pairs * pl.G.n_P;
             part_time = reinterpret_cast<double *>(ws);
             ws += align_up(cells * sizeof(double), 256);
             part_idx = reinterpret_cast<uint32_t *>(ws);
             ws += align_up(cells * sizeof(uint32_t), 256);
-        }
-        if (need_carry) {
-            tile_sum = reinterpret_cast<double *>(ws);
-            ws += align_up(pl.carry_bytes_per_table * nt, 256);
         }
         double *gaps = nullptr;
         if (pl.use_gaps && pl.inline_sweep && pl.n_seg > 0 && (predict || use_decide)) {
@@ -509,14 +504,6 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             int n_launches = 0;
             { LaunchTimer lt(h, PLOGP_KERNEL_SWEEP, st); CK(launch_sweep(sp, nt, &n_launches, st)); }
             g_launches += unsigned(n_launches);
-        }
-        if (need_carry) {
-            S1Params s{};
-            s.T = h->T; s.G = pl.G;
-            s.n_mtiles = pl.n_mtiles; s.n_ptiles = n_ptiles; s.passes_per_tile = passes_per_tile;
-            s.table0 = t0; s.n_tables_launch = nt; s.tile_sum = tile_sum;
-            { LaunchTimer lt(h, PLOGP_KERNEL_CHAIN_PREFIX, st); CK(launch_s1_tiles(s, st)); }
-            g_launches += 1;
         }
         GridDev Gf = pl.G;
         if (predict && pl.inline_sweep && pl.n_seg > 0) {
@@ -554,18 +541,30 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             Gf.n_s = 0;
             if (!Gf.mask) continue;
         }
+        if (use_scatter) {
+            ScatterParams sc{};
+            sc.T = h->T; sc.G = Gf;
+            const bool aligned = reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 &&
+                                 reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
+            sc.vec = aligned ? pl.sc_vec : 1;
+            sc.n_mtiles = (pl.G.n_m + 32 * sc.vec - 1) / (32 * sc.vec);
+            sc.n_ptiles = pl.sc_ptiles; sc.run_len = pl.sc_run;
+            sc.table0 = t0; sc.n_tables_launch = nt; sc.out_table0 = out.out_table0; sc.om = out.om;
+            sc.d_strategy = out.d_strategy; sc.d_sbytes = out.d_sbytes; sc.d_time = out.d_time;
+            { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_scatter(sc, st)); }
+            g_launches += 1;
+            continue;
+        }
         FusedParams fp = out;
         fp.T = h->T; fp.G = Gf;
-        fp.n_mtiles = pl.n_mtiles; fp.n_ptiles = n_ptiles; fp.passes_per_tile = passes_per_tile;
+        fp.n_mtiles = pl.n_mtiles; fp.n_ptiles = pl.n_ptiles; fp.passes_per_tile = pl.passes_per_tile;
         fp.table0 = t0; fp.n_tables_launch = nt;
-        fp.s1_sums = tile_sum;
         // part_time doubles as the "segmented minima come from the sweep kernel" switch
         fp.part_time = pl.inline_sweep ? nullptr : part_time;
         fp.part_idx = part_idx;
         fp.pair_base = pl.inline_sweep ? nullptr : reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_base);
         fp.n_pairs = pl.n_pairs; fp.n_seg = pl.n_seg;
-        if (use_scatter) { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_scatter(fp, st)); }
-        else { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, st)); }
+        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, st)); }
         g_launches += 1;
     }
     return PLOGP_OK;

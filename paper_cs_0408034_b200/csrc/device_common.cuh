@@ -102,34 +102,123 @@ __device__ __forceinline__ int interval_of(const double *s_tab, int npad, double
     return i;
 }
 
-// g(x) for a caller whose arguments never decrease: the current interval's line is kept in
-// registers and shared memory is touched only when x crosses into the next interval (keys past
-// the last interval are +inf, and npad >= n_bp leaves at least one such key, so the walk stops
-// inside the array).
-struct GapWalk {
-    int i = -1;
+// x rounded to a whole number, for 0 <= x < 2^51 (two additions; the rounding instruction has a quarter of their rate).
+// Of the two whole numbers around a quotient's true value the caller takes the right one by the sign of the remainder:
+// a product with the reciprocal is off by far less than one half, as j m < 2^53 and j <= 2^30.
+__device__ __forceinline__ double round_whole(double x)
+{
+    const double big = 6755399441055744.0;  // 1.5 * 2^52
+    return (x + big) - big;
+}
+
+// g(x) for a caller whose arguments never decrease (the Scatter Chain's j m): the current interval's line is kept in
+// registers and shared memory is touched only when x crosses into the next interval (keys past the last interval are
+// +inf, and npad >= n_bp leaves at least one such key, so the walk stops inside the array).  Below the table a
+// pseudo-interval with slope 0 holds g at its first value.
+struct ChainWalk {
+    int i;
     double key, next, slope, gap;
 
-    __device__ __forceinline__ void load(const double *s_tab, int npad)
+    __device__ __forceinline__ void start(const double *s_tab, int npad, double x)
     {
-        key = s_tab[i];
-        next = s_tab[i + 1];
-        slope = s_tab[2 * npad + i];
-        gap = s_tab[npad + i];
-    }
-    __device__ __forceinline__ double at(const double *s_tab, int npad, double x)
-    {
-        if (i < 0) {
+        if (x < s_tab[0]) {
+            i = -1; key = 0.0; next = s_tab[0]; slope = 0.0; gap = s_tab[npad];
+        } else {
             i = interval_of(s_tab, npad, x);
             load(s_tab, npad);
         }
+    }
+    __device__ __forceinline__ void load(const double *s_tab, int npad)
+    {
+        key = s_tab[i]; next = s_tab[i + 1]; slope = s_tab[2 * npad + i]; gap = s_tab[npad + i];
+    }
+    __device__ __forceinline__ void advance(const double *s_tab, int npad, double x)
+    {
         while (x >= next) {
+            // rare: keep it a branch (the barrier stops the compiler from turning the reload into
+            // loads and selects that would run at every step)
+            asm volatile("" ::: "memory");
             ++i;
             load(s_tab, npad);
         }
-        return fma(fmax(x - key, 0.0), slope, gap);
+    }
+    __device__ __forceinline__ double at(const double *s_tab, int npad, double x)
+    {
+        advance(s_tab, npad, x);
+        return fma(x - key, slope, gap);
+    }
+    // Sum of g(j m) for j = j0 .. j1 (whole numbers, j0 <= j1) in closed form: inside one interval g is a line, so its
+    // terms are an arithmetic series, n times g at their mean argument.  The loop runs over the intervals that the
+    // arguments cross (at most n_bp), not over j.
+    __device__ __forceinline__ double range(const double *s_tab, int npad, double md, double j0, double j1)
+    {
+        const double x1 = j1 * md;
+        double sum = 0.0;
+        advance(s_tab, npad, j0 * md);
+        if (x1 >= next) {
+            const double inv_m = 1.0 / md;
+            do {
+                // last j of the interval: the largest with j m < next (next <= x1 < 2^53: the products are exact)
+                double q = round_whole(next * inv_m);
+                if (fma(-q, md, next) <= 0.0) q -= 1.0;
+                sum = fma(q - j0 + 1.0, fma(0.5 * ((j0 + q) * md) - key, slope, gap), sum);
+                j0 = q + 1.0;
+                advance(s_tab, npad, j0 * md);
+            } while (x1 >= next);
+        }
+        return fma(j1 - j0 + 1.0, fma(0.5 * ((j0 + j1) * md) - key, slope, gap), sum);
     }
 };
+
+// Scatter Chain sum in front of each warp's run of process counts, for one message size per lane.  A CTA's kWarps warps
+// own the runs [e0, e1) of process-count indices, one after another from index c0 on.  The terms j <= P(c0) - 2, which
+// lie in front of the whole CTA, are split over its warps by table intervals (front); each warp adds the closed form of
+// its own run (own), which the warps behind it need.  A handful of intervals per warp instead of a pass over the process
+// counts, and nothing is carried between CTAs.  The caller puts a barrier between the two calls.
+static __device__ __noinline__ void chain_front_parts(const double *s_tab, int npad, int n_bp, const int32_t *P_list, int P_lo, double md, int c0, int e0,
+                                                      int e1, int warp, double *s_front, double *s_own, int stride)
+{
+    auto P_of = [&](int e) { return P_list ? P_list[e] : P_lo + e; };
+    double front = 0.0, own = 0.0;
+    if (c0 < e1) {  // the CTA has process counts (a warp without any still takes its share of the front)
+        const int P0 = P_of(c0);
+        const double jc = static_cast<double>(P0 - 2);
+        ChainWalk w;
+        if (jc >= 1.0) {
+            const double inv_m = 1.0 / md, x_end = jc * md;
+            const int n_int = n_bp - 1, i0 = n_int * warp / kWarps, i1 = n_int * (warp + 1) / kWarps;
+            auto first_j = [&](int i) {  // smallest j with j m >= key i; jc + 1 when that lies behind jc
+                const double key = s_tab[i];
+                const double q = round_whole(key * inv_m), j = fmax(fma(-q, md, key) > 0.0 ? q + 1.0 : q, 1.0);
+                return key > x_end ? jc + 1.0 : j;
+            };
+            double ja = first_j(i0);
+            if (warp == 0) front = (ja - 1.0) * s_tab[npad];  // below the table
+            // no branch depends on the lane, and the intervals do not wait for one another
+#pragma unroll 4
+            for (int i = i0; i < i1; ++i) {
+                const double jb = i + 1 < n_int ? first_j(i + 1) : jc + 1.0;
+                front = fma(jb - ja, fma(0.5 * ((ja + jb - 1.0) * md) - s_tab[i], s_tab[2 * npad + i], s_tab[npad + i]), front);
+                ja = jb;
+            }
+        }
+        if (e0 < e1 && warp < kWarps - 1) {
+            const double j0 = e0 == c0 ? jc + 1.0 : static_cast<double>(P_of(e0 - 1)), j1 = static_cast<double>(P_of(e1 - 1) - 1);
+            w.start(s_tab, npad, j0 * md);
+            own = w.range(s_tab, npad, md, j0, j1);
+        }
+    }
+    s_front[warp * stride] = front;
+    s_own[warp * stride] = own;
+}
+__device__ __forceinline__ double chain_front_sum(const double *s_front, const double *s_own, int stride, int warp)
+{
+    double run = 0.0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) run += s_front[w * stride];
+    for (int w = 0; w < warp; ++w) run += s_own[w * stride];
+    return run;
+}
 
 // Lexicographic minimum of (t, e) over a warp (all lanes receive it).
 __device__ __forceinline__ void warp_min_pair(double &t, int &e)
@@ -140,74 +229,6 @@ __device__ __forceinline__ void warp_min_pair(double &t, int &e)
         const int e2 = __shfl_xor_sync(0xffffffffu, e, off);
         if (t2 < t || (t2 == t && e2 < e)) { t = t2; e = e2; }
     }
-}
-
-// Sum of g(j m) for j = jlo .. jhi (jlo <= jhi) in closed form: inside one table interval g is a line, so the
-// terms whose arguments fall into it are an arithmetic series, n gap_i + slope_i (m (jlo' + jhi') n / 2 - n key_i);
-// the loop runs over the table intervals that the arguments cross (at most n_bp), not over j.  Below the first
-// size g is constant (its first value), above the last size the last interval's line goes on.  This is what
-// keeps a gap in a process-count list, or a first process count far above 2, from turning into a long loop.
-static __device__ __noinline__ double chain_range_sum(const double *s_tab, int npad, double md, long long jlo, long long jhi)
-{
-    double sum = 0.0;
-    long long j = jlo;
-    int i = -1;  // -1: below the table
-    if (static_cast<double>(j) * md >= s_tab[0]) i = interval_of(s_tab, npad, static_cast<double>(j) * md);
-    while (j <= jhi) {
-        const double next = s_tab[i + 1];  // first argument that belongs to the next interval (+inf after the last)
-        long long jend = jhi;
-        if (next <= static_cast<double>(jhi) * md) {
-            // largest j with j m < next (m, next and the products are integers below 2^53: exact)
-            long long q = static_cast<long long>(next / md);
-            while (static_cast<double>(q) * md >= next) --q;
-            while (static_cast<double>(q + 1) * md < next) ++q;
-            jend = q;
-        }
-        if (jend >= j) {
-            const double n = static_cast<double>(jend - j + 1);
-            if (i < 0) {
-                sum += n * s_tab[npad];
-            } else {
-                const double mean = 0.5 * (static_cast<double>(j + jend) * md) - s_tab[i];  // mean argument minus the key
-                sum += n * fma(mean, s_tab[2 * npad + i], s_tab[npad + i]);
-            }
-            j = jend + 1;
-        }
-        ++i;
-    }
-    return sum;
-}
-
-// One term of the Scatter Chain sum for the process count at index pidx: the gaps g(j m) for j
-// from the previous listed process count (1 before the first) up to P-1.  For a contiguous
-// range of P this is the single gap g((P-1) m); longer runs are summed interval by interval.
-// The walk state must only see non-decreasing arguments.
-__device__ __forceinline__ double s1_term(const double *s_tab, int npad, const GridDev &G, int pidx, double md, GapWalk &w)
-{
-    const int jhi = P_at(G, pidx) - 1;
-    const int jlo = pidx == 0 ? 1 : P_at(G, pidx - 1);
-    if (jlo == jhi) return w.at(s_tab, npad, static_cast<double>(jlo) * md);
-    return chain_range_sum(s_tab, npad, md, jlo, jhi);
-}
-
-// Scatter Chain sum in front of a warp's run when the P range is split over CTAs: the totals of the tiles
-// in front of this one (added up by the CTA's warps in a fixed order: warp w takes tiles w, w + 8, ...) plus
-// the shares of the lower warps of this tile.  sums is laid out [table][tile][9][m] (8 warp shares, then the
-// tile's total); s_buf holds kWarps * 32 doubles.  Called by all threads of the CTA (one barrier inside).
-__device__ __forceinline__ double chain_prefix(const double *sums, int trel, int n_ptiles, int ptile, int warp, int lane,
-                                               int n_m, int midx_c, double *s_buf)
-{
-    const double *tab0 = sums + static_cast<size_t>(trel) * n_ptiles * (kWarps + 1) * n_m + midx_c;
-    double part = 0.0;
-    for (int t = warp; t < ptile; t += kWarps) part += tab0[(static_cast<size_t>(t) * (kWarps + 1) + kWarps) * n_m];
-    s_buf[warp * 32 + lane] = part;
-    __syncthreads();
-    double run = 0.0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) run += s_buf[w * 32 + lane];
-    const double *mine = tab0 + static_cast<size_t>(ptile) * (kWarps + 1) * n_m;
-    for (int w = 0; w < warp; ++w) run += mine[static_cast<size_t>(w) * n_m];
-    return run;
 }
 
 }  // namespace plogp

@@ -93,7 +93,6 @@ struct FusedParams {
     int table0, n_tables_launch;
     int out_table0;  // table whose results sit at the start of the output arrays (0 unless the caller passes a window)
     OutMap om;
-    const double *s1_sums;  // [n_tables_launch][n_ptiles][9][n_m] Scatter Chain sums per warp run and per tile, or nullptr
     // segmented minima precomputed by the sweep kernel (nullptr => inline sweep)
     const double *part_time;
     const uint32_t *part_idx;
@@ -108,12 +107,17 @@ struct FusedParams {
     uint32_t *p_best_s;
 };
 
-struct S1Params {
+// Scatter half of the decision table: see scatter.cu
+struct ScatterParams {
     TableDev T;
     GridDev G;
-    int n_mtiles, n_ptiles, passes_per_tile;
-    int table0, n_tables_launch;
-    double *tile_sum;  // [n_tables_launch][n_ptiles][9][n_m]: the 8 warps' shares, then the tile's total
+    int vec;  // message sizes per lane, 1 or 2 (2: n_m even and the outputs aligned for it)
+    int n_mtiles, n_ptiles, run_len;  // CTAs along m (32 vec sizes each) and along P (kWarps runs of run_len process counts each)
+    int table0, n_tables_launch, out_table0;
+    OutMap om;
+    uint8_t *d_strategy;
+    uint32_t *d_sbytes;
+    double *d_time;
 };
 
 // Gap pre-pass (gaps.cu): g at every distinct argument of the lane <-> P kernels, once per table.
@@ -182,9 +186,8 @@ constexpr int kMaxInlineS = 64;
 
 size_t fused_smem_bytes(const TableDev &T, const GridDev &G, bool inline_sweep);
 cudaError_t launch_fused(const FusedParams &p, bool predict, cudaStream_t st);
-cudaError_t launch_scatter(const FusedParams &p, cudaStream_t st);  // decision table, Scatter strategies only
+cudaError_t launch_scatter(const ScatterParams &p, cudaStream_t st);  // decision table, Scatter strategies only
 cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st);
-cudaError_t launch_s1_tiles(const S1Params &p, cudaStream_t st);
 cudaError_t launch_decide(const DecideParams &p, cudaStream_t st);
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st);
 size_t segmin_smem_bytes(const TableDev &T, const GridDev &G);

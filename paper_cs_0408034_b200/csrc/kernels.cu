@@ -13,8 +13,6 @@
 //                  candidate lists inline or reduces the sweep kernel's partial minima, keeps the
 //                  Scatter Chain sum running along each warp's contiguous run of P, and writes either
 //                  the predicted planes or the decision table.  The general path.
-//   s1_tile_sum    per-tile and per-warp-run sums for the Scatter Chain sum when P is split over CTAs
-//                  (reduce-then-scan: the consumers add up the sums of the tiles in front of theirs).
 // Short candidate lists have faster, specialised kernels: decide.cu (Broadcast half of the decision
 // table), scatter.cu (Scatter half), segmin.cu (segmented planes of the predictions); the host routes
 // them there, so fused_kernel's own inline loop over short lists only serves callers of launch_fused
@@ -293,51 +291,6 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
 }
 
 // ------------------------------------------------------------------------------------------
-// Scatter Chain: per-tile sums of g(j m) (first phase of the reduce-then-scan over P)
-// ------------------------------------------------------------------------------------------
-
-__global__ void __launch_bounds__(kThreads) s1_tile_sum_kernel(const S1Params p)
-{
-    constexpr int R = kFusedR;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *s_tab = reinterpret_cast<double *>(smem_raw);
-    double *s_red = s_tab + 3 * p.T.npad;  // [kWarps][32]
-
-    int b = blockIdx.x;
-    const int mtile = b % p.n_mtiles;
-    b /= p.n_mtiles;
-    const int ptile = b % p.n_ptiles;
-    const int trel = b / p.n_ptiles;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int midx = mtile * 32 + lane;
-    const double md = static_cast<double>(p.G.m_list[min(midx, p.G.n_m - 1)]);
-
-    stage_table(s_tab, p.T, p.table0 + trel);
-    __syncthreads();
-
-    double acc = 0.0;
-    GapWalk walk;
-    const int run_len = p.passes_per_tile * R;
-    const int p_warp = ptile * (kWarps * run_len) + warp * run_len;
-    for (int e = 0; e < run_len; ++e)
-        if (p_warp + e < p.G.n_P) acc += s1_term(s_tab, p.T.npad, p.G, p_warp + e, md, walk);
-    // Per tile and message size: the shares of the 8 warps (each the sum over its run of process counts) and
-    // their total, laid out as [tile][9][m]; the kernels that follow turn them into the sum in front of a run.
-    s_red[warp * 32 + lane] = acc;
-    __syncthreads();
-    if (midx < p.G.n_m) {
-        double *row = p.tile_sum + (static_cast<size_t>(trel) * p.n_ptiles + ptile) * (kWarps + 1) * p.G.n_m + midx;
-        row[static_cast<size_t>(warp) * p.G.n_m] = acc;
-        if (warp == 0) {
-            double t = 0.0;
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) t += s_red[w * 32 + lane];
-            row[static_cast<size_t>(kWarps) * p.G.n_m] = t;
-        }
-    }
-}
-
-// ------------------------------------------------------------------------------------------
 // Fused evaluation: all strategies, strategy selection, stores
 // ------------------------------------------------------------------------------------------
 
@@ -437,21 +390,17 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
     const int run_len = p.passes_per_tile * R;
     const int p_warp = ptile * (kWarps * run_len) + warp * run_len;
 
-    // Scatter Chain: prefix of g(j m) in front of this thread's run = the tiles in front (sums from
-    // s1_tile_sum_kernel when the P range is split over CTAs) + the runs of the lower warps
-    double s1_run = 0.0;
-    GapWalk s1_walk;  // table interval of this thread's last Scatter Chain argument
+    // Scatter Chain: the sum of g(j m) in front of this thread's run, then a walk along it
+    double s1_run = 0.0, j_last = 0.0;
+    ChainWalk s1_walk;
     if ((mask >> 11) & 1u) {
-        if (p.s1_sums) {
-            s1_run = chain_prefix(p.s1_sums, trel, p.n_ptiles, ptile, warp, lane, p.G.n_m, midx_c, sm.tot);
-        } else {
-            double mine = 0.0;
-            for (int e = 0; e < run_len; ++e)
-                if (p_warp + e < p.G.n_P) mine += s1_term(sm.tab, npad, p.G, p_warp + e, md, s1_walk);
-            sm.tot[warp * 32 + lane] = mine;
-            __syncthreads();
-            for (int w = 0; w < warp; ++w) s1_run += sm.tot[w * 32 + lane];
-            s1_walk.i = -1;
+        const int c0 = ptile * (kWarps * run_len), e0 = min(p_warp, p.G.n_P), e1 = min(p_warp + run_len, p.G.n_P);
+        chain_front_parts(sm.tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md, c0, e0, e1, warp, sm.tot + lane, sm.tot + kWarps * 32 + lane, 32);
+        __syncthreads();
+        if (e0 < e1) {
+            s1_run = chain_front_sum(sm.tot + lane, sm.tot + kWarps * 32 + lane, 32, warp);
+            j_last = static_cast<double>(warp == 0 ? P_at(p.G, e0) - 2 : P_at(p.G, e0 - 1) - 1);
+            s1_walk.start(sm.tab, npad, (j_last + 1.0) * md);
         }
     }
 
@@ -476,7 +425,10 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
         if ((mask >> 11) & 1u) {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                if (ok[r]) s1_run += s1_term(sm.tab, npad, p.G, p0 + r, md, s1_walk);
+                if (ok[r]) {
+                    s1_run += j_last + 1.0 == pm1[r] ? s1_walk.at(sm.tab, npad, pm1[r] * md) : s1_walk.range(sm.tab, npad, md, j_last + 1.0, pm1[r]);
+                    j_last = pm1[r];
+                }
                 s1sum[r] = s1_run;
             }
         }
@@ -740,17 +692,6 @@ cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launche
         if (e == cudaSuccess) ++*launches;
     }
     return e;
-}
-
-cudaError_t launch_s1_tiles(const S1Params &p, cudaStream_t st)
-{
-    const size_t smem = (3 * static_cast<size_t>(p.T.npad) + kWarps * 32) * sizeof(double);
-    cudaError_t e = set_smem(s1_tile_sum_kernel, smem);
-    if (e != cudaSuccess) return e;
-    const long long blocks = static_cast<long long>(p.n_mtiles) * p.n_ptiles * p.n_tables_launch;
-    if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    s1_tile_sum_kernel<<<static_cast<unsigned>(blocks), kThreads, smem, st>>>(p);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st)
