@@ -49,10 +49,14 @@ int ceil_log2(int64_t P)
 // 2 floor(log2 P) + (P is no power of two): numbers the (floor, ceil) pairs in the order of P
 int log2_pair(int64_t P) { return 2 * ceil_log2(P) - ((P & (P - 1)) ? 1 : 0); }
 
-// Everything derived from a grid that the launches need; cached on the handle while the same
-// grid keeps being passed.
+// Everything derived from a grid that the launches need.  A handle keeps the plans of the last kMaxPlans grids it was
+// given (a tuner that asks for several collectives passes several masks in turn), each with its own device arrays.
+constexpr size_t kMaxPlans = 8;
 struct Plan {
-    std::vector<unsigned char> key;  // serialised grid, for the cache comparison
+    std::vector<unsigned char> key;  // serialised grid, for the cache comparison; empty: no plan
+    unsigned char *d_grid = nullptr; // the grid's device arrays
+    size_t grid_cap = 0;
+    uint64_t used = 0;               // handle's tick of its last use
     bool empty = true;
     GridDev G{};
     int n_seg = 0;
@@ -85,11 +89,11 @@ struct plogp_tables {
     TableDev T{};
     bool monotone = false;  // no table's gap ever decreases with the size (the envelope search relies on it)
     double *d_tab = nullptr, *d_lat = nullptr;
-    unsigned char *d_grid = nullptr;
-    size_t grid_cap = 0;
     unsigned char *d_ws = nullptr;
     size_t ws_cap = 0;
-    Plan plan;
+    std::vector<Plan> plans;
+    uint64_t tick = 0;
+    std::vector<unsigned char> key;  // of the grid at hand (kept for its memory)
     // optional per-kernel timing: event pairs recorded around every launch while enabled
     // host-output path: two device staging sets and a copy stream
     unsigned char *d_stage[2] = {nullptr, nullptr};
@@ -206,15 +210,15 @@ int validate_grid(const plogp_tables *h, const plogp_grid *g, int64_t *n_s_out)
     return PLOGP_OK;
 }
 
-// Builds (or reuses) the launch plan of a grid and makes its device arrays current.
-int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
+// Finds or builds the launch plan of a grid; *out is valid until the next call.
+int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **out)
 {
     if (!g || g->n_m < 0 || (g->n_m > 0 && !g->m)) return PLOGP_E_INVAL;
     if (g->P && g->n_P < 0) return PLOGP_E_INVAL;
     if ((g->strategy_mask & kSegBits) && g->s && g->n_s < 0) return PLOGP_E_INVAL;
     // ---- cache key: every input that the plan depends on ----
-    std::vector<unsigned char> key;
-    key.reserve(256 + size_t(std::max(g->n_m, 0)) * 8);
+    std::vector<unsigned char> &key = h->key;
+    key.clear();
     const int has_P = g->P != nullptr, has_s = g->s != nullptr;
     put(key, has_P);
     if (has_P) { put(key, g->n_P); put_array(key, g->P, size_t(std::max(g->n_P, 0))); }
@@ -228,19 +232,37 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
         if (has_s) { put(key, g->n_s); put_array(key, g->s, size_t(std::max<int64_t>(g->n_s, 0))); }
         else { put(key, g->s_lo); put(key, g->s_hi); put(key, g->s_step); }
     }
-    if (!h->plan.key.empty() && h->plan.key == key) return PLOGP_OK;
+    for (Plan &c : h->plans) {
+        if (c.key != key) continue;
+        c.used = ++h->tick;
+        *out = &c;
+        return PLOGP_OK;
+    }
 
     int64_t n_s64 = 0;
     int rc = validate_grid(h, g, &n_s64);
     if (rc != PLOGP_OK) return rc;
 
     Plan pl;
-    pl.key = std::move(key);
     const int n_P = g->P ? g->n_P : (g->P_hi - g->P_lo + 1);
     const int n_m = g->n_m;
     const int n_s = int(n_s64);
     pl.empty = (n_P == 0 || n_m == 0 || g->strategy_mask == 0);
-    if (pl.empty) { h->plan = std::move(pl); return PLOGP_OK; }
+    if (h->plans.capacity() < kMaxPlans) h->plans.reserve(kMaxPlans);
+    if (h->plans.size() < kMaxPlans) h->plans.emplace_back();
+    // the newest slot is still without a key, else the one that was not used for longest gives way
+    Plan &slot = h->plans.back().key.empty() ? h->plans.back()
+                                             : *std::min_element(h->plans.begin(), h->plans.end(), [](const Plan &a, const Plan &b) { return a.used < b.used; });
+    slot.key.clear();
+    auto keep = [&]() {
+        pl.d_grid = slot.d_grid; pl.grid_cap = slot.grid_cap;
+        pl.key = key;
+        pl.used = ++h->tick;
+        slot = std::move(pl);
+        *out = &slot;
+        return int(PLOGP_OK);
+    };
+    if (pl.empty) return keep();
 
     const int64_t P_hi = g->P ? g->P[n_P - 1] : g->P_hi;
     pl.n_seg = __builtin_popcount(g->strategy_mask & kSegBits);
@@ -378,29 +400,29 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
         pl.sweep_ptiles = (p_tiles + pl.sweep_wp - 1) / pl.sweep_wp;
     }
 
-    if (blob.size() > h->grid_cap) {
-        if (h->d_grid) CK(cudaFree(h->d_grid));
-        h->d_grid = nullptr;
-        h->grid_cap = 0;
-        const size_t cap = std::max<size_t>(blob.size() * 2, 4096);
-        CK(cudaMalloc(&h->d_grid, cap));
-        h->grid_cap = cap;
+    if (blob.size() > slot.grid_cap) {
+        if (slot.d_grid) CK(cudaFree(slot.d_grid));
+        slot.d_grid = nullptr;
+        slot.grid_cap = 0;
+        const size_t cap = std::max<size_t>(blob.size() + blob.size() / 4, 4096);
+        CK(cudaMalloc(&slot.d_grid, cap));
+        slot.grid_cap = cap;
     }
     // The source is pageable host memory: the runtime stages it before returning.
-    CK(cudaMemcpyAsync(h->d_grid, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(slot.d_grid, blob.data(), blob.size(), cudaMemcpyHostToDevice, st));
 
     GridDev &G = pl.G;
-    G.P_list = g->P ? reinterpret_cast<const int32_t *>(h->d_grid + off_P) : nullptr;
+    G.P_list = g->P ? reinterpret_cast<const int32_t *>(slot.d_grid + off_P) : nullptr;
     G.n_P = n_P;
     G.P_lo = g->P ? 0 : g->P_lo;
-    G.m_list = reinterpret_cast<const uint32_t *>(h->d_grid + off_m);
+    G.m_list = reinterpret_cast<const uint32_t *>(slot.d_grid + off_m);
     G.n_m = n_m;
-    G.s_list = (pl.n_seg && g->s) ? reinterpret_cast<const uint32_t *>(h->d_grid + off_s) : nullptr;
+    G.s_list = (pl.n_seg && g->s) ? reinterpret_cast<const uint32_t *>(slot.d_grid + off_s) : nullptr;
     G.n_s = pl.n_seg ? n_s : 0;
     G.s_lo = uint32_t(g->s_lo);
     G.s_step = uint32_t(g->s_step);
-    G.ns_of_m = reinterpret_cast<const int32_t *>(h->d_grid + off_ns);
-    G.k_list = short_lists ? reinterpret_cast<const double *>(h->d_grid + pl.off_k) : nullptr;
+    G.ns_of_m = reinterpret_cast<const int32_t *>(slot.d_grid + off_ns);
+    G.k_list = short_lists ? reinterpret_cast<const double *>(slot.d_grid + pl.off_k) : nullptr;
     G.mask = g->strategy_mask;
     G.k_mode = g->k_mode;
     G.lc_max = std::max(1, ceil_log2(P_hi));
@@ -432,8 +454,7 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st)
         if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(scratch)");
         h->ws_cap = pl.scratch_bytes;
     }
-    h->plan = std::move(pl);
-    return PLOGP_OK;
+    return keep();
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -452,9 +473,10 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
     int dev = 0;
     CK(cudaGetDevice(&dev));
     if (dev != h->device) return PLOGP_E_INVAL;
-    int rc = prepare(h, g, st);
-    if (rc != PLOGP_OK) { h->plan = Plan(); return rc; }
-    const Plan &pl = h->plan;
+    const Plan *plan = nullptr;
+    const int rc = prepare(h, g, st, &plan);
+    if (rc != PLOGP_OK) return rc;
+    const Plan &pl = *plan;
     if (pl.empty) return PLOGP_OK;
     // Short candidate lists with segmented strategies: the lane<->P decision kernel; everything else
     // (predictions, long lists reduced by the sweep kernel, Scatter-only grids) goes through fused_kernel.
@@ -496,9 +518,9 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         } else if (!pl.inline_sweep && pl.n_pairs > 0) {
             SweepParams sp{};
             sp.T = h->T; sp.G = pl.G;
-            sp.pair_m = reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_m);
-            sp.pair_chunk = reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_chunk);
-            sp.pair_row = reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_row);
+            sp.pair_m = reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_pair_m);
+            sp.pair_chunk = reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_pair_chunk);
+            sp.pair_row = reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_pair_row);
             sp.n_pairs = pl.n_pairs; sp.n_ptiles = pl.sweep_ptiles; sp.chunk_len = pl.chunk_len; sp.wp = pl.sweep_wp;
             sp.part_time = part_time; sp.part_idx = part_idx; sp.n_seg = pl.n_seg; sp.table0 = t0;
             int n_launches = 0;
@@ -517,7 +539,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;
             sp.vec_out = (pl.G.n_m % 2 == 0) && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
                          (!out.p_best_s || reinterpret_cast<uintptr_t>(out.p_best_s) % 8 == 0);
-            { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, st)); }
+            { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, gaps != nullptr, st)); }
             g_launches += 1;
             Gf.mask &= ~kSegBits;
             Gf.n_s = 0;
@@ -535,7 +557,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             dp.gaps = gaps; dp.gaps_stride = pl.gaps_stride;
             dp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
                          reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
-            { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, st)); }
+            { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, gaps != nullptr, st)); }
             g_launches += 1;
             Gf.mask &= 0x1C00u;
             Gf.n_s = 0;
@@ -551,7 +573,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sc.n_ptiles = pl.sc_ptiles; sc.run_len = pl.sc_run;
             sc.table0 = t0; sc.n_tables_launch = nt; sc.out_table0 = out.out_table0; sc.om = out.om;
             sc.d_strategy = out.d_strategy; sc.d_sbytes = out.d_sbytes; sc.d_time = out.d_time;
-            { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_scatter(sc, st)); }
+            { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_scatter(sc, use_decide, st)); }
             g_launches += 1;
             continue;
         }
@@ -562,9 +584,9 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         // part_time doubles as the "segmented minima come from the sweep kernel" switch
         fp.part_time = pl.inline_sweep ? nullptr : part_time;
         fp.part_idx = part_idx;
-        fp.pair_base = pl.inline_sweep ? nullptr : reinterpret_cast<const int32_t *>(h->d_grid + pl.off_pair_base);
+        fp.pair_base = pl.inline_sweep ? nullptr : reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_pair_base);
         fp.n_pairs = pl.n_pairs; fp.n_seg = pl.n_seg;
-        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, st)); }
+        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, pl.n_seg > 0 && (!pl.inline_sweep ? pl.envelope || pl.n_pairs > 0 : predict), st)); }
         g_launches += 1;
     }
     return PLOGP_OK;
@@ -677,7 +699,8 @@ int plogp_table_free(plogp_tables *h)
 {
     if (!h) return PLOGP_OK;
     int rc = PLOGP_OK;
-    void *bufs[] = {h->d_tab, h->d_lat, h->d_grid, h->d_ws, h->d_stage[0], h->d_stage[1]};
+    std::vector<void *> bufs = {h->d_tab, h->d_lat, h->d_ws, h->d_stage[0], h->d_stage[1]};
+    for (const Plan &c : h->plans) bufs.push_back(c.d_grid);
     for (int i = 0; i < 2; ++i) {
         if (h->ev_done[i]) cudaEventDestroy(h->ev_done[i]);
         if (h->ev_copied[i]) cudaEventDestroy(h->ev_copied[i]);
@@ -749,10 +772,11 @@ int plogp_select_best_host(plogp_tables *h, const plogp_grid *grid, uint8_t *h_s
     int dev = 0;
     CK(cudaGetDevice(&dev));
     if (dev != h->device) return PLOGP_E_INVAL;
-    int rc = prepare(h, grid, st);
-    if (rc != PLOGP_OK) { h->plan = Plan(); return rc; }
-    if (h->plan.empty) return PLOGP_OK;
-    const size_t cells = size_t(2) * h->plan.G.n_P * h->plan.G.n_m;  // per table
+    const Plan *plan = nullptr;
+    int rc = prepare(h, grid, st, &plan);
+    if (rc != PLOGP_OK) return rc;
+    if (plan->empty) return PLOGP_OK;
+    const size_t cells = size_t(2) * plan->G.n_P * plan->G.n_m;  // per table
     const size_t per_table = cells * 13 + 3 * 256;
     // tables per staging set: at most 512 MiB, at least one table
     const int batch = int(std::min<size_t>(h->T.n_tables, std::max<size_t>(1, (size_t(512) << 20) / per_table)));
@@ -844,10 +868,11 @@ int plogp_select_best_collective(plogp_tables *h, const plogp_grid *grid, int co
         int dev = 0;
         CK(cudaGetDevice(&dev));
         if (dev != h->device) return PLOGP_E_INVAL;
-        int rc = prepare(h, &g, st);
-        if (rc != PLOGP_OK) { h->plan = Plan(); return rc; }
-        if (h->plan.empty) return PLOGP_OK;  // no process count, no message size to carry the plan, or no strategy
-        CK(launch_barrier(h->T, h->plan.G, 0, h->T.n_tables, d_strategy, d_s_bytes, d_time, st));
+        const Plan *plan = nullptr;
+        const int rc = prepare(h, &g, st, &plan);
+        if (rc != PLOGP_OK) return rc;
+        if (plan->empty) return PLOGP_OK;  // no process count, no message size to carry the plan, or no strategy
+        CK(launch_barrier(h->T, plan->G, 0, h->T.n_tables, d_strategy, d_s_bytes, d_time, st));
         g_launches += 1;
         return PLOGP_OK;
     }
@@ -863,9 +888,10 @@ int plogp_segment_surface(plogp_tables *h, const plogp_grid *grid, double *d_sur
     int dev = 0;
     CK(cudaGetDevice(&dev));
     if (dev != h->device) return PLOGP_E_INVAL;
-    int rc = prepare(h, grid, st);
-    if (rc != PLOGP_OK) { h->plan = Plan(); return rc; }
-    const Plan &pl = h->plan;
+    const Plan *plan = nullptr;
+    const int rc = prepare(h, grid, st, &plan);
+    if (rc != PLOGP_OK) return rc;
+    const Plan &pl = *plan;
     if (pl.empty || pl.n_seg == 0 || pl.G.n_s == 0) return PLOGP_OK;
     for (int t0 = 0; t0 < h->T.n_tables; t0 += 65535) {
         SensParams sp{};
@@ -889,9 +915,10 @@ int plogp_segment_sensitivity(plogp_tables *h, const plogp_grid *grid, uint64_t 
     int dev = 0;
     CK(cudaGetDevice(&dev));
     if (dev != h->device) return PLOGP_E_INVAL;
-    int rc = prepare(h, grid, st);
-    if (rc != PLOGP_OK) { h->plan = Plan(); return rc; }
-    const Plan &pl = h->plan;
+    const Plan *plan = nullptr;
+    const int rc = prepare(h, grid, st, &plan);
+    if (rc != PLOGP_OK) return rc;
+    const Plan &pl = *plan;
     if (pl.empty || pl.n_seg == 0) return PLOGP_OK;
     // enough CTAs to fill the GPU, each with a run of process counts per warp
     const long long base_blocks = (long long)((pl.G.n_m + 31) / 32) * h->T.n_tables;

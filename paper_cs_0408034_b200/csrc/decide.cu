@@ -115,7 +115,9 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
+    dependents_may_start();
     if (!grow) stage_table(sm.tab, p.T, table);
+    else wait_for_kernel_in_front();  // the gap pre-pass
     for (int i = tid; i < n_p; i += kDecThreads) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
         sm.pm1[i] = static_cast<double>(P - 1);
@@ -474,24 +476,12 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     }
 }
 
-template <bool ENV>
-static cudaError_t launch_decide_t(const DecideParams &p, size_t smem, unsigned blocks, cudaStream_t st)
-{
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024)
-        e = cudaFuncSetAttribute(decide_kernel<ENV>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    decide_kernel<ENV><<<blocks, kDecThreads, smem, st>>>(p);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_decide(const DecideParams &p, cudaStream_t st)
+cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st)
 {
     const size_t smem = dec_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles, nullptr, nullptr);
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    return p.envelope ? launch_decide_t<true>(p, smem, static_cast<unsigned>(blocks), st)
-                      : launch_decide_t<false>(p, smem, static_cast<unsigned>(blocks), st);
+    return launch(p.envelope ? decide_kernel<true> : decide_kernel<false>, static_cast<unsigned>(blocks), 1, kDecThreads, smem, st, overlap, p);
 }
 
 }  // namespace plogp

@@ -8,6 +8,17 @@
 namespace plogp {
 
 // ------------------------------------------------------------------------------------------
+// Overlap of the kernels of one call
+// ------------------------------------------------------------------------------------------
+//
+// The first kernel of a call is launched as usual; the ones behind it may start once every CTA of the kernel in front
+// has started (dependents_may_start).  A kernel that reads what the one in front writes waits for its end first;
+// one that does not waits as the last thing thread 0 of each CTA does, so that the end of the call's last kernel is the
+// end of the call.
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_kernel_in_front() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ------------------------------------------------------------------------------------------
 // Table staging and g(x)
 // ------------------------------------------------------------------------------------------
 

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
     int *s_cnt = s_opt + p.max_coarse;                                // [32] + [32]
 
     const int midx = blockIdx.x, trel = blockIdx.y, table = p.table0 + trel;
+    dependents_may_start();
     const uint32_t m_u = p.G.m_list[midx];
     const int ns = p.G.ns_of_m[midx];
     if (ns == 0) return;  // no candidate fits: the consumer evaluates the whole message itself
@@ -208,14 +209,8 @@ size_t envelope_smem_bytes(const TableDev &T, int threads, int rep_cap, int max_
 cudaError_t launch_envelope(const EnvParams &p, int threads, cudaStream_t st)
 {
     const size_t smem = envelope_smem_bytes(p.T, threads, p.rep_cap, p.max_coarse);
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024)
-        e = cudaFuncSetAttribute(envelope_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     if (p.G.n_m <= 0 || p.n_tables_launch <= 0 || p.n_tables_launch > 65535) return cudaErrorInvalidConfiguration;
-    dim3 grid(static_cast<unsigned>(p.G.n_m), static_cast<unsigned>(p.n_tables_launch));
-    envelope_kernel<<<grid, threads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(envelope_kernel, static_cast<unsigned>(p.G.n_m), static_cast<unsigned>(p.n_tables_launch), static_cast<unsigned>(threads), smem, st, false, p);
 }
 
 }  // namespace plogp

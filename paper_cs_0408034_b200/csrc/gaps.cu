@@ -14,6 +14,7 @@ __global__ void __launch_bounds__(kGapsThreads) gaps_kernel(const GapsParams p)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *s_tab = reinterpret_cast<double *>(smem_raw);
     const int table = p.table0 + blockIdx.x;
+    dependents_may_start();
     stage_table(s_tab, p.T, table);
     __syncthreads();
     double *row = p.gaps + static_cast<size_t>(blockIdx.x) * p.stride;
@@ -28,13 +29,8 @@ __global__ void __launch_bounds__(kGapsThreads) gaps_kernel(const GapsParams p)
 
 cudaError_t launch_gaps(const GapsParams &p, cudaStream_t st)
 {
-    const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double);
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(gaps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     if (p.n_tables_launch <= 0) return cudaErrorInvalidConfiguration;
-    gaps_kernel<<<static_cast<unsigned>(p.n_tables_launch), kGapsThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(gaps_kernel, static_cast<unsigned>(p.n_tables_launch), 1, kGapsThreads, 3 * static_cast<size_t>(p.T.npad) * sizeof(double), st, false, p);
 }
 
 }  // namespace plogp

@@ -7,6 +7,23 @@
 
 namespace plogp {
 
+// Launches a kernel on a stream; overlap: it may start before the kernel in front of it has ended (device_common.cuh).
+template <typename P>
+inline cudaError_t launch(void (*kernel)(P), unsigned gx, unsigned gy, unsigned threads, size_t smem, cudaStream_t st, bool overlap, const P &params)
+{
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(gx, gy); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &attr; cfg.numAttrs = overlap ? 1u : 0u;
+    return cudaLaunchKernelEx(&cfg, kernel, params);
+}
+
 // Tables as they live in device memory.  Per table: three runs of `npad` doubles
 //   key[npad]   breakpoint sizes usable as interval starts (index <= n_bp-2), +inf beyond
 //   gap[npad]   g at the interval start
@@ -185,13 +202,13 @@ constexpr int kSweepSeeds = 128;  // log-spaced candidates that the upper bounds
 constexpr int kMaxInlineS = 64;
 
 size_t fused_smem_bytes(const TableDev &T, const GridDev &G, bool inline_sweep);
-cudaError_t launch_fused(const FusedParams &p, bool predict, cudaStream_t st);
-cudaError_t launch_scatter(const ScatterParams &p, cudaStream_t st);  // decision table, Scatter strategies only
+cudaError_t launch_fused(const FusedParams &p, bool predict, bool overlap, cudaStream_t st);
+cudaError_t launch_scatter(const ScatterParams &p, bool overlap, cudaStream_t st);  // decision table, Scatter strategies only
 cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st);
-cudaError_t launch_decide(const DecideParams &p, cudaStream_t st);
+cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st);
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st);
 size_t segmin_smem_bytes(const TableDev &T, const GridDev &G);
-cudaError_t launch_segmin(const SegminParams &p, cudaStream_t st);
+cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st);
 cudaError_t launch_gaps(const GapsParams &p, cudaStream_t st);
 cudaError_t launch_barrier(const TableDev &T, const GridDev &G, int table0, int n_tables_launch, uint8_t *d_strategy, uint32_t *d_sbytes,
                            double *d_time, cudaStream_t st);

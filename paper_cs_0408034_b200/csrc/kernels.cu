@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     const int s_end = min(ns, s_begin + p.chunk_len);
     const int n_sub = (s_end - s_begin + kSweepSub - 1) / kSweepSub;
 
+    dependents_may_start();
     stage_table(s_tab, p.T, table);
     const double L = p.T.lat[table];
 
@@ -288,6 +289,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
             p.part_idx[rbase * p.G.n_P + pidx] = bi;
         }
     }
+    if (IS9 && tid == 0) wait_for_kernel_in_front();  // the launch for ids 2 and 5; nothing of it is read here
 }
 
 // ------------------------------------------------------------------------------------------
@@ -346,7 +348,9 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
     const double md = static_cast<double>(m_u);
     const int ns = p.G.ns_of_m[midx_c];
 
+    dependents_may_start();
     stage_table(sm.tab, p.T, table);
+    if (!inline_sweep) wait_for_kernel_in_front();  // the partial minima
     __syncthreads();
 
     const double L = p.T.lat[table];
@@ -604,6 +608,7 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
         }
         if (mask & 0x1C00u) flush(1);
     }
+    if (threadIdx.x == 0) wait_for_kernel_in_front();  // nothing of it is read here unless it was waited for above
 }
 
 // ------------------------------------------------------------------------------------------
@@ -636,43 +641,24 @@ __global__ void __launch_bounds__(kThreads) fp64_probe_kernel(double *sink, int 
 // Launch wrappers
 // ------------------------------------------------------------------------------------------
 
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t bytes)
-{
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-}
-
-cudaError_t launch_fused(const FusedParams &p, bool predict, cudaStream_t st)
+cudaError_t launch_fused(const FusedParams &p, bool predict, bool overlap, cudaStream_t st)
 {
     const size_t smem = fused_smem_bytes(p.T, p.G, p.part_time == nullptr);
     const long long blocks = static_cast<long long>(p.n_mtiles) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    cudaError_t e;
-    if (predict) {
-        if ((e = set_smem(fused_kernel<true>, smem)) != cudaSuccess) return e;
-        fused_kernel<true><<<static_cast<unsigned>(blocks), kThreads, smem, st>>>(p);
-    } else {
-        if ((e = set_smem(fused_kernel<false>, smem)) != cudaSuccess) return e;
-        fused_kernel<false><<<static_cast<unsigned>(blocks), kThreads, smem, st>>>(p);
-    }
-    return cudaGetLastError();
+    return launch(predict ? fused_kernel<true> : fused_kernel<false>, static_cast<unsigned>(blocks), 1, kThreads, smem, st, overlap, p);
 }
 
 template <bool HAS2, bool HAS5, bool IS9>
-static cudaError_t launch_sweep_t(const SweepParams &p, int n_tables_launch, cudaStream_t st)
+static cudaError_t launch_sweep_t(const SweepParams &p, int n_tables_launch, bool overlap, cudaStream_t st)
 {
     constexpr int n_id = (HAS2 ? 1 : 0) + (HAS5 ? 1 : 0) + (IS9 ? 1 : 0);
     const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double) +
                         2 * kSweepSub * (sizeof(double2) + sizeof(double) + 3 * sizeof(float)) +
                         static_cast<size_t>(n_id) * kWarps * kSweepR * 32 * (sizeof(double) + sizeof(uint32_t));
-    cudaError_t e = set_smem(sweep_kernel<HAS2, HAS5, IS9>, smem);
-    if (e != cudaSuccess) return e;
     const long long bx = static_cast<long long>(p.n_pairs) * p.n_ptiles;
     if (bx <= 0 || bx > 0x7FFFFFFFLL || n_tables_launch > 65535) return cudaErrorInvalidConfiguration;
-    dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(n_tables_launch));
-    sweep_kernel<HAS2, HAS5, IS9><<<grid, kThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(sweep_kernel<HAS2, HAS5, IS9>, static_cast<unsigned>(bx), static_cast<unsigned>(n_tables_launch), kThreads, smem, st, overlap, p);
 }
 
 // Ids 2 and 5 share a launch (one set of coefficients, lines in P); id 9, whose lines are in floor(log2 P), has its own.
@@ -682,13 +668,13 @@ cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launche
     cudaError_t e = cudaSuccess;
     *launches = 0;
     if (has2 || has5) {
-        e = has2 && has5 ? launch_sweep_t<true, true, false>(p, n_tables_launch, st)
-                         : (has2 ? launch_sweep_t<true, false, false>(p, n_tables_launch, st) : launch_sweep_t<false, true, false>(p, n_tables_launch, st));
+        e = has2 && has5 ? launch_sweep_t<true, true, false>(p, n_tables_launch, false, st)
+                         : (has2 ? launch_sweep_t<true, false, false>(p, n_tables_launch, false, st) : launch_sweep_t<false, true, false>(p, n_tables_launch, false, st));
         if (e != cudaSuccess) return e;
         ++*launches;
     }
     if (has9) {
-        e = launch_sweep_t<false, false, true>(p, n_tables_launch, st);
+        e = launch_sweep_t<false, false, true>(p, n_tables_launch, has2 || has5, st);
         if (e == cudaSuccess) ++*launches;
     }
     return e;

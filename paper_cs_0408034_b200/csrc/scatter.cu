@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(kThreads, 4) scatter_kernel(const ScatterParam
 #pragma unroll
     for (int v = 0; v < V; ++v) md[v] = static_cast<double>(p.G.m_list[min(midx + v, p.G.n_m - 1)]);
 
+    dependents_may_start();
     stage_table(s_tab, p.T, table);
     __syncthreads();
     const double L = p.T.lat[table];
@@ -157,29 +158,26 @@ __global__ void __launch_bounds__(kThreads, 4) scatter_kernel(const ScatterParam
         if (CONTIG) { ++P; pm1 += 1.0; }
         else j_last = pm1;
     }
+    if (threadIdx.x == 0) wait_for_kernel_in_front();  // the Broadcast half; nothing of it is read here
 }
 
 template <bool CONTIG, bool ALL, int V>
-static cudaError_t launch_scatter_t(const ScatterParams &p, cudaStream_t st)
+static cudaError_t launch_scatter_t(const ScatterParams &p, bool overlap, cudaStream_t st)
 {
     const size_t smem = (3 * static_cast<size_t>(p.T.npad) + static_cast<size_t>(p.G.lc_max) * 32 * V + 2 * kWarps * 32 * V) * sizeof(double);
     const long long blocks = static_cast<long long>(p.n_mtiles) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024) e = cudaFuncSetAttribute(scatter_kernel<CONTIG, ALL, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    scatter_kernel<CONTIG, ALL, V><<<static_cast<unsigned>(blocks), kThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(scatter_kernel<CONTIG, ALL, V>, static_cast<unsigned>(blocks), 1, kThreads, smem, st, overlap, p);
 }
 
 template <int V>
-static cudaError_t launch_scatter_v(const ScatterParams &p, cudaStream_t st)
+static cudaError_t launch_scatter_v(const ScatterParams &p, bool overlap, cudaStream_t st)
 {
     const bool all = (p.G.mask & 0x1C00u) == 0x1C00u, contig = p.G.P_list == nullptr;
-    if (contig) return all ? launch_scatter_t<true, true, V>(p, st) : launch_scatter_t<true, false, V>(p, st);
-    return all ? launch_scatter_t<false, true, V>(p, st) : launch_scatter_t<false, false, V>(p, st);
+    if (contig) return all ? launch_scatter_t<true, true, V>(p, overlap, st) : launch_scatter_t<true, false, V>(p, overlap, st);
+    return all ? launch_scatter_t<false, true, V>(p, overlap, st) : launch_scatter_t<false, false, V>(p, overlap, st);
 }
 
-cudaError_t launch_scatter(const ScatterParams &p, cudaStream_t st) { return p.vec == 2 ? launch_scatter_v<2>(p, st) : launch_scatter_v<1>(p, st); }
+cudaError_t launch_scatter(const ScatterParams &p, bool overlap, cudaStream_t st) { return p.vec == 2 ? launch_scatter_v<2>(p, overlap, st) : launch_scatter_v<1>(p, overlap, st); }
 
 }  // namespace plogp

@@ -112,7 +112,9 @@ __global__ void __launch_bounds__(kSegThreads, 2) segmin_kernel(const SegminPara
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
+    dependents_may_start();
     if (!grow) stage_table(sm.tab, p.T, table);
+    else wait_for_kernel_in_front();  // the gap pre-pass
     for (int i = tid; i < kSegTileP; i += kSegThreads) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
         sm.lf[i] = static_cast<double>(31 - __clz(P));
@@ -337,17 +339,11 @@ __global__ void __launch_bounds__(kSegThreads, 2) segmin_kernel(const SegminPara
 
 size_t segmin_smem_bytes(const TableDev &T, const GridDev &G) { return seg_layout(T.npad, G.n_s, nullptr, nullptr); }
 
-cudaError_t launch_segmin(const SegminParams &p, cudaStream_t st)
+cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
 {
-    const size_t smem = segmin_smem_bytes(p.T, p.G);
-    cudaError_t e = cudaSuccess;
-    if (smem > 48 * 1024)
-        e = cudaFuncSetAttribute(segmin_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    segmin_kernel<<<static_cast<unsigned>(blocks), kSegThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(segmin_kernel, static_cast<unsigned>(blocks), 1, kSegThreads, segmin_smem_bytes(p.T, p.G), st, overlap, p);
 }
 
 }  // namespace plogp

@@ -205,8 +205,26 @@ def _as_grid(grid) -> GridArgs:
 
 def _stream_ptr(stream) -> int:
     import torch
-    st = torch.cuda.current_stream() if stream is None else stream
-    return int(st.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # the stream's handle without a Stream object around it (0.2 us instead of 3.4 on every call)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+BCAST_MASK, SCATTER_MASK, ALL_MASK, SEG_MASK = 0x3FF, 0x1C00, (1 << N_STRATEGIES) - 1, (1 << 2) | (1 << 5) | (1 << 9)
+REDUCE_MASK, BARRIER_MASK = 0x2ED, 0xC9  # printed ids that have a Reduce / Barrier counterpart
+
+
+def _new(shape, dtype, fill, whole):
+    """A new device tensor: left as it is where the call writes every element (``whole``), else filled."""
+    import torch
+    return torch.empty(shape, dtype=dtype, device="cuda") if whole else torch.full(shape, fill, dtype=dtype, device="cuda")
+
+
+def _new_decision(shape, whole) -> "DecisionTable":
+    import torch
+    return DecisionTable(_new(shape, torch.uint8, 255, whole), _new(shape, torch.int32, 0, whole),
+                         _new(shape, torch.float64, float("nan"), whole))
 
 
 @dataclass
@@ -227,9 +245,9 @@ def predict(tables: Tables, grid, out: Optional[Prediction] = None, stream=None,
     import torch
     g = _as_grid(grid)
     if out is None:
-        shape = (tables.n_tables, N_STRATEGIES, g.n_P, g.n_m)
-        time = torch.full(shape, float("nan"), dtype=torch.float64, device="cuda")
-        best = torch.zeros((tables.n_tables, 3, g.n_P, g.n_m), dtype=torch.int32, device="cuda") if want_best_s else None
+        mask = g.struct.strategy_mask
+        time = _new((tables.n_tables, N_STRATEGIES, g.n_P, g.n_m), torch.float64, float("nan"), mask == ALL_MASK)
+        best = _new((tables.n_tables, 3, g.n_P, g.n_m), torch.int32, 0, mask & SEG_MASK == SEG_MASK) if want_best_s else None
         out = Prediction(time, best)
     _check(lib.plogp_predict(tables.handle, g.ref, out.time.data_ptr(),
                              None if out.best_s is None else out.best_s.data_ptr(), _stream_ptr(stream)),
@@ -238,18 +256,15 @@ def predict(tables: Tables, grid, out: Optional[Prediction] = None, stream=None,
 
 
 def alloc_decision(n_tables: int, n_P: int, n_m: int) -> DecisionTable:
-    import torch
-    shape = (n_tables, 2, n_P, n_m)
-    return DecisionTable(torch.full(shape, 255, dtype=torch.uint8, device="cuda"),
-                         torch.zeros(shape, dtype=torch.int32, device="cuda"),
-                         torch.full(shape, float("nan"), dtype=torch.float64, device="cuda"))
+    return _new_decision((n_tables, 2, n_P, n_m), whole=False)
 
 
 def select_best(tables: Tables, grid, out: Optional[DecisionTable] = None, stream=None) -> DecisionTable:
     """``plogp_select_best``: best strategy, its segment size and predicted time per (collective, P, m)."""
     g = _as_grid(grid)
     if out is None:
-        out = alloc_decision(tables.n_tables, g.n_P, g.n_m)
+        mask = g.struct.strategy_mask
+        out = _new_decision((tables.n_tables, 2, g.n_P, g.n_m), bool(mask & BCAST_MASK) and bool(mask & SCATTER_MASK))
     _check(lib.plogp_select_best(tables.handle, g.ref, out.strategy.data_ptr(), out.s_bytes.data_ptr(),
                                  out.time.data_ptr(), _stream_ptr(stream)), "plogp_select_best")
     return out
@@ -330,7 +345,7 @@ def segment_surface(tables: Tables, grid, out=None, stream=None):
     import torch
     g = _as_grid(grid)
     if out is None:
-        out = torch.full((tables.n_tables, 3, g.n_P, g.n_m, n_candidates(g)), float("inf"), dtype=torch.float64, device="cuda")
+        out = _new((tables.n_tables, 3, g.n_P, g.n_m, n_candidates(g)), torch.float64, float("inf"), g.struct.strategy_mask & SEG_MASK == SEG_MASK)
     _check(lib.plogp_segment_surface(tables.handle, g.ref, out.data_ptr(), _stream_ptr(stream)), "plogp_segment_surface")
     return out
 
@@ -341,8 +356,9 @@ def segment_sensitivity(tables: Tables, grid, s_fixed: int, pred: Optional[Predi
     import torch
     g = _as_grid(grid)
     shape = (tables.n_tables, 3, g.n_P, g.n_m)
-    fixed = torch.full(shape, float("nan"), dtype=torch.float64, device="cuda")
-    ratio = None if pred is None else torch.full(shape, float("nan"), dtype=torch.float64, device="cuda")
+    whole = g.struct.strategy_mask & SEG_MASK == SEG_MASK
+    fixed = _new(shape, torch.float64, float("nan"), whole)
+    ratio = None if pred is None else _new(shape, torch.float64, float("nan"), whole)
     _check(lib.plogp_segment_sensitivity(tables.handle, g.ref, int(s_fixed), None if pred is None else pred.time.data_ptr(),
                                          fixed.data_ptr(), None if ratio is None else ratio.data_ptr(), _stream_ptr(stream)),
            "plogp_segment_sensitivity")
@@ -365,12 +381,10 @@ GATHER, REDUCE, BARRIER = 2, 3, 4
 def select_best_collective(tables: Tables, grid, collective: int, stream=None) -> DecisionTable:
     """``plogp_select_best_collective``: decision table of a derived collective (GATHER, REDUCE: [n_tables][n_P][n_m];
     BARRIER: [n_tables][n_P])."""
-    import torch
     g = _as_grid(grid)
     shape = (tables.n_tables, g.n_P) if collective == BARRIER else (tables.n_tables, g.n_P, g.n_m)
-    out = DecisionTable(torch.full(shape, 255, dtype=torch.uint8, device="cuda"),
-                        torch.zeros(shape, dtype=torch.int32, device="cuda"),
-                        torch.full(shape, float("nan"), dtype=torch.float64, device="cuda"))
+    out = _new_decision(shape, bool(g.struct.strategy_mask & {GATHER: SCATTER_MASK, REDUCE: REDUCE_MASK, BARRIER: BARRIER_MASK}.get(collective, 0))
+                        and g.n_m > 0)
     _check(lib.plogp_select_best_collective(tables.handle, g.ref, int(collective), out.strategy.data_ptr(), out.s_bytes.data_ptr(),
                                             out.time.data_ptr(), _stream_ptr(stream)), "plogp_select_best_collective")
     return out
