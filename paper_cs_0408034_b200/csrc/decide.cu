@@ -49,11 +49,12 @@ struct DecSmem {
     double2 *line;    // [kDecMG][slots]: coefficients by slot
     float *x;         // [n_p]: P-1 rounded down
     float *fa, *fc;   // [kDecWarps][cap]: the lines' coefficients rounded down, for the warp's current message size
-    double *q;        // [kDecWarps][n_s]: g(s) k, for the warp's current message size
+    double *q;        // [kDecWarps][cap_q]: g(s) k, for the warp's current message size
+    float *fq;        // [kDecWarps][cap_q]: the same rounded down
     uint32_t *sval;   // [256]: segment sizes by candidate index; [kCandNone] = 0
     uint16_t *code;   // [kDecMG][slots]: id << 8 | candidate index
     uint8_t *pair, *pos;  // [n_p]: pair of a process count; [kDecMG][pos_stride]: winners
-    int cap, slots, pos_stride;
+    int cap, cap_q, slots, pos_stride;
 };
 
 __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
@@ -63,22 +64,22 @@ __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a *
 __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int tiles, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(2 * nsv + 4, kStep), slots = cap + n_pairs, n_p = tiles * kDecTileP, pos_stride = n_p + 4;
+    const int cap = round_up(2 * nsv + 4, kStep), cap_q = round_up(nsv, 4), slots = cap + n_pairs, n_p = tiles * kDecTileP, pos_stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
                  o_line = take(size_t(kDecMG) * slots * 16), o_fa = take(size_t(kDecWarps) * cap * 4), o_fc = take(size_t(kDecWarps) * cap * 4),
-                 o_q = take(size_t(kDecWarps) * nsv * 8), o_sv = take(256 * 4), o_code = take(size_t(kDecMG) * slots * 2),
+                 o_q = take(size_t(kDecWarps) * cap_q * 8), o_fq = take(size_t(kDecWarps) * cap_q * 4), o_sv = take(256 * 4), o_code = take(size_t(kDecMG) * slots * 2),
                  o_pair = take(n_p), o_pos = take(size_t(kDecMG) * pos_stride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
         o->gm = reinterpret_cast<double *>(base + o_gm); o->pm1 = reinterpret_cast<double *>(base + o_pm);
         o->line = reinterpret_cast<double2 *>(base + o_line);
         o->fa = reinterpret_cast<float *>(base + o_fa); o->fc = reinterpret_cast<float *>(base + o_fc);
-        o->q = reinterpret_cast<double *>(base + o_q); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
+        o->q = reinterpret_cast<double *>(base + o_q); o->fq = reinterpret_cast<float *>(base + o_fq); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
         o->code = reinterpret_cast<uint16_t *>(base + o_code); o->pair = base + o_pair; o->pos = base + o_pos;
         o->x = reinterpret_cast<float *>(base + o_x);
-        o->cap = cap; o->slots = slots; o->pos_stride = pos_stride;
+        o->cap = cap; o->cap_q = cap_q; o->slots = slots; o->pos_stride = pos_stride;
     }
     return off;
 }
@@ -92,7 +93,7 @@ __device__ __forceinline__ int pair_of(int P) { return 2 * (31 - __clz(P)) + ((P
 
 // ENV: lower-envelope search (DecideParams::envelope), compiled apart so that the exhaustive kernel carries none of it.
 template <bool ENV>
-__global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecideParams p)
+__global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecideParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
@@ -164,17 +165,33 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
     const double fa = fid == 3 ? L : (fid == 4 ? rdv : 0.0);
     const double fc = fid == 0 ? L : (fid == 1 ? rdv : 0.0);
     const uint16_t fcode = static_cast<uint16_t>(idc(fid) | kCandNone);
-    const int pair_w = n_pairs <= 16 ? 16 : 32, pair_step = n_pairs <= 16 ? 2 : 1;
     float *const la = sm.fa + warp * sm.cap, *const lc = sm.fc + warp * sm.cap;
-    double *const lq = sm.q + warp * max(p.G.n_s, 1);
+    double *const lq = sm.q + warp * sm.cap_q;
+    float *const lqf = sm.fq + warp * sm.cap_q;
+
+    // what a message size reads from global memory is fetched while the one before it is worked on
+    const int n_s = p.G.n_s;
+    int ns_next = 0;
+    uint32_t m_next = 0;
+    double k_next[2] = {1.0, 1.0};  // Section 2's k of this lane's candidates, from the host's table
+    auto fetch = [&](int mi) {
+        if (mi >= n_mi) return;
+        const int midx = m0 + mi;
+        ns_next = p.G.ns_of_m[midx];
+        m_next = p.G.m_list[midx];
+        const double *krow = p.G.k_list + static_cast<size_t>(midx) * n_s;
+        if (lane < n_s) k_next[0] = krow[lane];
+        if (lane + 32 < n_s) k_next[1] = krow[lane + 32];
+    };
+    fetch(warp);
 
     for (int mi = warp; mi < n_mi; mi += kDecWarps) {
-        const int midx = m0 + mi;
-        const int ns = p.G.ns_of_m[midx];
+        const int ns = ns_next;
+        const uint32_t m_u = m_next;
+        const double k_of[2] = {k_next[0], k_next[1]};
+        fetch(mi + kDecWarps);
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
         const double gm = sm.gm[mi];
-        const uint32_t m_u = p.G.m_list[midx];
-        const double *krow = p.G.k_list + static_cast<size_t>(midx) * p.G.n_s;
         double2 *const line = sm.line + mi * sm.slots;
         uint16_t *const code = sm.code + mi * sm.slots;
         // Lower-envelope search (p.envelope, tables whose gaps never decrease): ids 2 and 9 keep only the candidate
@@ -188,8 +205,11 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
             const double x_first = sm.pm1[0], x_last = sm.pm1[n_valid - 1];
             double qb = CUDART_INF, tf = CUDART_INF, tl = CUDART_INF;
             int qc = kIntMax, ef = kIntMax, el = kIntMax;
-            for (int c = lane; c < ns; c += 32) {
-                const double gsv = sm.gs[c], k = krow[c];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = lane + 32 * h;
+                if (c >= ns) break;
+                const double gsv = sm.gs[c], k = k_of[h];
                 const double Q = gsv * k, B = gsv + L, C = gsv * (k - 1.0);
                 if (Q < qb) { qb = Q; qc = c; }
                 const double t1 = fma(x_first, B, C), t2 = fma(x_last, B, C);
@@ -212,6 +232,9 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
         unsigned pilot[kPilots];  // bound (without its last 8 bits) and slot in one number
 #pragma unroll
         for (int i = 0; i < kPilots; ++i) pilot[i] = 0xFFFFFFFFu;
+        unsigned q_pilot = 0xFFFFFFFFu;  // the smallest g(s) k, likewise
+        double t_two = CUDART_INF;       // P = 2: this lane's best line, exactly
+        unsigned at_two = 0xFFu;
         auto put = [&](int slot, double a, double c, uint32_t cd, bool twin) {
             const float af = __double2float_rd(a), cf = __double2float_rd(c);
             line[slot] = make_double2(a, c);
@@ -221,61 +244,79 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
 #pragma unroll
             for (int i = 0; i < kPilots; ++i)
                 pilot[i] = min(pilot[i], (__float_as_uint(__fmaf_rd(x_pilot[i], af, cf)) & ~0xFFu) | static_cast<unsigned>(slot));
+            if (two) {
+                const double t = fma(1.0, a, c);
+                if (t < t_two || (t == t_two && static_cast<unsigned>(slot) < at_two)) { t_two = t; at_two = static_cast<unsigned>(slot); }
+            }
         };
         if (f_on) put((fid < 3 ? 0 : o3 - n01) + __popc(mask & 0x1Bu & ((1u << fid) - 1u)), gm + fa, fc, fcode, false);
         if (lane >= 16 && n1 + lane - 16 < round_up(n1, kStep)) {  // padding: the bound is +inf
             la[n1 + lane - 16] = 0.0f;
             lc[n1 + lane - 16] = CUDART_INF_F;
         }
-        for (int c = lane; c < nsv; c += 32) {
-            // Section 2's k and the line coefficients of Table 1's segmented rows
+        if (lane >= 16 && lane < 20 && nsv + lane - 16 < round_up(nsv, 4)) lqf[nsv + lane - 16] = CUDART_INF_F;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            // the line coefficients of Table 1's segmented rows
+            const int c = lane + 32 * h;
+            if (c >= nsv) break;
             double gsv = gm, k = 1.0;
             uint32_t cand = kCandWhole;
             bool whole = true;  // one segment: the line of the unsegmented sibling, whose lower id wins the tie
             if (ns > 0) {
                 gsv = sm.gs[c];
-                k = krow[c];  // Section 2's k, from the host's table
+                k = k_of[h];
                 cand = static_cast<uint32_t>(c);
                 whole = sm.sval[c] == m_u;
             }
             const double Q = gsv * k;
+            const float Qf = __double2float_rd(Q);
             lq[c] = Q;
+            lqf[c] = Qf;
+            q_pilot = min(q_pilot, (__float_as_uint(Qf) & ~0xFFu) | static_cast<unsigned>(c));
             if (has2 && (!env || c == q_c)) put(o2 + (env ? 0 : c), Q, L, code2 | cand, whole && has0);  // (P-1) (g(s) k) + L
             if (has5 && (!env || (c >= lo5 && c < lo5 + n5)))                                            // (P-1) (g(s) + L) + g(s) (k-1)
                 put(o5 + (env ? c - lo5 : c), gsv + L, gsv * (k - 1.0), code5 | cand, whole && has3);
         }
 #pragma unroll
         for (int i = 0; i < kPilots; ++i) pilot[i] = __reduce_min_sync(kFull, pilot[i]) & 0xFFu;
+        q_pilot = env ? static_cast<unsigned>(q_c) : __reduce_min_sync(kFull, q_pilot) & 0xFFu;
+        if ((q_pilot & 31u) == static_cast<unsigned>(lane)) lqf[q_pilot] = CUDART_INF_F;  // written by this lane itself above
+        if (two && n1 > 0) {
+            const int h = __reduce_min_sync(kFull, at_two == 0xFFu ? kIntMax : hi32(t_two));
+            const bool on_h = at_two != 0xFFu && hi32(t_two) == h;
+            const unsigned l = __reduce_min_sync(kFull, on_h ? static_cast<unsigned>(__double2loint(t_two)) : 0xFFFFFFFFu);
+            at_two = __reduce_min_sync(kFull, on_h && static_cast<unsigned>(__double2loint(t_two)) == l ? at_two : 0xFFu);
+            t_two = __hiloint2double(h, static_cast<int>(l));
+        }
         __syncwarp();
 
-        // ---- the best of ids 6 to 9 per (floor, ceil) pair: half a warp where it is enough, the halves split the candidates ----
+        // ---- the best of ids 6 to 9 per (floor, ceil) pair, lanes <-> pairs ----
         if (any_log)
-        for (int b0 = 0; b0 < n_pairs; b0 += pair_w) {
-            const int pr = b0 + (lane & (pair_w - 1)), half = pair_w == 16 ? lane >> 4 : 0;
-            const int li = pair0 + pr;
+        for (int b0 = 0; b0 < n_pairs; b0 += 32) {
+            const int pr = b0 + lane, li = pair0 + min(pr, n_pairs - 1);
             const double lf = static_cast<double>(li >> 1), lcd = static_cast<double>((li >> 1) + (li & 1)), lcL = lcd * L;
             double t = CUDART_INF;
             uint32_t cd = 0;
-            if (has9) {  // floor(log2 P) g(s) k + ceil(log2 P) L; the half-warps take every other candidate
-                double tc = CUDART_INF;
-                int cb = 0x1000;
-                if (env) {
-                    tc = fma(lf, lq[q_c], lcL);
-                    cb = q_c;
-                } else {
-#pragma unroll 4
-                    for (int c = half; c < nsv; c += pair_step) {
-                        const double v = fma(lf, lq[c], lcL);
-                        if (v < tc) { tc = v; cb = c; }
+            if (has9) {  // floor(log2 P) g(s) k + ceil(log2 P) L: the smallest g(s) k, and bounds of all others
+                unsigned cb = q_pilot;
+                t = fma(lf, lq[cb], lcL);
+                if (!env) {
+                    const f32x2 x2 = splat2(static_cast<float>(li >> 1)), c2 = splat2(__double2float_rd(lcL));
+                    float low = CUDART_INF_F;
+                    for (int c = 0; c < nsv; c += 4) {
+                        const f32x2x2 qq = *reinterpret_cast<const f32x2x2 *>(lqf + c);
+                        low = min_with2(min_with2(low, fma2_down(x2, qq.x, c2)), fma2_down(x2, qq.y, c2));
                     }
-                    if (pair_w == 16) {
-                        const double t2 = __shfl_xor_sync(kFull, tc, 16);
-                        const int cb2 = __shfl_xor_sync(kFull, cb, 16);
-                        if (t2 < tc || (t2 == tc && cb2 < cb)) { tc = t2; cb = cb2; }
+                    if (__any_sync(kFull, low <= __double2float_ru(t))) {
+#pragma unroll 1
+                        for (int c = 0; c < nsv; ++c) {
+                            const double v = fma(lf, lq[c], lcL);
+                            if (v <= t && (v < t || static_cast<unsigned>(c) < cb)) { t = v; cb = static_cast<unsigned>(c); }
+                        }
                     }
                 }
-                t = tc;
-                cd = code9 | (ns > 0 ? static_cast<uint32_t>(min(cb, ns - 1)) : kCandWhole);
+                cd = code9 | (ns > 0 ? cb : kCandWhole);
             }
             // lower ids win ties: in descending order, '<='
             if (has8) {  // Binomial Tree Rendezvous: floor(log2 P) g(m) + ceil(log2 P) rdv
@@ -290,27 +331,13 @@ __global__ void __launch_bounds__(kDecThreads, 5) decide_kernel(const DecidePara
                 const double v = lcd * fma(2.0, gm, L);
                 if (v <= t) { t = v; cd = idc(6) | kCandNone; }
             }
-            if (half == 0 && pr < n_pairs) {
+            if (pr < n_pairs) {
                 line[sm.cap + pr] = make_double2(0.0, t);
                 code[sm.cap + pr] = static_cast<uint16_t>(cd);
             }
         }
 
         // ---- the pilots leave the lists: their own bounds would always pass ----
-        double t_two = CUDART_INF;
-        unsigned at_two = 0xFFu;
-        if (two && n1 > 0) {  // P = 2: the best line, exactly, lanes <-> lines
-            for (int u = lane; u < n1; u += 32) {
-                const double2 v = line[u];
-                const double t = fma(1.0, v.x, v.y);
-                if (t < t_two || at_two == 0xFFu) { t_two = t; at_two = static_cast<unsigned>(u); }
-            }
-            const int h = __reduce_min_sync(kFull, at_two == 0xFFu ? kIntMax : hi32(t_two));
-            const bool on_h = at_two != 0xFFu && hi32(t_two) == h;
-            const unsigned l = __reduce_min_sync(kFull, on_h ? static_cast<unsigned>(__double2loint(t_two)) : 0xFFFFFFFFu);
-            at_two = __reduce_min_sync(kFull, on_h && static_cast<unsigned>(__double2loint(t_two)) == l ? at_two : 0xFFu);
-            t_two = __hiloint2double(h, static_cast<int>(l));
-        }
         if (n1 > 0 && lane < kPilots) {
             unsigned mine = pilot[0];
 #pragma unroll
