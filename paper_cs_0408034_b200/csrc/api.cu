@@ -533,11 +533,11 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             // come from the lane<->P kernel; fused_kernel then writes the closed-form planes only.
             SegminParams sp{};
             sp.T = h->T; sp.G = pl.G;
-            sp.n_mgroups = (pl.G.n_m + kSegMG - 1) / kSegMG; sp.n_ptiles = (pl.G.n_P + kSegTileP - 1) / kSegTileP;
+            sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs;
             sp.table0 = t0; sp.n_tables_launch = nt; sp.out_table0 = out.out_table0;
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
             sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;
-            sp.vec_out = (pl.G.n_m % 2 == 0) && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
+            sp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
                          (!out.p_best_s || reinterpret_cast<uintptr_t>(out.p_best_s) % 8 == 0);
             { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, gaps != nullptr, st)); }
             g_launches += 1;

@@ -86,9 +86,6 @@ __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int
 
 __device__ __forceinline__ int hi32(double x) { return __double2hiint(x); }
 
-// (floor, ceil) of log2 P as one number that grows with P: 2 floor + (P is no power of two)
-__device__ __forceinline__ int pair_of(int P) { return 2 * (31 - __clz(P)) + ((P & (P - 1)) != 0 ? 1 : 0); }
-
 }  // namespace
 
 // ENV: lower-envelope search (DecideParams::envelope), compiled apart so that the exhaustive kernel carries none of it.

@@ -70,6 +70,9 @@ __device__ __forceinline__ uint32_t s_at(const GridDev &G, int si)
     return G.s_list ? G.s_list[si] : G.s_lo + static_cast<uint32_t>(si) * G.s_step;
 }
 
+// (floor, ceil) of log2 P as one number that grows with P: 2 floor + (P is no power of two)
+__device__ __forceinline__ int pair_of(int P) { return 2 * (31 - __clz(P)) + ((P & (P - 1)) != 0 ? 1 : 0); }
+
 // k of Section 2: number of segments of size s in a message of m bytes.
 __device__ __forceinline__ uint32_t segments(uint32_t m, uint32_t s, int k_mode)
 {

@@ -181,15 +181,17 @@ struct SegminParams {
     int gaps_stride;
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16-byte aligned times, 8-byte aligned sizes)
     int n_mgroups, n_ptiles;
+    int mg, tiles, n_pairs;  // as in DecideParams
     int table0, n_tables_launch, out_table0;
     double *p_time;      // [n_tables][13][n_P][n_m]: planes 2, 5, 9 are written
     uint32_t *p_best_s;  // [n_tables][3][n_P][n_m], or nullptr
 };
-constexpr int kSegThreads = 256;
+constexpr int kSegThreads = 128;
 constexpr int kSegWarps = kSegThreads / 32;
 constexpr int kSegR = 8;                 // process counts per thread
-constexpr int kSegTileP = 32 * kSegR;    // process counts per CTA
-constexpr int kSegMG = 16;               // message sizes per CTA, two per warp
+constexpr int kSegTileP = 32 * kSegR;    // process counts per tile
+constexpr int kSegMG = 16;               // message sizes per CTA (at most), split over the warps
+static_assert(kSegTileP == kDecTileP && kSegMG == kDecMG && kSegThreads == kDecThreads, "the host gives both lane <-> P kernels the same tiling");
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -207,7 +209,6 @@ cudaError_t launch_scatter(const ScatterParams &p, bool overlap, cudaStream_t st
 cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st);
 cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st);
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st);
-size_t segmin_smem_bytes(const TableDev &T, const GridDev &G);
 cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st);
 cudaError_t launch_gaps(const GapsParams &p, cudaStream_t st);
 cudaError_t launch_barrier(const TableDev &T, const GridDev &G, int table0, int n_tables_launch, uint8_t *d_strategy, uint32_t *d_sbytes,

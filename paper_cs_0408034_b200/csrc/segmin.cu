@@ -3,100 +3,83 @@
 // of the model over the candidate segment sizes and the smallest size that attains it.
 //
 // Same building blocks as decide_kernel (decide.cu), with one running minimum per strategy instead of one
-// over all of them.  One CTA (8 warps) owns one table, 16 consecutive message sizes (two per warp) and a tile
-// of 256 process counts (lane + 32 r, r = 0..7).  For a fixed message size the models are lines,
+// over all of them.  One CTA owns one table, up to 16 consecutive message sizes and one or two tiles of 256 process
+// counts (lane + 32 r, r = 0..7); its four warps split the message sizes.  For a fixed message size the models are
 //     id 2: fma(P-1, Q, L)      id 9: fma(floor(log2 P), Q, ceil(log2 P) L)      Q = g(s) k
 //     id 5: fma(P-1, B, C)      B = g(s) + L, C = g(s) (k-1)
-// so a warp first builds the coefficient lists of its message sizes (lanes <-> candidates); then the CTA takes
-// one strategy at a time: every warp sweeps that strategy's list for its message sizes, the results are staged
-// in shared memory as [m][P], and the whole CTA writes the strategy's plane out as rows of 16 consecutive m
-// (128-byte row segments) before the next strategy reuses the staging area.  In a sweep
-// every cell is evaluated with one DFMA and compared with the running minimum on the high
-// 32 bits only, in the integer pipe (times are non-negative); a group of four candidates in which some cell
-// can reach the minimum is re-evaluated with the exact comparison, (time, candidate) in lexicographic order,
-// for the rows of 32 process counts that need it.  The running minima start from a pilot: for ids 2 and 9 the
-// candidate with the smallest Q, which is their winner for every P (the sweep still visits every cell), for
-// id 5 the winner at the tile's middle process count.  The outputs are the prediction planes
+// so a warp builds the coefficient lists of a message size (lanes <-> candidates), searches id 9 once per
+// (floor, ceil) pair of log2 P (lanes <-> pairs) and sweeps ids 2 and 5 over the process counts: the running minimum
+// starts from pilots (id 2: the smallest Q; id 5: the winners at four process counts), every cell of every other
+// candidate is evaluated as a lower bound in FP32 (coefficients, process count and fused multiply-add rounded down, two
+// candidates per instruction), and rows of 32 process counts in which some bound is not above the running minimum are
+// searched exactly, (time, candidate) in lexicographic order.  Results are those of the exhaustive FP64 search, bit for
+// bit.  The winners are staged as candidate numbers, one byte per cell; the write-out, rows of consecutive m per process
+// count, evaluates the winner's model again (the same fma, the same double).  The outputs are the prediction planes
 // time[table][13][P][m] and best_s[table][3][P][m].
 #include "device_common.cuh"
 
 #include <algorithm>
-#include <type_traits>
 
 namespace plogp {
 
 namespace {
 
-constexpr int R = kSegR, U = 4;
+constexpr int R = kSegR;
+constexpr int kPilots = 4;
+constexpr int kStep = 16;  // candidates per vote of the exact search
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kIntMax = 0x7FFFFFFF;
-constexpr int kStride = kSegTileP + 1;   // doubles per staged row: the transposed reads stay conflict-free
-constexpr int kIStride = kSegTileP + 2;  // 16-bit candidate indices per staged row
-constexpr uint32_t kWhole = 0xFFFEu;     // no candidate fits: the whole message in one segment
-static_assert(kMaxInlineS <= 64, "warp_argmin_pilot keeps a candidate index in six bits");
+static_assert(kMaxInlineS <= 64, "a lane builds at most two candidates");
+
+__host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
 struct SegSmem {
-    double *tab, *gs, *gm, *lf, *lc, *pm1, *lq, *qp, *st_time;
-    double2 *l5, *ep;
+    double *tab, *gs, *gm, *pm1;
+    double2 *l5;      // [kSegMG][cap]: (B, C)
+    double *q;        // [kSegMG][cap]: Q
+    double *t9;       // [kSegMG][n_pairs]: id 9's minimum
+    float *x;         // [n_p]: P-1 rounded down
+    float *fb, *fc, *fq;  // [kSegWarps][cap]: the lists of the warp's current message size rounded down, without the pilots
     uint32_t *sval;
-    uint16_t *st_idx;
-    int *pc;
-    int cap;
+    uint8_t *i9;      // [kSegMG][n_pairs]: id 9's winner
+    uint8_t *pair;    // [n_p]: pair of a process count
+    uint8_t *pos2, *pos5;  // [kSegMG][stride]: winners of ids 2 and 5
+    int cap, stride;
 };
 
-__host__ __device__ inline size_t seg_layout(int npad, int n_s, unsigned char *base, SegSmem *o)
+__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int tiles, unsigned char *base, SegSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = (nsv + U - 1) / U * U;
+    const int cap = round_up(nsv, kStep), n_p = tiles * kSegTileP, stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
-    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_sv = take(size_t(nsv) * 4),
-                 o_gm = take(kSegMG * 8), o_lf = take(kSegTileP * 8), o_lc = take(kSegTileP * 8), o_pm = take(kSegTileP * 8),
-                 o_lq = take(size_t(kSegMG) * cap * 8), o_l5 = take(size_t(kSegMG) * cap * 16),
-                 o_qp = take(kSegMG * 8), o_ep = take(kSegMG * 16), o_pc = take(2 * kSegMG * 4),
-                 o_t = take(size_t(kSegMG) * kStride * 8), o_i = take(size_t(kSegMG) * kIStride * 2);
+    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kSegMG * 8), o_pm = take(size_t(n_p) * 8),
+                 o_l5 = take(size_t(kSegMG) * cap * 16), o_q = take(size_t(kSegMG) * cap * 8), o_t9 = take(size_t(kSegMG) * n_pairs * 8),
+                 o_x = take(size_t(n_p) * 4), o_fb = take(size_t(kSegWarps) * cap * 4), o_fc = take(size_t(kSegWarps) * cap * 4),
+                 o_fq = take(size_t(kSegWarps) * cap * 4), o_sv = take(size_t(nsv) * 4), o_i9 = take(size_t(kSegMG) * n_pairs), o_pair = take(n_p),
+                 o_p2 = take(size_t(kSegMG) * stride), o_p5 = take(size_t(kSegMG) * stride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
-        o->sval = reinterpret_cast<uint32_t *>(base + o_sv); o->gm = reinterpret_cast<double *>(base + o_gm);
-        o->lf = reinterpret_cast<double *>(base + o_lf); o->lc = reinterpret_cast<double *>(base + o_lc);
-        o->pm1 = reinterpret_cast<double *>(base + o_pm);
-        o->lq = reinterpret_cast<double *>(base + o_lq); o->l5 = reinterpret_cast<double2 *>(base + o_l5);
-        o->qp = reinterpret_cast<double *>(base + o_qp); o->ep = reinterpret_cast<double2 *>(base + o_ep);
-        o->pc = reinterpret_cast<int *>(base + o_pc);
-        o->st_time = reinterpret_cast<double *>(base + o_t); o->st_idx = reinterpret_cast<uint16_t *>(base + o_i);
-        o->cap = cap;
+        o->gm = reinterpret_cast<double *>(base + o_gm); o->pm1 = reinterpret_cast<double *>(base + o_pm);
+        o->l5 = reinterpret_cast<double2 *>(base + o_l5); o->q = reinterpret_cast<double *>(base + o_q);
+        o->t9 = reinterpret_cast<double *>(base + o_t9); o->x = reinterpret_cast<float *>(base + o_x);
+        o->fb = reinterpret_cast<float *>(base + o_fb); o->fc = reinterpret_cast<float *>(base + o_fc);
+        o->fq = reinterpret_cast<float *>(base + o_fq); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
+        o->i9 = base + o_i9; o->pair = base + o_pair; o->pos2 = base + o_p2; o->pos5 = base + o_p5;
+        o->cap = cap; o->stride = stride;
     }
     return off;
 }
 
-__device__ __forceinline__ int hi32(double x) { return __double2hiint(x); }
-
-// Index (< 64) of a smallest non-negative value over the warp, up to the last 6 bits of its low word: two integer
-// warp reductions (high word, then low word with the index in its last bits).  Good enough for a pilot: the sweep's
-// exact comparisons settle what the pilot leaves open.
-__device__ __forceinline__ int warp_argmin_pilot(double v, int idx)
-{
-    const int hmin = __reduce_min_sync(0xffffffffu, hi32(v));
-    const unsigned key = hi32(v) == hmin ? ((static_cast<unsigned>(__double2loint(v)) & ~0x3Fu) | static_cast<unsigned>(idx & 0x3F)) : 0xFFFFFFFFu;
-    return static_cast<int>(__reduce_min_sync(0xffffffffu, key) & 0x3Fu);
-}
-
-__device__ __forceinline__ void offer(double &bt, uint32_t &bidx, double t, uint32_t idx)
-{
-    if (t <= bt) {
-        if (t < bt || idx < bidx) { bt = t; bidx = idx; }
-    }
-}
-
 }  // namespace
 
-__global__ void __launch_bounds__(kSegThreads, 2) segmin_kernel(const SegminParams p)
+__global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
     SegSmem sm;
-    seg_layout(npad, p.G.n_s, smem_raw, &sm);
+    seg_layout(npad, p.G.n_s, p.n_pairs, p.tiles, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
+    const bool has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has9 = (mask >> 9) & 1u;
 
     int b = blockIdx.x;
     const int mgroup = b % p.n_mgroups;
@@ -105,21 +88,22 @@ __global__ void __launch_bounds__(kSegThreads, 2) segmin_kernel(const SegminPara
     const int trel = b / p.n_ptiles;
     const int table = p.table0 + trel;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int m0 = mgroup * kSegMG;
-    const int n_mi = min(kSegMG, p.G.n_m - m0);
-    const int tile0 = ptile * kSegTileP;
-    const int n_valid = min(kSegTileP, p.G.n_P - tile0);
+    const int m0 = mgroup * p.mg;
+    const int n_mi = min(p.mg, p.G.n_m - m0);
+    const int n_p = p.tiles * kSegTileP, tile0 = ptile * n_p;
+    const int n_valid = min(n_p, p.G.n_P - tile0);
+    const int pair0 = pair_of(P_at(p.G, tile0)), n_pairs = pair_of(P_at(p.G, tile0 + n_valid - 1)) - pair0 + 1;
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
     dependents_may_start();
     if (!grow) stage_table(sm.tab, p.T, table);
     else wait_for_kernel_in_front();  // the gap pre-pass
-    for (int i = tid; i < kSegTileP; i += kSegThreads) {
+    for (int i = tid; i < n_p; i += kSegThreads) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
-        sm.lf[i] = static_cast<double>(31 - __clz(P));
-        sm.lc[i] = static_cast<double>(32 - __clz(P - 1));
         sm.pm1[i] = static_cast<double>(P - 1);
+        sm.x[i] = __int2float_rd(P - 1);
+        sm.pair[i] = static_cast<uint8_t>(pair_of(P) - pair0);
     }
     __syncthreads();
     const double L = p.T.lat[table];
@@ -134,216 +118,268 @@ __global__ void __launch_bounds__(kSegThreads, 2) segmin_kernel(const SegminPara
     }
     __syncthreads();
 
-    const double x_mid = sm.pm1[n_valid / 2];
+    float x_pilot[kPilots];  // the winner of id 5 changes more often where P is small
+    {
+        const int at[kPilots] = {n_valid >> 5, n_valid * 5 >> 5, n_valid * 15 >> 5, n_valid - 1};
+#pragma unroll
+        for (int i = 0; i < kPilots; ++i) x_pilot[i] = sm.x[at[i]];
+    }
+    float *const fb = sm.fb + warp * sm.cap, *const fc = sm.fc + warp * sm.cap, *const fq = sm.fq + warp * sm.cap;
+    const float Lf = __double2float_rd(L);
+    const f32x2 L2 = splat2(Lf);
 
-    // ---- phase 0: the coefficient lists of the warp's message sizes (lanes <-> candidates) and the pilots ----
     for (int mi = warp; mi < n_mi; mi += kSegWarps) {
         const int midx = m0 + mi;
         const int ns = p.G.ns_of_m[midx];
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
-        const int np = (nsv + U - 1) / U * U;
+        const int np4 = round_up(nsv, 4), np16 = round_up(nsv, kStep);
         const double gm = sm.gm[mi];
-        const double *krow = p.G.k_list + static_cast<size_t>(midx) * p.G.n_s;
-        double *lq = sm.lq + mi * sm.cap;
-        double2 *l5 = sm.l5 + mi * sm.cap;
-        double qb = CUDART_INF, tb = CUDART_INF;
-        int qc = kIntMax, tc = kIntMax;
-        for (int c = lane; c < np; c += 32) {
-            double Q = CUDART_INF, B = CUDART_INF, C = CUDART_INF;  // padding never reaches a minimum
+        double *const q = sm.q + mi * sm.cap;
+        double2 *const l5 = sm.l5 + mi * sm.cap;
+
+        // ---- the lists (lanes <-> candidates) and the pilots: bound (without its last 8 bits) and index in one number ----
+        __syncwarp();  // the previous message size's sweeps are done with the lists
+        unsigned pilot[kPilots], q_pilot = 0xFFFFFFFFu;
+#pragma unroll
+        for (int i = 0; i < kPilots; ++i) pilot[i] = 0xFFFFFFFFu;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = lane + 32 * h;
+            if (c >= np16) break;
+            float Bf = 0.f, Cf = CUDART_INF_F, Qf = CUDART_INF_F;  // padding: the bound is +inf
             if (c < nsv) {
                 double gsv = gm, k = 1.0;
                 if (ns > 0) {
                     gsv = sm.gs[c];
-                    k = krow[c];  // Section 2's k, from the host's table
+                    k = p.G.k_list[static_cast<size_t>(midx) * p.G.n_s + c];  // Section 2's k, from the host's table
                 }
-                Q = gsv * k;
-                B = gsv + L;
-                C = gsv * (k - 1.0);
-                if (Q < qb) { qb = Q; qc = c; }
-                const double t = fma(x_mid, B, C);
-                if (t < tb) { tb = t; tc = c; }
+                const double Q = gsv * k, B = gsv + L, C = gsv * (k - 1.0);
+                q[c] = Q;
+                l5[c] = make_double2(B, C);
+                Qf = __double2float_rd(Q); Bf = __double2float_rd(B); Cf = __double2float_rd(C);
+                q_pilot = min(q_pilot, (__float_as_uint(Qf) & ~0xFFu) | static_cast<unsigned>(c));
+#pragma unroll
+                for (int i = 0; i < kPilots; ++i)
+                    pilot[i] = min(pilot[i], (__float_as_uint(__fmaf_rd(x_pilot[i], Bf, Cf)) & ~0xFFu) | static_cast<unsigned>(c));
             }
-            lq[c] = Q;
-            l5[c] = make_double2(B, C);
+            fb[c] = Bf; fc[c] = Cf; fq[c] = Qf;
         }
-        qc = warp_argmin_pilot(qb, qc);  // smallest Q: the winner of ids 2 and 9 for every P
-        tc = warp_argmin_pilot(tb, tc);  // id 5's winner at the middle of the tile
+        q_pilot = __reduce_min_sync(kFull, q_pilot) & 0xFFu;
+#pragma unroll
+        for (int i = 0; i < kPilots; ++i) pilot[i] = __reduce_min_sync(kFull, pilot[i]) & 0xFFu;
         __syncwarp();
-        // the pilots leave the lists (their own cells would always pass the filter); the running minima start from them
-        const double q_pilot = lq[qc];
-        const double2 e_pilot = l5[tc];
+        // the pilots leave the lists: their own bounds would always pass
+        if (lane < kPilots) {
+            unsigned mine = pilot[0];
+#pragma unroll
+            for (int i = 1; i < kPilots; ++i) mine = lane == i ? pilot[i] : mine;
+            fb[mine] = 0.0f;
+            fc[mine] = CUDART_INF_F;
+        }
+        if (lane == kPilots) fq[q_pilot] = CUDART_INF_F;
         __syncwarp();
-        if (lane == 0) {
-            lq[qc] = CUDART_INF;
-            l5[tc] = make_double2(CUDART_INF, CUDART_INF);
-            sm.qp[mi] = q_pilot; sm.ep[mi] = e_pilot;
-            sm.pc[2 * mi] = qc; sm.pc[2 * mi + 1] = tc;
+
+        // ---- id 9 per (floor, ceil) pair ----
+        if (has9)
+        for (int b0 = 0; b0 < n_pairs; b0 += 32) {
+            const int pr = b0 + lane, li = pair0 + min(pr, n_pairs - 1);
+            const double lf = static_cast<double>(li >> 1), lcL = static_cast<double>((li >> 1) + (li & 1)) * L;
+            const f32x2 x2 = splat2(static_cast<float>(li >> 1)), c2 = splat2(__double2float_rd(lcL));
+            unsigned at = q_pilot;
+            double t = fma(lf, q[at], lcL);
+            float low = CUDART_INF_F;
+            for (int c = 0; c < np4; c += 4) {
+                const f32x2x2 qq = *reinterpret_cast<const f32x2x2 *>(fq + c);
+                low = min_with2(min_with2(low, fma2_down(x2, qq.x, c2)), fma2_down(x2, qq.y, c2));
+            }
+            if (__any_sync(kFull, low <= __double2float_ru(t))) {
+#pragma unroll 1
+                for (int c = 0; c < nsv; ++c) {
+                    const double v = fma(lf, q[c], lcL);
+                    if (v <= t && (v < t || static_cast<unsigned>(c) < at)) { t = v; at = static_cast<unsigned>(c); }
+                }
+            }
+            if (pr < n_pairs) {
+                sm.t9[mi * p.n_pairs + pr] = t;
+                sm.i9[mi * p.n_pairs + pr] = static_cast<uint8_t>(at);
+            }
+        }
+
+        for (int tile = 0; tile < p.tiles; ++tile) {
+            if (tile * kSegTileP >= n_valid) break;
+            const double *const xd = sm.pm1 + tile * kSegTileP + lane;
+            uint8_t *const pos2 = sm.pos2 + mi * sm.stride + tile * kSegTileP + lane, *const pos5 = sm.pos5 + mi * sm.stride + tile * kSegTileP + lane;
+            f32x2 x2[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) x2[r] = splat2(sm.x[tile * kSegTileP + 32 * r + lane]);
+            unsigned hit = 0;  // bit r: id 5, bit 16 + r: id 2
+            if (has5) {
+                float T[R], mn[R];
+                {
+                    double t[R];
+                    unsigned at[R];
+                    const double2 e = l5[pilot[0]];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) { t[r] = fma(xd[32 * r], e.x, e.y); at[r] = pilot[0]; }
+#pragma unroll
+                    for (int i = 1; i < kPilots; ++i) {
+                        if (pilot[i] == pilot[i - 1]) continue;
+                        const double2 v = l5[pilot[i]];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            const double tt = fma(xd[32 * r], v.x, v.y);
+                            if (tt < t[r] || (tt == t[r] && pilot[i] < at[r])) { t[r] = tt; at[r] = pilot[i]; }
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) { T[r] = __double2float_ru(t[r]); pos5[32 * r] = static_cast<uint8_t>(at[r]); }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) mn[r] = CUDART_INF_F;
+#pragma unroll 2
+                for (int j = 0; j < np4; j += 4) {
+                    const f32x2x2 bb = *reinterpret_cast<const f32x2x2 *>(fb + j), cc = *reinterpret_cast<const f32x2x2 *>(fc + j);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], bb.x, cc.x));
+#pragma unroll
+                    for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], bb.y, cc.y));
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (mn[r] <= T[r]) hit |= 1u << r;
+            }
+            if (has2) {
+                float T[R], mn[R];
+                const double Q = q[q_pilot];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    T[r] = __double2float_ru(fma(xd[32 * r], Q, L));
+                    pos2[32 * r] = static_cast<uint8_t>(q_pilot);
+                    mn[r] = CUDART_INF_F;
+                }
+#pragma unroll 2
+                for (int j = 0; j < np4; j += 4) {
+                    const f32x2x2 qq = *reinterpret_cast<const f32x2x2 *>(fq + j);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], qq.x, L2));
+#pragma unroll
+                    for (int r = 0; r < R; ++r) mn[r] = min_with2(mn[r], fma2_down(x2[r], qq.y, L2));
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (mn[r] <= T[r]) hit |= 0x10000u << r;
+            }
+
+            // ---- exact search of the rows in which some bound is not above the running minimum ----
+#pragma unroll 1
+            for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
+                const int bit = __ffs(rows) - 1, r = bit & 15;
+                const bool two = bit >> 4;  // id 2
+                const double x = xd[32 * r];
+                const f32x2 xx = splat2(sm.x[tile * kSegTileP + 32 * r + lane]);
+                uint8_t *const pos = two ? pos2 : pos5;
+                unsigned at = pos[32 * r];
+                double t = two ? fma(x, q[at], L) : fma(x, l5[at].x, l5[at].y);
+                const bool mine = (hit >> bit) & 1u;
+                float T = mine ? __double2float_ru(t) : -1.0f;
+#pragma unroll 1
+                for (int j = 0; j < nsv; j += kStep) {
+                    float low[kStep / 4];
+#pragma unroll
+                    for (int u = 0; u < kStep / 4; ++u) {
+                        const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>((two ? fq : fb) + j + 4 * u);
+                        f32x2x2 cc;
+                        cc.x = cc.y = L2;
+                        if (!two) cc = *reinterpret_cast<const f32x2x2 *>(fc + j + 4 * u);
+                        low[u] = min_with2(min_with2(CUDART_INF_F, fma2_down(xx, aa.x, cc.x)), fma2_down(xx, aa.y, cc.y));
+                    }
+                    if (!__any_sync(kFull, fminf(fminf(low[0], low[1]), fminf(low[2], low[3])) <= T)) continue;
+#pragma unroll
+                    for (int u = 0; u < kStep / 4; ++u) {
+                        if (!__any_sync(kFull, low[u] <= T)) continue;
+                        const int c0 = j + 4 * u;
+#pragma unroll
+                        for (int c = c0; c < c0 + 4; ++c) {
+                            if (c >= nsv) break;
+                            const double2 e = l5[c];
+                            const double tt = two ? fma(x, q[c], L) : fma(x, e.x, e.y);
+                            if (tt <= t && (tt < t || static_cast<unsigned>(c) < at)) { t = tt; at = static_cast<unsigned>(c); }
+                        }
+                        if (mine) T = __double2float_ru(t);
+                    }
+                }
+                pos[32 * r] = static_cast<uint8_t>(at);
+            }
         }
     }
-    __syncwarp();  // the lists and pilots of a message size are read by the warp that wrote them
+    __syncthreads();
 
+    // ---- transposed write-out: rows of p.mg consecutive m per process count, one plane after another ----
     const size_t plane = static_cast<size_t>(p.G.n_P) * p.G.n_m;
+    const size_t cell0 = static_cast<size_t>(tile0) * p.G.n_m + m0;
     const int ids[3] = {2, 5, 9};
-    // ---- one strategy at a time: every warp sweeps it for its message sizes, then the CTA writes the plane ----
 #pragma unroll 1
-    for (int q = 0; q < 3; ++q) {
-        if (!((mask >> ids[q]) & 1u)) continue;
-        for (int mi = warp; mi < n_mi; mi += kSegWarps) {
-            const int midx = m0 + mi;
-            const int ns = p.G.ns_of_m[midx];
-            const int np = (max(ns, 1) + U - 1) / U * U;
-            const double *lq = sm.lq + mi * sm.cap;
-            const double2 *l5 = sm.l5 + mi * sm.cap;
-            const uint32_t whole = ns > 0 ? 0u : 1u;
-            auto stage = [&](const double *bt, const uint32_t *bidx) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    sm.st_time[mi * kStride + 32 * r + lane] = bt[r];
-                    sm.st_idx[mi * kIStride + 32 * r + lane] = static_cast<uint16_t>(whole ? kWhole : bidx[r]);
-                }
-            };
-            // Filter of a group of U candidates: the smallest high word of the U times minus the high word of the running
-            // minimum says whether a cell can reach it (<= 0); the differences of all R process counts are folded into one
-            // integer minimum and one vote decides whether the group needs the exact pass.
-            auto sweep_q = [&](auto is9_tag) {
-                constexpr bool IS9 = decltype(is9_tag)::value;
-                // id 2: fma(P-1, Q, L); id 9: fma(floor(log2 P), Q, ceil(log2 P) L)
-                const double q_pilot = sm.qp[mi];
-                const int qc = sm.pc[2 * mi];
-                double x[R], c9[IS9 ? R : 1];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    x[r] = IS9 ? sm.lf[32 * r + lane] : sm.pm1[32 * r + lane];
-                    if (IS9) c9[r] = sm.lc[32 * r + lane] * L;
-                }
-                if (!IS9) c9[0] = L;
-                double bt[R];
-                uint32_t bidx[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) { bt[r] = fma(x[r], q_pilot, c9[IS9 ? r : 0]); bidx[r] = static_cast<uint32_t>(qc); }
-#pragma unroll 1
-                for (int j = 0; j < np; j += U) {
-                    const double2 q01 = *reinterpret_cast<const double2 *>(lq + j), q23 = *reinterpret_cast<const double2 *>(lq + j + 2);
-                    int acc = kIntMax;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double c = c9[IS9 ? r : 0];
-                        const int h0 = hi32(fma(x[r], q01.x, c)), h1 = hi32(fma(x[r], q01.y, c));
-                        const int h2 = hi32(fma(x[r], q23.x, c)), h3 = hi32(fma(x[r], q23.y, c));
-                        acc = min(acc, min(min(h0, h1), min(h2, h3)) - hi32(bt[r]));
-                    }
-                    if (__any_sync(kFull, acc <= 0)) {
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            const double c = c9[IS9 ? r : 0];
-                            const int h0 = hi32(fma(x[r], q01.x, c)), h1 = hi32(fma(x[r], q01.y, c));
-                            const int h2 = hi32(fma(x[r], q23.x, c)), h3 = hi32(fma(x[r], q23.y, c));
-                            if (__any_sync(kFull, min(min(h0, h1), min(h2, h3)) <= hi32(bt[r]))) {
-#pragma unroll 1
-                                for (int u = 0; u < U; ++u) offer(bt[r], bidx[r], fma(x[r], lq[j + u], c), static_cast<uint32_t>(j + u));
-                            }
-                        }
-                    }
-                }
-                stage(bt, bidx);
-            };
-            if (q == 0) sweep_q(std::false_type{});
-            else if (q == 2) sweep_q(std::true_type{});
-            else {
-                // ---- id 5: list of (B, C) ----
-                const double2 e_pilot = sm.ep[mi];
-                const int tc = sm.pc[2 * mi + 1];
-                double pm1[R], bt[R];
-                uint32_t bidx[R];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    pm1[r] = sm.pm1[32 * r + lane];
-                    bt[r] = fma(pm1[r], e_pilot.x, e_pilot.y);
-                    bidx[r] = static_cast<uint32_t>(tc);
-                }
-#pragma unroll 1
-                for (int j = 0; j < np; j += U) {
-                    const double2 e0 = l5[j], e1 = l5[j + 1], e2 = l5[j + 2], e3 = l5[j + 3];
-                    int acc = kIntMax;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const int h0 = hi32(fma(pm1[r], e0.x, e0.y)), h1 = hi32(fma(pm1[r], e1.x, e1.y));
-                        const int h2 = hi32(fma(pm1[r], e2.x, e2.y)), h3 = hi32(fma(pm1[r], e3.x, e3.y));
-                        acc = min(acc, min(min(h0, h1), min(h2, h3)) - hi32(bt[r]));
-                    }
-                    if (__any_sync(kFull, acc <= 0)) {
-#pragma unroll
-                        for (int r = 0; r < R; ++r) {
-                            const int h0 = hi32(fma(pm1[r], e0.x, e0.y)), h1 = hi32(fma(pm1[r], e1.x, e1.y));
-                            const int h2 = hi32(fma(pm1[r], e2.x, e2.y)), h3 = hi32(fma(pm1[r], e3.x, e3.y));
-                            if (__any_sync(kFull, min(min(h0, h1), min(h2, h3)) <= hi32(bt[r]))) {
-#pragma unroll 1
-                                for (int u = 0; u < U; ++u) {
-                                    const double2 e = l5[j + u];
-                                    offer(bt[r], bidx[r], fma(pm1[r], e.x, e.y), static_cast<uint32_t>(j + u));
-                                }
-                            }
-                        }
-                    }
-                }
-                stage(bt, bidx);
+    for (int w = 0; w < 3; ++w) {
+        if (!((mask >> ids[w]) & 1u)) continue;
+        double *plane_t = p.p_time + (static_cast<size_t>(table - p.out_table0) * 13 + ids[w]) * plane + cell0;
+        uint32_t *plane_s = p.p_best_s ? p.p_best_s + (static_cast<size_t>(table - p.out_table0) * 3 + w) * plane + cell0 : nullptr;
+        const uint8_t *const pos = w == 0 ? sm.pos2 : sm.pos5;
+        // winner and time of one cell
+        auto cell = [&](int mi, int pr, double x, unsigned &at) {
+            if (w == 2) {
+                const int i = mi * p.n_pairs + sm.pair[pr];
+                at = sm.i9[i];
+                return sm.t9[i];
             }
-        }
-        __syncthreads();
-
-        // transposed write-out of the strategy's plane: rows of 16 consecutive m per process count
-        double *plane_t = p.p_time + (static_cast<size_t>(table - p.out_table0) * 13 + ids[q]) * plane;
-        uint32_t *plane_s = p.p_best_s ? p.p_best_s + (static_cast<size_t>(table - p.out_table0) * 3 + q) * plane : nullptr;
+            at = pos[mi * sm.stride + pr];
+            if (w == 0) return fma(x, sm.q[mi * sm.cap + at], L);
+            const double2 e = sm.l5[mi * sm.cap + at];
+            return fma(x, e.x, e.y);
+        };
         if (p.vec_out) {
-            // two message sizes per lane (16-byte and 8-byte stores; the host has checked the alignment), running pointers
-            constexpr int kHalf = kSegMG / 2, kRows = 32 / kHalf, kStep = kSegWarps * kRows;
-            const int mi = 2 * (lane & (kHalf - 1)), pr0 = warp * kRows + lane / kHalf;
+            // two message sizes per lane (16-byte and 8-byte stores; the host has checked the alignment)
+            const int half = p.mg >> 1;
+            const int mi = 2 * (lane & (half - 1)), rows = 32 / half, step = kSegWarps * rows, pr0 = warp * rows + lane / half;
             if (mi < n_mi) {  // n_m is even, so mi + 1 is a message size of the grid too
                 const uint32_t m_u0 = p.G.m_list[m0 + mi], m_u1 = p.G.m_list[m0 + mi + 1];
-                const size_t cell0 = static_cast<size_t>(tile0 + pr0) * p.G.n_m + static_cast<size_t>(m0 + mi);
-                const size_t step = static_cast<size_t>(kStep) * p.G.n_m;
-                const double *st0 = sm.st_time + mi * kStride + pr0, *st1 = st0 + kStride;
-                const uint16_t *si0 = sm.st_idx + mi * kIStride + pr0, *si1 = si0 + kIStride;
-                double *out_t = plane_t + cell0;
-                uint32_t *out_s = plane_s ? plane_s + cell0 : nullptr;
-                for (int pr = pr0; pr < n_valid; pr += kStep) {
-                    *reinterpret_cast<double2 *>(out_t) = make_double2(*st0, *st1);
+                const bool w0 = p.G.ns_of_m[m0 + mi] == 0, w1 = p.G.ns_of_m[m0 + mi + 1] == 0;  // the whole message
+                const size_t o = static_cast<size_t>(pr0) * p.G.n_m + mi, go = static_cast<size_t>(step) * p.G.n_m;
+                double *out_t = plane_t + o;
+                uint32_t *out_s = plane_s ? plane_s + o : nullptr;
+                for (int pr = pr0; pr < n_valid; pr += step) {
+                    const double x = sm.pm1[pr];
+                    unsigned a0, a1;
+                    const double t0 = cell(mi, pr, x, a0), t1 = cell(mi + 1, pr, x, a1);
+                    *reinterpret_cast<double2 *>(out_t) = make_double2(t0, t1);
+                    out_t += go;
                     if (out_s) {
-                        const uint32_t i0 = *si0, i1 = *si1;
-                        *reinterpret_cast<uint2 *>(out_s) = make_uint2(i0 == kWhole ? m_u0 : sm.sval[i0], i1 == kWhole ? m_u1 : sm.sval[i1]);
-                        out_s += step;
+                        *reinterpret_cast<uint2 *>(out_s) = make_uint2(w0 ? m_u0 : sm.sval[a0], w1 ? m_u1 : sm.sval[a1]);
+                        out_s += go;
                     }
-                    out_t += step;
-                    st0 += kStep; st1 += kStep; si0 += kStep; si1 += kStep;
                 }
             }
         } else {
-            const int mi = lane & (kSegMG - 1), prow = lane / kSegMG, rows = 32 / kSegMG;
+            const int mi = lane & (p.mg - 1), rows = 32 / p.mg;
             if (mi < n_mi) {
                 const uint32_t m_u = p.G.m_list[m0 + mi];
-                const double *st = sm.st_time + mi * kStride;
-                const uint16_t *si = sm.st_idx + mi * kIStride;
-                for (int pr = warp * rows + prow; pr < n_valid; pr += kSegWarps * rows) {
-                    const size_t o = static_cast<size_t>(tile0 + pr) * p.G.n_m + static_cast<size_t>(m0 + mi);
-                    plane_t[o] = st[pr];
-                    if (plane_s) {
-                        const uint32_t idx = si[pr];
-                        plane_s[o] = idx == kWhole ? m_u : sm.sval[idx];
-                    }
+                const bool whole = p.G.ns_of_m[m0 + mi] == 0;
+                for (int pr = warp * rows + lane / p.mg; pr < n_valid; pr += kSegWarps * rows) {
+                    const size_t o = static_cast<size_t>(pr) * p.G.n_m + mi;
+                    unsigned at;
+                    plane_t[o] = cell(mi, pr, sm.pm1[pr], at);
+                    if (plane_s) plane_s[o] = whole ? m_u : sm.sval[at];
                 }
             }
         }
-        __syncthreads();  // the staging area is free again
     }
 }
-
-size_t segmin_smem_bytes(const TableDev &T, const GridDev &G) { return seg_layout(T.npad, G.n_s, nullptr, nullptr); }
 
 cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
 {
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    return launch(segmin_kernel, static_cast<unsigned>(blocks), 1, kSegThreads, segmin_smem_bytes(p.T, p.G), st, overlap, p);
+    return launch(segmin_kernel, static_cast<unsigned>(blocks), 1, kSegThreads, seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles, nullptr, nullptr), st,
+                  overlap, p);
 }
 
 }  // namespace plogp
