@@ -63,7 +63,7 @@ struct Plan {
     bool inline_sweep = true;
     bool envelope = false;        // envelope_kernel instead of the sweep kernel (long candidate lists)
     bool envelope_short = false;  // the decision kernel prunes its candidate lists (short candidate lists)
-    int env_threads = 256, env_rep_cap = 0, env_coarse = 64, env_max_coarse = 0;
+    int env_threads = 256, env_rep_cap = 0, env_coarse_log = 5, env_max_coarse = 0;
     // fused kernel tiling
     int n_mtiles = 0, n_ptiles = 1, passes_per_tile = 1;
     // Scatter decision kernel: its own split of P (vec = 2: two message sizes per lane, where the outputs allow it)
@@ -373,8 +373,9 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
         // short lists: small CTAs; the list of representatives of one message size lives in shared memory
         pl.env_threads = ns_max <= 64 ? 64 : (ns_max <= 4096 ? 256 : 1024);
         pl.env_rep_cap = std::min(std::max(ns_max, 1), 6144);
-        pl.env_coarse = std::max(64, (n_P + 1023) / 1024);
-        pl.env_max_coarse = (std::max(n_P, 1) - 1 + pl.env_coarse - 1) / pl.env_coarse + 1;
+        pl.env_coarse_log = 5;
+        while ((2 << pl.env_coarse_log) < (n_P + 1023) / 1024) ++pl.env_coarse_log;
+        pl.env_max_coarse = envelope_coarse_of(n_P - 1, pl.env_coarse_log) + 2;
     } else if (!pl.inline_sweep) {
         pl.chunk_len = std::max(2048, ((ns_max + 31) / 32 + kSweepSub - 1) / kSweepSub * kSweepSub);
         std::vector<int32_t> pair_base(n_m + 1, 0);
@@ -512,7 +513,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             ep.T = h->T; ep.G = pl.G;
             ep.table0 = t0; ep.n_tables_launch = nt;
             ep.part_time = part_time; ep.part_idx = part_idx; ep.n_seg = pl.n_seg;
-            ep.rep_cap = pl.env_rep_cap; ep.coarse = pl.env_coarse; ep.max_coarse = pl.env_max_coarse;
+            ep.rep_cap = pl.env_rep_cap; ep.coarse_log = pl.env_coarse_log; ep.max_coarse = pl.env_max_coarse;
             { LaunchTimer lt(h, PLOGP_KERNEL_ENVELOPE, st); CK(launch_envelope(ep, pl.env_threads, st)); }
             g_launches += 1;
         } else if (!pl.inline_sweep && pl.n_pairs > 0) {

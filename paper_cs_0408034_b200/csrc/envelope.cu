@@ -9,12 +9,17 @@
 // For id 5 the minimum over s is the lower envelope of the lines.  When g does not decrease along the
 // candidate sizes (the host only selects this kernel for such tables) two facts hold:
 //   * among candidates with the same segment count k the smallest s has the smallest B and C, so
-//     only the first candidate of every run of equal k can ever win (its "representative");
+//     only the first candidate of every run of equal k can ever win (its "representative"), for id 5 as for ids 2 and 9;
 //   * the representatives are sorted by slope B, hence the index of the winner does not grow with P:
 //     the winners at two process counts bracket the winners at all counts in between.
-// The kernel therefore (A) lists the representatives in shared memory, (B) finds the winner at every
-// `coarse`-th process count over the whole list and (C) searches, for each process count, only the
-// bracket given by its two coarse neighbours (widened by one entry on each side, which absorbs a
+// Where the candidates are equally spaced the representatives are found without visiting the others: below
+// s = sqrt(m step) almost every candidate has a segment count of its own and is looked at, above it the counts are few
+// and the first candidate of each is computed (4096 instead of 262144 candidates for m = 16 MB and every multiple of
+// 4 B up to 1 MB: 298 -> 22 us for 128 message sizes).
+// The kernel therefore (A) lists the representatives in shared memory, (B) finds the winners at a sequence of coarse
+// process-count indices (all of the first 16, then ever wider apart up to `2 << coarse_log`: the winner moves fastest
+// where P is small), every eighth over the whole list, the others between those, and (C) searches, for each
+// process count, only the bracket given by its two coarse neighbours (widened by one entry on each side, which absorbs a
 // winner that rounding moved across a bracket end).  All comparisons are the exact ones of the
 // exhaustive search: (time, s) in lexicographic order.
 //
@@ -28,7 +33,23 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// coarse number c <-> process-count index: 0..15, then runs of 8 with distances 2, 4, 8, .. up to 2 << g_max, which stays
+__device__ __forceinline__ int coarse_index(int c, int g_max)
+{
+    if (c < 16) return c;
+    const int g = min((c - 16) >> 3, g_max);
+    return (16 << g) + (c - 16 - 8 * g) * (2 << g);
+}
+
 }  // namespace
+
+__host__ __device__ int envelope_coarse_of(int pidx, int g_max)
+{
+    if (pidx < 16) return pidx;
+    int g = 0;
+    while (g < g_max && (32 << g) <= pidx) ++g;
+    return 16 + 8 * g + (pidx - (16 << g)) / (2 << g);
+}
 
 __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
 {
@@ -62,25 +83,51 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
     double qmin = CUDART_INF;
     int qidx = 0x7FFFFFFF;
     int n_rep = 0;  // all representatives (of every window), known after the first pass
-    constexpr int V = 4;  // consecutive candidates per thread and chunk (independent searches and divisions in flight)
+    constexpr int V = 4;  // consecutive items per thread and chunk (independent searches and divisions in flight)
+    // Items in ascending order of s: the first n_low candidates, then (equally spaced candidates only) one item for every
+    // smaller segment count.  An item is a representative if its candidate's count differs from the one in front of it.
+    int n_low = ns, n_items = ns;
+    uint32_t k_low = 0;  // segment count of candidate n_low - 1
+    if (!p.G.s_list) {
+        n_low = min(ns, static_cast<int>(sqrtf(static_cast<float>(m_u) / static_cast<float>(p.G.s_step))) + 1);
+        k_low = segments(m_u, s_at(p.G, n_low - 1), p.G.k_mode);
+        n_items = n_low + static_cast<int>(k_low - segments(m_u, s_at(p.G, ns - 1), p.G.k_mode));
+    }
     auto list_pass = [&](int win) {
         int base = 0;
-        uint32_t carry_k = 0;  // thread 0: k of the last candidate of the previous chunk
-        for (int c0 = 0; c0 < ns; c0 += V * T) {
+        uint32_t carry_k = 0;  // thread 0: k of the last item of the previous chunk
+        for (int c0 = 0; c0 < n_items; c0 += V * T) {
             double gs[V];
             uint32_t k[V];
+            int cand[V];
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const int si = c0 + V * tid + v;
+                const int it = c0 + V * tid + v;
+                int si = it;
                 gs[v] = 0.0;
                 k[v] = 0;
-                if (si < ns) {
+                bool real = it < n_items;
+                uint32_t want = 0;
+                if (real && it >= n_low) {
+                    // the smallest candidate with at most `want` segments: s >= m / want (k = ceil), s > m / (want + 1) (k = floor)
+                    want = k_low - 1u - static_cast<uint32_t>(it - n_low);
+                    uint32_t t;
+                    if (p.G.k_mode == 0) { t = m_u / want; t += t * want != m_u ? 1u : 0u; }
+                    else t = m_u / (want + 1u) + 1u;
+                    si = t <= p.G.s_lo ? 0 : static_cast<int>((static_cast<unsigned long long>(t - p.G.s_lo) + p.G.s_step - 1u) / p.G.s_step);
+                    real = si < ns;
+                }
+                cand[v] = si;
+                if (real) {
                     const uint32_t s = s_at(p.G, si);
-                    gs[v] = gap_at(s_tab, npad, static_cast<double>(s));
                     k[v] = segments(m_u, s, p.G.k_mode);
-                    if (win == 0) {
-                        const double Q = gs[v] * static_cast<double>(k[v]);
-                        if (Q < qmin) { qmin = Q; qidx = si; }  // ascending si per thread: the smallest index stays
+                    if (it >= n_low && k[v] != want) k[v] = 0;  // no candidate has that count
+                    else {
+                        gs[v] = gap_at(s_tab, npad, static_cast<double>(s));
+                        if (win == 0) {
+                            const double Q = gs[v] * static_cast<double>(k[v]);
+                            if (Q < qmin) { qmin = Q; qidx = si; }  // ascending si per thread: the smallest index stays
+                        }
                     }
                 }
             }
@@ -91,8 +138,9 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
             int cnt = 0;
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-                const int si = c0 + V * tid + v;
-                if (si < ns && (si == 0 || k[v] != k_prev)) { rep |= 1u << v; ++cnt; }
+                const int it = c0 + V * tid + v;
+                // behind n_low every item that has a candidate is a representative
+                if (it < n_items && k[v] != 0 && (it == 0 || it >= n_low || k[v] != k_prev)) { rep |= 1u << v; ++cnt; }
                 k_prev = k[v];
             }
             // ordered positions: inclusive scan of the counts over the warp, then the warps' totals
@@ -118,7 +166,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
                     if (pos >= 0 && pos < p.rep_cap) {
                         s_B[pos] = gs[v] + L;
                         s_C[pos] = gs[v] * (static_cast<double>(k[v]) - 1.0);
-                        s_I[pos] = static_cast<uint32_t>(c0 + V * tid + v);
+                        s_I[pos] = static_cast<uint32_t>(cand[v]);
                     }
                     ++pos;
                 }
@@ -157,7 +205,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
     if (!has5) return;
 
     // ---- id 5: lower envelope over the representatives, one window of the list at a time ----
-    const int n_c = (n_P - 1 + p.coarse - 1) / p.coarse + 1;  // coarse process-count indices 0, coarse, ..., n_P - 1
+    const int n_c = envelope_coarse_of(n_P - 1, p.coarse_log) + 2;  // the last one stands for n_P - 1
     const int n_win = (n_rep + p.rep_cap - 1) / p.rep_cap;
     for (int win = 0; win < n_win; ++win) {
         if (win > 0) {
@@ -166,24 +214,38 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
         }
         __syncthreads();
         const int n_e = min(p.rep_cap, n_rep - win * p.rep_cap);
-        // (B) winners at the coarse process counts, over the whole window
-        for (int c = warp; c < n_c; c += n_warps) {
-            const double x = static_cast<double>(P_at(p.G, min(c * p.coarse, n_P - 1)) - 1);
+        // (B) winners at the coarse process counts: every eighth and the last over the whole window, then the others
+        auto coarse_winner = [&](int c, int lo, int hi) {
+            const double x = static_cast<double>(P_at(p.G, min(coarse_index(c, p.coarse_log), n_P - 1)) - 1);
             double tb = CUDART_INF;
             int eb = 0x7FFFFFFF;
-            for (int e = lane; e < n_e; e += 32) {
+#pragma unroll 4
+            for (int e = lo + lane; e <= hi; e += 32) {
                 const double t = fma(x, s_B[e], s_C[e]);
                 if (t < tb) { tb = t; eb = e; }
             }
             warp_min_pair(tb, eb);
-            if (lane == 0) s_opt[c] = eb;
+            if (lane == 0) s_opt[c] = min(eb, n_e - 1);
+        };
+        auto bracket = [&](int a, int b, int &lo, int &hi) {
+            lo = max(min(a, b) - 1, 0);
+            hi = min(max(a, b) + 1, n_e - 1);
+        };
+        const int n_8 = (n_c - 1 + 7) / 8 + 1;  // 0, 8, 16, .. and n_c - 1
+        for (int i = warp; i < n_8; i += n_warps) coarse_winner(min(8 * i, n_c - 1), 0, n_e - 1);
+        __syncthreads();
+        for (int c = warp; c < n_c - 1; c += n_warps) {
+            if ((c & 7) == 0) continue;
+            int lo, hi;
+            bracket(s_opt[c & ~7], s_opt[min((c & ~7) + 8, n_c - 1)], lo, hi);
+            coarse_winner(c, lo, hi);
         }
         __syncthreads();
         // (C) every process count: the bracket of its coarse neighbours, one entry wider on each side
         for (int pidx = tid; pidx < n_P; pidx += T) {
-            const int c = pidx / p.coarse;
-            const int a = s_opt[min(c + 1, n_c - 1)], b = s_opt[c];
-            const int lo = max(min(a, b) - 1, 0), hi = min(max(a, b) + 1, n_e - 1);
+            const int c = envelope_coarse_of(pidx, p.coarse_log);
+            int lo, hi;
+            bracket(s_opt[c], s_opt[min(c + 1, n_c - 1)], lo, hi);
             const double x = static_cast<double>(P_at(p.G, pidx) - 1);
             double tb = CUDART_INF;
             int eb = lo;

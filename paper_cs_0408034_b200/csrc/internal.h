@@ -87,7 +87,7 @@ struct EnvParams {
     uint32_t *part_idx;  // same shape: index of s in the candidate list
     int n_seg;
     int rep_cap;     // entries of the shared-memory list of representatives (longer lists go through it in windows)
-    int coarse;      // distance between the coarse process-count indices
+    int coarse_log;  // the coarse process-count indices are at most 2 << coarse_log apart
     int max_coarse;  // capacity of the coarse-winner array (>= number of coarse indices)
 };
 
@@ -217,6 +217,7 @@ cudaError_t launch_surface(const SensParams &p, cudaStream_t st);
 cudaError_t launch_fixed(const SensParams &p, cudaStream_t st);
 cudaError_t launch_boundaries(const uint8_t *d_strategy, uint8_t *d_boundary, long long n_planes, int n_P, int n_m, int sm_count, cudaStream_t st);
 size_t envelope_smem_bytes(const TableDev &T, int threads, int rep_cap, int max_coarse);
+__host__ __device__ int envelope_coarse_of(int pidx, int g_max);  // number of the last coarse index at or below pidx
 cudaError_t launch_envelope(const EnvParams &p, int threads, cudaStream_t st);
 
 }  // namespace plogp

@@ -55,3 +55,30 @@ def test_times_outside_the_range_of_fp32(plogp, scale, long_list):
     if long_list:
         w = replace(w, P_hi=70, s_list=None, s_lo=4, s_hi=4 * 300, s_step=4)
     both(plogp, w)
+
+
+@pytest.mark.parametrize("s_lo,s_step,n_s,k_mode", [(4, 4, 66, 0), (4, 4, 3000, 1), (4, 12, 900, 0), (1000, 20, 1500, 1), (20000, 4, 500, 0),
+                                                    (4, 4000, 300, 0), (4, 4000, 300, 1)])
+def test_envelope_over_equally_spaced_candidates(plogp, s_lo, s_step, n_s, k_mode):
+    """The first candidate of every segment count, where counts change with every candidate, with some and with few of
+    them, and where counts are skipped; message sizes below, inside and above the list."""
+    base = wl.config4(n_tables=2, P_hi=130, n_m=4, seed_offset=n_s)
+    m = np.array([4, 48, 1000, 3996, 4000, 4004, 20004, 65536, 1000000, 1 << 24], dtype=np.uint64)
+    both(plogp, replace(base, m=m, s_list=None, s_lo=s_lo, s_hi=s_lo + s_step * (n_s - 1), s_step=s_step, k_mode=k_mode, search_mode=1))
+
+
+def test_alternating_grids_keep_their_plans(plogp):
+    """Twelve grids in turn on one handle (more than it keeps plans for), twice: every result is the one of a handle that
+    has seen no other grid."""
+    import torch
+    base = wl.config4(n_tables=3, P_hi=40, n_m=9, n_s=12, seed_offset=3)
+    grids = [replace(base, P_hi=10 + 3 * i, strategy_mask=wl.ALL_STRATEGIES if i % 3 else 0x1C07) for i in range(12)]
+    fresh = []
+    for w in grids:
+        with plogp.Tables.from_workload(w) as tabs:
+            fresh.append(plogp.select_best(tabs, w))
+    with plogp.Tables.from_workload(base) as tabs:
+        for w, f in list(zip(grids, fresh)) * 2:
+            d = plogp.select_best(tabs, w)
+            assert torch.equal(d.strategy, f.strategy) and torch.equal(d.s_bytes, f.s_bytes) and torch.equal(d.time, f.time)
+        torch.cuda.synchronize()
