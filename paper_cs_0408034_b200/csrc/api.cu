@@ -315,17 +315,23 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
         pl.sc_ptiles = (n_P + kWarps * pl.sc_run - 1) / (kWarps * pl.sc_run);
     }
 
-    pl.dec_ptiles = (n_P + kDecTileP - 1) / kDecTileP;
-    // 16 message sizes per CTA give the widest output rows; small grids trade that for more CTAs
-    // (never fewer than one message size per warp)
-    pl.dec_mg = kDecMG;
-    while (pl.dec_mg > kDecWarps && (long long)((n_m + pl.dec_mg - 1) / pl.dec_mg) * pl.dec_ptiles * h->T.n_tables < (long long)h->sm_count * 4)
-        pl.dec_mg >>= 1;
-    pl.dec_mgroups = (n_m + pl.dec_mg - 1) / pl.dec_mg;
-    // two tiles per CTA share the candidate lists, where that leaves enough CTAs
-    if (pl.dec_ptiles % 2 == 0 && (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables >= (long long)h->sm_count * 40) {
-        pl.dec_tiles = 2;
-        pl.dec_ptiles /= 2;
+    // Tiling of the lane <-> P kernels.  Wide CTAs (16 message sizes: 128-byte output rows; two tiles of process counts: the
+    // candidate lists are built once for both) against the last wave of CTAs: the choice with the smallest number of
+    // waves times the cost of a CTA, in cycles as measured on the batched workload (a message size's lists and pairs
+    // 5000, each of its tiles 5500, 3500 besides; narrower rows cost about a tenth more per halving).  64 tables, P = 2..512, 128 m: 16 x 2 takes 45 us, 16 x 1 70.
+    {
+        const int p_tiles = (n_P + kDecTileP - 1) / kDecTileP;
+        long long best = 0;
+        for (int tiles = std::min(2, p_tiles); tiles >= 1; --tiles) {
+            for (int mg = kDecMG; mg >= kDecWarps; mg >>= 1) {  // never fewer than one message size per warp
+                const int groups = (n_m + mg - 1) / mg, p_ctas = (p_tiles + tiles - 1) / tiles;
+                const long long waves = ((long long)groups * p_ctas * h->T.n_tables + h->sm_count * 4 - 1) / (h->sm_count * 4);
+                const long long cost = waves * (3500 + (std::min(mg, n_m) + kDecWarps - 1) / kDecWarps * (5000 + 5500LL * tiles)) * (kDecMG / mg + 9);
+                if (best && cost >= best) continue;
+                best = cost;
+                pl.dec_mg = mg; pl.dec_tiles = tiles; pl.dec_mgroups = groups; pl.dec_ptiles = p_ctas;
+            }
+        }
     }
     const int dec_p = pl.dec_tiles * kDecTileP;
     for (int t = 0; t < pl.dec_ptiles; ++t) {

@@ -182,13 +182,9 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
         warp_min_pair(qmin, qidx);
         if (lane == 0) { s_redt[warp] = qmin; s_cnt[32 + warp] = qidx; }
         __syncthreads();
-        double q = s_redt[0];
-        int qi = s_cnt[32];
-        for (int w = 1; w < n_warps; ++w) {
-            const double q2 = s_redt[w];
-            const int i2 = s_cnt[32 + w];
-            if (q2 < q || (q2 == q && i2 < qi)) { q = q2; qi = i2; }
-        }
+        double q = lane < n_warps ? s_redt[lane] : CUDART_INF;
+        int qi = lane < n_warps ? s_cnt[32 + lane] : 0x7FFFFFFF;
+        warp_min_pair(q, qi);
         for (int pidx = tid; pidx < n_P; pidx += T) {
             const int P = P_at(p.G, pidx);
             if (has2) {
@@ -247,6 +243,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
             int lo, hi;
             bracket(s_opt[c], s_opt[min(c + 1, n_c - 1)], lo, hi);
             const double x = static_cast<double>(P_at(p.G, pidx) - 1);
+            if (coarse_index(c, p.coarse_log) == pidx) lo = hi = s_opt[c];  // a coarse one itself: already found
             double tb = CUDART_INF;
             int eb = lo;
             for (int e = lo; e <= hi; ++e) {
