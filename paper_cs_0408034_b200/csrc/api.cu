@@ -785,8 +785,10 @@ int plogp_select_best_host(plogp_tables *h, const plogp_grid *grid, uint8_t *h_s
     if (plan->empty) return PLOGP_OK;
     const size_t cells = size_t(2) * plan->G.n_P * plan->G.n_m;  // per table
     const size_t per_table = cells * 13 + 3 * 256;
-    // tables per staging set: at most 512 MiB, at least one table
+    // Tables per staging set: at most 512 MiB, at least one table.  The first set is an eighth of the whole (4 MiB or more),
+    // so that the first copy starts early and its kernels are all that the copies do not hide.
     const int batch = int(std::min<size_t>(h->T.n_tables, std::max<size_t>(1, (size_t(512) << 20) / per_table)));
+    const int first = int(std::min<size_t>(batch, std::max<size_t>((h->T.n_tables + 7) / 8, (size_t(4) << 20) / per_table + 1)));
     const size_t need = per_table * batch;
     if (need > h->stage_cap) {
         for (int i = 0; i < 2; ++i) {
@@ -810,13 +812,13 @@ int plogp_select_best_host(plogp_tables *h, const plogp_grid *grid, uint8_t *h_s
     }
     auto align = [](size_t x) { return (x + 255) / 256 * 256; };
     int slot = 0;
-    for (int t0 = 0; t0 < h->T.n_tables; t0 += batch, slot ^= 1) {
-        const int nt = std::min(batch, h->T.n_tables - t0);
+    for (int t0 = 0, nt; t0 < h->T.n_tables; t0 += nt, slot ^= 1) {
+        nt = std::min(t0 == 0 ? first : batch, h->T.n_tables - t0);
         // layout of a staging set: time | segment size | strategy, each for nt tables
         double *s_time = reinterpret_cast<double *>(h->d_stage[slot]);
         uint32_t *s_sb = reinterpret_cast<uint32_t *>(h->d_stage[slot] + align(cells * 8 * batch));
         uint8_t *s_id = h->d_stage[slot] + align(cells * 8 * batch) + align(cells * 4 * batch);
-        if (t0 >= 2 * batch) {  // the set's previous copy has left
+        if (t0 >= first + batch) {  // the set's previous copy has left
             cudaError_t ew = cudaStreamWaitEvent(st, h->ev_copied[slot], 0);
             if (ew != cudaSuccess) { rc = cuda_fail(ew, "cudaStreamWaitEvent"); break; }
         }
@@ -900,11 +902,14 @@ int plogp_segment_surface(plogp_tables *h, const plogp_grid *grid, double *d_sur
     if (rc != PLOGP_OK) return rc;
     const Plan &pl = *plan;
     if (pl.empty || pl.n_seg == 0 || pl.G.n_s == 0) return PLOGP_OK;
+    // up to four message sizes per warp, while that leaves eight CTAs per SM
+    int surf_m = 32;
+    while (surf_m > 8 && (long long)((pl.G.n_m + surf_m - 1) / surf_m) * ((pl.G.n_P + 7) / 8) * h->T.n_tables < (long long)h->sm_count * 8) surf_m >>= 1;
     for (int t0 = 0; t0 < h->T.n_tables; t0 += 65535) {
         SensParams sp{};
         sp.T = h->T; sp.G = pl.G;
         sp.table0 = t0; sp.n_tables_launch = std::min(65535, h->T.n_tables - t0); sp.out_table0 = 0;
-        sp.surface = d_surface;
+        sp.surface = d_surface; sp.surf_m = surf_m;
         CK(launch_surface(sp, st));
         g_launches += 1;
     }
@@ -928,14 +933,16 @@ int plogp_segment_sensitivity(plogp_tables *h, const plogp_grid *grid, uint64_t 
     const Plan &pl = *plan;
     if (pl.empty || pl.n_seg == 0) return PLOGP_OK;
     // enough CTAs to fill the GPU, each with a run of process counts per warp
-    const long long base_blocks = (long long)((pl.G.n_m + 31) / 32) * h->T.n_tables;
+    const bool aligned = (reinterpret_cast<uintptr_t>(d_pred_time) | reinterpret_cast<uintptr_t>(d_time_fixed) | reinterpret_cast<uintptr_t>(d_ratio)) % 16 == 0;
+    const int vec = pl.G.n_m % 2 == 0 && aligned && (pl.G.n_m + 63) / 64 * 2 == (pl.G.n_m + 31) / 32 ? 2 : 1;
+    const long long base_blocks = (long long)((pl.G.n_m + 32 * vec - 1) / (32 * vec)) * h->T.n_tables;
     int p_per_cta = pl.G.n_P;
     while (p_per_cta > 8 && base_blocks * ((pl.G.n_P + p_per_cta - 1) / p_per_cta) < (long long)h->sm_count * 8) p_per_cta = (p_per_cta + 1) / 2;
     for (int t0 = 0; t0 < h->T.n_tables; t0 += 65535) {
         SensParams sp{};
         sp.T = h->T; sp.G = pl.G;
         sp.table0 = t0; sp.n_tables_launch = std::min(65535, h->T.n_tables - t0); sp.out_table0 = 0;
-        sp.s_fixed = uint32_t(s_fixed); sp.p_per_cta = p_per_cta;
+        sp.s_fixed = uint32_t(s_fixed); sp.p_per_cta = p_per_cta; sp.vec = vec;
         sp.pred_time = d_pred_time; sp.time_fixed = d_time_fixed; sp.ratio = d_ratio;
         CK(launch_fixed(sp, st));
         g_launches += 1;

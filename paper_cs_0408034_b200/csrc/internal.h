@@ -96,9 +96,11 @@ struct SensParams {
     TableDev T;
     GridDev G;
     int table0, n_tables_launch, out_table0;
+    int surf_m;                // message sizes per CTA (surface_kernel)
     double *surface;           // [n_tables][3][n_P][n_m][n_s]
     uint32_t s_fixed;          // the fixed segment size (fixed_kernel)
     int p_per_cta;             // process counts per CTA (fixed_kernel)
+    int vec;                   // message sizes per lane (fixed_kernel): 2 where n_m is even and the arrays are 16-byte aligned
     const double *pred_time;   // [n_tables][13][n_P][n_m] from plogp_predict, or nullptr together with ratio
     double *time_fixed, *ratio;  // [n_tables][3][n_P][n_m]
 };

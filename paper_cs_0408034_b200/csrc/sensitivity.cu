@@ -11,89 +11,140 @@
 
 namespace plogp {
 
-// One CTA: one table, one message size, kSurfP consecutive process counts; threads <-> candidate sizes, so
-// g(s), k and the line coefficients are computed once per candidate and serve 3 x kSurfP outputs, and every
-// store is a run of consecutive s.
-constexpr int kSurfP = 8;
+// One CTA: one table, p.surf_m message sizes (its warps stride over them), kSurfP consecutive process counts; lanes <->
+// candidate sizes, so g(s) is computed once per CTA, k and the line coefficients once per (m, s), and every store is a
+// run of consecutive s.
+constexpr int kSurfP = 8, kSurfW = 8, kSurfS = 32 * kSurfW;
 
-__global__ void __launch_bounds__(256) surface_kernel(const SensParams p)
+__global__ void __launch_bounds__(kSurfS) surface_kernel(const SensParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *s_tab = reinterpret_cast<double *>(smem_raw);
-    const int midx = blockIdx.x % p.G.n_m, pchunk = blockIdx.x / p.G.n_m, trel = blockIdx.y;
+    double *s_gs = s_tab + 3 * p.T.npad;  // [kSurfS]
+    const int n_s = p.G.n_s, n_P = p.G.n_P, n_m = p.G.n_m;
+    const int n_mg = (n_m + p.surf_m - 1) / p.surf_m;
+    const int mgroup = blockIdx.x % n_mg, pchunk = blockIdx.x / n_mg, trel = blockIdx.y;
     const int table = p.table0 + trel;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     stage_table(s_tab, p.T, table);
     __syncthreads();
     const double L = p.T.lat[table];
-    const uint32_t m_u = p.G.m_list[midx];
-    const uint32_t mask = p.G.mask;
-    const int n_s = p.G.n_s, n_P = p.G.n_P, n_m = p.G.n_m;
+    const bool on2 = (p.G.mask >> 2) & 1u, on5 = (p.G.mask >> 5) & 1u, on9 = (p.G.mask >> 9) & 1u;
     const int p0 = pchunk * kSurfP, p1 = min(p0 + kSurfP, n_P);
     const double nan = CUDART_NAN;
-    for (int si = threadIdx.x; si < n_s; si += blockDim.x) {
-        const uint32_t s = s_at(p.G, si);
-        const bool fits = s <= m_u;
-        double B = nan, C = nan, Q = nan;
-        if (fits) {
-            const double gs = gap_at(s_tab, p.T.npad, static_cast<double>(s));
-            const double k = static_cast<double>(segments(m_u, s, p.G.k_mode));
-            B = gs + L;
-            C = gs * (k - 1.0);
-            Q = gs * k;
+    const size_t plane = static_cast<size_t>(n_P) * n_m * n_s, step = static_cast<size_t>(n_m) * n_s;
+    for (int s0 = 0; s0 < n_s; s0 += kSurfS) {
+        const int si_t = s0 + threadIdx.x;
+        if (s0 > 0) __syncthreads();  // the previous chunk's gaps have been read
+        if (si_t < n_s) s_gs[threadIdx.x] = gap_at(s_tab, p.T.npad, static_cast<double>(s_at(p.G, si_t)));
+        __syncthreads();
+        for (int midx = mgroup * p.surf_m + warp; midx < min((mgroup + 1) * p.surf_m, n_m); midx += kSurfW) {
+        const uint32_t m_u = p.G.m_list[midx];
+        for (int c = lane; c < min(kSurfS, n_s - s0); c += 32) {
+            const uint32_t s = s_at(p.G, s0 + c);
+            const bool fits = s <= m_u;
+            double B = nan, C = nan, Q = nan;
+            if (fits) {
+                const double gs = s_gs[c], k = static_cast<double>(segments(m_u, s, p.G.k_mode));
+                B = gs + L;
+                C = gs * (k - 1.0);
+                Q = gs * k;
+            }
+            double *out = p.surface + (static_cast<size_t>(table - p.out_table0) * 3 * n_P + p0) * step + static_cast<size_t>(midx) * n_s + s0 + c;
+            for (int pi = p0; pi < p1; ++pi, out += step) {
+                const int P = P_at(p.G, pi);
+                const double pm1 = static_cast<double>(P - 1);
+                if (on2) out[0] = fits ? fma(pm1, Q, L) : nan;      // (P-1) (g(s) k) + L
+                if (on5) out[plane] = fits ? fma(pm1, B, C) : nan;  // (P-1) (g(s)+L) + g(s)(k-1)
+                if (on9)                                            // floor(log2 P) g(s) k + ceil(log2 P) L
+                    out[2 * plane] = fits ? fma(static_cast<double>(31 - __clz(P)), Q, static_cast<double>(32 - __clz(P - 1)) * L) : nan;
+            }
         }
-        for (int pi = p0; pi < p1; ++pi) {
-            const int P = P_at(p.G, pi);
-            const double pm1 = static_cast<double>(P - 1);
-            const size_t o = ((static_cast<size_t>(table - p.out_table0) * 3 * n_P + pi) * n_m + midx) * n_s + si;
-            const size_t plane = static_cast<size_t>(n_P) * n_m * n_s;
-            if ((mask >> 2) & 1u) p.surface[o] = fits ? fma(pm1, Q, L) : nan;                      // (P-1) (g(s) k) + L
-            if ((mask >> 5) & 1u) p.surface[o + plane] = fits ? fma(pm1, B, C) : nan;              // (P-1) (g(s)+L) + g(s)(k-1)
-            if ((mask >> 9) & 1u)                                                                  // floor(log2 P) g(s) k + ceil(log2 P) L
-                p.surface[o + 2 * plane] = fits ? fma(static_cast<double>(31 - __clz(P)), Q, static_cast<double>(32 - __clz(P - 1)) * L) : nan;
         }
     }
 }
 
-// One CTA: one table, 32 consecutive message sizes (lanes), a chunk of process counts (warps stride over it).
+// One CTA: one table, 32 V consecutive message sizes (V per lane), a chunk of process counts (warps stride over it).
+// Bound by HBM: three planes read, six written.  256 tables, P = 2..512, 128 m (1.2 GB): 257 us with one size per lane
+// and 64-bit index arithmetic per store, 207 us (5.8 TB/s) with two, running pointers and the loads first.
+template <int V> struct FixedVec;
+template <> struct FixedVec<1> {
+    static __device__ __forceinline__ void load(double *v, const double *p) { v[0] = __ldcs(p); }
+    static __device__ __forceinline__ void store(double *p, const double *v) { __stcs(p, v[0]); }
+};
+template <> struct FixedVec<2> {
+    static __device__ __forceinline__ void load(double *v, const double *p)
+    {
+        const double2 t = __ldcs(reinterpret_cast<const double2 *>(p));
+        v[0] = t.x; v[1] = t.y;
+    }
+    static __device__ __forceinline__ void store(double *p, const double *v) { __stcs(reinterpret_cast<double2 *>(p), make_double2(v[0], v[1])); }
+};
+
+template <int V>
 __global__ void __launch_bounds__(256) fixed_kernel(const SensParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *s_tab = reinterpret_cast<double *>(smem_raw);
-    const int n_mtiles = (p.G.n_m + 31) / 32;
+    const int n_mtiles = (p.G.n_m + 32 * V - 1) / (32 * V);
     const int mtile = blockIdx.x % n_mtiles, pchunk = blockIdx.x / n_mtiles, trel = blockIdx.y;
     const int table = p.table0 + trel;
     stage_table(s_tab, p.T, table);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    const int midx = mtile * 32 + lane;
-    if (midx >= p.G.n_m) return;  // no barriers below
+    const int midx = mtile * 32 * V + lane * V;
+    if (midx >= p.G.n_m) return;  // no barriers below; V = 2 is taken for even n_m only
     const double L = p.T.lat[table];
-    const uint32_t m_u = p.G.m_list[midx];
-    // the fixed size where it fits, else the whole message in one segment (Section 3.1)
-    const uint32_t s_eff = p.s_fixed <= m_u ? p.s_fixed : m_u;
-    const double gs = gap_at(s_tab, p.T.npad, static_cast<double>(s_eff));
-    const double k = static_cast<double>(segments(m_u, s_eff, p.G.k_mode));
-    const double B = gs + L, C = gs * (k - 1.0), Q = gs * k;
+    double B[V], C[V], Q[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const uint32_t m_u = p.G.m_list[midx + v];
+        // the fixed size where it fits, else the whole message in one segment (Section 3.1)
+        const uint32_t s_eff = p.s_fixed <= m_u ? p.s_fixed : m_u;
+        const double gs = gap_at(s_tab, p.T.npad, static_cast<double>(s_eff));
+        const double k = static_cast<double>(segments(m_u, s_eff, p.G.k_mode));
+        B[v] = gs + L; C[v] = gs * (k - 1.0); Q[v] = gs * k;
+    }
     const uint32_t mask = p.G.mask;
+    const bool on[3] = {((mask >> 2) & 1u) != 0, ((mask >> 5) & 1u) != 0, ((mask >> 9) & 1u) != 0};
+    const int ids[3] = {2, 5, 9};
     const int n_P = p.G.n_P, n_m = p.G.n_m;
     const size_t plane = static_cast<size_t>(n_P) * n_m;
     const int p0 = pchunk * p.p_per_cta, p1 = min(p0 + p.p_per_cta, n_P);
+    const size_t cell = static_cast<size_t>(p0 + warp) * n_m + midx, step = static_cast<size_t>(n_warps) * n_m;
+    double *out = p.time_fixed + static_cast<size_t>(table - p.out_table0) * 3 * plane + cell;
+    double *rat = p.ratio ? p.ratio + static_cast<size_t>(table - p.out_table0) * 3 * plane + cell : nullptr;
+    const double *in = p.pred_time ? p.pred_time + static_cast<size_t>(table - p.out_table0) * 13 * plane + cell : nullptr;
     for (int pi = p0 + warp; pi < p1; pi += n_warps) {
-        const int P = P_at(p.G, pi);
-        const double pm1 = static_cast<double>(P - 1);
-        const size_t cell = static_cast<size_t>(pi) * n_m + midx;
-        const size_t o3 = static_cast<size_t>(table - p.out_table0) * 3 * plane + cell;
-        const size_t o13 = static_cast<size_t>(table - p.out_table0) * 13 * plane + cell;
-        double t[3];
-        t[0] = fma(pm1, Q, L);
-        t[1] = fma(pm1, B, C);
-        t[2] = fma(static_cast<double>(31 - __clz(P)), Q, static_cast<double>(32 - __clz(P - 1)) * L);
-        const int ids[3] = {2, 5, 9};
+        double best[3][V];
+        if (rat) {
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (!((mask >> ids[q]) & 1u)) continue;
-            p.time_fixed[o3 + q * plane] = t[q];
-            if (p.ratio) p.ratio[o3 + q * plane] = t[q] / p.pred_time[o13 + ids[q] * plane];
+            for (int q = 0; q < 3; ++q)
+                if (on[q]) FixedVec<V>::load(best[q], in + ids[q] * plane);
+            in += step;
+        }
+        const int P = P_at(p.G, pi);
+        const double pm1 = static_cast<double>(P - 1), lf = static_cast<double>(31 - __clz(P)), lcL = static_cast<double>(32 - __clz(P - 1)) * L;
+        double t[3][V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            t[0][v] = fma(pm1, Q[v], L);
+            t[1][v] = fma(pm1, B[v], C[v]);
+            t[2][v] = fma(lf, Q[v], lcL);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (on[q]) FixedVec<V>::store(out + q * plane, t[q]);
+        out += step;
+        if (rat) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                if (!on[q]) continue;
+#pragma unroll
+                for (int v = 0; v < V; ++v) t[q][v] /= best[q][v];
+                FixedVec<V>::store(rat + q * plane, t[q]);
+            }
+            rat += step;
         }
     }
 }
@@ -112,63 +163,68 @@ __global__ void boundary_kernel(const uint8_t *strategy, uint8_t *boundary, long
     }
 }
 
-// The same, eight consecutive message sizes per thread (n_m a multiple of 8, both arrays 8-byte aligned):
-// one 8-byte load of the row, one of the next row, one 8-byte store.
-__global__ void boundary8_kernel(const uint8_t *strategy, uint8_t *boundary, long long n_planes, int n_P, int n_m)
+// The same, 4 W consecutive message sizes per thread (n_m a multiple of that, arrays aligned for it), walking down
+// kBndRows process counts, so that every row is read once and the index arithmetic is shared (256 tables, P = 2..512,
+// 128 m, 67 MB: 29 us with one row of 8 sizes per thread, 17 us so).
+constexpr int kBndRows = 8;
+template <int W>
+__global__ void __launch_bounds__(256) boundary_rows_kernel(const uint8_t *strategy, uint8_t *boundary, long long n_planes, int n_P, int n_m)
 {
-    const int groups = n_m >> 3;
-    const long long total = n_planes * n_P * groups;
-    for (long long gidx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; gidx < total;
-         gidx += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int g = static_cast<int>(gidx % groups), ip = static_cast<int>((gidx / groups) % n_P);
-        const long long i = (gidx / groups) * n_m + 8LL * g;
-        const unsigned long long row = *reinterpret_cast<const unsigned long long *>(strategy + i);
-        const unsigned long long below = ip + 1 < n_P ? *reinterpret_cast<const unsigned long long *>(strategy + i + n_m) : row;
-        // the right neighbours: this group shifted by one byte, its last byte taken from the next group (or itself
-        // at the end of the row, which has no neighbour)
-        const unsigned long long last = g + 1 < groups ? strategy[i + 8] : (row >> 56);
-        const unsigned long long right = (row >> 8) | (last << 56);
-        unsigned long long out = 0;
+    struct __align__(4 * W) Words { unsigned w[W]; };
+    const int groups = n_m / (4 * W), chunks = (n_P + kBndRows - 1) / kBndRows;
+    const long long total = n_planes * chunks * groups;
+    for (long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; idx < total; idx += static_cast<long long>(gridDim.x) * blockDim.x) {
+        const long long rest = idx / groups;
+        const int g = static_cast<int>(idx - rest * groups);
+        const long long pl = rest / chunks;
+        const int ip0 = static_cast<int>(rest - pl * chunks) * kBndRows, ip1 = min(ip0 + kBndRows, n_P);
+        const uint8_t *in = strategy + (pl * n_P + ip0) * n_m + 4LL * W * g;
+        uint8_t *out = boundary + (in - strategy);
+        Words row = *reinterpret_cast<const Words *>(in);
+        for (int ip = ip0; ip < ip1; ++ip, in += n_m, out += n_m) {
+            const Words below = ip + 1 < n_P ? *reinterpret_cast<const Words *>(in + n_m) : row;
+            // the right neighbours: this group shifted by one byte, its last byte taken from the next group (or itself
+            // at the end of the row, which has no neighbour)
+            const unsigned last = g + 1 < groups ? in[4 * W] : row.w[W - 1] >> 24;
+            Words o;
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const unsigned long long sh = 8ull * b;
-            const unsigned f = (((row >> sh) & 0xFF) != ((below >> sh) & 0xFF) ? 1u : 0u) |
-                               (((row >> sh) & 0xFF) != ((right >> sh) & 0xFF) ? 2u : 0u);
-            out |= static_cast<unsigned long long>(f) << sh;
+            for (int w = 0; w < W; ++w) {
+                const unsigned right = __funnelshift_r(row.w[w], w + 1 < W ? row.w[w + 1] : last, 8);
+                o.w[w] = __vsetne4(row.w[w], below.w[w]) | __vsetne4(row.w[w], right) << 1;
+            }
+            *reinterpret_cast<Words *>(out) = o;
+            row = below;
         }
-        *reinterpret_cast<unsigned long long *>(boundary + i) = out;
     }
 }
 
 cudaError_t launch_surface(const SensParams &p, cudaStream_t st)
 {
-    const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double);
-    const long long bx = static_cast<long long>(p.G.n_m) * ((p.G.n_P + kSurfP - 1) / kSurfP);
+    const size_t smem = (3 * static_cast<size_t>(p.T.npad) + kSurfS) * sizeof(double);
+    const long long bx = static_cast<long long>((p.G.n_m + p.surf_m - 1) / p.surf_m) * ((p.G.n_P + kSurfP - 1) / kSurfP);
     if (bx <= 0 || bx > 0x7FFFFFFFLL || p.n_tables_launch <= 0 || p.n_tables_launch > 65535) return cudaErrorInvalidConfiguration;
-    const int threads = std::min(256, std::max(32, (p.G.n_s + 31) / 32 * 32));
-    dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(p.n_tables_launch));
-    surface_kernel<<<grid, threads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(surface_kernel, static_cast<unsigned>(bx), static_cast<unsigned>(p.n_tables_launch), kSurfS, smem, st, false, p);
 }
 
 cudaError_t launch_fixed(const SensParams &p, cudaStream_t st)
 {
     const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double);
-    const long long bx = static_cast<long long>((p.G.n_m + 31) / 32) * ((p.G.n_P + p.p_per_cta - 1) / p.p_per_cta);
+    const int per_cta = 32 * p.vec;
+    const long long bx = static_cast<long long>((p.G.n_m + per_cta - 1) / per_cta) * ((p.G.n_P + p.p_per_cta - 1) / p.p_per_cta);
     if (bx <= 0 || bx > 0x7FFFFFFFLL || p.n_tables_launch <= 0 || p.n_tables_launch > 65535) return cudaErrorInvalidConfiguration;
-    dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(p.n_tables_launch));
-    fixed_kernel<<<grid, 256, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch(p.vec == 2 ? fixed_kernel<2> : fixed_kernel<1>, static_cast<unsigned>(bx), static_cast<unsigned>(p.n_tables_launch), 256, smem, st, false, p);
 }
 
 cudaError_t launch_boundaries(const uint8_t *d_strategy, uint8_t *d_boundary, long long n_planes, int n_P, int n_m, int sm_count, cudaStream_t st)
 {
     const long long total = n_planes * n_P * n_m;
     if (total <= 0) return cudaSuccess;
-    const bool wide = n_m % 8 == 0 && reinterpret_cast<uintptr_t>(d_strategy) % 8 == 0 && reinterpret_cast<uintptr_t>(d_boundary) % 8 == 0;
-    const long long want = ((wide ? total / 8 : total) + 255) / 256;
-    const unsigned blocks = static_cast<unsigned>(std::min<long long>(want, static_cast<long long>(sm_count) * 32));
-    if (wide) boundary8_kernel<<<blocks, 256, 0, st>>>(d_strategy, d_boundary, n_planes, n_P, n_m);
+    const uintptr_t both = reinterpret_cast<uintptr_t>(d_strategy) | reinterpret_cast<uintptr_t>(d_boundary);
+    const int w = n_m % 16 == 0 && both % 16 == 0 ? 4 : (n_m % 8 == 0 && both % 8 == 0 ? 2 : 0);
+    const long long items = w ? n_planes * ((n_P + kBndRows - 1) / kBndRows) * (n_m / (4 * w)) : total;
+    const unsigned blocks = static_cast<unsigned>(std::min<long long>((items + 255) / 256, static_cast<long long>(sm_count) * 32));
+    if (w == 4) boundary_rows_kernel<4><<<blocks, 256, 0, st>>>(d_strategy, d_boundary, n_planes, n_P, n_m);
+    else if (w == 2) boundary_rows_kernel<2><<<blocks, 256, 0, st>>>(d_strategy, d_boundary, n_planes, n_P, n_m);
     else boundary_kernel<<<blocks, 256, 0, st>>>(d_strategy, d_boundary, n_planes, n_P, n_m);
     return cudaGetLastError();
 }

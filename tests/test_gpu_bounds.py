@@ -82,3 +82,15 @@ def test_alternating_grids_keep_their_plans(plogp):
             d = plogp.select_best(tabs, w)
             assert torch.equal(d.strategy, f.strategy) and torch.equal(d.s_bytes, f.s_bytes) and torch.equal(d.time, f.time)
         torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n_m", [7, 8, 16, 24, 32, 40])
+@pytest.mark.parametrize("n_P", [1, 7, 8, 9, 17])
+def test_boundaries_of_random_maps(plogp, n_m, n_P):
+    """One byte, 8 and 16 bytes per thread; runs of 8 process counts that end inside, at and past a table's last row."""
+    import torch
+    from oracle import plogp_oracle as po
+    rng = np.random.default_rng(n_m * 100 + n_P)
+    s = rng.integers(0, 3, size=(3, 2, n_P, n_m)).astype(np.uint8) * 200  # neighbouring bytes must not touch one another
+    dec = plogp.DecisionTable(torch.as_tensor(s, device="cuda"), None, None)
+    assert np.array_equal(plogp.decision_boundaries(dec).cpu().numpy(), po.decision_boundaries(s))
