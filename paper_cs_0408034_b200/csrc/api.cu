@@ -69,7 +69,7 @@ struct Plan {
     // Scatter decision kernel: its own split of P (vec = 2: two message sizes per lane, where the outputs allow it)
     int sc_vec = 1, sc_ptiles = 1, sc_run = 1;
     // decision kernel tiling (short candidate lists)
-    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_tiles = 1, dec_pairs = 1;
+    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_rows = 8, dec_tiles = 1, dec_pairs = 1;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
     size_t off_pair_m = 0, off_pair_chunk = 0, off_pair_row = 0, off_pair_base = 0;
@@ -316,24 +316,29 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
     }
 
     // Tiling of the lane <-> P kernels.  Wide CTAs (16 message sizes: 128-byte output rows; two tiles of process counts: the
-    // candidate lists are built once for both) against the last wave of CTAs: the choice with the smallest number of
-    // waves times the cost of a CTA, in cycles as measured on the batched workload (a message size's lists and pairs
-    // 5000, each of its tiles 5500, 3500 besides; narrower rows cost about a tenth more per halving).  64 tables, P = 2..512, 128 m: 16 x 2 takes 45 us, 16 x 1 70.
+    // candidate lists are built once for both; 8 process counts per lane) against the last wave of CTAs: the choice with the
+    // smallest number of waves times the cost of a CTA, in cycles as measured on the batched workload (a message size's
+    // lists and pairs 5000, each of its tiles 5500 with 8 rows and 3200 with 4, 3500 besides; narrower output rows cost
+    // about a tenth more per halving).  64 tables, P = 2..512, 128 m: 16 x 2 tiles takes 45 us, 16 x 1 70; one table,
+    // P = 2..1024, 256 m, 64 candidates: 4 x 1 tile of 4 rows 14.7 us, of 8 rows 19.
     {
-        const int p_tiles = (n_P + kDecTileP - 1) / kDecTileP;
         long long best = 0;
-        for (int tiles = std::min(2, p_tiles); tiles >= 1; --tiles) {
-            for (int mg = kDecMG; mg >= kDecWarps; mg >>= 1) {  // never fewer than one message size per warp
-                const int groups = (n_m + mg - 1) / mg, p_ctas = (p_tiles + tiles - 1) / tiles;
-                const long long waves = ((long long)groups * p_ctas * h->T.n_tables + h->sm_count * 4 - 1) / (h->sm_count * 4);
-                const long long cost = waves * (3500 + (std::min(mg, n_m) + kDecWarps - 1) / kDecWarps * (5000 + 5500LL * tiles)) * (kDecMG / mg + 9);
-                if (best && cost >= best) continue;
-                best = cost;
-                pl.dec_mg = mg; pl.dec_tiles = tiles; pl.dec_mgroups = groups; pl.dec_ptiles = p_ctas;
+        for (int rows = 8; rows >= 4; rows -= 4) {
+            const int p_tiles = (n_P + 32 * rows - 1) / (32 * rows);
+            for (int tiles = std::min(2, p_tiles); tiles >= 1; --tiles) {
+                for (int mg = kDecMG; mg >= kDecWarps; mg >>= 1) {  // never fewer than one message size per warp
+                    const int groups = (n_m + mg - 1) / mg, p_ctas = (p_tiles + tiles - 1) / tiles;
+                    const long long waves = ((long long)groups * p_ctas * h->T.n_tables + h->sm_count * 4 - 1) / (h->sm_count * 4);
+                    const long long per_m = 5000 + (rows == 8 ? 5500LL : 3200LL) * tiles;
+                    const long long cost = waves * (3500 + (std::min(mg, n_m) + kDecWarps - 1) / kDecWarps * per_m) * (kDecMG / mg + 9);
+                    if (best && cost >= best) continue;
+                    best = cost;
+                    pl.dec_rows = rows; pl.dec_mg = mg; pl.dec_tiles = tiles; pl.dec_mgroups = groups; pl.dec_ptiles = p_ctas;
+                }
             }
         }
     }
-    const int dec_p = pl.dec_tiles * kDecTileP;
+    const int dec_p = pl.dec_tiles * 32 * pl.dec_rows;
     for (int t = 0; t < pl.dec_ptiles; ++t) {
         const int first = t * dec_p, last = std::min(n_P, first + dec_p) - 1;
         const int64_t P0 = g->P ? g->P[first] : int64_t(g->P_lo) + first, P1 = g->P ? g->P[last] : int64_t(g->P_lo) + last;
@@ -540,7 +545,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             // come from the lane<->P kernel; fused_kernel then writes the closed-form planes only.
             SegminParams sp{};
             sp.T = h->T; sp.G = pl.G;
-            sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs;
+            sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs;
             sp.table0 = t0; sp.n_tables_launch = nt; sp.out_table0 = out.out_table0;
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
             sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;
@@ -557,7 +562,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             DecideParams dp{};
             dp.T = h->T; dp.G = pl.G;
             dp.G.mask &= 0x3FFu;
-            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs;
+            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.rows = pl.dec_rows; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs;
             dp.table0 = t0; dp.n_tables_launch = nt; dp.out_table0 = out.out_table0; dp.om = out.om;
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
             dp.envelope = pl.envelope_short ? 1 : 0;

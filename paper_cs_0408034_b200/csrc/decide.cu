@@ -36,11 +36,11 @@ namespace plogp {
 
 namespace {
 
-constexpr int R = kDecR;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr uint32_t kCandNone = 255;   // winner is an unsegmented strategy
 constexpr uint32_t kCandWhole = 254;  // segmented winner with no fitting candidate: the whole message
 constexpr int kPilots = 4;
+static_assert(kMaxInlineS <= 64, "a lane builds at most two candidates");
 constexpr int kStep = 16;  // lines per vote of the exact search
 constexpr int kIntMax = 0x7FFFFFFF;
 
@@ -61,10 +61,10 @@ __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a *
 
 // Shared-memory layout.  cap: lines of one message size (a multiple of kStep); n_pairs: (floor, ceil) pairs of a CTA at most.
 // A slot number fits a byte: at most 144 lines and 61 pairs.
-__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int tiles, unsigned char *base, DecSmem *o)
+__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int n_p, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(2 * nsv + 4, kStep), cap_q = round_up(nsv, 4), slots = cap + n_pairs, n_p = tiles * kDecTileP, pos_stride = n_p + 4;
+    const int cap = round_up(2 * nsv + 4, kStep), cap_q = round_up(nsv, 4), slots = cap + n_pairs, pos_stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
@@ -89,13 +89,16 @@ __device__ __forceinline__ int hi32(double x) { return __double2hiint(x); }
 }  // namespace
 
 // ENV: lower-envelope search (DecideParams::envelope), compiled apart so that the exhaustive kernel carries none of it.
-template <bool ENV>
+// R: process counts per lane and tile, 8, or 4 on grids that leave the GPU part empty (twice as many, shorter CTAs).
+template <bool ENV, int R>
 __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecideParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
     DecSmem sm;
-    dec_layout(npad, p.G.n_s, p.n_pairs, p.tiles, smem_raw, &sm);
+    constexpr int kTileP = 32 * R;
+    const int n_p = p.tiles * kTileP;
+    dec_layout(npad, p.G.n_s, p.n_pairs, n_p, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
 
     int b = blockIdx.x;
@@ -107,13 +110,31 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = mgroup * p.mg;  // p.mg <= kDecMG message sizes per CTA (fewer on small grids, for more CTAs)
     const int n_mi = min(p.mg, p.G.n_m - m0);
-    const int n_p = p.tiles * kDecTileP, tile0 = ptile * n_p;
+    const int tile0 = ptile * n_p;
     const int n_valid = min(n_p, p.G.n_P - tile0);
     const int pair0 = pair_of(P_at(p.G, tile0)), n_pairs = pair_of(P_at(p.G, tile0 + n_valid - 1)) - pair0 + 1;
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
     dependents_may_start();
+    // what the set-up reads from global memory is on its way while the table is
+    const double L = p.T.lat[table];
+    const uint32_t m_mine = m0 + (tid & (kDecMG - 1)) < p.G.n_m ? p.G.m_list[m0 + (tid & (kDecMG - 1))] : 0u;
+    const uint32_t s_mine = tid < p.G.n_s ? s_at(p.G, tid) : 0u;
+    const int n_s = p.G.n_s;  // at most kMaxInlineS, fewer than the threads
+    int ns_next = 0;
+    uint32_t m_next = 0;
+    double k_next[2] = {1.0, 1.0};  // Section 2's k of this lane's candidates, from the host's table
+    auto fetch = [&](int mi) {
+        if (mi >= n_mi) return;
+        const int midx = m0 + mi;
+        ns_next = p.G.ns_of_m[midx];
+        m_next = p.G.m_list[midx];
+        const double *krow = p.G.k_list + static_cast<size_t>(midx) * n_s;
+        if (lane < n_s) k_next[0] = krow[lane];
+        if (lane + 32 < n_s) k_next[1] = krow[lane + 32];
+    };
+    fetch(warp);
     if (!grow) stage_table(sm.tab, p.T, table);
     else wait_for_kernel_in_front();  // the gap pre-pass
     for (int i = tid; i < n_p; i += kDecThreads) {
@@ -123,18 +144,16 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
         sm.pair[i] = static_cast<uint8_t>(min(pair_of(P) - pair0, n_pairs - 1));
     }
     __syncthreads();
-    const double L = p.T.lat[table];
-    for (int si = tid; si < p.G.n_s; si += kDecThreads) {
-        const uint32_t s = s_at(p.G, si);
-        sm.sval[si] = s;
-        sm.gs[si] = grow ? grow[1 + si] : gap_at(sm.tab, npad, static_cast<double>(s));
+    if (tid < n_s) {
+        sm.sval[tid] = s_mine;
+        sm.gs[tid] = grow ? grow[1 + tid] : gap_at(sm.tab, npad, static_cast<double>(s_mine));
     }
     if (tid == 0) sm.sval[kCandNone] = 0u;
     if (tid >= kDecThreads - kDecMG) {  // g(m) of the group's message sizes, by the last threads
         const int mi = tid - (kDecThreads - kDecMG);
-        if (mi < n_mi) sm.gm[mi] = grow ? grow[1 + p.G.n_s + m0 + mi] : gap_at(sm.tab, npad, static_cast<double>(p.G.m_list[m0 + mi]));
+        if (mi < n_mi) sm.gm[mi] = grow ? grow[1 + n_s + m0 + mi] : gap_at(sm.tab, npad, static_cast<double>(m_mine));
     }
-    const double g1 = grow ? grow[0] : gap_at(sm.tab, npad, 1.0);
+    const double g1 = grow ? grow[0] : gap_at_one(sm.tab, npad);
     const double rdv = 2.0 * g1 + 3.0 * L;  // rendezvous handshake: 2 g(1) + 3 L
     __syncthreads();
 
@@ -167,21 +186,6 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
     float *const lqf = sm.fq + warp * sm.cap_q;
 
     // what a message size reads from global memory is fetched while the one before it is worked on
-    const int n_s = p.G.n_s;
-    int ns_next = 0;
-    uint32_t m_next = 0;
-    double k_next[2] = {1.0, 1.0};  // Section 2's k of this lane's candidates, from the host's table
-    auto fetch = [&](int mi) {
-        if (mi >= n_mi) return;
-        const int midx = m0 + mi;
-        ns_next = p.G.ns_of_m[midx];
-        m_next = p.G.m_list[midx];
-        const double *krow = p.G.k_list + static_cast<size_t>(midx) * n_s;
-        if (lane < n_s) k_next[0] = krow[lane];
-        if (lane + 32 < n_s) k_next[1] = krow[lane + 32];
-    };
-    fetch(warp);
-
     for (int mi = warp; mi < n_mi; mi += kDecWarps) {
         const int ns = ns_next;
         const uint32_t m_u = m_next;
@@ -345,9 +349,9 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
         __syncwarp();
 
         for (int tile = 0; tile < p.tiles; ++tile) {
-            if (tile * kDecTileP >= n_valid) break;
-            const double *const xd = sm.pm1 + tile * kDecTileP + lane;
-            uint8_t *const pos = sm.pos + mi * sm.pos_stride + tile * kDecTileP + lane;
+            if (tile * kTileP >= n_valid) break;
+            const double *const xd = sm.pm1 + tile * kTileP + lane;
+            uint8_t *const pos = sm.pos + mi * sm.pos_stride + tile * kTileP + lane;
             float T[R];
             // ---- start of the running minima: the best of the pilots and the pair ----
             {
@@ -374,7 +378,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
                 if (any_log) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        const unsigned slot = sm.cap + sm.pair[tile * kDecTileP + 32 * r + lane];
+                        const unsigned slot = sm.cap + sm.pair[tile * kTileP + 32 * r + lane];
                         const double tl = line[slot].y;
                         if (tl < t[r] || n1 == 0) { t[r] = tl; at[r] = slot; }  // lines have the lower ids
                     }
@@ -391,7 +395,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
             float mn[R];
             f32x2 x2[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) { mn[r] = CUDART_INF_F; x2[r] = splat2(sm.x[tile * kDecTileP + 32 * r + lane]); }
+            for (int r = 0; r < R; ++r) { mn[r] = CUDART_INF_F; x2[r] = splat2(sm.x[tile * kTileP + 32 * r + lane]); }
 #pragma unroll 2
             for (int j = 0; j < n1p; j += 4) {
                 const f32x2x2 aa = *reinterpret_cast<const f32x2x2 *>(la + j), cc = *reinterpret_cast<const f32x2x2 *>(lc + j);
@@ -502,10 +506,12 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
 
 cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st)
 {
-    const size_t smem = dec_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles, nullptr, nullptr);
+    const size_t smem = dec_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, nullptr, nullptr);
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    return launch(p.envelope ? decide_kernel<true> : decide_kernel<false>, static_cast<unsigned>(blocks), 1, kDecThreads, smem, st, overlap, p);
+    const auto kernel = p.rows == 8 ? (p.envelope ? decide_kernel<true, 8> : decide_kernel<false, 8>)
+                                    : (p.envelope ? decide_kernel<true, 4> : decide_kernel<false, 4>);
+    return launch(kernel, static_cast<unsigned>(blocks), 1, kDecThreads, smem, st, overlap, p);
 }
 
 }  // namespace plogp

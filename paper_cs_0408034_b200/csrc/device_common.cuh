@@ -60,6 +60,13 @@ __device__ __forceinline__ double gap_at(const double *s_tab, int npad, double x
     return fma(dx, s_tab[2 * npad + i], s_tab[npad + i]);
 }
 
+// g(1): sizes are whole numbers, so 1 lies below the table or in one of its first two intervals
+__device__ __forceinline__ double gap_at_one(const double *s_tab, int npad)
+{
+    const int i = s_tab[1] <= 1.0 ? 1 : 0;
+    return fma(fmax(1.0 - s_tab[i], 0.0), s_tab[2 * npad + i], s_tab[npad + i]);
+}
+
 __device__ __forceinline__ int P_at(const GridDev &G, int pidx)
 {
     return G.P_list ? G.P_list[pidx] : G.P_lo + pidx;

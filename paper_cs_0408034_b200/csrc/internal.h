@@ -157,7 +157,8 @@ struct DecideParams {
     int gaps_stride;
     int n_mgroups, n_ptiles;
     int mg;  // message sizes per CTA, 1..kDecMG
-    int tiles;    // tiles of kDecTileP process counts per CTA
+    int rows;     // process counts per lane and tile: 8 or 4
+    int tiles;    // tiles of 32 x rows process counts per CTA
     int n_pairs;  // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most
     int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cu)
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16 / 8 / 2-byte aligned bases)
@@ -171,8 +172,6 @@ struct DecideParams {
 
 constexpr int kDecThreads = 128;
 constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kDecR = 8;                               // process counts per thread
-constexpr int kDecTileP = 32 * kDecR;                  // 256 process counts per CTA, shared by its warps
 constexpr int kDecMG = 16;                             // message sizes per CTA (at most), split over the warps
 
 // segmin_kernel (segmented minima of plogp_predict on short candidate lists, lanes <-> P): see segmin.cu
@@ -183,17 +182,15 @@ struct SegminParams {
     int gaps_stride;
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16-byte aligned times, 8-byte aligned sizes)
     int n_mgroups, n_ptiles;
-    int mg, tiles, n_pairs;  // as in DecideParams
+    int mg, rows, tiles, n_pairs;  // as in DecideParams
     int table0, n_tables_launch, out_table0;
     double *p_time;      // [n_tables][13][n_P][n_m]: planes 2, 5, 9 are written
     uint32_t *p_best_s;  // [n_tables][3][n_P][n_m], or nullptr
 };
 constexpr int kSegThreads = 128;
 constexpr int kSegWarps = kSegThreads / 32;
-constexpr int kSegR = 8;                 // process counts per thread
-constexpr int kSegTileP = 32 * kSegR;    // process counts per tile
 constexpr int kSegMG = 16;               // message sizes per CTA (at most), split over the warps
-static_assert(kSegTileP == kDecTileP && kSegMG == kDecMG && kSegThreads == kDecThreads, "the host gives both lane <-> P kernels the same tiling");
+static_assert(kSegMG == kDecMG && kSegThreads == kDecThreads, "the host gives both lane <-> P kernels the same tiling");
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;

@@ -349,12 +349,12 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
     const int ns = p.G.ns_of_m[midx_c];
 
     dependents_may_start();
+    const double L = p.T.lat[table];
     stage_table(sm.tab, p.T, table);
     if (!inline_sweep) wait_for_kernel_in_front();  // the partial minima
     __syncthreads();
 
-    const double L = p.T.lat[table];
-    const double g1 = gap_at(sm.tab, npad, 1.0);
+    const double g1 = gap_at_one(sm.tab, npad);
     const double gm = gap_at(sm.tab, npad, md);
 
     // Scatter Binomial Tree: running sums of g(2^j m), j = 0..lc_max-1 (Table 2, third row)

@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(kThreads, 4) scatter_kernel(const ScatterParam
     for (int v = 0; v < V; ++v) md[v] = static_cast<double>(p.G.m_list[min(midx + v, p.G.n_m - 1)]);
 
     dependents_may_start();
+    const double L = p.T.lat[table];
     stage_table(s_tab, p.T, table);
     __syncthreads();
-    const double L = p.T.lat[table];
 #pragma unroll
     for (int v = 0; v < V; ++v) gm[v] = gap_at(s_tab, npad, md[v]);
 

@@ -24,7 +24,6 @@ namespace plogp {
 
 namespace {
 
-constexpr int R = kSegR;
 constexpr int kPilots = 4;
 constexpr int kStep = 16;  // candidates per vote of the exact search
 constexpr unsigned kFull = 0xffffffffu;
@@ -46,10 +45,10 @@ struct SegSmem {
     int cap, stride;
 };
 
-__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int tiles, unsigned char *base, SegSmem *o)
+__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int n_p, unsigned char *base, SegSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(nsv, kStep), n_p = tiles * kSegTileP, stride = n_p + 4;
+    const int cap = round_up(nsv, kStep), stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kSegMG * 8), o_pm = take(size_t(n_p) * 8),
@@ -72,12 +71,16 @@ __host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int
 
 }  // namespace
 
+// R: as in decide_kernel.
+template <int R>
 __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
     SegSmem sm;
-    seg_layout(npad, p.G.n_s, p.n_pairs, p.tiles, smem_raw, &sm);
+    constexpr int kTileP = 32 * R;
+    const int n_p = p.tiles * kTileP;
+    seg_layout(npad, p.G.n_s, p.n_pairs, n_p, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
     const bool has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has9 = (mask >> 9) & 1u;
 
@@ -90,13 +93,28 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = mgroup * p.mg;
     const int n_mi = min(p.mg, p.G.n_m - m0);
-    const int n_p = p.tiles * kSegTileP, tile0 = ptile * n_p;
+    const int tile0 = ptile * n_p;
     const int n_valid = min(n_p, p.G.n_P - tile0);
     const int pair0 = pair_of(P_at(p.G, tile0)), n_pairs = pair_of(P_at(p.G, tile0 + n_valid - 1)) - pair0 + 1;
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
     dependents_may_start();
+    // what the set-up reads from global memory is on its way while the table is
+    const double L = p.T.lat[table];
+    const uint32_t m_mine = m0 + (tid & (kSegMG - 1)) < p.G.n_m ? p.G.m_list[m0 + (tid & (kSegMG - 1))] : 0u;
+    const uint32_t s_mine = tid < p.G.n_s ? s_at(p.G, tid) : 0u;
+    const int n_s = p.G.n_s;  // at most kMaxInlineS, fewer than the threads
+    int ns_next = 0;
+    double k_next[2] = {1.0, 1.0};  // Section 2's k of this lane's candidates, from the host's table
+    auto fetch = [&](int mi) {
+        if (mi >= n_mi) return;
+        ns_next = p.G.ns_of_m[m0 + mi];
+        const double *krow = p.G.k_list + static_cast<size_t>(m0 + mi) * n_s;
+        if (lane < n_s) k_next[0] = krow[lane];
+        if (lane + 32 < n_s) k_next[1] = krow[lane + 32];
+    };
+    fetch(warp);
     if (!grow) stage_table(sm.tab, p.T, table);
     else wait_for_kernel_in_front();  // the gap pre-pass
     for (int i = tid; i < n_p; i += kSegThreads) {
@@ -106,15 +124,13 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
         sm.pair[i] = static_cast<uint8_t>(pair_of(P) - pair0);
     }
     __syncthreads();
-    const double L = p.T.lat[table];
-    for (int si = tid; si < p.G.n_s; si += kSegThreads) {
-        const uint32_t s = s_at(p.G, si);
-        sm.sval[si] = s;
-        sm.gs[si] = grow ? grow[1 + si] : gap_at(sm.tab, npad, static_cast<double>(s));
+    if (tid < n_s) {
+        sm.sval[tid] = s_mine;
+        sm.gs[tid] = grow ? grow[1 + tid] : gap_at(sm.tab, npad, static_cast<double>(s_mine));
     }
     if (tid >= kSegThreads - kSegMG) {
         const int mi = tid - (kSegThreads - kSegMG);
-        if (mi < n_mi) sm.gm[mi] = grow ? grow[1 + p.G.n_s + m0 + mi] : gap_at(sm.tab, npad, static_cast<double>(p.G.m_list[m0 + mi]));
+        if (mi < n_mi) sm.gm[mi] = grow ? grow[1 + n_s + m0 + mi] : gap_at(sm.tab, npad, static_cast<double>(m_mine));
     }
     __syncthreads();
 
@@ -129,8 +145,10 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
     const f32x2 L2 = splat2(Lf);
 
     for (int mi = warp; mi < n_mi; mi += kSegWarps) {
-        const int midx = m0 + mi;
-        const int ns = p.G.ns_of_m[midx];
+        // what a message size reads from global memory is fetched while the one before it is worked on
+        const int ns = ns_next;
+        const double k_of[2] = {k_next[0], k_next[1]};
+        fetch(mi + kSegWarps);
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
         const int np4 = round_up(nsv, 4), np16 = round_up(nsv, kStep);
         const double gm = sm.gm[mi];
@@ -151,7 +169,7 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
                 double gsv = gm, k = 1.0;
                 if (ns > 0) {
                     gsv = sm.gs[c];
-                    k = p.G.k_list[static_cast<size_t>(midx) * p.G.n_s + c];  // Section 2's k, from the host's table
+                    k = k_of[h];
                 }
                 const double Q = gsv * k, B = gsv + L, C = gsv * (k - 1.0);
                 q[c] = Q;
@@ -206,12 +224,12 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
         }
 
         for (int tile = 0; tile < p.tiles; ++tile) {
-            if (tile * kSegTileP >= n_valid) break;
-            const double *const xd = sm.pm1 + tile * kSegTileP + lane;
-            uint8_t *const pos2 = sm.pos2 + mi * sm.stride + tile * kSegTileP + lane, *const pos5 = sm.pos5 + mi * sm.stride + tile * kSegTileP + lane;
+            if (tile * kTileP >= n_valid) break;
+            const double *const xd = sm.pm1 + tile * kTileP + lane;
+            uint8_t *const pos2 = sm.pos2 + mi * sm.stride + tile * kTileP + lane, *const pos5 = sm.pos5 + mi * sm.stride + tile * kTileP + lane;
             f32x2 x2[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) x2[r] = splat2(sm.x[tile * kSegTileP + 32 * r + lane]);
+            for (int r = 0; r < R; ++r) x2[r] = splat2(sm.x[tile * kTileP + 32 * r + lane]);
             unsigned hit = 0;  // bit r: id 5, bit 16 + r: id 2
             if (has5) {
                 float T[R], mn[R];
@@ -276,7 +294,7 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
                 const int bit = __ffs(rows) - 1, r = bit & 15;
                 const bool two = bit >> 4;  // id 2
                 const double x = xd[32 * r];
-                const f32x2 xx = splat2(sm.x[tile * kSegTileP + 32 * r + lane]);
+                const f32x2 xx = splat2(sm.x[tile * kTileP + 32 * r + lane]);
                 uint8_t *const pos = two ? pos2 : pos5;
                 unsigned at = pos[32 * r];
                 double t = two ? fma(x, q[at], L) : fma(x, l5[at].x, l5[at].y);
@@ -378,8 +396,8 @@ cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
 {
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    return launch(segmin_kernel, static_cast<unsigned>(blocks), 1, kSegThreads, seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles, nullptr, nullptr), st,
-                  overlap, p);
+    const size_t smem = seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, nullptr, nullptr);
+    return launch(p.rows == 8 ? segmin_kernel<8> : segmin_kernel<4>, static_cast<unsigned>(blocks), 1, kSegThreads, smem, st, overlap, p);
 }
 
 }  // namespace plogp
