@@ -470,6 +470,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
             const uint16_t *c0 = sm.code + mi * sm.slots, *c1 = c0 + sm.slots;
             const uint8_t *p0 = sm.pos + mi * sm.pos_stride + pr0, *p1 = p0 + sm.pos_stride;
             const double *px = sm.pm1 + pr0;
+#pragma unroll 1  // (unrolled by the compiler it is 1.3 % slower on the batched workload)
             for (int pr = pr0; pr < n_valid; pr += prs) {
                 const unsigned at0 = *p0, at1 = *p1;
                 const double x = *px;
