@@ -19,6 +19,7 @@
 #include "device_common.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace plogp {
 
@@ -73,7 +74,7 @@ __host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int
 
 // R: as in decide_kernel.
 template <int R>
-__global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminParams p)
+__global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
@@ -335,11 +336,9 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
     // ---- transposed write-out: rows of p.mg consecutive m per process count, one plane after another ----
     const size_t plane = static_cast<size_t>(p.G.n_P) * p.G.n_m;
     const size_t cell0 = static_cast<size_t>(tile0) * p.G.n_m + m0;
-    const int ids[3] = {2, 5, 9};
-#pragma unroll 1
-    for (int w = 0; w < 3; ++w) {
-        if (!((mask >> ids[w]) & 1u)) continue;
-        double *plane_t = p.p_time + (static_cast<size_t>(table - p.out_table0) * 13 + ids[w]) * plane + cell0;
+    auto write_plane = [&](auto w_tag, int strategy) {
+        constexpr int w = decltype(w_tag)::value;  // 0, 1, 2: ids 2, 5, 9
+        double *plane_t = p.p_time + (static_cast<size_t>(table - p.out_table0) * 13 + strategy) * plane + cell0;
         uint32_t *plane_s = p.p_best_s ? p.p_best_s + (static_cast<size_t>(table - p.out_table0) * 3 + w) * plane + cell0 : nullptr;
         const uint8_t *const pos = w == 0 ? sm.pos2 : sm.pos5;
         // winner and time of one cell
@@ -364,6 +363,7 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
                 const size_t o = static_cast<size_t>(pr0) * p.G.n_m + mi, go = static_cast<size_t>(step) * p.G.n_m;
                 double *out_t = plane_t + o;
                 uint32_t *out_s = plane_s ? plane_s + o : nullptr;
+#pragma unroll 1
                 for (int pr = pr0; pr < n_valid; pr += step) {
                     const double x = sm.pm1[pr];
                     unsigned a0, a1;
@@ -389,7 +389,10 @@ __global__ void __launch_bounds__(kSegThreads, 4) segmin_kernel(const SegminPara
                 }
             }
         }
-    }
+    };
+    if (has2) write_plane(std::integral_constant<int, 0>{}, 2);
+    if (has5) write_plane(std::integral_constant<int, 1>{}, 5);
+    if (has9) write_plane(std::integral_constant<int, 2>{}, 9);
 }
 
 cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
