@@ -496,6 +496,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
     // the kernel that follows the (optional) Broadcast decision kernel: Scatter strategies only => scatter_kernel
     const bool use_scatter = !predict && ((use_decide ? pl.G.mask & 0x1C00u : pl.G.mask) & 0x3FFu) == 0;
 
+    const bool overlap = !h->profiling;  // the times of overlapping kernels would not add up
     if (t_end < 0) t_end = h->T.n_tables;
     for (int t0 = t_begin; t0 < t_end; t0 += pl.tables_per_batch) {
         const int nt = std::min(pl.tables_per_batch, t_end - t0);
@@ -551,7 +552,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;
             sp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
                          (!out.p_best_s || reinterpret_cast<uintptr_t>(out.p_best_s) % 8 == 0);
-            { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, gaps != nullptr, st)); }
+            { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= ~kSegBits;
             Gf.n_s = 0;
@@ -569,7 +570,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             dp.gaps = gaps; dp.gaps_stride = pl.gaps_stride;
             dp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
                          reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
-            { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, gaps != nullptr, st)); }
+            { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= 0x1C00u;
             Gf.n_s = 0;
@@ -585,7 +586,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sc.n_ptiles = pl.sc_ptiles; sc.run_len = pl.sc_run;
             sc.table0 = t0; sc.n_tables_launch = nt; sc.out_table0 = out.out_table0; sc.om = out.om;
             sc.d_strategy = out.d_strategy; sc.d_sbytes = out.d_sbytes; sc.d_time = out.d_time;
-            { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_scatter(sc, use_decide, st)); }
+            { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_scatter(sc, overlap && use_decide, st)); }
             g_launches += 1;
             continue;
         }
@@ -598,7 +599,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         fp.part_idx = part_idx;
         fp.pair_base = pl.inline_sweep ? nullptr : reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_pair_base);
         fp.n_pairs = pl.n_pairs; fp.n_seg = pl.n_seg;
-        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, pl.n_seg > 0 && (!pl.inline_sweep ? pl.envelope || pl.n_pairs > 0 : predict), st)); }
+        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, overlap && pl.n_seg > 0 && (!pl.inline_sweep ? pl.envelope || pl.n_pairs > 0 : predict), st)); }
         g_launches += 1;
     }
     return PLOGP_OK;

@@ -116,7 +116,6 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
 
     // g at the kernel's arguments: read from the gap pre-pass where the host has run it, else interpolated here
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
-    dependents_may_start();
     // what the set-up reads from global memory is on its way while the table is
     const double L = p.T.lat[table];
     const uint32_t m_mine = m0 + (tid & (kDecMG - 1)) < p.G.n_m ? p.G.m_list[m0 + (tid & (kDecMG - 1))] : 0u;
@@ -137,6 +136,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
     fetch(warp);
     if (!grow) stage_table(sm.tab, p.T, table);
     else wait_for_kernel_in_front();  // the gap pre-pass
+    dependents_may_start();
     for (int i = tid; i < n_p; i += kDecThreads) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
         sm.pm1[i] = static_cast<double>(P - 1);
@@ -503,6 +503,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
             }
         }
     }
+    last_block_waits(tid);
 }
 
 cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st)

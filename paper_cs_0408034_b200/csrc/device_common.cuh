@@ -12,11 +12,16 @@ namespace plogp {
 // ------------------------------------------------------------------------------------------
 //
 // The first kernel of a call is launched as usual; the ones behind it may start once every CTA of the kernel in front
-// has started (dependents_may_start).  A kernel that reads what the one in front writes waits for its end first;
-// one that does not waits as the last thing thread 0 of each CTA does, so that the end of the call's last kernel is the
-// end of the call.
+// has called dependents_may_start.  A kernel that reads what the one in front writes waits for its end first.  Each kernel's
+// last CTA waits for the end of the kernel in front before it ends itself, so that the end of a call's last kernel is the
+// end of the call.  Nothing here spins: the waits are the hardware's, and a kernel's CTAs only start when all CTAs of the
+// kernel in front have their place.
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_kernel_in_front() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void last_block_waits(int tid)  // call at the end; thread 0 of a kernel's last CTA must get here
+{
+    if (tid == 0 && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1) wait_for_kernel_in_front();
+}
 
 // ------------------------------------------------------------------------------------------
 // Table staging and g(x)

@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
             p.part_idx[rbase * p.G.n_P + pidx] = bi;
         }
     }
-    if (IS9 && tid == 0) wait_for_kernel_in_front();  // the launch for ids 2 and 5; nothing of it is read here
+    last_block_waits(tid);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
         }
         if (mask & 0x1C00u) flush(1);
     }
-    if (threadIdx.x == 0) wait_for_kernel_in_front();  // nothing of it is read here unless it was waited for above
+    last_block_waits(tid);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kThreads, 4) scatter_kernel(const ScatterParam
         if (CONTIG) { ++P; pm1 += 1.0; }
         else j_last = pm1;
     }
-    if (threadIdx.x == 0) wait_for_kernel_in_front();  // the Broadcast half; nothing of it is read here
+    last_block_waits(threadIdx.x);
 }
 
 template <bool CONTIG, bool ALL, int V>
