@@ -68,6 +68,9 @@ struct Plan {
     int n_mtiles = 0, n_ptiles = 1, passes_per_tile = 1;
     // Scatter decision kernel: its own split of P (vec = 2: two message sizes per lane, where the outputs allow it)
     int sc_vec = 1, sc_ptiles = 1, sc_run = 1;
+    // both halves in one launch, and then the Scatter half's split of P
+    bool select = false;
+    int sel_ptiles = 1, sel_run = 1;
     // decision kernel tiling (short candidate lists)
     int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_rows = 8, dec_tiles = 1, dec_pairs = 1;
     // sweep kernel
@@ -338,6 +341,16 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
             }
         }
     }
+    // One launch for both halves where the GPU holds all their CTAs at once (four per SM; its Scatter CTAs have four warps)
+    {
+        const long long decide = (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
+        const long long room = (long long)h->sm_count * 4 - decide;
+        pl.select = room >= base && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
+        if (pl.select) {
+            pl.sel_run = int(std::max<long long>(4, (n_P + kDecWarps * (room / base) - 1) / (kDecWarps * (room / base))));
+            pl.sel_ptiles = (n_P + kDecWarps * pl.sel_run - 1) / (kDecWarps * pl.sel_run);
+        }
+    }
     const int dec_p = pl.dec_tiles * 32 * pl.dec_rows;
     for (int t = 0; t < pl.dec_ptiles; ++t) {
         const int first = t * dec_p, last = std::min(n_P, first + dec_p) - 1;
@@ -570,6 +583,18 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             dp.gaps = gaps; dp.gaps_stride = pl.gaps_stride;
             dp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
                          reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
+            if (pl.select && !gaps && overlap) {
+                SelectParams sl{};
+                sl.decide = dp;
+                ScatterParams &sc = sl.scatter;
+                sc.T = h->T; sc.G = pl.G;
+                sc.vec = 1; sc.n_mtiles = pl.n_mtiles; sc.n_ptiles = pl.sel_ptiles; sc.run_len = pl.sel_run;
+                sc.table0 = t0; sc.n_tables_launch = nt; sc.out_table0 = out.out_table0; sc.om = out.om;
+                sc.d_strategy = out.d_strategy; sc.d_sbytes = out.d_sbytes; sc.d_time = out.d_time;
+                CK(launch_select(sl, st));
+                g_launches += 1;
+                continue;
+            }
             { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= 0x1C00u;

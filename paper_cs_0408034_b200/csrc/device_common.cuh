@@ -196,13 +196,13 @@ struct ChainWalk {
     }
 };
 
-// Scatter Chain sum in front of each warp's run of process counts, for one message size per lane.  A CTA's kWarps warps
+// Scatter Chain sum in front of each warp's run of process counts, for one message size per lane.  A CTA's n_warps warps
 // own the runs [e0, e1) of process-count indices, one after another from index c0 on.  The terms j <= P(c0) - 2, which
 // lie in front of the whole CTA, are split over its warps by table intervals (front); each warp adds the closed form of
 // its own run (own), which the warps behind it need.  A handful of intervals per warp instead of a pass over the process
 // counts, and nothing is carried between CTAs.  The caller puts a barrier between the two calls.
 static __device__ __noinline__ void chain_front_parts(const double *s_tab, int npad, int n_bp, const int32_t *P_list, int P_lo, double md, int c0, int e0,
-                                                      int e1, int warp, double *s_front, double *s_own, int stride)
+                                                      int e1, int warp, int n_warps, double *s_front, double *s_own, int stride)
 {
     auto P_of = [&](int e) { return P_list ? P_list[e] : P_lo + e; };
     double front = 0.0, own = 0.0;
@@ -212,7 +212,7 @@ static __device__ __noinline__ void chain_front_parts(const double *s_tab, int n
         ChainWalk w;
         if (jc >= 1.0) {
             const double inv_m = 1.0 / md, x_end = jc * md;
-            const int n_int = n_bp - 1, i0 = n_int * warp / kWarps, i1 = n_int * (warp + 1) / kWarps;
+            const int n_int = n_bp - 1, i0 = n_int * warp / n_warps, i1 = n_int * (warp + 1) / n_warps;
             auto first_j = [&](int i) {  // smallest j with j m >= key i; jc + 1 when that lies behind jc
                 const double key = s_tab[i];
                 const double q = round_whole(key * inv_m), j = fmax(fma(-q, md, key) > 0.0 ? q + 1.0 : q, 1.0);
@@ -228,7 +228,7 @@ static __device__ __noinline__ void chain_front_parts(const double *s_tab, int n
                 ja = jb;
             }
         }
-        if (e0 < e1 && warp < kWarps - 1) {
+        if (e0 < e1 && warp < n_warps - 1) {
             const double j0 = e0 == c0 ? jc + 1.0 : static_cast<double>(P_of(e0 - 1)), j1 = static_cast<double>(P_of(e1 - 1) - 1);
             w.start(s_tab, npad, j0 * md);
             own = w.range(s_tab, npad, md, j0, j1);
@@ -237,11 +237,11 @@ static __device__ __noinline__ void chain_front_parts(const double *s_tab, int n
     s_front[warp * stride] = front;
     s_own[warp * stride] = own;
 }
-__device__ __forceinline__ double chain_front_sum(const double *s_front, const double *s_own, int stride, int warp)
+__device__ __forceinline__ double chain_front_sum(const double *s_front, const double *s_own, int stride, int warp, int n_warps)
 {
     double run = 0.0;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) run += s_front[w * stride];
+    for (int w = 0; w < n_warps; ++w) run += s_front[w * stride];
     for (int w = 0; w < warp; ++w) run += s_own[w * stride];
     return run;
 }

@@ -207,6 +207,15 @@ cudaError_t launch_fused(const FusedParams &p, bool predict, bool overlap, cudaS
 cudaError_t launch_scatter(const ScatterParams &p, bool overlap, cudaStream_t st);  // decision table, Scatter strategies only
 cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st);
 cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st);
+// both halves of a decision table in one launch: see select.cu (launch_select fills in n_decide)
+struct SelectParams {
+    DecideParams decide;
+    ScatterParams scatter;
+    int n_decide;
+};
+size_t decide_smem_bytes(const DecideParams &p);
+size_t scatter_smem_bytes(const ScatterParams &p, int warps);
+cudaError_t launch_select(SelectParams &p, cudaStream_t st);
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st);
 cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st);
 cudaError_t launch_gaps(const GapsParams &p, cudaStream_t st);

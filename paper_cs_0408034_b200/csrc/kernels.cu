@@ -399,10 +399,10 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
     ChainWalk s1_walk;
     if ((mask >> 11) & 1u) {
         const int c0 = ptile * (kWarps * run_len), e0 = min(p_warp, p.G.n_P), e1 = min(p_warp + run_len, p.G.n_P);
-        chain_front_parts(sm.tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md, c0, e0, e1, warp, sm.tot + lane, sm.tot + kWarps * 32 + lane, 32);
+        chain_front_parts(sm.tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md, c0, e0, e1, warp, kWarps, sm.tot + lane, sm.tot + kWarps * 32 + lane, 32);
         __syncthreads();
         if (e0 < e1) {
-            s1_run = chain_front_sum(sm.tot + lane, sm.tot + kWarps * 32 + lane, 32, warp);
+            s1_run = chain_front_sum(sm.tot + lane, sm.tot + kWarps * 32 + lane, 32, warp, kWarps);
             j_last = static_cast<double>(warp == 0 ? P_at(p.G, e0) - 2 : P_at(p.G, e0 - 1) - 1);
             s1_walk.start(sm.tab, npad, (j_last + 1.0) * md);
         }

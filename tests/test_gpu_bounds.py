@@ -94,3 +94,23 @@ def test_boundaries_of_random_maps(plogp, n_m, n_P):
     s = rng.integers(0, 3, size=(3, 2, n_P, n_m)).astype(np.uint8) * 200  # neighbouring bytes must not touch one another
     dec = plogp.DecisionTable(torch.as_tensor(s, device="cuda"), None, None)
     assert np.array_equal(plogp.decision_boundaries(dec).cpu().numpy(), po.decision_boundaries(s))
+
+
+@pytest.mark.parametrize("n_P,n_m,n_s,n_tables,listed,search", [(1, 1, 1, 1, False, 0), (3, 5, 64, 1, False, 0), (129, 33, 7, 1, True, 0), (257, 37, 33, 2, False, 1),
+                                                               (600, 70, 20, 1, False, 0), (127, 300, 12, 1, True, 1), (1500, 64, 3, 2, False, 0)])
+def test_both_halves_in_one_launch_and_in_two(plogp, n_P, n_m, n_s, n_tables, listed, search):
+    """Small grids: one launch for both halves (tiles of 128 process counts, four warps per Scatter CTA); the same call
+    with per-kernel timing on makes the two launches.  Both match the oracle and one another bit for bit."""
+    import torch
+    w = wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=n_s, seed_offset=n_P)
+    if listed:
+        w = replace(w, P_list=np.unique(np.rint(2 * 1500 ** (np.arange(n_P) / max(1, n_P - 1)))).astype(np.int32))
+    w = replace(w, search_mode=search)
+    both(plogp, w)
+    with plogp.Tables.from_workload(w) as tabs:
+        a = plogp.select_best(tabs, w)
+        plogp.profile_enable(tabs)
+        b = plogp.select_best(tabs, w)
+        torch.cuda.synchronize()
+        assert len(plogp.profile_read(tabs)) >= 2
+        assert torch.equal(a.strategy, b.strategy) and torch.equal(a.s_bytes, b.s_bytes) and torch.equal(a.time, b.time)
