@@ -11,7 +11,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) decide_kernel(const DecidePara
     last_block_waits(threadIdx.x);
 }
 
-size_t decide_smem_bytes(const DecideParams &p) { return decide::dec_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, nullptr, nullptr); }
+size_t decide_smem_bytes(const DecideParams &p) { return decide::dec_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, p.mg, nullptr, nullptr); }
 
 cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st)
 {

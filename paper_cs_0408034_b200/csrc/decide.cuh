@@ -48,14 +48,14 @@ constexpr int kIntMax = 0x7FFFFFFF;
 
 struct DecSmem {
     double *tab, *gs, *gm, *pm1;
-    double2 *line;    // [kDecMG][slots]: coefficients by slot
+    double2 *line;    // [mg][slots]: coefficients by slot
     float *x;         // [n_p]: P-1 rounded down
     float *fa, *fc;   // [kDecWarps][cap]: the lines' coefficients rounded down, for the warp's current message size
     double *q;        // [kDecWarps][cap_q]: g(s) k, for the warp's current message size
     float *fq;        // [kDecWarps][cap_q]: the same rounded down
     uint32_t *sval;   // [256]: segment sizes by candidate index; [kCandNone] = 0
-    uint16_t *code;   // [kDecMG][slots]: id << 8 | candidate index
-    uint8_t *pair, *pos;  // [n_p]: pair of a process count; [kDecMG][pos_stride]: winners
+    uint16_t *code;   // [mg][slots]: id << 8 | candidate index
+    uint8_t *pair, *pos;  // [n_p]: pair of a process count; [mg][pos_stride]: winners
     int cap, cap_q, slots, pos_stride;
 };
 
@@ -63,16 +63,16 @@ __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a *
 
 // Shared-memory layout.  cap: lines of one message size (a multiple of kStep); n_pairs: (floor, ceil) pairs of a CTA at most.
 // A slot number fits a byte: at most 144 lines and 61 pairs.
-__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int n_p, unsigned char *base, DecSmem *o)
+__host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int n_p, int mg, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
     const int cap = round_up(2 * nsv + 4, kStep), cap_q = round_up(nsv, 4), slots = cap + n_pairs, pos_stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
-    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kDecMG * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
-                 o_line = take(size_t(kDecMG) * slots * 16), o_fa = take(size_t(kDecWarps) * cap * 4), o_fc = take(size_t(kDecWarps) * cap * 4),
-                 o_q = take(size_t(kDecWarps) * cap_q * 8), o_fq = take(size_t(kDecWarps) * cap_q * 4), o_sv = take(256 * 4), o_code = take(size_t(kDecMG) * slots * 2),
-                 o_pair = take(n_p), o_pos = take(size_t(kDecMG) * pos_stride);
+    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(mg * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
+                 o_line = take(size_t(mg) * slots * 16), o_fa = take(size_t(kDecWarps) * cap * 4), o_fc = take(size_t(kDecWarps) * cap * 4),
+                 o_q = take(size_t(kDecWarps) * cap_q * 8), o_fq = take(size_t(kDecWarps) * cap_q * 4), o_sv = take(256 * 4), o_code = take(size_t(mg) * slots * 2),
+                 o_pair = take(n_p), o_pos = take(size_t(mg) * pos_stride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
         o->gm = reinterpret_cast<double *>(base + o_gm); o->pm1 = reinterpret_cast<double *>(base + o_pm);
@@ -100,7 +100,7 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
     DecSmem sm;
     constexpr int kTileP = 32 * R;
     const int n_p = p.tiles * kTileP;
-    dec_layout(npad, p.G.n_s, p.n_pairs, n_p, smem_raw, &sm);
+    dec_layout(npad, p.G.n_s, p.n_pairs, n_p, p.mg, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
 
     int b = block;
@@ -437,13 +437,16 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
 #pragma unroll
                     for (int q = 0; q < kStep / 4; ++q) {
                         if (!__any_sync(kFull, low[q] <= Tr)) continue;
-                        const int u0 = j + 4 * q;
+                        double tt[4];  // four loads in flight; behind the last line the last one again
 #pragma unroll
-                        for (int u = u0; u < u0 + 4; ++u) {
-                            if (u >= n1) break;
-                            const double2 v = line[u];
-                            const double tt = fma(x, v.x, v.y);
-                            if (tt <= t && (tt < t || static_cast<unsigned>(u) < at)) { t = tt; at = static_cast<unsigned>(u); }
+                        for (int u = 0; u < 4; ++u) {
+                            const double2 v = line[min(j + 4 * q + u, n1 - 1)];
+                            tt[u] = fma(x, v.x, v.y);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const unsigned slot = static_cast<unsigned>(min(j + 4 * q + u, n1 - 1));
+                            if (tt[u] < t || (tt[u] == t && slot < at)) { t = tt[u]; at = slot; }
                         }
                         if (Tr >= 0.0f) Tr = __double2float_ru(t);
                     }

@@ -34,29 +34,29 @@ __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a *
 
 struct SegSmem {
     double *tab, *gs, *gm, *pm1;
-    double2 *l5;      // [kSegMG][cap]: (B, C)
-    double *q;        // [kSegMG][cap]: Q
-    double *t9;       // [kSegMG][n_pairs]: id 9's minimum
+    double2 *l5;      // [mg][cap]: (B, C)
+    double *q;        // [mg][cap]: Q
+    double *t9;       // [mg][n_pairs]: id 9's minimum
     float *x;         // [n_p]: P-1 rounded down
     float *fb, *fc, *fq;  // [kSegWarps][cap]: the lists of the warp's current message size rounded down, without the pilots
     uint32_t *sval;
-    uint8_t *i9;      // [kSegMG][n_pairs]: id 9's winner
+    uint8_t *i9;      // [mg][n_pairs]: id 9's winner
     uint8_t *pair;    // [n_p]: pair of a process count
-    uint8_t *pos2, *pos5;  // [kSegMG][stride]: winners of ids 2 and 5
+    uint8_t *pos2, *pos5;  // [mg][stride]: winners of ids 2 and 5
     int cap, stride;
 };
 
-__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int n_p, unsigned char *base, SegSmem *o)
+__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int n_p, int mg, unsigned char *base, SegSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
     const int cap = round_up(nsv, kStep), stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
-    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(kSegMG * 8), o_pm = take(size_t(n_p) * 8),
-                 o_l5 = take(size_t(kSegMG) * cap * 16), o_q = take(size_t(kSegMG) * cap * 8), o_t9 = take(size_t(kSegMG) * n_pairs * 8),
+    const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(mg * 8), o_pm = take(size_t(n_p) * 8),
+                 o_l5 = take(size_t(mg) * cap * 16), o_q = take(size_t(mg) * cap * 8), o_t9 = take(size_t(mg) * n_pairs * 8),
                  o_x = take(size_t(n_p) * 4), o_fb = take(size_t(kSegWarps) * cap * 4), o_fc = take(size_t(kSegWarps) * cap * 4),
-                 o_fq = take(size_t(kSegWarps) * cap * 4), o_sv = take(size_t(nsv) * 4), o_i9 = take(size_t(kSegMG) * n_pairs), o_pair = take(n_p),
-                 o_p2 = take(size_t(kSegMG) * stride), o_p5 = take(size_t(kSegMG) * stride);
+                 o_fq = take(size_t(kSegWarps) * cap * 4), o_sv = take(size_t(nsv) * 4), o_i9 = take(size_t(mg) * n_pairs), o_pair = take(n_p),
+                 o_p2 = take(size_t(mg) * stride), o_p5 = take(size_t(mg) * stride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
         o->gm = reinterpret_cast<double *>(base + o_gm); o->pm1 = reinterpret_cast<double *>(base + o_pm);
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
     SegSmem sm;
     constexpr int kTileP = 32 * R;
     const int n_p = p.tiles * kTileP;
-    seg_layout(npad, p.G.n_s, p.n_pairs, n_p, smem_raw, &sm);
+    seg_layout(npad, p.G.n_s, p.n_pairs, n_p, p.mg, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
     const bool has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has9 = (mask >> 9) & 1u;
 
@@ -316,13 +316,17 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
 #pragma unroll
                     for (int u = 0; u < kStep / 4; ++u) {
                         if (!__any_sync(kFull, low[u] <= T)) continue;
-                        const int c0 = j + 4 * u;
+                        double tt[4];  // four loads in flight; behind the last candidate the last one again
 #pragma unroll
-                        for (int c = c0; c < c0 + 4; ++c) {
-                            if (c >= nsv) break;
-                            const double2 e = l5[c];
-                            const double tt = two ? fma(x, q[c], L) : fma(x, e.x, e.y);
-                            if (tt <= t && (tt < t || static_cast<unsigned>(c) < at)) { t = tt; at = static_cast<unsigned>(c); }
+                        for (int v = 0; v < 4; ++v) {
+                            const int c = min(j + 4 * u + v, nsv - 1);
+                            const double2 e = two ? make_double2(q[c], L) : l5[c];
+                            tt[v] = fma(x, e.x, e.y);
+                        }
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const unsigned c = static_cast<unsigned>(min(j + 4 * u + v, nsv - 1));
+                            if (tt[v] < t || (tt[v] == t && c < at)) { t = tt[v]; at = c; }
                         }
                         if (mine) T = __double2float_ru(t);
                     }
@@ -400,7 +404,7 @@ cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
 {
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    const size_t smem = seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, nullptr, nullptr);
+    const size_t smem = seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, p.mg, nullptr, nullptr);
     return launch(p.rows == 8 ? segmin_kernel<8> : segmin_kernel<4>, static_cast<unsigned>(blocks), 1, kSegThreads, smem, st, overlap, p);
 }
 
