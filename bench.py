@@ -38,8 +38,7 @@ NOMINAL_FP64_FMA_RATE = 148 * 64 * 1.965e9  # SMs x FP64 lanes per SM x max SM c
 # under profiles/ (batched workload cut to 1024 tables: 0.87 GB of output per kernel, far beyond the L2,
 # so what is still cached when the kernel ends is a few percent; traffic grows in proportion to the table
 # count).  An entry is None while its kernel has changed since the last capture.
-NCU_TRAFFIC_BYTES_PER_TABLE = {"decide_kernel": (813.820672e6 + 1.456128e6) / 1024, "scatter_kernel": (812.184320e6 + 1.679872e6) / 1024,
-                               "sweep_kernel": None}
+NCU_TRAFFIC_BYTES_PER_TABLE = {"decide_kernel": None, "scatter_kernel": None, "sweep_kernel": None}
 NCU_TRAFFIC_NOTE = "bytes per launch = bytes per table of the 1024-table ncu capture in profiles/ x tables"
 FALLBACK_HBM_GBS = 6650.0
 
@@ -65,10 +64,14 @@ def make_workload(name: str, scale: str, rank: int):
 
 
 def work_counts(w):
-    """Cells of one step and the algorithmic work of each kernel: a segmented cell
-    is one DFMA and one compare (2 FP64 issue slots), an unsegmented cell one DFMA, a Scatter Chain
-    element one interpolation DFMA, one running-sum DADD and the model's DFMA; HBM bytes are the decision
-    table written once (13 B per decision cell)."""
+    """Cells of one step and the algorithmic work of each kernel, in issue slots of a 64-lane pipe (the FP64 pipe's
+    measured rate is the peak).  The lane <-> P kernels evaluate every cell of a line in P as a lower bound in FP32:
+    half a slot for the packed multiply-add (two cells per instruction, 64 lane pairs) and half a slot for its share of a
+    three-input minimum, one slot together; what the bounds leave open is compared in FP64 and not counted.  Models that
+    depend on floor and ceil of log2 P alone (ids 6 to 9) have the same value for all process counts in between and are
+    searched once for them: not counted as slots there.  Elsewhere an unsegmented cell is one DFMA, a Scatter Chain element
+    one interpolation DFMA, one running-sum DADD and the model's DFMA.  HBM bytes are the decision table written once
+    (13 B per decision cell)."""
     mask = w.strategy_mask
     seg_ids = [b for b in (2, 5, 9) if (mask >> b) & 1]
     unseg_b = [b for b in (0, 1, 3, 4, 6, 7, 8) if (mask >> b) & 1]
@@ -77,18 +80,18 @@ def work_counts(w):
     seg_cells = w.n_tables * w.n_P * len(seg_ids) * int(w.n_candidates().sum())
     bcast_dec = cells_pm if (seg_ids or unseg_b) else 0
     scat_dec = cells_pm if scat else 0
+    n_cand = w.n_tables * w.n_P * int(w.n_candidates().sum())
+    line_slots = n_cand * sum((mask >> b) & 1 for b in (2, 5))
+    line_unseg = cells_pm * sum((mask >> b) & 1 for b in (0, 1, 3, 4))
     scat_slots = cells_pm * (((mask >> 10) & 1) + 3 * ((mask >> 11) & 1) + ((mask >> 12) & 1))
     long_lists = bool(seg_ids) and len(w.s_values()) > 64
     per_kernel = {}
     if long_lists:
-        per_kernel["sweep_kernel"] = {"fp64_slots": 2 * seg_cells, "hbm_bytes": 0}
+        per_kernel["sweep_kernel"] = {"fp64_slots": seg_cells, "hbm_bytes": 0}
         per_kernel["fused_kernel"] = {"fp64_slots": len(unseg_b) * cells_pm + scat_slots, "hbm_bytes": 13 * (bcast_dec + scat_dec)}
     else:
         if seg_ids:
-            # selection_slots: the strategy-selection compares per decision cell (enabled Broadcast strategies - 1), which
-            # the per-unit table of the roofline also lists as FP64 work; reported beside `frac`, not inside it
-            per_kernel["decide_kernel"] = {"fp64_slots": 2 * seg_cells + len(unseg_b) * cells_pm, "hbm_bytes": 13 * bcast_dec,
-                                           "selection_slots": (len(seg_ids) + len(unseg_b) - 1) * cells_pm}
+            per_kernel["decide_kernel"] = {"fp64_slots": line_slots + line_unseg, "hbm_bytes": 13 * bcast_dec}
             if scat:
                 per_kernel["scatter_kernel"] = {"fp64_slots": scat_slots, "hbm_bytes": 13 * scat_dec}
         elif unseg_b:
@@ -96,7 +99,7 @@ def work_counts(w):
         elif scat:
             per_kernel["scatter_kernel"] = {"fp64_slots": scat_slots, "hbm_bytes": 13 * scat_dec}
     total_slots = sum(k["fp64_slots"] for k in per_kernel.values())
-    return {"model_cells": seg_cells + (len(unseg_b) + len(scat)) * cells_pm, "segmented_cells": seg_cells,
+    return {"line_slots": line_slots, "model_cells": seg_cells + (len(unseg_b) + len(scat)) * cells_pm, "segmented_cells": seg_cells,
             "decision_cells": bcast_dec + scat_dec, "fp64_slots": total_slots, "hbm_bytes": 13 * (bcast_dec + scat_dec),
             "per_kernel": per_kernel}
 
@@ -258,17 +261,17 @@ def predict_counts(w, counts):
     cells_pm = w.n_tables * w.n_P * w.n_m
     out_bytes = cells_pm * (8 * n_on + 4 * n_seg)
     seg_bytes = cells_pm * 12 * n_seg
-    slots = counts["fp64_slots"]
-    seg_slots = 2 * counts["segmented_cells"]
+    unseg = n_on - n_seg + 2 * ((w.strategy_mask >> 11) & 1)  # the closed-form planes, in FP64
     c = dict(counts)
     if "sweep_kernel" in counts["per_kernel"]:
         sweep = counts["per_kernel"]["sweep_kernel"]
-        c["per_kernel"] = {"sweep_kernel": sweep, "fused_kernel": {"fp64_slots": slots - sweep["fp64_slots"], "hbm_bytes": out_bytes}}
+        c["per_kernel"] = {"sweep_kernel": sweep, "fused_kernel": {"fp64_slots": unseg * cells_pm, "hbm_bytes": out_bytes}}
     elif n_seg:
-        c["per_kernel"] = {"segmin_kernel": {"fp64_slots": seg_slots, "hbm_bytes": seg_bytes},
-                           "fused_kernel": {"fp64_slots": slots - seg_slots, "hbm_bytes": out_bytes - seg_bytes}}
+        c["per_kernel"] = {"segmin_kernel": {"fp64_slots": counts["line_slots"], "hbm_bytes": seg_bytes},
+                           "fused_kernel": {"fp64_slots": unseg * cells_pm, "hbm_bytes": out_bytes - seg_bytes}}
     else:
-        c["per_kernel"] = {"fused_kernel": {"fp64_slots": slots, "hbm_bytes": out_bytes}}
+        c["per_kernel"] = {"fused_kernel": {"fp64_slots": unseg * cells_pm, "hbm_bytes": out_bytes}}
+    c["fp64_slots"] = sum(k["fp64_slots"] for k in c["per_kernel"].values())
     c["hbm_bytes"] = out_bytes
     return c
 
@@ -302,7 +305,8 @@ class Bench:
 
     def time_device(self, w, predict, steps, warmup, clocks_uuid=None):
         """Device-resident timing of `steps` steps of one call on one workload.  Returns the measured
-        dictionary; the per-kernel times come from events the library records around each launch."""
+        dictionary; the per-kernel times come from a few more steps in which the library records events around each
+        launch (its kernels do not overlap then, so they add up to a little more than a step)."""
         torch, plogp = self.torch, self.plogp
         counts = work_counts(w)
         grid = plogp.GridArgs.from_workload(w)
@@ -332,7 +336,6 @@ class Bench:
                 flush.fill_(1)
         self.barrier()
         launches0 = plogp.kernel_launches()
-        plogp.profile_enable(tabs, True)
         events = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(steps)]
         with ClockSampler(clocks_uuid) as clocks:
             self.barrier()
@@ -344,11 +347,17 @@ class Bench:
                     flush.fill_(1)
             self.barrier()
         launches = plogp.kernel_launches() - launches0
-        kernel_ms = plogp.profile_read(tabs)   # {kernel: (ms over the timed region, launches)}
+        kernel_steps = max(3, min(steps, 10))
+        plogp.profile_enable(tabs, True)
+        for _ in range(kernel_steps):
+            step()
+            if flush is not None:
+                flush.fill_(1)
+        kernel_ms = plogp.profile_read(tabs)   # {kernel: (ms over these steps, launches)}
         plogp.profile_enable(tabs, False)
         total_ms = max_over_ranks(sum(a.elapsed_time(b) for a, b in events), self.world, "cuda")
         return {"w": w, "predict": predict, "counts": counts, "steps": steps, "ms_per_step": total_ms / steps, "launches": launches,
-                "kernel_ms": kernel_ms, "out_bytes": out_bytes, "flushed": flush is not None, "clocks": clocks,
+                "kernel_ms": kernel_ms, "kernel_steps": kernel_steps, "out_bytes": out_bytes, "flushed": flush is not None, "clocks": clocks,
                 "tabs": tabs, "grid": grid}
 
     def time_e2e(self, m, steps):
@@ -476,12 +485,11 @@ class Bench:
         if self.fma_rate is None:
             self.fma_rate = self.plogp.fp64_fma_rate(100.0)
         fma_rate, hbm_gbs = self.fma_rate, self.hbm_gbs
-        counts, steps, w = m["counts"], m["steps"], m["w"]
-        seg_cells = counts["segmented_cells"]
+        counts, steps, w = m["counts"], m["kernel_steps"], m["w"]
 
         def roof(name, ms_total, n_launch):
             # algorithmic work per launch / average launch duration (CUDA events recorded by the library on
-            # the launching stream during the timed region)
+            # the launching stream)
             work = counts["per_kernel"].get(name)
             if work is None or n_launch == 0:
                 return {"kernel": name, "launches": n_launch, "ms_total": ms_total, "avg_ms": ms_total / max(n_launch, 1)}
@@ -494,18 +502,14 @@ class Bench:
                  "bound": "alu" if alu else "hbm",
                  "achieved": slots / dur / 1e12 if alu else nbytes / dur / 1e9,
                  "peak": fma_rate / 1e12 if alu else hbm_gbs,
-                 "unit": "T FP64 thread-instr/s" if alu else "GB/s",
+                 "unit": "T slots/s of a 64-lane pipe" if alu else "GB/s",
                  "frac": max(t_alu, t_hbm) / dur,
                  "alu_time_ms": t_alu * 1e3, "hbm_time_ms": t_hbm * 1e3,
                  "peak_source": ("DFMA issue rate measured in this run by plogp_fp64_fma_rate, of measured (nominal %.2f T/s = 148 SMs x 64 lanes x 1.965 GHz)"
                                  % (NOMINAL_FP64_FMA_RATE / 1e12)) if alu else "HBM copy bandwidth, of %s" % self.peak_src}
-            if alu and work.get("selection_slots"):
-                r["frac_with_selection_compares"] = max((slots + work["selection_slots"] * per_launch) / fma_rate, t_hbm) / dur
             if alu and name in ("sweep_kernel", "decide_kernel", "segmin_kernel"):
-                # stricter accounting: the compare of a segmented cell runs in the integer pipe, so only its DFMA
-                # is an FP64 slot (1 instead of 2 per segmented cell)
-                strict = (work["fp64_slots"] - seg_cells) * per_launch
-                r["frac_dfma_only"] = max(strict / fma_rate, t_hbm) / dur
+                # stricter: the minima run beside the multiply-adds in another pipe, so only the latter count
+                r["frac_multiply_adds_only"] = max(0.5 * slots / fma_rate, t_hbm) / dur
             return r
 
         kernels = [roof(k, v[0], v[1]) for k, v in m["kernel_ms"].items()]
@@ -520,7 +524,7 @@ class Bench:
         t_alu = counts["fp64_slots"] / fma_rate
         t_hbm = counts["hbm_bytes"] / (hbm_gbs * 1e9)
         dominant["step"] = {"frac": max(t_alu, t_hbm) / (m["ms_per_step"] * 1e-3), "alu_time_ms": t_alu * 1e3, "hbm_time_ms": t_hbm * 1e3,
-                            "note": "whole step (all kernels) against max(FP64 issue, HBM bytes)"}
+                            "note": "whole step (all kernels) against max(issue slots, HBM bytes)"}
         return kernels, dominant
 
     def config_of(self, m):
@@ -529,6 +533,9 @@ class Bench:
                 "P": [w.P_lo, w.P_hi], "n_m": w.n_m, "n_s": int(len(w.s_values())), "strategy_mask": w.strategy_mask,
                 "model_cells_per_gpu": counts["model_cells"], "decision_cells_per_gpu": counts["decision_cells"],
                 "parallelism": "tables sharded, %d rank(s)" % self.world,
+                "evaluation": "every (P, m, s) cell of a line in P as a lower bound in FP32 (operands and multiply-add rounded down), decided in "
+                              "FP64 wherever the bound does not rule it out; ids 6 to 9 once per (floor, ceil) of log2 P; results are "
+                              "those of the exhaustive FP64 search",
                 "l2": "256 MB written between timed steps to flush L2" if m["flushed"]
                 else "outputs (%.1f GB per step) exceed the 126 MB L2" % (m["out_bytes"] / 1e9)}
 
