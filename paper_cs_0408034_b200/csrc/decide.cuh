@@ -286,11 +286,9 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
         q_pilot = env ? static_cast<unsigned>(q_c) : __reduce_min_sync(kFull, q_pilot) & 0xFFu;
         if ((q_pilot & 31u) == static_cast<unsigned>(lane)) lqf[q_pilot] = CUDART_INF_F;  // written by this lane itself above
         if (two && n1 > 0) {
-            const int h = __reduce_min_sync(kFull, at_two == 0xFFu ? kIntMax : hi32(t_two));
-            const bool on_h = at_two != 0xFFu && hi32(t_two) == h;
-            const unsigned l = __reduce_min_sync(kFull, on_h ? static_cast<unsigned>(__double2loint(t_two)) : 0xFFFFFFFFu);
-            at_two = __reduce_min_sync(kFull, on_h && static_cast<unsigned>(__double2loint(t_two)) == l ? at_two : 0xFFu);
-            t_two = __hiloint2double(h, static_cast<int>(l));
+            int e = at_two == 0xFFu ? kIntMax : static_cast<int>(at_two);
+            warp_min_pair(t_two, e);
+            at_two = static_cast<unsigned>(e);
         }
         __syncwarp();
 

@@ -246,15 +246,15 @@ __device__ __forceinline__ double chain_front_sum(const double *s_front, const d
     return run;
 }
 
-// Lexicographic minimum of (t, e) over a warp (all lanes receive it).
+// Lexicographic minimum of (t, e) over a warp (all lanes receive it), t >= 0 and e >= 0: three integer warp reductions,
+// of the high word, the low word where it ties, and e where both do.
 __device__ __forceinline__ void warp_min_pair(double &t, int &e)
 {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double t2 = __shfl_xor_sync(0xffffffffu, t, off);
-        const int e2 = __shfl_xor_sync(0xffffffffu, e, off);
-        if (t2 < t || (t2 == t && e2 < e)) { t = t2; e = e2; }
-    }
+    const int h = __reduce_min_sync(0xffffffffu, __double2hiint(t));
+    const bool on_h = __double2hiint(t) == h;
+    const unsigned l = __reduce_min_sync(0xffffffffu, on_h ? static_cast<unsigned>(__double2loint(t)) : 0xffffffffu);
+    e = __reduce_min_sync(0xffffffffu, on_h && static_cast<unsigned>(__double2loint(t)) == l ? e : 0x7fffffff);
+    t = __hiloint2double(h, static_cast<int>(l));
 }
 
 }  // namespace plogp
