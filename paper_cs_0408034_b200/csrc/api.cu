@@ -91,7 +91,9 @@ struct plogp_tables {
     int sm_count = 148;
     TableDev T{};
     bool monotone = false;  // no table's gap ever decreases with the size (the envelope search relies on it)
-    double *d_tab = nullptr, *d_lat = nullptr;
+    double *d_tab = nullptr;           // T.tab
+    unsigned char *d_raw = nullptr;    // behind it, in the same allocation: the caller's arrays (T.lat first)
+    std::vector<unsigned char> pack;   // the same on the host, kept for its memory
     unsigned char *d_ws = nullptr;
     size_t ws_cap = 0;
     std::vector<Plan> plans;
@@ -634,44 +636,58 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
 
 extern "C" {
 
-// Validates host tables and lays them out as the kernels read them (key | gap | slope, padded).
-static int build_tables(int n_tables, int n_bp, int npad, const uint64_t *sizes_bytes, int sizes_shared,
-                        const double *gap, const double *latency, std::vector<double> &tab, std::vector<double> &lat,
-                        bool *monotone)
+// Checks host tables; on success packs them as [latency][gap][sizes] for one copy to the device.
+static int check_tables(int n_tables, int n_bp, const uint64_t *sizes_bytes, int sizes_shared, const double *gap, const double *latency,
+                        std::vector<unsigned char> &pack, bool *monotone)
 {
-    *monotone = true;
-    try {
-        tab.assign(size_t(n_tables) * 3 * npad, 0.0);
-        lat.assign(latency, latency + n_tables);
-    } catch (const std::bad_alloc &) { return PLOGP_E_NOMEM; }
-
-    const double inf = std::numeric_limits<double>::infinity();
+    const double most = std::numeric_limits<double>::max();
+    bool falls = false;
     for (int t = 0; t < n_tables; ++t) {
         const uint64_t *sz = sizes_bytes + (sizes_shared ? 0 : size_t(t) * n_bp);
         const double *gp = gap + size_t(t) * n_bp;
-        if (!std::isfinite(lat[t]) || lat[t] < 0.0) return PLOGP_E_INVAL;
-        for (int i = 0; i < n_bp; ++i) {
-            if (!std::isfinite(gp[i]) || gp[i] < 0.0) return PLOGP_E_INVAL;
-            if (i && sz[i] <= sz[i - 1]) return PLOGP_E_INVAL;
-            if (i && gp[i] < gp[i - 1]) *monotone = false;
-            if (double(sz[i]) >= kTwo53) return PLOGP_E_RANGE;
+        if (!(latency[t] >= 0.0 && latency[t] <= most)) return PLOGP_E_INVAL;
+        // all values first, without a branch per value; which error it is, only where there is one
+        unsigned bad = 0, down = 0;
+        for (int i = 0; i < n_bp; ++i) bad |= unsigned(!(gp[i] >= 0.0)) | unsigned(!(gp[i] <= most));
+        for (int i = 1; i < n_bp; ++i) down |= unsigned(gp[i] < gp[i - 1]);
+        if (t == 0 || !sizes_shared) {
+            for (int i = 1; i < n_bp; ++i) bad |= unsigned(sz[i] <= sz[i - 1]);
+            bad |= unsigned(double(sz[n_bp - 1]) >= kTwo53);
         }
-        // Above the last size the last interval's line is continued: a falling line would turn g negative for
-        // large arguments, and the kernels compare times through their (sign-free) high words.
-        if (gp[n_bp - 1] < gp[n_bp - 2]) return PLOGP_E_RANGE;
-        double *key = tab.data() + size_t(t) * 3 * npad, *g0 = key + npad, *sl = g0 + npad;
-        for (int i = 0; i < npad; ++i) {
-            if (i <= n_bp - 2) {
-                key[i] = double(sz[i]);
-                g0[i] = gp[i];
-                sl[i] = (gp[i + 1] - gp[i]) / double(sz[i + 1] - sz[i]);
-            } else {
-                key[i] = inf;
-                g0[i] = 0.0;
-                sl[i] = 0.0;
+        if (bad)
+            for (int i = 0; i < n_bp; ++i) {
+                if (!std::isfinite(gp[i]) || gp[i] < 0.0) return PLOGP_E_INVAL;
+                if (i && sz[i] <= sz[i - 1]) return PLOGP_E_INVAL;
+                if (double(sz[i]) >= kTwo53) return PLOGP_E_RANGE;
             }
-        }
+        // Above the last size the last interval's line is continued: a falling line would turn g negative for
+        // large arguments, and the kernels' lower bounds and comparisons rely on times that are not.
+        if (gp[n_bp - 1] < gp[n_bp - 2]) return PLOGP_E_RANGE;
+        falls |= down != 0;
     }
+    *monotone = !falls;
+    const size_t lat = size_t(n_tables) * 8, gaps = size_t(n_tables) * n_bp * 8, sizes = (sizes_shared ? size_t(1) : size_t(n_tables)) * n_bp * 8;
+    try {
+        pack.resize(lat + gaps + sizes);
+    } catch (const std::bad_alloc &) { return PLOGP_E_NOMEM; }
+    std::memcpy(pack.data(), latency, lat);
+    std::memcpy(pack.data() + lat, gap, gaps);
+    std::memcpy(pack.data() + lat + gaps, sizes_bytes, sizes);
+    return PLOGP_OK;
+}
+
+// Enqueues the packed tables' copy and their layout.
+static int upload_tables(plogp_tables *h, int sizes_shared, cudaStream_t st)
+{
+    // pageable source: the runtime stages it before returning
+    CK(cudaMemcpyAsync(h->d_raw, h->pack.data(), h->pack.size(), cudaMemcpyHostToDevice, st));
+    LayoutParams lp{};
+    lp.gap = reinterpret_cast<const double *>(h->d_raw) + h->T.n_tables;
+    lp.sizes = reinterpret_cast<const uint64_t *>(lp.gap + size_t(h->T.n_tables) * h->T.n_bp);
+    lp.tab = h->d_tab;
+    lp.n_tables = h->T.n_tables; lp.n_bp = h->T.n_bp; lp.npad = h->T.npad; lp.sizes_shared = sizes_shared;
+    CK(launch_layout(lp, st));
+    g_launches += 1;
     return PLOGP_OK;
 }
 
@@ -684,9 +700,9 @@ int plogp_table_load(int n_tables, int n_bp, const uint64_t *sizes_bytes, int si
     int npad = 2;
     while (npad < n_bp) npad <<= 1;  // >= n_bp: at least one +inf key follows the last interval
 
-    std::vector<double> tab, lat;
+    std::vector<unsigned char> pack;
     bool monotone = false;
-    const int brc = build_tables(n_tables, n_bp, npad, sizes_bytes, sizes_shared, gap, latency, tab, lat, &monotone);
+    const int brc = check_tables(n_tables, n_bp, sizes_bytes, sizes_shared, gap, latency, pack, &monotone);
     if (brc != PLOGP_OK) return brc;
 
     plogp_tables *h = new (std::nothrow) plogp_tables();
@@ -696,20 +712,21 @@ int plogp_table_load(int n_tables, int n_bp, const uint64_t *sizes_bytes, int si
     if ((e = cudaGetDevice(&h->device)) != cudaSuccess) return fail(cuda_fail(e, "cudaGetDevice"));
     if ((e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device)) != cudaSuccess)
         return fail(cuda_fail(e, "cudaDeviceGetAttribute"));
-    if ((e = cudaMalloc(&h->d_tab, tab.size() * sizeof(double))) != cudaSuccess)
+    // one allocation: the kernels' layout, then room for the caller's arrays [latency][gap][sizes per table]
+    const size_t tab = size_t(n_tables) * 3 * npad * sizeof(double), raw = size_t(n_tables) * (1 + 2 * size_t(n_bp)) * 8;
+    if ((e = cudaMalloc(&h->d_tab, tab + raw)) != cudaSuccess)
         return fail(e == cudaErrorMemoryAllocation ? (cudaGetLastError(), PLOGP_E_NOMEM) : cuda_fail(e, "cudaMalloc(tables)"));
-    if ((e = cudaMalloc(&h->d_lat, lat.size() * sizeof(double))) != cudaSuccess)
-        return fail(e == cudaErrorMemoryAllocation ? (cudaGetLastError(), PLOGP_E_NOMEM) : cuda_fail(e, "cudaMalloc(latency)"));
-    if ((e = cudaMemcpy(h->d_tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return fail(cuda_fail(e, "cudaMemcpy(tables)"));
-    if ((e = cudaMemcpy(h->d_lat, lat.data(), lat.size() * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return fail(cuda_fail(e, "cudaMemcpy(latency)"));
+    h->d_raw = reinterpret_cast<unsigned char *>(h->d_tab) + tab;
+    h->pack.swap(pack);
     h->T.tab = h->d_tab;
-    h->T.lat = h->d_lat;
+    h->T.lat = reinterpret_cast<const double *>(h->d_raw);
     h->T.n_tables = n_tables;
     h->T.n_bp = n_bp;
     h->T.npad = npad;
     h->monotone = monotone;
+    const int urc = upload_tables(h, sizes_shared, nullptr);
+    if (urc != PLOGP_OK) return fail(urc);
+    if ((e = cudaStreamSynchronize(nullptr)) != cudaSuccess) return fail(cuda_fail(e, "cudaStreamSynchronize(tables)"));
     *out = h;
     return PLOGP_OK;
 }
@@ -721,23 +738,18 @@ int plogp_table_update(plogp_tables *h, const uint64_t *sizes_bytes, int sizes_s
     int dev = 0;
     CK(cudaGetDevice(&dev));
     if (dev != h->device) return PLOGP_E_INVAL;
-    std::vector<double> tab, lat;
     bool monotone = false;
-    const int brc = build_tables(h->T.n_tables, h->T.n_bp, h->T.npad, sizes_bytes, sizes_shared, gap, latency, tab, lat, &monotone);
+    const int brc = check_tables(h->T.n_tables, h->T.n_bp, sizes_bytes, sizes_shared, gap, latency, h->pack, &monotone);
     if (brc != PLOGP_OK) return brc;  // the tables on the device are untouched
     h->monotone = monotone;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // pageable sources: the runtime stages them before returning, so the vectors may go out of scope
-    CK(cudaMemcpyAsync(h->d_tab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(h->d_lat, lat.data(), lat.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    return PLOGP_OK;
+    return upload_tables(h, sizes_shared, static_cast<cudaStream_t>(stream));
 }
 
 int plogp_table_free(plogp_tables *h)
 {
     if (!h) return PLOGP_OK;
     int rc = PLOGP_OK;
-    std::vector<void *> bufs = {h->d_tab, h->d_lat, h->d_ws, h->d_stage[0], h->d_stage[1]};
+    std::vector<void *> bufs = {h->d_tab, h->d_ws, h->d_stage[0], h->d_stage[1]};
     for (const Plan &c : h->plans) bufs.push_back(c.d_grid);
     for (int i = 0; i < 2; ++i) {
         if (h->ev_done[i]) cudaEventDestroy(h->ev_done[i]);

@@ -139,6 +139,15 @@ struct ScatterParams {
     double *d_time;
 };
 
+// Tables as the caller has them -> TableDev's layout: see layout.cu
+struct LayoutParams {
+    const uint64_t *sizes;  // [n_bp] (shared) or [n_tables][n_bp]
+    const double *gap;      // [n_tables][n_bp]
+    double *tab;            // [n_tables][3 * npad]
+    int n_tables, n_bp, npad, sizes_shared;
+};
+cudaError_t launch_layout(const LayoutParams &p, cudaStream_t st);
+
 // Gap pre-pass (gaps.cu): g at every distinct argument of the lane <-> P kernels, once per table.
 // Row of a table: [0] = g(1), [1 .. n_s] = g(s_i), [1 + n_s .. 1 + n_s + n_m) = g(m_j).
 struct GapsParams {
