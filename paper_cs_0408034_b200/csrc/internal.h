@@ -112,7 +112,7 @@ struct FusedParams {
     int table0, n_tables_launch;
     int out_table0;  // table whose results sit at the start of the output arrays (0 unless the caller passes a window)
     OutMap om;
-    // segmented minima precomputed by the sweep kernel (nullptr => inline sweep)
+    // segmented minima from the sweep or envelope kernel (nullptr: no segmented strategy in the mask)
     const double *part_time;
     const uint32_t *part_idx;
     const int32_t *pair_base;  // device [n_m+1]
@@ -211,7 +211,6 @@ constexpr int kSweepBatch = 128; // candidates per comparison of the bounds with
 constexpr int kSweepSeeds = 128;  // log-spaced candidates that the upper bounds start from
 constexpr int kMaxInlineS = 64;
 
-size_t fused_smem_bytes(const TableDev &T, const GridDev &G, bool inline_sweep);
 cudaError_t launch_fused(const FusedParams &p, bool predict, bool overlap, cudaStream_t st);
 cudaError_t launch_scatter(const ScatterParams &p, bool overlap, cudaStream_t st);  // decision table, Scatter strategies only
 cudaError_t launch_sweep(const SweepParams &p, int n_tables_launch, int *launches, cudaStream_t st);

@@ -9,14 +9,13 @@
 //                  cell costs half a packed FP32 multiply-add and half a minimum; what the FP32 bounds leave
 //                  open is decided in FP64.  Used when the candidate list is long.
 //   fused_kernel   lane <-> message size m (32 consecutive m per warp, so every output row is
-//                  written as full, aligned segments).  Evaluates all enabled strategies, runs short
-//                  candidate lists inline or reduces the sweep kernel's partial minima, keeps the
+//                  written as full, aligned segments).  Evaluates all enabled strategies, reduces the sweep
+//                  kernel's partial minima where segmented ones are among them, keeps the
 //                  Scatter Chain sum running along each warp's contiguous run of P, and writes either
 //                  the predicted planes or the decision table.  The general path.
 // Short candidate lists have faster, specialised kernels: decide.cu (Broadcast half of the decision
 // table), scatter.cu (Scatter half), segmin.cu (segmented planes of the predictions); the host routes
-// them there, so fused_kernel's own inline loop over short lists only serves callers of launch_fused
-// that pass segmented strategies without partial minima.
+// them there, and fused_kernel writes the closed-form planes only.
 #include "device_common.cuh"
 
 namespace plogp {
@@ -296,43 +295,22 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
 // Fused evaluation: all strategies, strategy selection, stores
 // ------------------------------------------------------------------------------------------
 
-struct FusedSmem {
-    double *tab, *cum, *tot, *gs, *cB, *cC, *cQ;
-};
-
-__host__ __device__ inline size_t fused_smem_layout(int npad, int lc_max, int n_inline, FusedSmem *out)
+// table | Scatter Binomial sums [lc_max][32] | Scatter Chain [2][warps][32]
+static size_t fused_smem_bytes(const TableDev &T, const GridDev &G)
 {
-    size_t off = 0;
-    auto take = [&](size_t n) { size_t o = off; off += n; return o; };
-    const size_t o_tab = take(3 * (size_t)npad), o_cum = take((size_t)lc_max * 32),
-                 o_tot = take(2 * kWarps * 32), o_gs = take(n_inline), o_B = take((size_t)n_inline * 32),
-                 o_C = take((size_t)n_inline * 32), o_Q = take((size_t)n_inline * 32);
-    if (out) {
-        double *base = out->tab;
-        out->tab = base + o_tab; out->cum = base + o_cum; out->tot = base + o_tot; out->gs = base + o_gs;
-        out->cB = base + o_B; out->cC = base + o_C; out->cQ = base + o_Q;
-    }
-    return off * sizeof(double);
+    return (3 * static_cast<size_t>(T.npad) + static_cast<size_t>(G.lc_max) * 32 + 2 * kWarps * 32) * sizeof(double);
 }
 
-size_t fused_smem_bytes(const TableDev &T, const GridDev &G, bool inline_sweep)
-{
-    return fused_smem_layout(T.npad, G.lc_max, inline_sweep ? max(G.n_s, 1) : 1, nullptr);
-}
-
+// (Four warps per CTA instead of eight halve the set-up per process count and are 1 to 25 % slower, whatever the grid.)
 template <bool PREDICT>
 __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
 {
     constexpr int R = kFusedR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const bool inline_sweep = p.part_time == nullptr;
-    const int n_inline = inline_sweep ? max(p.G.n_s, 1) : 1;
-    FusedSmem sm;
-    sm.tab = reinterpret_cast<double *>(smem_raw);
-    fused_smem_layout(p.T.npad, p.G.lc_max, n_inline, &sm);
+    double *const s_tab = reinterpret_cast<double *>(smem_raw);
     const int npad = p.T.npad;
     const uint32_t mask = p.G.mask;
-    const bool any_seg = (mask & ((1u << 2) | (1u << 5) | (1u << 9))) != 0;
+    double *const s_cum = s_tab + 3 * npad, *const s_tot = s_cum + p.G.lc_max * 32;
 
     int b = blockIdx.x;
     const int mtile = b % p.n_mtiles;
@@ -350,40 +328,24 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
 
     dependents_may_start();
     const double L = p.T.lat[table];
-    stage_table(sm.tab, p.T, table);
-    if (!inline_sweep) wait_for_kernel_in_front();  // the partial minima
+    stage_table(s_tab, p.T, table);
+    if (p.part_time) wait_for_kernel_in_front();  // the partial minima
     __syncthreads();
 
-    const double g1 = gap_at_one(sm.tab, npad);
-    const double gm = gap_at(sm.tab, npad, md);
+    const double g1 = gap_at_one(s_tab, npad);
+    const double gm = gap_at(s_tab, npad, md);
 
     // Scatter Binomial Tree: running sums of g(2^j m), j = 0..lc_max-1 (Table 2, third row)
     // (the gaps are looked up by all warps, one j per warp at a time; warp 0 then adds them up)
     if ((mask >> 12) & 1u) {
         for (int d = warp; d < p.G.lc_max; d += kWarps)
-            sm.cum[d * 32 + lane] = gap_at(sm.tab, npad, md * static_cast<double>(1ull << d));
+            s_cum[d * 32 + lane] = gap_at(s_tab, npad, md * static_cast<double>(1ull << d));
         __syncthreads();
         if (warp == 0) {
             double acc = 0.0;
             for (int d = 0; d < p.G.lc_max; ++d) {
-                acc += sm.cum[d * 32 + lane];
-                sm.cum[d * 32 + lane] = acc;
-            }
-        }
-    }
-    // Inline candidate list: g(s) once per s, then the line coefficients per (s, m)
-    if (inline_sweep && any_seg) {
-        for (int si = tid; si < p.G.n_s; si += kThreads)
-            sm.gs[si] = gap_at(sm.tab, npad, static_cast<double>(s_at(p.G, si)));
-        __syncthreads();
-        for (int si = warp; si < p.G.n_s; si += kWarps) {
-            if (si < ns) {
-                const uint32_t s = s_at(p.G, si);
-                const double gs = sm.gs[si];
-                const double k = static_cast<double>(segments(m_u, s, p.G.k_mode));
-                sm.cB[si * 32 + lane] = gs + L;
-                sm.cC[si * 32 + lane] = gs * (k - 1.0);
-                sm.cQ[si * 32 + lane] = gs * k;
+                acc += s_cum[d * 32 + lane];
+                s_cum[d * 32 + lane] = acc;
             }
         }
     }
@@ -399,12 +361,12 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
     ChainWalk s1_walk;
     if ((mask >> 11) & 1u) {
         const int c0 = ptile * (kWarps * run_len), e0 = min(p_warp, p.G.n_P), e1 = min(p_warp + run_len, p.G.n_P);
-        chain_front_parts(sm.tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md, c0, e0, e1, warp, kWarps, sm.tot + lane, sm.tot + kWarps * 32 + lane, 32);
+        chain_front_parts(s_tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md, c0, e0, e1, warp, kWarps, s_tot + lane, s_tot + kWarps * 32 + lane, 32);
         __syncthreads();
         if (e0 < e1) {
-            s1_run = chain_front_sum(sm.tot + lane, sm.tot + kWarps * 32 + lane, 32, warp, kWarps);
+            s1_run = chain_front_sum(s_tot + lane, s_tot + kWarps * 32 + lane, 32, warp, kWarps);
             j_last = static_cast<double>(warp == 0 ? P_at(p.G, e0) - 2 : P_at(p.G, e0 - 1) - 1);
-            s1_walk.start(sm.tab, npad, (j_last + 1.0) * md);
+            s1_walk.start(s_tab, npad, (j_last + 1.0) * md);
         }
     }
 
@@ -430,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 if (ok[r]) {
-                    s1_run += j_last + 1.0 == pm1[r] ? s1_walk.at(sm.tab, npad, pm1[r] * md) : s1_walk.range(sm.tab, npad, md, j_last + 1.0, pm1[r]);
+                    s1_run += j_last + 1.0 == pm1[r] ? s1_walk.at(s_tab, npad, pm1[r] * md) : s1_walk.range(s_tab, npad, md, j_last + 1.0, pm1[r]);
                     j_last = pm1[r];
                 }
                 s1sum[r] = s1_run;
@@ -500,19 +462,6 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
                     st[r] = two_coef ? fma(a[r], gm + L, 0.0) : fma(a[r], gm, c[r]);
                     sb[r] = m_u;
                 }
-            } else if (inline_sweep) {
-                const double *c1 = two_coef ? sm.cB : sm.cQ;
-                for (int si = 0; si < ns; ++si) {
-                    const double k1 = c1[si * 32 + lane];
-                    const double k2 = two_coef ? sm.cC[si * 32 + lane] : 0.0;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const double t = fma(a[r], k1, two_coef ? k2 : c[r]);
-                        if (t < st[r]) { st[r] = t; si_best[r] = static_cast<uint32_t>(si); }
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < R; ++r) sb[r] = s_at(p.G, static_cast<int>(si_best[r]));
             } else {
                 // partial minima from the sweep kernel, chunks in ascending candidate order
                 const int r0 = p.pair_base[midx_c], r1 = p.pair_base[midx_c + 1];
@@ -603,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 2) fused_kernel(const FusedParams p)
         }
         if ((mask >> 12) & 1u) {  // Binomial Tree
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = sm.cum[(32 - __clz(Pv[r] - 1) - 1) * 32 + lane] + lcL[r];
+            for (int r = 0; r < R; ++r) v[r] = s_cum[(32 - __clz(Pv[r] - 1) - 1) * 32 + lane] + lcL[r];
             consider(12, v, nullptr);
         }
         if (mask & 0x1C00u) flush(1);
@@ -643,7 +592,7 @@ __global__ void __launch_bounds__(kThreads) fp64_probe_kernel(double *sink, int 
 
 cudaError_t launch_fused(const FusedParams &p, bool predict, bool overlap, cudaStream_t st)
 {
-    const size_t smem = fused_smem_bytes(p.T, p.G, p.part_time == nullptr);
+    const size_t smem = fused_smem_bytes(p.T, p.G);
     const long long blocks = static_cast<long long>(p.n_mtiles) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
     return launch(predict ? fused_kernel<true> : fused_kernel<false>, static_cast<unsigned>(blocks), 1, kThreads, smem, st, overlap, p);
