@@ -562,6 +562,16 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             SegminParams sp{};
             sp.T = h->T; sp.G = pl.G;
             sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs;
+            sp.warps = kDecWarps;
+            // Eight warps and 32 message sizes per CTA instead of four and 16 where rows are no multiple of a 32-byte sector, on
+            // grids of many CTAs: a row segment of 16 message sizes then is two write requests instead of one, a segment of 32
+            // three instead of two, each with part of a sector at either end (1024 tables, P = 2..513, 32 sizes, 16 -> 32: n_m =
+            // 127 1.70 -> 1.36 ms, 130 1.65 -> 1.33, 145 1.96 -> 1.51).  Whole sectors gain nothing (132: 1.17 -> 1.19 ms).
+            if (pl.G.n_m % 4 != 0 && pl.dec_mg == kDecMG && pl.dec_rows == 8 &&
+                (long long)pl.dec_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * 16) {
+                sp.warps = 2 * kDecWarps; sp.mg = 2 * kDecMG;
+                sp.n_mgroups = (pl.G.n_m + sp.mg - 1) / sp.mg;
+            }
             sp.table0 = t0; sp.n_tables_launch = nt; sp.out_table0 = out.out_table0;
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
             sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;

@@ -191,16 +191,12 @@ struct SegminParams {
     int gaps_stride;
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16-byte aligned times, 8-byte aligned sizes)
     int n_mgroups, n_ptiles;
-    int mg, rows, tiles, n_pairs;  // as in DecideParams
+    int mg, rows, tiles, n_pairs;  // as in DecideParams (mg up to 4 * warps)
+    int warps;  // per CTA: 4, or 8 (rows = 8)
     int table0, n_tables_launch, out_table0;
     double *p_time;      // [n_tables][13][n_P][n_m]: planes 2, 5, 9 are written
     uint32_t *p_best_s;  // [n_tables][3][n_P][n_m], or nullptr
 };
-constexpr int kSegThreads = 128;
-constexpr int kSegWarps = kSegThreads / 32;
-constexpr int kSegMG = 16;               // message sizes per CTA (at most), split over the warps
-static_assert(kSegMG == kDecMG && kSegThreads == kDecThreads, "the host gives both lane <-> P kernels the same tiling");
-
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kFusedR = 4;   // process counts per thread and pass in the fused kernel

@@ -3,8 +3,8 @@
 // of the model over the candidate segment sizes and the smallest size that attains it.
 //
 // Same building blocks as decide_kernel (decide.cu), with one running minimum per strategy instead of one
-// over all of them.  One CTA owns one table, up to 16 consecutive message sizes and one or two tiles of 256 process
-// counts (lane + 32 r, r = 0..7); its four warps split the message sizes.  For a fixed message size the models are
+// over all of them.  One CTA owns one table, up to 16 consecutive message sizes (32 with eight warps) and one or two tiles
+// of 256 process counts (lane + 32 r, r = 0..7); its four (eight) warps split the message sizes.  For a fixed message size the models are
 //     id 2: fma(P-1, Q, L)      id 9: fma(floor(log2 P), Q, ceil(log2 P) L)      Q = g(s) k
 //     id 5: fma(P-1, B, C)      B = g(s) + L, C = g(s) (k-1)
 // so a warp builds the coefficient lists of a message size (lanes <-> candidates), searches id 9 once per
@@ -38,7 +38,7 @@ struct SegSmem {
     double *q;        // [mg][cap]: Q
     double *t9;       // [mg][n_pairs]: id 9's minimum
     float *x;         // [n_p]: P-1 rounded down
-    float *fb, *fc, *fq;  // [kSegWarps][cap]: the lists of the warp's current message size rounded down, without the pilots
+    float *fb, *fc, *fq;  // [warps][cap]: the lists of the warp's current message size rounded down, without the pilots
     uint32_t *sval;
     uint8_t *i9;      // [mg][n_pairs]: id 9's winner
     uint8_t *pair;    // [n_p]: pair of a process count
@@ -46,7 +46,7 @@ struct SegSmem {
     int cap, stride;
 };
 
-__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int n_p, int mg, unsigned char *base, SegSmem *o)
+__host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int n_p, int mg, int warps, unsigned char *base, SegSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
     const int cap = round_up(nsv, kStep), stride = n_p + 4;
@@ -54,8 +54,8 @@ __host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(mg * 8), o_pm = take(size_t(n_p) * 8),
                  o_l5 = take(size_t(mg) * cap * 16), o_q = take(size_t(mg) * cap * 8), o_t9 = take(size_t(mg) * n_pairs * 8),
-                 o_x = take(size_t(n_p) * 4), o_fb = take(size_t(kSegWarps) * cap * 4), o_fc = take(size_t(kSegWarps) * cap * 4),
-                 o_fq = take(size_t(kSegWarps) * cap * 4), o_sv = take(size_t(nsv) * 4), o_i9 = take(size_t(mg) * n_pairs), o_pair = take(n_p),
+                 o_x = take(size_t(n_p) * 4), o_fb = take(size_t(warps) * cap * 4), o_fc = take(size_t(warps) * cap * 4),
+                 o_fq = take(size_t(warps) * cap * 4), o_sv = take(size_t(nsv) * 4), o_i9 = take(size_t(mg) * n_pairs), o_pair = take(n_p),
                  o_p2 = take(size_t(mg) * stride), o_p5 = take(size_t(mg) * stride);
     if (o) {
         o->tab = reinterpret_cast<double *>(base + o_tab); o->gs = reinterpret_cast<double *>(base + o_gs);
@@ -72,16 +72,16 @@ __host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int
 
 }  // namespace
 
-// R: as in decide_kernel.
-template <int R>
-__global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminParams p)
+// R: as in decide_kernel.  W: warps, four of them per 16 message sizes (the host says when eight are better).
+template <int R, int W>
+__global__ void __launch_bounds__(32 * W, W == 4 ? 5 : 2) segmin_kernel(const SegminParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad;
     SegSmem sm;
     constexpr int kTileP = 32 * R;
     const int n_p = p.tiles * kTileP;
-    seg_layout(npad, p.G.n_s, p.n_pairs, n_p, p.mg, smem_raw, &sm);
+    seg_layout(npad, p.G.n_s, p.n_pairs, n_p, p.mg, W, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
     const bool has2 = (mask >> 2) & 1u, has5 = (mask >> 5) & 1u, has9 = (mask >> 9) & 1u;
 
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
     const double *grow = p.gaps ? p.gaps + static_cast<size_t>(trel) * p.gaps_stride : nullptr;
     // what the set-up reads from global memory is on its way while the table is
     const double L = p.T.lat[table];
-    const uint32_t m_mine = m0 + (tid & (kSegMG - 1)) < p.G.n_m ? p.G.m_list[m0 + (tid & (kSegMG - 1))] : 0u;
+    const uint32_t m_mine = m0 + (tid & (4 * W - 1)) < p.G.n_m ? p.G.m_list[m0 + (tid & (4 * W - 1))] : 0u;
     const uint32_t s_mine = tid < p.G.n_s ? s_at(p.G, tid) : 0u;
     const int n_s = p.G.n_s;  // at most kMaxInlineS, fewer than the threads
     int ns_next = 0;
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
     if (!grow) stage_table(sm.tab, p.T, table);
     else wait_for_kernel_in_front();  // the gap pre-pass
     dependents_may_start();
-    for (int i = tid; i < n_p; i += kSegThreads) {
+    for (int i = tid; i < n_p; i += 32 * W) {
         const int P = P_at(p.G, min(tile0 + i, p.G.n_P - 1));
         sm.pm1[i] = static_cast<double>(P - 1);
         sm.x[i] = __int2float_rd(P - 1);
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
         sm.sval[tid] = s_mine;
         sm.gs[tid] = grow ? grow[1 + tid] : gap_at(sm.tab, npad, static_cast<double>(s_mine));
     }
-    if (tid >= kSegThreads - kSegMG) {
-        const int mi = tid - (kSegThreads - kSegMG);
+    if (tid >= 28 * W) {
+        const int mi = tid - 28 * W;
         if (mi < n_mi) sm.gm[mi] = grow ? grow[1 + n_s + m0 + mi] : gap_at(sm.tab, npad, static_cast<double>(m_mine));
     }
     __syncthreads();
@@ -145,11 +145,11 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
     const float Lf = __double2float_rd(L);
     const f32x2 L2 = splat2(Lf);
 
-    for (int mi = warp; mi < n_mi; mi += kSegWarps) {
+    for (int mi = warp; mi < n_mi; mi += W) {
         // what a message size reads from global memory is fetched while the one before it is worked on
         const int ns = ns_next;
         const double k_of[2] = {k_next[0], k_next[1]};
-        fetch(mi + kSegWarps);
+        fetch(mi + W);
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
         const int np4 = round_up(nsv, 4), np16 = round_up(nsv, kStep);
         const double gm = sm.gm[mi];
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
         if (p.vec_out) {
             // two message sizes per lane (16-byte and 8-byte stores; the host has checked the alignment)
             const int half = p.mg >> 1;
-            const int mi = 2 * (lane & (half - 1)), rows = 32 / half, step = kSegWarps * rows, pr0 = warp * rows + lane / half;
+            const int mi = 2 * (lane & (half - 1)), rows = 32 / half, step = W * rows, pr0 = warp * rows + lane / half;
             if (mi < n_mi) {  // n_m is even, so mi + 1 is a message size of the grid too
                 const uint32_t m_u0 = p.G.m_list[m0 + mi], m_u1 = p.G.m_list[m0 + mi + 1];
                 const bool w0 = p.G.ns_of_m[m0 + mi] == 0, w1 = p.G.ns_of_m[m0 + mi + 1] == 0;  // the whole message
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kSegThreads, 5) segmin_kernel(const SegminPara
             if (mi < n_mi) {
                 const uint32_t m_u = p.G.m_list[m0 + mi];
                 const bool whole = p.G.ns_of_m[m0 + mi] == 0;
-                for (int pr = warp * rows + lane / p.mg; pr < n_valid; pr += kSegWarps * rows) {
+                for (int pr = warp * rows + lane / p.mg; pr < n_valid; pr += W * rows) {
                     const size_t o = static_cast<size_t>(pr) * p.G.n_m + mi;
                     unsigned at;
                     plane_t[o] = cell(mi, pr, sm.pm1[pr], at);
@@ -404,8 +404,9 @@ cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
 {
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    const size_t smem = seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, p.mg, nullptr, nullptr);
-    return launch(p.rows == 8 ? segmin_kernel<8> : segmin_kernel<4>, static_cast<unsigned>(blocks), 1, kSegThreads, smem, st, overlap, p);
+    const size_t smem = seg_layout(p.T.npad, p.G.n_s, p.n_pairs, p.tiles * 32 * p.rows, p.mg, p.warps, nullptr, nullptr);
+    const auto kernel = p.warps == 8 ? segmin_kernel<8, 8> : (p.rows == 8 ? segmin_kernel<8, 4> : segmin_kernel<4, 4>);
+    return launch(kernel, static_cast<unsigned>(blocks), 1, 32u * p.warps, smem, st, overlap, p);
 }
 
 }  // namespace plogp

@@ -114,3 +114,22 @@ def test_both_halves_in_one_launch_and_in_two(plogp, n_P, n_m, n_s, n_tables, li
         torch.cuda.synchronize()
         assert len(plogp.profile_read(tabs)) >= 2
         assert torch.equal(a.strategy, b.strategy) and torch.equal(a.s_bytes, b.s_bytes) and torch.equal(a.time, b.time)
+
+
+@pytest.mark.parametrize("n_m,n_P,n_s,k_mode", [(17, 300, 33, 0), (33, 257, 5, 1), (65, 129, 64, 0), (97, 513, 20, 0), (98, 70, 32, 0)])
+def test_prediction_rows_off_the_sectors_on_many_tables(plogp, n_m, n_P, n_s, k_mode):
+    """Rows of message sizes that are no multiple of 32 bytes, on enough tables for CTAs of 32 message sizes (the last one
+    ragged): the first and last table match the oracle, and the searches of five tables at either end a call
+    over these alone, bit for bit."""
+    import torch
+    n = 2368 // max(1, n_m // 16) + 8
+    w = replace(wl.config4(n_tables=n, P_hi=n_P + 1, n_m=n_m, n_s=n_s, seed_offset=n_m), k_mode=k_mode)
+    with plogp.Tables.from_workload(w) as tabs:
+        a = plogp.predict(tabs, w)
+    p_idx = np.unique(np.r_[0:n_P:7, n_P - 1])
+    assert check_prediction(w, oracle_tables(w), a, tables=(0, n - 1), p_idx=p_idx) > 0
+    for lo in (0, n - 5):
+        few = replace(w, gaps=np.ascontiguousarray(w.gaps[lo:lo + 5]), latency=w.latency[lo:lo + 5])
+        with plogp.Tables.from_workload(few) as tabs:
+            b = plogp.predict(tabs, few)
+        assert torch.equal(a.time[lo:lo + 5, [2, 5, 9]], b.time[:, [2, 5, 9]]) and torch.equal(a.best_s[lo:lo + 5], b.best_s)
