@@ -627,6 +627,29 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             g_launches += 1;
             continue;
         }
+        bool behind = pl.n_seg > 0 && (!pl.inline_sweep ? pl.envelope || pl.n_pairs > 0 : predict);  // a kernel of this call is in front
+        // Rows that are no multiple of a 32-byte sector: the planes that need no sum along P are written cell by cell as they
+        // lie in memory (planes.cu).  Whole calls, all ids, 32 sizes, without -> with: 1024 tables, P = 2..513, n_m = 127 3.34 ->
+        // 2.36 ms, 33 1.05 -> 0.86, whole sectors 136 2.05 -> 1.98 and 72 1.07 -> 1.10.  It is one launch more, so the line is
+        // where it starts to gain: rows of one warp are written one after another anyhow (n_m = 17: 0.40 -> 0.46 ms), planes of
+        // few rows spend it on their set-up (P = 2..101, 145 m, 4000 tables 2.37 -> 2.40, P = 2..201, 2000 tables 2.64 -> 2.14),
+        // and the L2 takes what is smaller than it (P = 2..512, 99 m: 32 tables 92 -> 93 us, 100 300 -> 277).
+        const size_t cells = size_t(pl.G.n_P) * pl.G.n_m;
+        if (predict && pl.inline_sweep && pl.G.n_m % 4 != 0 && pl.G.n_m > 32 && pl.G.n_m <= kPlanesMaxM && pl.G.n_P >= 160 && cells * nt >= (size_t(1) << 22)) {
+            PlanesParams pp{};
+            pp.T = h->T; pp.G = pl.G; pp.mask = Gf.mask & kPlanesMask;
+            // whole planes per CTA, split while that leaves fewer than eight CTAs per SM
+            const size_t split = std::max<size_t>(1, (size_t(h->sm_count) * 8 + nt - 1) / nt);
+            pp.seg_cells = (long long)std::max<size_t>(2048, ((cells + 31 + split - 1) / split + 255) / 256 * 256);
+            pp.table0 = t0; pp.n_tables_launch = nt; pp.out_table0 = out.out_table0; pp.p_time = out.p_time;
+            if (pp.mask) {
+                { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_planes(pp, overlap && behind, st)); }
+                g_launches += 1;
+                behind = true;
+                Gf.mask &= ~kPlanesMask;
+                if (!Gf.mask) continue;
+            }
+        }
         FusedParams fp = out;
         fp.T = h->T; fp.G = Gf;
         fp.n_mtiles = pl.n_mtiles; fp.n_ptiles = pl.n_ptiles; fp.passes_per_tile = pl.passes_per_tile;
@@ -636,7 +659,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         fp.part_idx = part_idx;
         fp.pair_base = pl.inline_sweep ? nullptr : reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_pair_base);
         fp.n_pairs = pl.n_pairs; fp.n_seg = pl.n_seg;
-        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, overlap && pl.n_seg > 0 && (!pl.inline_sweep ? pl.envelope || pl.n_pairs > 0 : predict), st)); }
+        { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_fused(fp, predict, overlap && behind, st)); }
         g_launches += 1;
     }
     return PLOGP_OK;

@@ -126,6 +126,19 @@ struct FusedParams {
     uint32_t *p_best_s;
 };
 
+// Closed-form prediction planes cell by cell as they lie in memory: see planes.cu
+struct PlanesParams {
+    TableDev T;
+    GridDev G;
+    uint32_t mask;        // of kPlanesMask
+    long long seg_cells;  // cells of a plane per CTA, a multiple of 256
+    int table0, n_tables_launch, out_table0;
+    double *p_time;       // [n_tables][13][n_P][n_m]
+};
+constexpr uint32_t kPlanesMask = 0x5DBu;  // ids 0 1 3 4 6 7 8 10
+constexpr int kPlanesMaxM = 4096;         // g(m) of all message sizes in shared memory
+cudaError_t launch_planes(const PlanesParams &p, bool overlap, cudaStream_t st);
+
 // Scatter half of the decision table: see scatter.cu
 struct ScatterParams {
     TableDev T;

@@ -133,3 +133,19 @@ def test_prediction_rows_off_the_sectors_on_many_tables(plogp, n_m, n_P, n_s, k_
         with plogp.Tables.from_workload(few) as tabs:
             b = plogp.predict(tabs, few)
         assert torch.equal(a.time[lo:lo + 5, [2, 5, 9]], b.time[:, [2, 5, 9]]) and torch.equal(a.best_s[lo:lo + 5], b.best_s)
+
+
+@pytest.mark.parametrize("n_m,n_P,n_tables,listed,ids", [(33, 160, 796, False, range(13)), (35, 163, 736, True, (0, 1, 3, 10)), (255, 161, 103, False, (4, 6, 7, 8)),
+                                                         (257, 409, 40, False, range(13)), (1031, 4100, 1, True, (0, 2, 6, 10, 11))])
+def test_closed_form_planes_cell_by_cell(plogp, n_m, n_P, n_tables, listed, ids):
+    """Planes written as they lie in memory (rows off the sectors, at least 2^22 cells): starts of planes at all 32 offsets
+    from a 256-byte boundary, rows shorter and longer than a CTA, with and without the kernel of the Scatter sums behind."""
+    base = wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=3, seed_offset=n_P)
+    w = replace(base, m=np.arange(4, 4 + 4 * n_m, 4, dtype=np.uint64) ** 2 // 4, strategy_mask=sum(1 << i for i in ids))
+    if listed:
+        w = replace(w, P_list=(2 + 3 * np.arange(n_P)).astype(np.int32))
+    assert w.n_m == n_m and w.n_P == n_P and n_P * n_m * n_tables >= 1 << 22
+    with plogp.Tables.from_workload(w) as tabs:
+        pred = plogp.predict(tabs, w)
+    p_idx, m_idx = np.unique(np.r_[0:4, 0:n_P:29, n_P - 2, n_P - 1]), np.unique(np.r_[0:n_m:7, n_m - 1])
+    assert check_prediction(w, oracle_tables(w), pred, tables=sorted({0, n_tables // 2, n_tables - 1}), p_idx=p_idx, m_idx=m_idx) > 0
