@@ -613,6 +613,28 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             Gf.n_s = 0;
             if (!Gf.mask) continue;
         }
+        // Rows of message sizes that are no multiple of a 32-byte sector: the Scatter sums go out as one piece per CTA (rows.cu).
+        // Decision tables, 32 sizes, without -> with: 2048 tables, P = 2..513, n_m = 127 1.83 -> 1.45 ms, 130 1.88 -> 1.58, 145
+        // 2.16 -> 1.74, 66 0.98 -> 0.83, whole sectors 132 1.64 -> 1.56, 136 1.52 -> 1.59 and 72 0.84 -> 0.87.  A warp more for
+        // a few message sizes past 32 costs what it gains (42: 0.525 -> 0.546 ms, 46 of 4096 tables 560 -> 552 us); what the L2
+        // takes gains nothing (200 tables 207 -> 205 us); a CTA sums up in front of its run what eight warps did elsewhere, so
+        // its run is at least as long as the table (1024 tables of 200 sizes 947 -> 818 us, 512 of 256 497 -> 451, of 1000 sizes
+        // 1104 -> 1202) and at most 256, split until there are 16 CTAs per SM.
+        const size_t cells = size_t(pl.G.n_P) * pl.G.n_m;
+        const bool rows_off = pl.G.n_m % 4 != 0 && pl.G.n_m >= 44 && pl.G.n_m <= kRowsMaxM && h->T.npad <= 256 && cells * nt >= (size_t(1) << 23);
+        RowsParams rp{};
+        rp.T = h->T; rp.G = Gf;
+        rp.run_len = std::min(pl.G.n_P, std::max(h->T.n_bp, int(std::min<long long>(256, (long long)pl.G.n_P * nt / (h->sm_count * 16LL)))));
+        rp.n_ptiles = (pl.G.n_P + rp.run_len - 1) / rp.run_len;
+        rp.table0 = t0; rp.n_tables_launch = nt; rp.out_table0 = out.out_table0;
+        if (use_scatter && rows_off && reinterpret_cast<uintptr_t>(out.d_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 16 == 0 &&
+            reinterpret_cast<uintptr_t>(out.d_strategy) % 4 == 0) {
+            rp.om = out.om;
+            rp.d_strategy = out.d_strategy; rp.d_sbytes = out.d_sbytes; rp.d_time = out.d_time;
+            { LaunchTimer lt(h, PLOGP_KERNEL_SCATTER, st); CK(launch_rows(rp, false, overlap && use_decide, st)); }
+            g_launches += 1;
+            continue;
+        }
         if (use_scatter) {
             ScatterParams sc{};
             sc.T = h->T; sc.G = Gf;
@@ -634,7 +656,6 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         // where it starts to gain: rows of one warp are written one after another anyhow (n_m = 17: 0.40 -> 0.46 ms), planes of
         // few rows spend it on their set-up (P = 2..101, 145 m, 4000 tables 2.37 -> 2.40, P = 2..201, 2000 tables 2.64 -> 2.14),
         // and the L2 takes what is smaller than it (P = 2..512, 99 m: 32 tables 92 -> 93 us, 100 300 -> 277).
-        const size_t cells = size_t(pl.G.n_P) * pl.G.n_m;
         if (predict && pl.inline_sweep && pl.G.n_m % 4 != 0 && pl.G.n_m > 32 && pl.G.n_m <= kPlanesMaxM && pl.G.n_P >= 160 && cells * nt >= (size_t(1) << 22)) {
             PlanesParams pp{};
             pp.T = h->T; pp.G = pl.G; pp.mask = Gf.mask & kPlanesMask;
@@ -648,6 +669,14 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
                 behind = true;
                 Gf.mask &= ~kPlanesMask;
                 if (!Gf.mask) continue;
+            }
+            if (rows_off && !(Gf.mask & ~0x1800u) && reinterpret_cast<uintptr_t>(out.p_time) % 32 == 0) {
+                rp.G = Gf;
+                rp.om.planes = 13;
+                rp.d_time = out.p_time;
+                { LaunchTimer lt(h, PLOGP_KERNEL_FUSED, st); CK(launch_rows(rp, true, overlap && behind, st)); }
+                g_launches += 1;
+                continue;
             }
         }
         FusedParams fp = out;

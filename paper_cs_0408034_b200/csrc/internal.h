@@ -152,6 +152,20 @@ struct ScatterParams {
     double *d_time;
 };
 
+// Scatter half of the decision table, or the predictions of ids 11 and 12, rows off the sectors: see rows.cu
+struct RowsParams {
+    TableDev T;
+    GridDev G;
+    int n_ptiles, run_len;  // CTAs along P and process counts of each
+    int table0, n_tables_launch, out_table0;
+    OutMap om;  // predictions: 13 planes per table, nothing else is read
+    uint8_t *d_strategy;  // aligned for four cells per store: 4,
+    uint32_t *d_sbytes;   // 16 and
+    double *d_time;       // 32 bytes
+};
+constexpr int kRowsMaxM = 256;
+cudaError_t launch_rows(const RowsParams &p, bool predict, bool overlap, cudaStream_t st);
+
 // Tables as the caller has them -> TableDev's layout: see layout.cu
 struct LayoutParams {
     const uint64_t *sizes;  // [n_bp] (shared) or [n_tables][n_bp]

@@ -6,7 +6,7 @@
 // and P, so here the cells of a plane are taken as they lie in memory: a warp's store is 32 cells from a 256-byte boundary,
 // whatever row they belong to, and each thread follows its process count and message size as it steps through the plane.
 // g(m) of all message sizes is in shared memory.  1024 tables, P = 2..513, n_m = 145: the eight planes take 0.90 ms (5.4 TB/s)
-// and the two that stay with fused_kernel 0.57, where that kernel took 2.45 for all ten (n_m = 127: 0.81 + 0.47 for 2.09).
+// where fused_kernel took 1.88 (2.45 for all ten; n_m = 127: 0.81 for 1.61).
 #include "device_common.cuh"
 
 namespace plogp {

@@ -149,3 +149,23 @@ def test_closed_form_planes_cell_by_cell(plogp, n_m, n_P, n_tables, listed, ids)
         pred = plogp.predict(tabs, w)
     p_idx, m_idx = np.unique(np.r_[0:4, 0:n_P:29, n_P - 2, n_P - 1]), np.unique(np.r_[0:n_m:7, n_m - 1])
     assert check_prediction(w, oracle_tables(w), pred, tables=sorted({0, n_tables // 2, n_tables - 1}), p_idx=p_idx, m_idx=m_idx) > 0
+
+
+@pytest.mark.parametrize("n_m,n_P,n_tables,n_bp,listed,ids", [(45, 257, 740, 64, False, range(13)), (255, 161, 206, 12, True, range(13)), (97, 2000, 45, 256, False, (2, 10, 12)),
+                                                              (150, 300, 200, 30, False, (5, 11)), (46, 16, 11500, 5, False, (10, 11, 12)), (129, 65100, 1, 100, True, (0, 11, 12))])
+def test_scatter_rows_off_the_sectors(plogp, n_m, n_P, n_tables, n_bp, listed, ids):
+    """Pieces of the Scatter plane per CTA (rows off the sectors, at least 2^23 cells): ragged last runs and flushes, pieces
+    that start at all four offsets from a group of cells, one to eight warps, sums in front of a run, some ids alone."""
+    base = wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=3, seed_offset=n_P)
+    sizes = wl.log_spaced_multiples(4, 256 << 20, n_bp)
+    gaps = np.stack([np.interp(sizes.astype(float), base.sizes.astype(float), g) for g in base.gaps])
+    w = replace(base, sizes=sizes, gaps=gaps, strategy_mask=sum(1 << i for i in ids))
+    if listed:
+        w = replace(w, P_list=(2 + 2 * np.arange(n_P)).astype(np.int32))
+    assert w.n_P == n_P and n_P * n_m * n_tables >= 1 << 23
+    p_idx, m_idx = np.unique(np.r_[0:4, 0:n_P:max(1, n_P // 40), n_P - 2, n_P - 1]), np.unique(np.r_[0:n_m:11, n_m - 1])
+    ot = oracle_tables(w)
+    sample = dict(tables=sorted({0, 1 % n_tables, n_tables // 2, n_tables - 1}), p_idx=p_idx, m_idx=m_idx)
+    with plogp.Tables.from_workload(w) as tabs:
+        assert check_decision(w, ot, plogp.select_best(tabs, w), **sample) > 0
+        assert check_prediction(w, ot, plogp.predict(tabs, w), **sample) > 0
