@@ -619,9 +619,10 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         // a few message sizes past 32 costs what it gains (42: 0.525 -> 0.546 ms, 46 of 4096 tables 560 -> 552 us); what the L2
         // takes gains nothing (200 tables 207 -> 205 us); a CTA sums up in front of its run what eight warps did elsewhere, so
         // its run is at least as long as the table (1024 tables of 200 sizes 947 -> 818 us, 512 of 256 497 -> 451, of 1000 sizes
-        // 1104 -> 1202) and at most 256, split until there are 16 CTAs per SM.
+        // 1104 -> 1202) and at most 256, split until there are 16 CTAs per SM.  Listed process counts are summed up by intervals,
+        // which is most of a cell there (1000 tables, 203 process counts, 101 m: 339 -> 370 us).
         const size_t cells = size_t(pl.G.n_P) * pl.G.n_m;
-        const bool rows_off = pl.G.n_m % 4 != 0 && pl.G.n_m >= 44 && pl.G.n_m <= kRowsMaxM && h->T.npad <= 256 && cells * nt >= (size_t(1) << 23);
+        const bool rows_off = !pl.G.P_list && pl.G.n_m % 4 != 0 && pl.G.n_m >= 44 && pl.G.n_m <= kRowsMaxM && h->T.npad <= 256 && cells * nt >= (size_t(1) << 23);
         RowsParams rp{};
         rp.T = h->T; rp.G = Gf;
         rp.run_len = std::min(pl.G.n_P, std::max(h->T.n_bp, int(std::min<long long>(256, (long long)pl.G.n_P * nt / (h->sm_count * 16LL)))));

@@ -152,7 +152,8 @@ struct ScatterParams {
     double *d_time;
 };
 
-// Scatter half of the decision table, or the predictions of ids 11 and 12, rows off the sectors: see rows.cu
+// Scatter half of the decision table, or the predictions of ids 11 and 12, for a range of process counts and rows off the
+// sectors: see rows.cu
 struct RowsParams {
     TableDev T;
     GridDev G;

@@ -3,7 +3,7 @@
 //
 // Bound by memory writes.  scatter_kernel and fused_kernel store row by row, 32 or 64 message sizes at a time; with such
 // rows every store straddles lines and sectors.  Here a CTA has all message sizes of a table, one per thread, and walks one
-// run of process counts: its cells are one piece of the plane.  The results of a few rows are put together in shared
+// run of consecutive process counts: its cells are one piece of the plane.  The results of a few rows are put together in shared
 // memory (two buffers, one barrier per flush) and go out from aligned addresses, whatever row they belong to.
 // 2048 tables, P = 2..513, n_m = 127: 0.37 ms (4.7 TB/s) where scatter_kernel took 0.73; n_m = 145 0.46 for 0.88 (its rows of
 // 128: 0.30).  Predictions, 1024 tables, n_m = 127: 0.30 ms for both ids where fused_kernel took 0.48, n_m = 145 0.34 for 0.57.
@@ -26,8 +26,8 @@ __device__ __forceinline__ void store4(double *out, const double *s)
     asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(out), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
 }
 
-// PREDICT: times of ids 11 and 12 instead of the decision.  CONTIG, ALL: as in scatter_block.
-template <bool PREDICT, bool CONTIG, bool ALL>
+// PREDICT: times of ids 11 and 12 instead of the decision.  ALL: all ids that the kernel writes are enabled.
+template <bool PREDICT, bool ALL>
 __global__ void __launch_bounds__(kRowsThreads, 4) scatter_rows_kernel(const RowsParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -51,14 +51,14 @@ __global__ void __launch_bounds__(kRowsThreads, 4) scatter_rows_kernel(const Row
     __syncthreads();
     const double gm = on10 ? gap_at(s_tab, npad, md) : 0.0;
 
-    int P = P_at(p.G, e0), lc = 0, P_next_lc = 2;  // ceil(log2 P) is lc below P_next_lc
+    int P = p.G.P_lo + e0, lc = 0, P_next_lc = 2;  // ceil(log2 P) is lc below P_next_lc
     double pm1 = static_cast<double>(P - 1), cum = 0.0, s2 = 0.0;  // cum: sum of g(2^d m), d < lc
-    double run = 0.0, j_last = static_cast<double>(P - 2);         // Chain: sum of g(j m) up to j_last
+    double run = 0.0;                                              // Chain: sum of g(j m), j < P - 1
     ChainWalk walk;
     if (on11) {
-        chain_front_parts(s_tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md, e0, e0, e1, 0, 1, s_t + tid, s_t + threads + tid, 0);
+        chain_front_parts(s_tab, npad, p.T.n_bp, nullptr, p.G.P_lo, md, e0, e0, e1, 0, 1, s_t + tid, s_t + threads + tid, 0);
         run = s_t[tid];
-        walk.start(s_tab, npad, (j_last + 1.0) * md);
+        walk.start(s_tab, npad, pm1 * md);
         __syncthreads();  // the buffers are now the rows'
     }
 
@@ -76,10 +76,6 @@ __global__ void __launch_bounds__(kRowsThreads, 4) scatter_rows_kernel(const Row
             double *ct = t_rows + shift + tid, *ct12 = t_rows + cap + shift12 + tid;
             uint8_t *ci = id_rows + shift + tid;
             for (int r = 0; r < rows; ++r) {
-                if (!CONTIG) {
-                    P = P_at(p.G, e + r);
-                    pm1 = static_cast<double>(P - 1);
-                }
                 if (on12 && P >= P_next_lc) {  // P passed a power of two
                     do {
                         cum += gap_at(s_tab, npad, md * static_cast<double>(1ull << lc));
@@ -90,7 +86,7 @@ __global__ void __launch_bounds__(kRowsThreads, 4) scatter_rows_kernel(const Row
                 }
                 double t11 = CUDART_INF;
                 if (on11) {
-                    run += CONTIG ? walk.at(s_tab, npad, pm1 * md) : walk.range(s_tab, npad, md, j_last + 1.0, pm1);
+                    run += walk.at(s_tab, npad, pm1 * md);
                     t11 = fma(pm1, L, run);
                 }
                 if (PREDICT) {
@@ -108,8 +104,8 @@ __global__ void __launch_bounds__(kRowsThreads, 4) scatter_rows_kernel(const Row
                     ci += n_m;
                 }
                 ct += n_m;
-                if (CONTIG) { ++P; pm1 += 1.0; }
-                else j_last = pm1;
+                ++P;
+                pm1 += 1.0;
             }
         }
         __syncthreads();  // also: everyone is past the flush of the other buffer
@@ -153,12 +149,9 @@ cudaError_t launch_rows(const RowsParams &p, bool predict, bool overlap, cudaStr
     const long long blocks = static_cast<long long>(p.n_ptiles) * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL || p.G.n_m > kRowsThreads) return cudaErrorInvalidConfiguration;
     const uint32_t ids = predict ? 0x1800u : 0x1C00u;
-    const bool all = (p.G.mask & ids) == ids, contig = p.G.P_list == nullptr;
-    void (*kernel)(RowsParams);
-    if (predict) kernel = contig ? (all ? scatter_rows_kernel<true, true, true> : scatter_rows_kernel<true, true, false>)
-                                 : (all ? scatter_rows_kernel<true, false, true> : scatter_rows_kernel<true, false, false>);
-    else kernel = contig ? (all ? scatter_rows_kernel<false, true, true> : scatter_rows_kernel<false, true, false>)
-                         : (all ? scatter_rows_kernel<false, false, true> : scatter_rows_kernel<false, false, false>);
+    const bool all = (p.G.mask & ids) == ids;
+    const auto kernel = predict ? (all ? scatter_rows_kernel<true, true> : scatter_rows_kernel<true, false>)
+                                : (all ? scatter_rows_kernel<false, true> : scatter_rows_kernel<false, false>);
     return launch(kernel, static_cast<unsigned>(blocks), 1, static_cast<unsigned>(rows_threads(p.G.n_m)), smem, st, overlap, p);
 }
 
