@@ -641,7 +641,10 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sc.T = h->T; sc.G = Gf;
             const bool aligned = reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 &&
                                  reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
-            sc.vec = aligned ? pl.sc_vec : 1;
+            // The table of sums is built by every CTA and takes 512 bytes per interval: 1000 tables, 200 process counts, 128 m,
+            // closed forms along the run -> table: 64 sizes 449 -> 429 us, 128 468 -> 471, 200 486 -> 542.
+            sc.chain_table = pl.G.P_list && h->T.n_bp <= 96;
+            sc.vec = aligned && !sc.chain_table ? pl.sc_vec : 1;
             sc.n_mtiles = (pl.G.n_m + 32 * sc.vec - 1) / (32 * sc.vec);
             sc.n_ptiles = pl.sc_ptiles; sc.run_len = pl.sc_run;
             sc.table0 = t0; sc.n_tables_launch = nt; sc.out_table0 = out.out_table0; sc.om = out.om;

@@ -246,6 +246,71 @@ __device__ __forceinline__ double chain_front_sum(const double *s_front, const d
     return run;
 }
 
+// The same sums for listed process counts, from a table per message size (lane) of the CTA: s_ja[i] = the first j whose
+// argument j m lies in interval i or behind it, s_before[i] = the sum of g(j m) over all j in front of it.  The sum up to any
+// j is then one arithmetic series, whatever the distance to the process count before it.  Built by all warps, each a chunk
+// of the intervals; a barrier of the caller's goes between the calls and one behind them.
+struct ChainTable {
+    double *ja, *before, *tot;  // [n_bp - 1][32], the same, [warps][32]; at the lane's column
+
+    __device__ __forceinline__ void build(const double *s_tab, int npad, int n_bp, double md, double j_max, int warp, int warps) const
+    {
+        const double inv_m = 1.0 / md, x_max = j_max * md;
+        const int n_int = n_bp - 1, i0 = n_int * warp / warps, i1 = n_int * (warp + 1) / warps;
+        auto first_j = [&](int i) {  // smallest j with j m >= key i; j_max + 1 when that lies behind j_max
+            const double key = s_tab[i];
+            const double q = round_whole(key * inv_m), j = fmax(fma(-q, md, key) > 0.0 ? q + 1.0 : q, 1.0);
+            return key > x_max ? j_max + 1.0 : j;
+        };
+        double j = first_j(i0), sum = warp == 0 ? (j - 1.0) * s_tab[npad] : 0.0;  // below the table
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i) {
+            const double jb = i + 1 < n_int ? first_j(i + 1) : j_max + 1.0;
+            ja[32 * i] = j;
+            before[32 * i] = sum;
+            sum = fma(jb - j, fma(0.5 * ((j + jb - 1.0) * md) - s_tab[i], s_tab[2 * npad + i], s_tab[npad + i]), sum);
+            j = jb;
+        }
+        tot[32 * warp] = sum;
+    }
+    __device__ __forceinline__ void add_up(int n_bp, int warp, int warps) const
+    {
+        const int n_int = n_bp - 1, i0 = n_int * warp / warps, i1 = n_int * (warp + 1) / warps;
+        double front = 0.0;
+        for (int w = 0; w < warp; ++w) front += tot[32 * w];
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i) before[32 * i] += front;
+    }
+};
+struct ChainAt {  // a lane's place in it; arguments never decrease
+    int i;
+    double key, next, slope, gap, ja, before;
+
+    __device__ __forceinline__ void start(const double *s_tab, int npad, const ChainTable &c, double x)
+    {
+        if (x < s_tab[0]) {
+            i = -1; key = 0.0; next = s_tab[0]; slope = 0.0; gap = s_tab[npad]; ja = 1.0; before = 0.0;
+        } else {
+            i = interval_of(s_tab, npad, x);
+            load(s_tab, npad, c);
+        }
+    }
+    __device__ __forceinline__ void load(const double *s_tab, int npad, const ChainTable &c)
+    {
+        key = s_tab[i]; next = s_tab[i + 1]; slope = s_tab[2 * npad + i]; gap = s_tab[npad + i];
+        ja = c.ja[32 * i]; before = c.before[32 * i];
+    }
+    __device__ __forceinline__ double sum(const double *s_tab, int npad, const ChainTable &c, double md, double j)
+    {
+        const double x = j * md;
+        if (x >= next) {
+            do { ++i; next = s_tab[i + 1]; } while (x >= next);
+            load(s_tab, npad, c);
+        }
+        return fma(j - ja + 1.0, fma(0.5 * ((ja + j) * md) - key, slope, gap), before);
+    }
+};
+
 // Lexicographic minimum of (t, e) over a warp (all lanes receive it), t >= 0 and e >= 0: three integer warp reductions,
 // of the high word, the low word where it ties, and e where both do.
 __device__ __forceinline__ void warp_min_pair(double &t, int &e)

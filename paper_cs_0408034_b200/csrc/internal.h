@@ -144,6 +144,7 @@ struct ScatterParams {
     TableDev T;
     GridDev G;
     int vec;  // message sizes per lane, 1 or 2 (2: n_m even and the outputs aligned for it)
+    int chain_table;  // listed process counts: sums per interval in shared memory (vec 1)
     int n_mtiles, n_ptiles, run_len;  // CTAs along m (32 vec sizes each) and along P (kWarps runs of run_len process counts each)
     int table0, n_tables_launch, out_table0;
     OutMap om;

@@ -1,6 +1,10 @@
 // scatter_block: one CTA of the Scatter half of the decision table (Table 2 of the paper: Flat Tree, Chain,
 // Binomial Tree; selection as in Sections 1 and 5).
 //
+// Listed process counts: the Chain's sum up to any j from a table of sums per interval in shared memory (ChainTable), with
+// no loop over the intervals between two process counts and no division per cell.  1000 tables of 50 sizes, 203 process
+// counts up to 3000, 101 message sizes: 124 -> 110 us (issue, 0.75 of the slots); the call 339 -> 324 us.
+//
 // Lanes are message sizes (32 V consecutive m per warp, V = 1 or 2 neighbours per lane, so every store is one aligned
 // row segment); each warp owns a contiguous run of process counts and walks it in ascending order, which turns
 // the Chain model's sum over j = 1..P-1 of g(j m) into a running sum along the thread: the argument
@@ -12,6 +16,8 @@
 #include "device_common.cuh"
 
 namespace plogp {
+
+constexpr int kChainRun = 0, kChainRange = 1, kChainTable = 2;
 
 namespace scatter {
 
@@ -33,15 +39,18 @@ template <> struct Out<2> {
 
 }  // namespace scatter
 
-// CONTIG: the process counts are the contiguous range P_lo + index (one new gap per step).
+// CHAIN, the Scatter Chain's sums: kChainRun for the contiguous range P_lo + index (one new gap per step), kChainTable for
+// listed process counts from a table of sums per interval (V = 1), kChainRange for them by closed forms along the run.
 // ALL: the three Scatter strategies are enabled (the usual case), known at compile time.
 // V: message sizes per lane.  W: warps of the CTA.
-template <bool CONTIG, bool ALL, int V, int W>
+template <int CHAIN, bool ALL, int V, int W>
 __device__ __forceinline__ void scatter_block(const ScatterParams &p, int block, unsigned char *smem_raw)
 {
     double *s_tab = reinterpret_cast<double *>(smem_raw);
     double *s_cum = s_tab + 3 * p.T.npad;          // [lc_max][32 V]
-    double *s_sum = s_cum + p.G.lc_max * 32 * V;   // [2][W][32 V]
+    double *s_sum = s_cum + p.G.lc_max * 32 * V;   // [2][W][32 V]; kChainTable: [W][32], then [2][n_bp - 1][32]
+    constexpr bool CONTIG = CHAIN == kChainRun;
+    static_assert(CHAIN != kChainTable || V == 1, "a column per lane");
     const int npad = p.T.npad;
     const uint32_t mask = p.G.mask;
     const bool on10 = ALL || ((mask >> 10) & 1u), on11 = ALL || ((mask >> 11) & 1u), on12 = ALL || ((mask >> 12) & 1u);
@@ -79,10 +88,13 @@ __device__ __forceinline__ void scatter_block(const ScatterParams &p, int block,
 
     // ---- Chain: the sum in front of the run ----
     ChainWalk walk[V];
+    const ChainTable ct{s_sum + W * 32 + (threadIdx.x & 31), s_sum + (W + p.T.n_bp - 1) * 32 + (threadIdx.x & 31), s_sum + (threadIdx.x & 31)};
+    ChainAt place;
     double run[V], j_last = 0.0;  // sum up to j_last
 #pragma unroll
     for (int v = 0; v < V; ++v) run[v] = 0.0;
-    if (on11) {
+    if (on11 && CHAIN == kChainTable) ct.build(s_tab, npad, p.T.n_bp, md[0], static_cast<double>(p.G.P_list[p.G.n_P - 1] - 1), warp, W);
+    if (on11 && CHAIN != kChainTable) {
 #pragma unroll
         for (int v = 0; v < V; ++v)
             chain_front_parts(s_tab, npad, p.T.n_bp, p.G.P_list, p.G.P_lo, md[v], c0, e0, e1, warp, W, s_sum + v * 32 + lane, s_sum + (W * V + v) * 32 + lane, 32 * V);
@@ -98,11 +110,13 @@ __device__ __forceinline__ void scatter_block(const ScatterParams &p, int block,
             }
         }
     }
-    if (on12) __syncthreads();
-    if (e0 >= e1 || !m_ok) return;  // no barriers below
+    if (on11 && CHAIN == kChainTable) ct.add_up(p.T.n_bp, warp, W);
+    if (on12 || (on11 && CHAIN == kChainTable)) __syncthreads();
+    if (e0 >= e1 || (CHAIN != kChainTable && !m_ok)) return;  // no barriers below; kChainTable shares process counts over the lanes
 
     int P = P_at(p.G, e0);
-    if (on11) {
+    if (on11 && CHAIN == kChainTable) place.start(s_tab, npad, ct, static_cast<double>(P - 1) * md[0]);
+    if (on11 && CHAIN != kChainTable) {
         j_last = warp == 0 ? static_cast<double>(P - 2) : static_cast<double>(P_at(p.G, e0 - 1) - 1);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -123,9 +137,15 @@ __device__ __forceinline__ void scatter_block(const ScatterParams &p, int block,
 #pragma unroll
     for (int v = 0; v < V; ++v) { s2[v] = 0.0; x[v] = pm1 * md[v]; }
 
+    int P_lane = P;  // kChainTable: 32 listed process counts, one per lane
     for (int e = e0; e < e1; ++e) {
         if (!CONTIG) {
-            P = P_at(p.G, e);
+            if (CHAIN == kChainTable) {
+                if (((e - e0) & 31) == 0) P_lane = p.G.P_list[min(e + lane, e1 - 1)];
+                P = __shfl_sync(0xffffffffu, P_lane, (e - e0) & 31);
+            } else {
+                P = P_at(p.G, e);
+            }
             pm1 = static_cast<double>(P - 1);
         }
         if (P >= P_next_lc) {  // P passed a power of two
@@ -146,6 +166,8 @@ __device__ __forceinline__ void scatter_block(const ScatterParams &p, int block,
                 if (CONTIG) {
                     run[v] += walk[v].at(s_tab, npad, x[v]);
                     x[v] += md[v];  // exact: j m < 2^53
+                } else if (CHAIN == kChainTable) {
+                    run[v] = place.sum(s_tab, npad, ct, md[v], pm1);
                 } else {
                     run[v] += walk[v].range(s_tab, npad, md[v], j_last + 1.0, pm1);
                 }
@@ -154,7 +176,7 @@ __device__ __forceinline__ void scatter_block(const ScatterParams &p, int block,
             }
             if (on12 && s2[v] < bt[v]) { bt[v] = s2[v]; bid[v] = id12; }  // Binomial Tree
         }
-        scatter::Out<V>::put(out_t, out_s, out_id, bt, bid);
+        if (CHAIN != kChainTable || m_ok) scatter::Out<V>::put(out_t, out_s, out_id, bt, bid);
         out_t += row; out_id += row; out_s += row;
         if (CONTIG) { ++P; pm1 += 1.0; }
         else j_last = pm1;

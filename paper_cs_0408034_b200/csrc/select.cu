@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) select_kernel(const SelectPara
         if (p.decide.rows == 8) decide_block<ENV, 8>(p.decide, blockIdx.x, smem_raw);
         else decide_block<ENV, 4>(p.decide, blockIdx.x, smem_raw);
     } else {
-        scatter_block<CONTIG, false, 1, kDecWarps>(p.scatter, blockIdx.x - p.n_decide, smem_raw);
+        scatter_block<CONTIG ? kChainRun : kChainRange, false, 1, kDecWarps>(p.scatter, blockIdx.x - p.n_decide, smem_raw);
     }
 }
 

@@ -169,3 +169,19 @@ def test_scatter_rows_off_the_sectors(plogp, n_m, n_P, n_tables, n_bp, listed, i
     with plogp.Tables.from_workload(w) as tabs:
         assert check_decision(w, ot, plogp.select_best(tabs, w), **sample) > 0
         assert check_prediction(w, ot, plogp.predict(tabs, w), **sample) > 0
+
+
+@pytest.mark.parametrize("n_bp,n_P,n_m,first,ids", [(2, 1, 33, 2, (10, 11, 12)), (3, 40, 5, 900, (11,)), (9, 33, 64, 2, (11, 12)), (96, 301, 97, 3, range(13)), (97, 301, 97, 3, range(13))])
+def test_listed_scatter_sums_by_interval(plogp, n_bp, n_P, n_m, first, ids):
+    """Sums per table interval for listed process counts: fewer intervals than warps, lists that start far from 2 and skip
+    intervals, arguments below and above the table, message sizes with idle lanes, the longest table that takes them."""
+    n = 1400 // n_m + 8
+    base = wl.config4(n_tables=n, P_hi=5000, n_m=n_m, n_s=3, seed_offset=n_bp)
+    sizes = wl.log_spaced_multiples(64, 64 << 20, n_bp)
+    gaps = np.stack([np.interp(sizes.astype(float), base.sizes.astype(float), g) for g in base.gaps])
+    P_list = np.unique(np.r_[first, first + np.rint(1.03 ** np.arange(n_P * 3)).astype(int)])[:n_P].astype(np.int32)
+    w = replace(base, sizes=sizes, gaps=gaps, strategy_mask=sum(1 << i for i in ids), P_list=P_list)
+    ot = oracle_tables(w)
+    with plogp.Tables.from_workload(w) as tabs:
+        plogp.profile_enable(tabs)  # two launches
+        assert check_decision(w, ot, plogp.select_best(tabs, w), tables=(0, 1, n - 1)) > 0
