@@ -116,7 +116,9 @@ typedef struct {
     uint32_t strategy_mask; /* bit i enables strategy id i */
     int32_t k_mode;         /* 0: k = ceil(m/s); 1: k = floor(m/s) */
     int32_t search_mode;    /* how the minimum over s of Section 3.1 is found; the results are the same:
-                               0: exhaustive, every (P, m, s) cell is evaluated (the default);
+                               0: exhaustive (the default): every (P, m, s) cell is bounded from below in FP32 and
+                                  compared in FP64 where the bound does not rule it out (ids 6 to 9 are evaluated
+                                  once per pair of floor(log2 P) and ceil(log2 P), on which alone they depend);
                                1: lower envelope: ids 2 and 9 take the s with the smallest g(s) k once per m, id 5
                                   walks the lower envelope of its lines in P (only for tables whose gaps never
                                   decrease with the size; other tables silently take the exhaustive search) */

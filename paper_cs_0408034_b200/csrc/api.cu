@@ -1,6 +1,6 @@
 // Host side of the C ABI declared in include/plogp.h: argument validation, table upload, the
 // launch plan for a grid (tiling, chunking of long candidate lists, scratch layout) and the
-// kernel launches.  Every step of the evaluation itself runs in kernels.cu.
+// kernel launches.  Every step of the evaluation itself runs on the device.
 #include "../../include/plogp.h"
 #include "internal.h"
 

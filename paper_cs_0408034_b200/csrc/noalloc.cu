@@ -1,7 +1,7 @@
 // plogp_scatter_chain_static: the Scatter Chain model (Table 2, second row) for callers that
-// cannot allocate device memory.  It is a self-contained variant of the reduce-then-scan that the
-// main path runs for this model; the per-tile partial sums, which the main path keeps in scratch
-// it allocates, live here in one fixed array that is part of the library image.
+// cannot allocate device memory.  It is a self-contained reduce-then-scan over the
+// terms (the main path takes the sums in front of a run in closed form inside its kernels); the per-tile partial sums live
+// in one fixed array that is part of the library image.
 //
 // The array is shared by every call on a device and keeps whatever the last call left in it.
 // Nothing in it has to start at zero: phase 1 writes every entry that phases 2 and 3 of the same
