@@ -588,11 +588,18 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             DecideParams dp{};
             dp.T = h->T; dp.G = pl.G;
             dp.G.mask &= 0x3FFu;
-            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.rows = pl.dec_rows; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs;
+            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.rows = pl.dec_rows; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs | 1;
             dp.table0 = t0; dp.n_tables_launch = nt; dp.out_table0 = out.out_table0; dp.om = out.om;
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
             dp.envelope = pl.envelope_short ? 1 : 0;
             dp.gaps = gaps; dp.gaps_stride = pl.gaps_stride;
+            // Five CTAs per SM instead of four where their shared memory fits (228 KB with 1 KB per CTA besides; 32 candidates
+            // over two tiles just do) and the grid has many of them: 4096 tables, P = 2..512, 128 m, 32 sizes 2.65 -> 2.53 ms,
+            // 2048 tables and 8 sizes 0.93 -> 0.90, 300 tables 224 -> 215 us.  Shorter grids wait for the last CTAs, which five
+            // on an SM make later (200 tables 150 -> 153 us, 64 tables 62 -> 65), and 96 registers alone are 1.5 % slower
+            // (64 sizes, which do not fit).
+            dp.ctas_per_sm = pl.dec_rows == 8 && 5 * (decide_smem_bytes(dp) + 1024) <= 228 * 1024 &&
+                             (long long)pl.dec_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * 16 ? 5 : 4;
             dp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
                          reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
             if (pl.select && !gaps && overlap) {

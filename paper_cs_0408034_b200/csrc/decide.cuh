@@ -56,17 +56,18 @@ struct DecSmem {
     uint32_t *sval;   // [256]: segment sizes by candidate index; [kCandNone] = 0
     uint16_t *code;   // [mg][slots]: id << 8 | candidate index
     uint8_t *pair, *pos;  // [n_p]: pair of a process count; [mg][pos_stride]: winners
-    int cap, cap_q, slots, pos_stride;
+    int cap, lines, cap_q, slots, pos_stride;
 };
 
 __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
-// Shared-memory layout.  cap: lines of one message size (a multiple of kStep); n_pairs: (floor, ceil) pairs of a CTA at most.
-// A slot number fits a byte: at most 144 lines and 61 pairs.
+// Shared-memory layout.  npad: 0 where the gap pre-pass has run; cap: the warps' lists of lines (a multiple of kStep); lines:
+// of one message size at most; n_pairs: (floor, ceil) pairs of a CTA at most.  A slot number fits a byte: at most 132 lines and
+// 61 pairs.
 __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int n_p, int mg, unsigned char *base, DecSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(2 * nsv + 4, kStep), cap_q = round_up(nsv, 4), slots = cap + n_pairs, pos_stride = n_p + 4;
+    const int lines = 2 * nsv + 4, cap = round_up(lines, kStep), cap_q = round_up(nsv, 4), slots = lines + n_pairs, pos_stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(mg * 8), o_pm = take(size_t(n_p) * 8), o_x = take(size_t(n_p) * 4),
@@ -81,7 +82,7 @@ __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int
         o->q = reinterpret_cast<double *>(base + o_q); o->fq = reinterpret_cast<float *>(base + o_fq); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
         o->code = reinterpret_cast<uint16_t *>(base + o_code); o->pair = base + o_pair; o->pos = base + o_pos;
         o->x = reinterpret_cast<float *>(base + o_x);
-        o->cap = cap; o->cap_q = cap_q; o->slots = slots; o->pos_stride = pos_stride;
+        o->cap = cap; o->lines = lines; o->cap_q = cap_q; o->slots = slots; o->pos_stride = pos_stride;
     }
     return off;
 }
@@ -100,7 +101,7 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
     DecSmem sm;
     constexpr int kTileP = 32 * R;
     const int n_p = p.tiles * kTileP;
-    dec_layout(npad, p.G.n_s, p.n_pairs, n_p, p.mg, smem_raw, &sm);
+    dec_layout(p.gaps ? 0 : npad, p.G.n_s, p.n_pairs, n_p, p.mg, smem_raw, &sm);
     const uint32_t mask = p.G.mask;
 
     int b = block;
@@ -333,8 +334,8 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
                 if (v <= t) { t = v; cd = idc(6) | kCandNone; }
             }
             if (pr < n_pairs) {
-                line[sm.cap + pr] = make_double2(0.0, t);
-                code[sm.cap + pr] = static_cast<uint16_t>(cd);
+                line[sm.lines + pr] = make_double2(0.0, t);
+                code[sm.lines + pr] = static_cast<uint16_t>(cd);
             }
         }
 
@@ -378,7 +379,7 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
                 if (any_log) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
-                        const unsigned slot = sm.cap + sm.pair[tile * kTileP + 32 * r + lane];
+                        const unsigned slot = sm.lines + sm.pair[tile * kTileP + 32 * r + lane];
                         const double tl = line[slot].y;
                         if (tl < t[r] || n1 == 0) { t[r] = tl; at[r] = slot; }  // lines have the lower ids
                     }

@@ -197,7 +197,9 @@ struct DecideParams {
     int mg;  // message sizes per CTA, 1..kDecMG
     int rows;     // process counts per lane and tile: 8 or 4
     int tiles;    // tiles of 32 x rows process counts per CTA
-    int n_pairs;  // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most
+    int n_pairs;  // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most, made odd: with an even number of
+                  // lines in front, neighbouring message sizes then start in different banks (an even one cost 6 % of a call)
+    int ctas_per_sm;  // 4 or 5
     int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cu)
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16 / 8 / 2-byte aligned bases)
     int table0, n_tables_launch;

@@ -185,3 +185,21 @@ def test_listed_scatter_sums_by_interval(plogp, n_bp, n_P, n_m, first, ids):
     with plogp.Tables.from_workload(w) as tabs:
         plogp.profile_enable(tabs)  # two launches
         assert check_decision(w, ot, plogp.select_best(tabs, w), tables=(0, 1, n - 1)) > 0
+
+
+@pytest.mark.parametrize("n_m,n_P,n_s,search", [(16, 257, 32, 0), (17, 300, 32, 1), (40, 250, 8, 0), (64, 520, 33, 0), (33, 700, 20, 1)])
+def test_decisions_on_many_tables(plogp, n_m, n_P, n_s, search):
+    """Grids of many CTAs (five per SM where their shared memory fits): the first and last table match the oracle, five
+    tables at either end a call over these alone (fewer CTAs per SM, other tiles), bit for bit in the Broadcast half."""
+    import torch
+    n = 2368 // max(1, n_m // 16) + 8
+    w = replace(wl.config4(n_tables=n, P_hi=n_P + 1, n_m=n_m, n_s=n_s, seed_offset=n_m), search_mode=search)
+    with plogp.Tables.from_workload(w) as tabs:
+        a = plogp.select_best(tabs, w)
+    assert check_decision(w, oracle_tables(w), a, tables=(0, n - 1), p_idx=np.unique(np.r_[0:n_P:7, n_P - 1])) > 0
+    for lo in (0, n - 5):
+        few = replace(w, gaps=np.ascontiguousarray(w.gaps[lo:lo + 5]), latency=w.latency[lo:lo + 5])
+        with plogp.Tables.from_workload(few) as tabs:
+            b = plogp.select_best(tabs, few)
+        for x, y in ((a.strategy, b.strategy), (a.s_bytes, b.s_bytes), (a.time, b.time)):
+            assert torch.equal(x[lo:lo + 5, 0], y[:, 0])
