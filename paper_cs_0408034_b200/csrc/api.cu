@@ -561,7 +561,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             // come from the lane<->P kernel; fused_kernel then writes the closed-form planes only.
             SegminParams sp{};
             sp.T = h->T; sp.G = pl.G;
-            sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs;
+            sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs | 1;
             sp.warps = kDecWarps;
             // Eight warps and 32 message sizes per CTA instead of four and 16 where rows are no multiple of a 32-byte sector, on
             // grids of many CTAs: a row segment of 16 message sizes then is two write requests instead of one, a segment of 32

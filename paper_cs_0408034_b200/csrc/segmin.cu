@@ -34,8 +34,8 @@ __host__ __device__ inline int round_up(int x, int a) { return (x + a - 1) / a *
 
 struct SegSmem {
     double *tab, *gs, *gm, *pm1;
-    double2 *l5;      // [mg][cap]: (B, C)
-    double *q;        // [mg][cap]: Q
+    double2 *l5;      // [mg][list]: (B, C)
+    double *q;        // [mg][list]: Q
     double *t9;       // [mg][n_pairs]: id 9's minimum
     float *x;         // [n_p]: P-1 rounded down
     float *fb, *fc, *fq;  // [warps][cap]: the lists of the warp's current message size rounded down, without the pilots
@@ -43,17 +43,17 @@ struct SegSmem {
     uint8_t *i9;      // [mg][n_pairs]: id 9's winner
     uint8_t *pair;    // [n_p]: pair of a process count
     uint8_t *pos2, *pos5;  // [mg][stride]: winners of ids 2 and 5
-    int cap, stride;
+    int cap, list, stride;  // list: odd, so that neighbouring message sizes start in different banks
 };
 
 __host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int n_p, int mg, int warps, unsigned char *base, SegSmem *o)
 {
     const int nsv = n_s > 0 ? n_s : 1;
-    const int cap = round_up(nsv, kStep), stride = n_p + 4;
+    const int cap = round_up(nsv, kStep), list = nsv | 1, stride = n_p + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off += (bytes + 15) & ~size_t(15); return at; };
     const size_t o_tab = take(3 * size_t(npad) * 8), o_gs = take(size_t(nsv) * 8), o_gm = take(mg * 8), o_pm = take(size_t(n_p) * 8),
-                 o_l5 = take(size_t(mg) * cap * 16), o_q = take(size_t(mg) * cap * 8), o_t9 = take(size_t(mg) * n_pairs * 8),
+                 o_l5 = take(size_t(mg) * list * 16), o_q = take(size_t(mg) * list * 8), o_t9 = take(size_t(mg) * n_pairs * 8),
                  o_x = take(size_t(n_p) * 4), o_fb = take(size_t(warps) * cap * 4), o_fc = take(size_t(warps) * cap * 4),
                  o_fq = take(size_t(warps) * cap * 4), o_sv = take(size_t(nsv) * 4), o_i9 = take(size_t(mg) * n_pairs), o_pair = take(n_p),
                  o_p2 = take(size_t(mg) * stride), o_p5 = take(size_t(mg) * stride);
@@ -65,7 +65,7 @@ __host__ __device__ inline size_t seg_layout(int npad, int n_s, int n_pairs, int
         o->fb = reinterpret_cast<float *>(base + o_fb); o->fc = reinterpret_cast<float *>(base + o_fc);
         o->fq = reinterpret_cast<float *>(base + o_fq); o->sval = reinterpret_cast<uint32_t *>(base + o_sv);
         o->i9 = base + o_i9; o->pair = base + o_pair; o->pos2 = base + o_p2; o->pos5 = base + o_p5;
-        o->cap = cap; o->stride = stride;
+        o->cap = cap; o->list = list; o->stride = stride;
     }
     return off;
 }
@@ -153,8 +153,8 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 5 : 2) segmin_kernel(const Se
         const int nsv = max(ns, 1);  // candidates actually evaluated (none fits: the whole message, k = 1)
         const int np4 = round_up(nsv, 4), np16 = round_up(nsv, kStep);
         const double gm = sm.gm[mi];
-        double *const q = sm.q + mi * sm.cap;
-        double2 *const l5 = sm.l5 + mi * sm.cap;
+        double *const q = sm.q + mi * sm.list;
+        double2 *const l5 = sm.l5 + mi * sm.list;
 
         // ---- the lists (lanes <-> candidates) and the pilots: bound (without its last 8 bits) and index in one number ----
         __syncwarp();  // the previous message size's sweeps are done with the lists
@@ -353,8 +353,8 @@ __global__ void __launch_bounds__(32 * W, W == 4 ? 5 : 2) segmin_kernel(const Se
                 return sm.t9[i];
             }
             at = pos[mi * sm.stride + pr];
-            if (w == 0) return fma(x, sm.q[mi * sm.cap + at], L);
-            const double2 e = sm.l5[mi * sm.cap + at];
+            if (w == 0) return fma(x, sm.q[mi * sm.list + at], L);
+            const double2 e = sm.l5[mi * sm.list + at];
             return fma(x, e.x, e.y);
         };
         if (p.vec_out) {
