@@ -72,6 +72,7 @@ struct Plan {
     bool select = false;
     int sel_ptiles = 1, sel_run = 1;
     // decision kernel tiling (short candidate lists)
+    int bc_mg = kDecMG, bc_mgroups = 0;  // message sizes per CTA of the decision kernel
     int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_rows = 8, dec_tiles = 1, dec_pairs = 1;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
@@ -343,9 +344,18 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
             }
         }
     }
+    // The decision kernel's CTAs of 16 message sizes and two tiles are long: with few of them per SM, some SMs have one more than
+    // others and all end together.  Half as many message sizes then: P = 2..511, 128 m, 32 sizes: 64 tables (3.5 per SM) 64 -> 58
+    // us, 100 (5.4) 91 -> 81; 48 tables of 100 m (2.3) 54 -> 42; 200 (10.8) 147 -> 148.
+    pl.bc_mg = pl.dec_mg;
+    if (pl.dec_mg == kDecMG && pl.dec_rows == 8 && pl.dec_tiles == 2 && n_m > kDecMG / 2) {
+        const long long ctas = (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables;
+        if (ctas > (long long)h->sm_count * 2 && ctas < (long long)h->sm_count * 8) pl.bc_mg = kDecMG / 2;
+    }
+    pl.bc_mgroups = (n_m + pl.bc_mg - 1) / pl.bc_mg;
     // One launch for both halves where the GPU holds all their CTAs at once (four per SM; its Scatter CTAs have four warps)
     {
-        const long long decide = (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
+        const long long decide = (long long)pl.bc_mgroups * pl.dec_ptiles * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
         const long long room = (long long)h->sm_count * 4 - decide;
         pl.select = room >= base && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
         if (pl.select) {
@@ -588,7 +598,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             DecideParams dp{};
             dp.T = h->T; dp.G = pl.G;
             dp.G.mask &= 0x3FFu;
-            dp.n_mgroups = pl.dec_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.dec_mg; dp.rows = pl.dec_rows; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs | 1;
+            dp.n_mgroups = pl.bc_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.bc_mg; dp.rows = pl.dec_rows; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs | 1;
             dp.table0 = t0; dp.n_tables_launch = nt; dp.out_table0 = out.out_table0; dp.om = out.om;
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
             dp.envelope = pl.envelope_short ? 1 : 0;
@@ -597,10 +607,10 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             // over two tiles just do) and the grid has many of them: 4096 tables, P = 2..512, 128 m, 32 sizes 2.65 -> 2.53 ms,
             // 2048 tables and 8 sizes 0.93 -> 0.90, 300 tables 224 -> 215 us.  Shorter grids wait for the last CTAs, which five
             // on an SM make later (200 tables 150 -> 153 us, 64 tables 62 -> 65), and 96 registers alone are 1.5 % slower
-            // (64 sizes, which do not fit).
+            // (64 sizes, which do not fit).  CTAs of fewer message sizes are short enough from 4 per SM on (100 tables 83 -> 81 us).
             dp.ctas_per_sm = pl.dec_rows == 8 && 5 * (decide_smem_bytes(dp) + 1024) <= 228 * 1024 &&
-                             (long long)pl.dec_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * 16 ? 5 : 4;
-            dp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
+                             (long long)pl.bc_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * (pl.bc_mg == kDecMG ? 16 : 4) ? 5 : 4;
+            dp.vec_out = (pl.G.n_m % 2 == 0) && pl.bc_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
                          reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
             if (pl.select && !gaps && overlap) {
                 SelectParams sl{};

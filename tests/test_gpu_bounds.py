@@ -203,3 +203,12 @@ def test_decisions_on_many_tables(plogp, n_m, n_P, n_s, search):
             b = plogp.select_best(tabs, few)
         for x, y in ((a.strategy, b.strategy), (a.s_bytes, b.s_bytes), (a.time, b.time)):
             assert torch.equal(x[lo:lo + 5, 0], y[:, 0])
+
+
+@pytest.mark.parametrize("n_tables,n_m,n_P,search", [(100, 33, 512, 0), (110, 56, 300, 1), (40, 129, 700, 0)])
+def test_decisions_on_a_few_ctas_per_sm(plogp, n_tables, n_m, n_P, search):
+    """Grids on which the decision kernel takes 8 message sizes per CTA instead of 16, the last group ragged."""
+    w = replace(wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=24, seed_offset=n_m), search_mode=search)
+    with plogp.Tables.from_workload(w) as tabs:
+        a = plogp.select_best(tabs, w)
+    assert check_decision(w, oracle_tables(w), a, tables=(0, n_tables - 1), p_idx=np.unique(np.r_[0:n_P:5, n_P - 1])) > 0
