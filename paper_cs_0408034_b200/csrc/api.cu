@@ -72,7 +72,7 @@ struct Plan {
     bool select = false;
     int sel_ptiles = 1, sel_run = 1;
     // decision kernel tiling (short candidate lists)
-    int bc_mg = kDecMG, bc_mgroups = 0;  // message sizes per CTA of the decision kernel
+    int bc_mg = kDecMG, bc_mgroups = 0;  // message sizes per CTA of decide_kernel and segmin_kernel as launched
     int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_rows = 8, dec_tiles = 1, dec_pairs = 1;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
@@ -344,9 +344,10 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
             }
         }
     }
-    // The decision kernel's CTAs of 16 message sizes and two tiles are long: with few of them per SM, some SMs have one more than
+    // The lane <-> P kernels' CTAs of 16 message sizes and two tiles are long: with few of them per SM, some SMs have one more than
     // others and all end together.  Half as many message sizes then: P = 2..511, 128 m, 32 sizes: 64 tables (3.5 per SM) 64 -> 58
     // us, 100 (5.4) 91 -> 81; 48 tables of 100 m (2.3) 54 -> 42; 200 (10.8) 147 -> 148.
+    // Predictions, which wait for memory besides: 48 tables of 100 m 101 -> 94 us, 140 of 128 238 -> 236.
     pl.bc_mg = pl.dec_mg;
     if (pl.dec_mg == kDecMG && pl.dec_rows == 8 && pl.dec_tiles == 2 && n_m > kDecMG / 2) {
         const long long ctas = (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables;
@@ -571,13 +572,13 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             // come from the lane<->P kernel; fused_kernel then writes the closed-form planes only.
             SegminParams sp{};
             sp.T = h->T; sp.G = pl.G;
-            sp.n_mgroups = pl.dec_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.dec_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs | 1;
+            sp.n_mgroups = pl.bc_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.bc_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs | 1;
             sp.warps = kDecWarps;
             // Eight warps and 32 message sizes per CTA instead of four and 16 where rows are no multiple of a 32-byte sector, on
             // grids of many CTAs: a row segment of 16 message sizes then is two write requests instead of one, a segment of 32
             // three instead of two, each with part of a sector at either end (1024 tables, P = 2..513, 32 sizes, 16 -> 32: n_m =
             // 127 1.70 -> 1.36 ms, 130 1.65 -> 1.33, 145 1.96 -> 1.51).  Whole sectors gain nothing (132: 1.17 -> 1.19 ms).
-            if (pl.G.n_m % 4 != 0 && pl.dec_mg == kDecMG && pl.dec_rows == 8 &&
+            if (pl.G.n_m % 4 != 0 && pl.bc_mg == kDecMG && pl.dec_rows == 8 &&
                 (long long)pl.dec_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * 16) {
                 sp.warps = 2 * kDecWarps; sp.mg = 2 * kDecMG;
                 sp.n_mgroups = (pl.G.n_m + sp.mg - 1) / sp.mg;
@@ -585,7 +586,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             sp.table0 = t0; sp.n_tables_launch = nt; sp.out_table0 = out.out_table0;
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
             sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;
-            sp.vec_out = (pl.G.n_m % 2 == 0) && pl.dec_mg >= 2 && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
+            sp.vec_out = (pl.G.n_m % 2 == 0) && pl.bc_mg >= 2 && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
                          (!out.p_best_s || reinterpret_cast<uintptr_t>(out.p_best_s) % 8 == 0);
             { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, overlap && gaps, st)); }
             g_launches += 1;

@@ -207,8 +207,9 @@ def test_decisions_on_many_tables(plogp, n_m, n_P, n_s, search):
 
 @pytest.mark.parametrize("n_tables,n_m,n_P,search", [(100, 33, 512, 0), (110, 56, 300, 1), (40, 129, 700, 0)])
 def test_decisions_on_a_few_ctas_per_sm(plogp, n_tables, n_m, n_P, search):
-    """Grids on which the decision kernel takes 8 message sizes per CTA instead of 16, the last group ragged."""
+    """Grids on which the lane <-> P kernels take 8 message sizes per CTA instead of 16, the last group ragged."""
     w = replace(wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=24, seed_offset=n_m), search_mode=search)
     with plogp.Tables.from_workload(w) as tabs:
-        a = plogp.select_best(tabs, w)
-    assert check_decision(w, oracle_tables(w), a, tables=(0, n_tables - 1), p_idx=np.unique(np.r_[0:n_P:5, n_P - 1])) > 0
+        a, b = plogp.select_best(tabs, w), plogp.predict(tabs, w)
+    ot, sample = oracle_tables(w), dict(tables=(0, n_tables - 1), p_idx=np.unique(np.r_[0:n_P:5, n_P - 1]))
+    assert check_decision(w, ot, a, **sample) + check_prediction(w, ot, b, **sample) > 0
