@@ -15,7 +15,7 @@
 //                  the predicted planes or the decision table.  The general path.
 // Short candidate lists have faster, specialised kernels: decide.cu (Broadcast half of the decision
 // table), scatter.cu (Scatter half), segmin.cu (segmented planes of the predictions); the host routes
-// them there, and fused_kernel writes the closed-form planes only.
+// them there, and fused_kernel writes the closed-form planes only.  Rows off the sectors on large grids go to planes.cu and rows.cu.
 #include "device_common.cuh"
 
 namespace plogp {
