@@ -604,13 +604,6 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
             dp.envelope = pl.envelope_short ? 1 : 0;
             dp.gaps = gaps; dp.gaps_stride = pl.gaps_stride;
-            // Five CTAs per SM instead of four where their shared memory fits (228 KB with 1 KB per CTA besides; 32 candidates
-            // over two tiles just do) and the grid has many of them: 4096 tables, P = 2..512, 128 m, 32 sizes 2.65 -> 2.53 ms,
-            // 2048 tables and 8 sizes 0.93 -> 0.90, 300 tables 224 -> 215 us.  Shorter grids wait for the last CTAs, which five
-            // on an SM make later (200 tables 150 -> 153 us, 64 tables 62 -> 65), and 96 registers alone are 1.5 % slower
-            // (64 sizes, which do not fit).  CTAs of fewer message sizes are short enough from 4 per SM on (100 tables 83 -> 81 us).
-            dp.ctas_per_sm = pl.dec_rows == 8 && 5 * (decide_smem_bytes(dp) + 1024) <= 228 * 1024 &&
-                             (long long)pl.bc_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * (pl.bc_mg == kDecMG ? 16 : 4) ? 5 : 4;
             dp.vec_out = (pl.G.n_m % 2 == 0) && pl.bc_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
                          reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
             if (pl.select && !gaps && overlap) {
@@ -625,6 +618,19 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
                 g_launches += 1;
                 continue;
             }
+            // Long lists: three CTAs of 16 message sizes are less than four or five of 8 (2048 tables, P = 2..513, 128 m: 64 sizes
+            // 2.08 -> 1.89 ms; 45 sizes, of which four fit, 1.56 either way).
+            if (dp.mg == kDecMG && 4 * (decide_smem_bytes(dp) + 1024) > 228 * 1024) {
+                dp.mg = kDecMG / 2;
+                dp.n_mgroups = (pl.G.n_m + dp.mg - 1) / dp.mg;
+            }
+            // Five CTAs per SM instead of four where their shared memory fits (228 KB with 1 KB per CTA besides; 32 candidates
+            // over two tiles just do) and the grid has many of them: 4096 tables, P = 2..512, 128 m, 32 sizes 2.65 -> 2.53 ms,
+            // 2048 tables and 8 sizes 0.93 -> 0.90, 300 tables 224 -> 215 us.  Shorter grids wait for the last CTAs, which five
+            // on an SM make later (200 tables 150 -> 153 us, 64 tables 62 -> 65), and 96 registers alone are 1.5 % slower
+            // (64 sizes, which do not fit).  CTAs of fewer message sizes are short enough from 4 per SM on (100 tables 83 -> 81 us).
+            dp.ctas_per_sm = pl.dec_rows == 8 && 5 * (decide_smem_bytes(dp) + 1024) <= 228 * 1024 &&
+                             (long long)dp.n_mgroups * dp.n_ptiles * nt >= (long long)h->sm_count * (dp.mg == kDecMG ? 16 : 4) ? 5 : 4;
             { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= 0x1C00u;

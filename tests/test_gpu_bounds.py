@@ -187,7 +187,7 @@ def test_listed_scatter_sums_by_interval(plogp, n_bp, n_P, n_m, first, ids):
         assert check_decision(w, ot, plogp.select_best(tabs, w), tables=(0, 1, n - 1)) > 0
 
 
-@pytest.mark.parametrize("n_m,n_P,n_s,search", [(16, 257, 32, 0), (17, 300, 32, 1), (40, 250, 8, 0), (64, 520, 33, 0), (33, 700, 20, 1)])
+@pytest.mark.parametrize("n_m,n_P,n_s,search", [(16, 257, 32, 0), (17, 300, 32, 1), (40, 250, 8, 0), (64, 520, 33, 0), (33, 700, 20, 1), (41, 512, 64, 0), (24, 512, 57, 1)])
 def test_decisions_on_many_tables(plogp, n_m, n_P, n_s, search):
     """Grids of many CTAs (five per SM where their shared memory fits): the first and last table match the oracle, five
     tables at either end a call over these alone (fewer CTAs per SM, other tiles), bit for bit in the Broadcast half."""
