@@ -216,6 +216,22 @@ int validate_grid(const plogp_tables *h, const plogp_grid *g, int64_t *n_s_out)
     return PLOGP_OK;
 }
 
+// Grows the handle's scratch to what a plan needs.  Asked for by every call that launches kernels on it, with a kept plan too:
+// a growth that fails for one grid leaves the handle without scratch for all of them.
+int ensure_scratch(plogp_tables *h, size_t bytes)
+{
+    if (bytes <= h->ws_cap) return PLOGP_OK;
+    if (h->d_ws) CK(cudaFree(h->d_ws));
+    h->d_ws = nullptr;
+    h->ws_cap = 0;
+    cudaError_t e = cudaMalloc(&h->d_ws, bytes);
+    if (e != cudaSuccess) h->d_ws = nullptr;
+    if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return PLOGP_E_NOMEM; }
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(scratch)");
+    h->ws_cap = bytes;
+    return PLOGP_OK;
+}
+
 // Finds or builds the launch plan of a grid; *out is valid until the next call.
 int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **out)
 {
@@ -483,16 +499,8 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
         pl.tables_per_batch = int(std::max<size_t>(1, kSweepScratchLimit / per_table));
     pl.tables_per_batch = std::min(pl.tables_per_batch, 65535);
     pl.scratch_bytes = per_table ? per_table * pl.tables_per_batch + 1024 : 0;  // the sections start on 256-byte boundaries
-    if (pl.scratch_bytes > h->ws_cap) {
-        if (h->d_ws) CK(cudaFree(h->d_ws));
-        h->d_ws = nullptr;
-        h->ws_cap = 0;
-        cudaError_t e = cudaMalloc(&h->d_ws, pl.scratch_bytes);
-        if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return PLOGP_E_NOMEM; }
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(scratch)");
-        h->ws_cap = pl.scratch_bytes;
-    }
-    return keep();
+    rc = ensure_scratch(h, pl.scratch_bytes);
+    return rc == PLOGP_OK ? keep() : rc;
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -512,10 +520,12 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
     CK(cudaGetDevice(&dev));
     if (dev != h->device) return PLOGP_E_INVAL;
     const Plan *plan = nullptr;
-    const int rc = prepare(h, g, st, &plan);
+    int rc = prepare(h, g, st, &plan);
     if (rc != PLOGP_OK) return rc;
     const Plan &pl = *plan;
     if (pl.empty) return PLOGP_OK;
+    rc = ensure_scratch(h, pl.scratch_bytes);
+    if (rc != PLOGP_OK) return rc;
     // Short candidate lists with segmented strategies: the lane<->P decision kernel; everything else
     // (predictions, long lists reduced by the sweep kernel, Scatter-only grids) goes through fused_kernel.
     const bool use_decide = !predict && pl.inline_sweep && pl.n_seg > 0;

@@ -1,0 +1,74 @@
+"""csrc/api.cu against a CUDA runtime made of host memory (fake_cuda.cpp): what the calls do when memory runs out."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_cs_0408034_b200 import plogp
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+OUT = C.c_void_p(1 << 20)  # outputs are passed on to the kernels, which the fake ones leave alone
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "libplogp_fake.so")
+    csrc = os.path.join(ROOT, "paper_cs_0408034_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I/usr/local/cuda/include", "-x", "c++",
+                    os.path.join(csrc, "api.cu"), os.path.join(ROOT, "tests", "fake_cuda.cpp"), "-o", so], check=True)
+    lib = C.CDLL(so)
+    lib.plogp_table_load.argtypes = [C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+    lib.plogp_select_best.argtypes = [C.c_void_p] * 6
+    lib.plogp_predict.argtypes = [C.c_void_p] * 5
+    lib.plogp_select_best_collective.argtypes = [C.c_void_p, C.c_void_p, C.c_int] + [C.c_void_p] * 4
+    lib.plogp_table_free.argtypes = [C.c_void_p]
+    lib.fake_refuse_from.argtypes = [C.c_longlong]
+    for f in ("fake_bad_accesses", "fake_launches", "fake_live_bytes"):
+        getattr(lib, f).restype = C.c_longlong
+    return lib
+
+
+def load(lib, n_tables):
+    sizes = np.array([4, 1024, 1 << 20], dtype=np.uint64)
+    gaps = np.ascontiguousarray(np.tile([1.0, 2.0, 900.0], (n_tables, 1)))
+    h = C.c_void_p()
+    lat = np.full(n_tables, 5.0)
+    assert lib.plogp_table_load(n_tables, 3, sizes.ctypes.data, 1, gaps.ctypes.data, lat.ctypes.data, C.byref(h)) == plogp.OK
+    return h
+
+
+def long_list(P_hi, n_m, **kw):
+    return plogp.GridArgs(np.arange(1, n_m + 1) * 65536, None, 2, P_hi, None, s_lo=4, s_hi=4096, s_step=4, **kw)
+
+
+@pytest.mark.parametrize("kind", ["sweep", "envelope", "gaps", "predict"])
+def test_scratch_that_does_not_grow_leaves_no_call_without_it(lib, kind):
+    """A grid whose scratch is refused: its call says so, and a call on a grid that the handle has kept a plan for either
+    gets scratch of its own or says so too, before any kernel is launched."""
+    short = plogp.GridArgs(np.arange(1, 129) * 4096, None, 2, 700, np.array([64, 256, 1024, 4096]))
+    small = short if kind in ("gaps", "predict") else long_list(40, 3, search_mode=int(kind == "envelope"))
+    large = long_list(3000, 60)
+    h = load(lib, 300)
+
+    def call():
+        if kind == "predict":
+            return lib.plogp_predict(h, small.ref, OUT, None, None)
+        return lib.plogp_select_best(h, small.ref, OUT, OUT, OUT, None)
+
+    try:
+        assert call() == plogp.OK
+        for refused_too in (False, True):
+            lib.fake_refuse_from((64 << 10) if refused_too else (64 << 20))
+            assert lib.plogp_select_best(h, large.ref, OUT, OUT, OUT, None) == plogp.E_NOMEM
+            n = lib.fake_launches()
+            assert call() == (plogp.E_NOMEM if refused_too else plogp.OK)
+            assert lib.fake_bad_accesses() == 0 and (lib.fake_launches() == n) == refused_too
+            lib.fake_refuse_from(-1)
+            assert call() == plogp.OK and lib.fake_bad_accesses() == 0
+        assert lib.plogp_select_best(h, large.ref, OUT, OUT, OUT, None) == plogp.OK and lib.fake_bad_accesses() == 0
+    finally:
+        lib.fake_refuse_from(-1)
+        lib.plogp_table_free(h)
+    assert lib.fake_live_bytes() == 0
