@@ -215,10 +215,11 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
                 if (c >= ns) break;
                 const double gsv = sm.gs[c], k = k_of[h];
                 const double Q = gsv * k, B = gsv + L, C = gsv * (k - 1.0);
-                if (Q < qb) { qb = Q; qc = c; }
-                const double t1 = fma(x_first, B, C), t2 = fma(x_last, B, C);
-                if (t1 < tf) { tf = t1; ef = c; }
-                if (t2 < tl) { tl = t2; el = c; }
+                // a lane's first candidate always counts, and inf * 0 as inf: where times overflow, the indices are still candidates
+                if (h == 0 || Q < qb) { qb = Q; qc = c; }
+                const double t1 = fmin(fma(x_first, B, C), CUDART_INF), t2 = fmin(fma(x_last, B, C), CUDART_INF);
+                if (h == 0 || t1 < tf) { tf = t1; ef = c; }
+                if (h == 0 || t2 < tl) { tl = t2; el = c; }
             }
             warp_min_pair(qb, qc);
             warp_min_pair(tf, ef);
