@@ -35,7 +35,9 @@
  *   - candidate segment sizes for a message m are the grid values s <= m; if none fits, the
  *     message is sent whole (s = m, k = 1) and best_s reports m.
  *   - ties: the smallest segment size, then the lowest strategy id.  (With search_mode 1 two segment sizes of
- *     ids 2 / 9 whose g(s) k differ but whose predicted times round to the same double may resolve to either.)
+ *     ids 2 / 9 whose g(s) k differ but whose predicted times round to the same double may resolve to either, and
+ *     among segment sizes of id 5 with the same k the smallest is taken, also where rounding makes the interpolated
+ *     g a last bit smaller at a larger one.)
  *
  * Threading: calls on one plogp_tables handle must not overlap in time on the host, and their
  * device work must be ordered (use one stream, or order the streams yourself): a handle owns

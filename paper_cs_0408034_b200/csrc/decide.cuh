@@ -200,33 +200,39 @@ __device__ __forceinline__ void decide_block(const DecideParams &p, int block, u
         uint16_t *const code = sm.code + mi * sm.slots;
         // Lower-envelope search (p.envelope, tables whose gaps never decrease): ids 2 and 9 keep only the candidate
         // with the smallest g(s) k (their minimum over s for every P at once, a rounded fused multiply-add being
-        // monotone in it), id 5 only the candidates between its winners at the tile's last and first process
-        // count, one more on each side (the lines are sorted by slope g(s) + L, so the winner's index does not
-        // grow with P).  Otherwise every candidate enters the lists.
+        // monotone in it), id 5 only the candidates between its best ones at the tile's last and first process
+        // count (envelope_near, device_common.cuh).  Otherwise every candidate enters the lists.
         const bool env = ENV && ns > 0;
         int q_c = 0, lo5 = 0, n5 = nsv;
         if constexpr (ENV) if (env) {
             const double x_first = sm.pm1[0], x_last = sm.pm1[n_valid - 1];
-            double qb = CUDART_INF, tf = CUDART_INF, tl = CUDART_INF;
-            int qc = kIntMax, ef = kIntMax, el = kIntMax;
+            double qb = CUDART_INF, t1[2] = {CUDART_INF, CUDART_INF}, t2[2] = {CUDART_INF, CUDART_INF};
+            int qc = kIntMax;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int c = lane + 32 * h;
                 if (c >= ns) break;
                 const double gsv = sm.gs[c], k = k_of[h];
                 const double Q = gsv * k, B = gsv + L, C = gsv * (k - 1.0);
-                // a lane's first candidate always counts, and inf * 0 as inf: where times overflow, the indices are still candidates
+                // a lane's first candidate always counts, and inf * 0 as inf: where times overflow, the index is still a candidate's
                 if (h == 0 || Q < qb) { qb = Q; qc = c; }
-                const double t1 = fmin(fma(x_first, B, C), CUDART_INF), t2 = fmin(fma(x_last, B, C), CUDART_INF);
-                if (h == 0 || t1 < tf) { tf = t1; ef = c; }
-                if (h == 0 || t2 < tl) { tl = t2; el = c; }
+                t1[h] = fmin(fma(x_first, B, C), CUDART_INF);
+                t2[h] = fmin(fma(x_last, B, C), CUDART_INF);
             }
             warp_min_pair(qb, qc);
-            warp_min_pair(tf, ef);
-            warp_min_pair(tl, el);
             q_c = qc;
-            lo5 = max(min(ef, el) - 1, 0);
-            n5 = min(max(ef, el) + 1, ns - 1) - lo5 + 1;
+            const double m1 = warp_min(fmin(t1[0], t1[1])), m2 = warp_min(fmin(t2[0], t2[1]));
+            const double r = static_cast<double>(__fdividef(sm.x[n_valid - 1], sm.x[0]));  // to 1e-6: envelope_near has a third to spare
+            const double up_to1 = fma(m1, envelope_near(r), m1), up_to2 = fma(m2, envelope_near(1.0), m2);
+            int lo = kIntMax, hi = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = lane + 32 * h;
+                if (c < ns && t2[h] <= up_to2) lo = min(lo, c);
+                if (c < ns && t1[h] <= up_to1) hi = c;
+            }
+            lo5 = __reduce_min_sync(kFull, lo);
+            n5 = __reduce_max_sync(kFull, hi) - lo5 + 1;
         }
         const int nq = env ? 1 : nsv;  // entries of ids 2 and 9
         const int o2 = n01, o3 = o2 + (has2 ? nq : 0), o5 = o3 + n34, n1 = o5 + (has5 ? n5 : 0);

@@ -321,5 +321,20 @@ __device__ __forceinline__ void warp_min_pair(double &t, int &e)
     e = __reduce_min_sync(0xffffffffu, on_h && static_cast<unsigned>(__double2loint(t)) == l ? e : 0x7fffffff);
     t = __hiloint2double(h, static_cast<int>(l));
 }
+__device__ __forceinline__ double warp_min(double t)  // t >= 0
+{
+    const int h = __reduce_min_sync(0xffffffffu, __double2hiint(t));
+    return __hiloint2double(h, static_cast<int>(__reduce_min_sync(0xffffffffu, __double2hiint(t) == h ? static_cast<unsigned>(__double2loint(t)) : 0xffffffffu)));
+}
+
+// The lower envelope of the lines t_e(x) = fma(x, B_e, C_e) of the Segmented Chain, slopes ascending with the candidate e: the
+// best line's index does not grow with x.  For the computed, rounded times that holds up to lines that differ by rounding,
+// which may be any number of entries apart (a latency far above the gaps makes almost all slopes equal).  With u = 2^-53:
+// slopes ascend up to 5 u (g is interpolated), a time is off by u.  An entry below every one whose time at x2 is within
+// (1 + e) of the best there loses at all x <= x2 if e > 12 u: its distance does not shrink towards smaller x.  One above
+// every such entry at x1 loses at all x in x1 .. r x1 if e > 4 u + 8 u r: its distance does not shrink, the best time grows by r
+// at most.  So the winners between x1 and x2 lie between the smallest entry within envelope_near at x2 and the largest within
+// envelope_near(x2 / x1) at x1.
+__device__ __forceinline__ double envelope_near(double r) { return 0x1p-49 * r; }
 
 }  // namespace plogp

@@ -11,16 +11,16 @@
 //   * among candidates with the same segment count k the smallest s has the smallest B and C, so
 //     only the first candidate of every run of equal k can ever win (its "representative"), for id 5 as for ids 2 and 9;
 //   * the representatives are sorted by slope B, hence the index of the winner does not grow with P:
-//     the winners at two process counts bracket the winners at all counts in between.
+//     the winners at two process counts bracket the winners at all counts in between.  Rounded times keep that up to lines
+//     that differ by rounding, so a bracket ends where times are further off than that (envelope_near, device_common.cuh).
 // Where the candidates are equally spaced the representatives are found without visiting the others: below
 // s = sqrt(m step) almost every candidate has a segment count of its own and is looked at, above it the counts are few
 // and the first candidate of each is computed (4096 instead of 262144 candidates for m = 16 MB and every multiple of
 // 4 B up to 1 MB: 298 -> 22 us for 128 message sizes).
-// The kernel therefore (A) lists the representatives in shared memory, (B) finds the winners at a sequence of coarse
-// process-count indices (all of the first 16, then ever wider apart up to `2 << coarse_log`: the winner moves fastest
+// The kernel therefore (A) lists the representatives in shared memory, (B) finds the range of the best entries at a sequence of
+// coarse process-count indices (all of the first 16, then ever wider apart up to `2 << coarse_log`: the winner moves fastest
 // where P is small), every eighth over the whole list, the others between those, and (C) searches, for each
-// process count, only the bracket given by its two coarse neighbours (widened by one entry on each side, which absorbs a
-// winner that rounding moved across a bracket end).  All comparisons are the exact ones of the
+// process count, only the bracket given by its two coarse neighbours.  All comparisons are the exact ones of the
 // exhaustive search: (time, s) in lexicographic order.
 //
 // One CTA per (table, m).  Results go to the scratch layout that the sweep kernel uses, one row per
@@ -32,6 +32,7 @@ namespace plogp {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int kPad = 128;  // entries behind the list of representatives that never win
 
 // coarse number c <-> process-count index: 0..15, then runs of 8 with distances 2, 4, 8, .. up to 2 << g_max, which stays
 __device__ __forceinline__ int coarse_index(int c, int g_max)
@@ -56,13 +57,12 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int npad = p.T.npad, T = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = T >> 5;
     double *s_tab = reinterpret_cast<double *>(smem_raw);
-    double *s_B = s_tab + 3 * npad;                                   // [rep_cap]
-    double *s_C = s_B + p.rep_cap;                                    // [rep_cap]
-    double *s_redt = s_C + p.rep_cap;                                 // [32]
+    double2 *s_line = reinterpret_cast<double2 *>(s_tab + 3 * npad);         // [rep_cap + kPad] (B, C)
+    double *s_redt = reinterpret_cast<double *>(s_line + p.rep_cap + kPad);  // [32]
     uint32_t *s_I = reinterpret_cast<uint32_t *>(s_redt + 32);        // [rep_cap] candidate index of an entry
     uint32_t *s_k = s_I + p.rep_cap;                                  // [T] exchange of k
-    int *s_opt = reinterpret_cast<int *>(s_k + T);                    // [max_coarse]
-    int *s_cnt = s_opt + p.max_coarse;                                // [32] + [32]
+    unsigned *s_near = s_k + T;                                       // [max_coarse] first and (<< 16) last of the best entries
+    int *s_cnt = reinterpret_cast<int *>(s_near + p.max_coarse);      // [32] + [32]
 
     const int midx = blockIdx.x, trel = blockIdx.y, table = p.table0 + trel;
     dependents_may_start();
@@ -164,8 +164,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
             for (int v = 0; v < V; ++v) {
                 if ((rep >> v) & 1u) {
                     if (pos >= 0 && pos < p.rep_cap) {
-                        s_B[pos] = gs[v] + L;
-                        s_C[pos] = gs[v] * (static_cast<double>(k[v]) - 1.0);
+                        s_line[pos] = make_double2(gs[v] + L, fmin(gs[v] * (static_cast<double>(k[v]) - 1.0), CUDART_INF));  // inf * 0 as inf
                         s_I[pos] = static_cast<uint32_t>(cand[v]);
                     }
                     ++pos;
@@ -208,46 +207,80 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
             __syncthreads();  // the previous window's searches are done with the list
             list_pass(win);
         }
-        __syncthreads();
         const int n_e = min(p.rep_cap, n_rep - win * p.rep_cap);
-        // (B) winners at the coarse process counts: every eighth and the last over the whole window, then the others
-        auto coarse_winner = [&](int c, int lo, int hi) {
-            const double x = static_cast<double>(P_at(p.G, min(coarse_index(c, p.coarse_log), n_P - 1)) - 1);
-            double tb = CUDART_INF;
-            int eb = 0x7FFFFFFF;
-#pragma unroll 4
-            for (int e = lo + lane; e <= hi; e += 32) {
-                const double t = fma(x, s_B[e], s_C[e]);
-                if (t < tb) { tb = t; eb = e; }
-            }
-            warp_min_pair(tb, eb);
-            if (lane == 0) s_opt[c] = min(eb, n_e - 1);
-        };
+        for (int i = tid; i < kPad; i += T) s_line[n_e + i] = make_double2(0.0, CUDART_INF);
+        __syncthreads();
+        // (B) the entries whose time is within (1 + near) of the best at the coarse process counts (a few more where times
+        // close in on it in steps as small as that): every eighth and the last over the whole window, then the others
+        auto x_of = [&](int c) { return static_cast<double>(P_at(p.G, min(coarse_index(c, p.coarse_log), n_P - 1)) - 1); };
+        // between coarse indices a and b: from the first of the best at b to the last at a
         auto bracket = [&](int a, int b, int &lo, int &hi) {
-            lo = max(min(a, b) - 1, 0);
-            hi = min(max(a, b) + 1, n_e - 1);
+            hi = static_cast<int>(s_near[a] >> 16);
+            lo = min(static_cast<int>(s_near[b] & 0xFFFFu), hi);
         };
-        const int n_8 = (n_c - 1 + 7) / 8 + 1;  // 0, 8, 16, .. and n_c - 1
-        for (int i = warp; i < n_8; i += n_warps) coarse_winner(min(8 * i, n_c - 1), 0, n_e - 1);
-        __syncthreads();
-        for (int c = warp; c < n_c - 1; c += n_warps) {
-            if ((c & 7) == 0) continue;
-            int lo, hi;
-            bracket(s_opt[c & ~7], s_opt[min((c & ~7) + 8, n_c - 1)], lo, hi);
-            coarse_winner(c, lo, hi);
+#pragma unroll 1
+        for (int level = 8; level >= 1; level -= 7) {
+            const int n = level == 8 ? (n_c - 1 + 7) / 8 + 1 : n_c - 1;  // 0, 8, 16, .. and n_c - 1
+#pragma unroll 1
+            for (int i = warp; i < n; i += n_warps) {
+                const int c = min(level * i, n_c - 1);
+                if (level == 1 && (c & 7) == 0) continue;
+                const double x = x_of(c), r = __fdividef(static_cast<float>(x_of(min(c + level, n_c - 1))), static_cast<float>(x));  // to 1e-6
+                int lo = 0, hi = n_e - 1;
+                if (level == 1) bracket(c & ~7, min((c & ~7) + 8, n_c - 1), lo, hi);
+                // What is within `near` at an index in between must be inside the bracket as well, so that of every eighth
+                // is wider: twice, and by the ratio of process counts once more.
+                const double near = envelope_near(level == 8 ? 2.0 * r * r : r);
+                // One read of the range, which is what this costs (16 bytes an entry out of shared memory; the nearest times
+                // in a second read 4 us of the kernel's 40): per lane the entries from the first to the last whose high word is
+                // at most one above the smallest.  Those behind hi are the list's as well, then kPad that never win.
+                int h = 0x7FFFFFFE, first = n_e - 1, last = 0;
+#pragma unroll 1
+                for (int e = lo + lane; e <= hi; e += 128) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int v = __double2hiint(fma(x, s_line[e + 32 * u].x, s_line[e + 32 * u].y));
+                        first = v < h - 1 ? e + 32 * u : first;  // so much better than all before that none of them counts
+                        last = v <= h + 1 ? e + 32 * u : last;
+                        h = min(h, v);
+                    }
+                }
+                bool on = h <= __reduce_min_sync(kFull, h) + 1;
+                first = __reduce_min_sync(kFull, on ? first : n_e - 1);
+                last = __reduce_max_sync(kFull, on ? min(last, n_e - 1) : 0);
+                if (near > 0x1p-21) { first = lo; last = hi; }  // more than a high word's last bit
+                // of these the ones that are within `near`
+                double tb = CUDART_INF, up_to = CUDART_INF;
+                const int begin = first + lane, end = last;
+                first = n_e - 1; last = 0;
+#pragma unroll 1
+                for (int e = begin; e <= end; e += 32) {
+                    const double t = fma(x, s_line[e].x, s_line[e].y);
+                    if (t <= up_to) {
+                        const double t_up = fma(t, near, t);
+                        first = t_up < tb ? e : min(first, e);
+                        last = e;
+                        if (t < tb) { tb = t; up_to = t_up; }
+                    }
+                }
+                const double m = warp_min(tb);
+                on = tb <= fma(m, near, m);
+                first = __reduce_min_sync(kFull, on ? first : n_e - 1);
+                last = __reduce_max_sync(kFull, on ? last : 0);
+                if (lane == 0) s_near[c] = static_cast<unsigned>(min(first, last)) | static_cast<unsigned>(last) << 16;
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        // (C) every process count: the bracket of its coarse neighbours, one entry wider on each side
+        // (C) every process count: the bracket of its coarse neighbours
         for (int pidx = tid; pidx < n_P; pidx += T) {
             const int c = envelope_coarse_of(pidx, p.coarse_log);
             int lo, hi;
-            bracket(s_opt[c], s_opt[min(c + 1, n_c - 1)], lo, hi);
+            bracket(c, coarse_index(c, p.coarse_log) == pidx ? c : min(c + 1, n_c - 1), lo, hi);
             const double x = static_cast<double>(P_at(p.G, pidx) - 1);
-            if (coarse_index(c, p.coarse_log) == pidx) lo = hi = s_opt[c];  // a coarse one itself: already found
             double tb = CUDART_INF;
             int eb = lo;
             for (int e = lo; e <= hi; ++e) {
-                const double t = fma(x, s_B[e], s_C[e]);
+                const double t = fma(x, s_line[e].x, s_line[e].y);
                 if (t < tb) { tb = t; eb = e; }  // ascending e: the smallest s stays on ties
             }
             const size_t o = out_row(slot5) + pidx;
@@ -261,7 +294,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
 
 size_t envelope_smem_bytes(const TableDev &T, int threads, int rep_cap, int max_coarse)
 {
-    return (3 * static_cast<size_t>(T.npad) + 2 * static_cast<size_t>(rep_cap) + 32) * sizeof(double) +
+    return (3 * static_cast<size_t>(T.npad) + 2 * (static_cast<size_t>(rep_cap) + kPad) + 32) * sizeof(double) +
            (static_cast<size_t>(rep_cap) + threads) * sizeof(uint32_t) + (static_cast<size_t>(max_coarse) + 64) * sizeof(int);
 }
 
