@@ -7,12 +7,16 @@
 
 namespace plogp {
 
+constexpr int kMaxSmem = 227 * 1024;  // shared memory of a CTA, at most
+
 // Launches a kernel on a stream; overlap: it may start before the kernel in front of it has ended (device_common.cuh).
 template <typename P>
 inline cudaError_t launch(void (*kernel)(P), unsigned gx, unsigned gy, unsigned threads, size_t smem, cudaStream_t st, bool overlap, const P &params)
 {
+    // The limit is the kernel's, for all threads: it is only ever raised to what an SM has, or a thread with a smaller call could
+    // lower it between another's two lines here.
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchAttribute attr{};

@@ -1,5 +1,10 @@
 // A CUDA runtime and kernels made of host memory, for csrc/api.cu on a machine without a GPU: allocations are counted and can
 // be refused, every launch checks that the scratch it is given lies inside a live allocation, and nothing is computed.
+#include <cuda_runtime.h>
+
+template <typename F>  // as nvcc has it
+static cudaError_t cudaFuncSetAttribute(F *f, cudaFuncAttribute a, int v) { return cudaFuncSetAttribute(reinterpret_cast<const void *>(f), a, v); }
+
 #include "../paper_cs_0408034_b200/csrc/internal.h"
 
 #include <cstdlib>
@@ -60,6 +65,37 @@ cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { *ms = 0.f; return cudaSuccess; }
+}
+
+// A kernel's limit on dynamic shared memory, for all threads; another thread's call may come in between any two of a call's own.
+namespace {
+int limit = 48 * 1024;
+void (*other_thread)() = nullptr;
+void kernel(int) {}
+}  // namespace
+extern "C" {
+cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int v)
+{
+    limit = v;
+    if (auto f = other_thread) { other_thread = nullptr; f(); }
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *, void **)
+{
+    return static_cast<int>(c->dynamicSmemBytes) <= limit ? cudaSuccess : cudaErrorInvalidValue;
+}
+// a launch with `mine` bytes while another thread launches the same kernel with `theirs`
+int fake_launch_beside(int mine, int theirs_)
+{
+    static int theirs;
+    static cudaError_t e;
+    theirs = theirs_;
+    e = cudaSuccess;
+    other_thread = [] { e = plogp::launch(kernel, 1, 1, 32, theirs, nullptr, false, 0); };
+    const cudaError_t own = plogp::launch(kernel, 1, 1, 32, mine, nullptr, false, 0);
+    if (other_thread) { auto f = other_thread; other_thread = nullptr; f(); }
+    return own == cudaSuccess && e == cudaSuccess;
+}
 }
 
 namespace plogp {

@@ -1,4 +1,5 @@
-"""csrc/api.cu against a CUDA runtime made of host memory (fake_cuda.cpp): what the calls do when memory runs out."""
+"""csrc/api.cu against a CUDA runtime made of host memory (fake_cuda.cpp): what the calls do when memory runs out, and
+beside one another."""
 import ctypes as C
 import os
 import subprocess
@@ -72,3 +73,10 @@ def test_scratch_that_does_not_grow_leaves_no_call_without_it(lib, kind):
         lib.fake_refuse_from(-1)
         lib.plogp_table_free(h)
     assert lib.fake_live_bytes() == 0
+
+
+@pytest.mark.parametrize("mine,theirs", [(100 << 10, 60 << 10), (60 << 10, 100 << 10), (227 << 10, 49 << 10), (100 << 10, 1 << 10)])
+def test_launches_of_one_kernel_from_two_threads(lib, mine, theirs):
+    """Handles are independent: a call that needs less shared memory does not lower a kernel's limit for one on another thread
+    that has just raised it."""
+    assert lib.fake_launch_beside(mine, theirs)
