@@ -8,6 +8,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <limits>
 #include <new>
 #include <string>
@@ -22,7 +23,9 @@ std::atomic<unsigned long long> g_launches{0};
 
 int cuda_fail(cudaError_t e, const char *what)
 {
-    g_cuda_error = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
+    try {
+        g_cuda_error = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
+    } catch (const std::bad_alloc &) { g_cuda_error.clear(); }
     cudaGetLastError();  // clear the sticky-free error state
     return PLOGP_E_CUDA;
 }
@@ -132,8 +135,11 @@ struct LaunchTimer {
     ~LaunchTimer()
     {
         if (!a) return;
-        if (cudaEventRecord(b, st) == cudaSuccess) h->timed.push_back({kind, a, b});
-        else { cudaEventDestroy(a); cudaEventDestroy(b); cudaGetLastError(); }
+        bool kept = false;
+        try {
+            if (cudaEventRecord(b, st) == cudaSuccess) { h->timed.push_back({kind, a, b}); kept = true; }
+        } catch (const std::bad_alloc &) {}
+        if (!kept) { cudaEventDestroy(a); cudaEventDestroy(b); cudaGetLastError(); }
     }
 };
 
@@ -232,8 +238,9 @@ int ensure_scratch(plogp_tables *h, size_t bytes)
     return PLOGP_OK;
 }
 
-// Finds or builds the launch plan of a grid; *out is valid until the next call.
-int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **out)
+// Finds or builds the launch plan of a grid; *out is valid until the next call.  Throws where host memory runs out; a plan that
+// was being built is then no plan.
+int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **out)
 {
     if (!g || g->n_m < 0 || (g->n_m > 0 && !g->m)) return PLOGP_E_INVAL;
     if (g->P && g->n_P < 0) return PLOGP_E_INVAL;
@@ -459,7 +466,10 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
         slot.d_grid = nullptr;
         slot.grid_cap = 0;
         const size_t cap = std::max<size_t>(blob.size() + blob.size() / 4, 4096);
-        CK(cudaMalloc(&slot.d_grid, cap));
+        const cudaError_t e = cudaMalloc(&slot.d_grid, cap);
+        if (e != cudaSuccess) slot.d_grid = nullptr;
+        if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); return PLOGP_E_NOMEM; }
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(grid)");
         slot.grid_cap = cap;
     }
     // The source is pageable host memory: the runtime stages it before returning.
@@ -501,6 +511,14 @@ int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **
     pl.scratch_bytes = per_table ? per_table * pl.tables_per_batch + 1024 : 0;  // the sections start on 256-byte boundaries
     rc = ensure_scratch(h, pl.scratch_bytes);
     return rc == PLOGP_OK ? keep() : rc;
+}
+
+// The same for the C calls, which throw nothing
+int prepare(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const Plan **out)
+{
+    try {
+        return find_or_build(h, g, st, out);
+    } catch (const std::exception &) { return PLOGP_E_NOMEM; }  // bad_alloc, or a length no vector can have
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -769,7 +787,7 @@ static int check_tables(int n_tables, int n_bp, const uint64_t *sizes_bytes, int
     const size_t lat = size_t(n_tables) * 8, gaps = size_t(n_tables) * n_bp * 8, sizes = (sizes_shared ? size_t(1) : size_t(n_tables)) * n_bp * 8;
     try {
         pack.resize(lat + gaps + sizes);
-    } catch (const std::bad_alloc &) { return PLOGP_E_NOMEM; }
+    } catch (const std::exception &) { return PLOGP_E_NOMEM; }
     std::memcpy(pack.data(), latency, lat);
     std::memcpy(pack.data() + lat, gap, gaps);
     std::memcpy(pack.data() + lat + gaps, sizes_bytes, sizes);
@@ -849,19 +867,17 @@ int plogp_table_free(plogp_tables *h)
 {
     if (!h) return PLOGP_OK;
     int rc = PLOGP_OK;
-    std::vector<void *> bufs = {h->d_tab, h->d_ws, h->d_stage[0], h->d_stage[1]};
-    for (const Plan &c : h->plans) bufs.push_back(c.d_grid);
     for (int i = 0; i < 2; ++i) {
         if (h->ev_done[i]) cudaEventDestroy(h->ev_done[i]);
         if (h->ev_copied[i]) cudaEventDestroy(h->ev_copied[i]);
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
-    for (void *b : bufs) {
-        if (b) {
-            cudaError_t e = cudaFree(b);
-            if (e != cudaSuccess) rc = cuda_fail(e, "cudaFree");
-        }
-    }
+    auto release = [&](void *b) {
+        const cudaError_t e = b ? cudaFree(b) : cudaSuccess;
+        if (e != cudaSuccess) rc = cuda_fail(e, "cudaFree");
+    };
+    for (void *b : {static_cast<void *>(h->d_tab), static_cast<void *>(h->d_ws), static_cast<void *>(h->d_stage[0]), static_cast<void *>(h->d_stage[1])}) release(b);
+    for (const Plan &c : h->plans) release(c.d_grid);
     for (auto &t : h->timed) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
     delete h;
     return rc;

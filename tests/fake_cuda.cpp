@@ -10,6 +10,7 @@ static cudaError_t cudaFuncSetAttribute(F *f, cudaFuncAttribute a, int v) { retu
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 
 namespace {
 std::map<const unsigned char *, size_t> live;
@@ -22,10 +23,21 @@ void inside(const void *p, size_t bytes)
     --it;
     if (static_cast<const unsigned char *>(p) + bytes > it->first + it->second) ++bad;
 }
+long long refuse_host_at = -1;  // likewise for operator new, api.cu's own
 cudaError_t launched() { ++launches; return cudaSuccess; }
 }  // namespace
 
+void *operator new(size_t n)
+{
+    if (refuse_host_at >= 0 && static_cast<long long>(n) >= refuse_host_at) throw std::bad_alloc();
+    if (void *p = std::malloc(n ? n : 1)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, size_t) noexcept { std::free(p); }
+
 extern "C" {
+void fake_refuse_host_from(long long bytes) { refuse_host_at = bytes; }
 void fake_refuse_from(long long bytes) { refuse_at = bytes; }
 long long fake_bad_accesses() { return bad; }
 long long fake_launches() { return launches; }

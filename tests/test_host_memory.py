@@ -25,7 +25,10 @@ def lib(tmp_path_factory):
     lib.plogp_predict.argtypes = [C.c_void_p] * 5
     lib.plogp_select_best_collective.argtypes = [C.c_void_p, C.c_void_p, C.c_int] + [C.c_void_p] * 4
     lib.plogp_table_free.argtypes = [C.c_void_p]
-    lib.fake_refuse_from.argtypes = [C.c_longlong]
+    lib.plogp_select_best_host.argtypes = [C.c_void_p] * 6
+    lib.plogp_segment_surface.argtypes = [C.c_void_p] * 4
+    lib.plogp_profile_read.argtypes = [C.c_void_p] * 3
+    lib.fake_refuse_from.argtypes = lib.fake_refuse_host_from.argtypes = [C.c_longlong]
     for f in ("fake_bad_accesses", "fake_launches", "fake_live_bytes"):
         getattr(lib, f).restype = C.c_longlong
     return lib
@@ -80,3 +83,48 @@ def test_launches_of_one_kernel_from_two_threads(lib, mine, theirs):
     """Handles are independent: a call that needs less shared memory does not lower a kernel's limit for one on another thread
     that has just raised it."""
     assert lib.fake_launch_beside(mine, theirs)
+
+
+def in_a_child(f):
+    """Exit status of f() in a process of its own: an exception that leaves a C call ends it with a signal."""
+    pid = os.fork()
+    if pid == 0:
+        os._exit(0 if f() else 1)
+    return os.waitpid(pid, 0)[1]
+
+
+@pytest.mark.parametrize("refuse", [1, 64, 600, 5000])
+def test_host_memory_that_runs_out_is_a_status(lib, refuse):
+    """Allocations of a size and up fail while a plan is built: every call returns PLOGP_E_NOMEM (or succeeds), nothing throws,
+    and the calls go on afterwards."""
+    grids = [long_list(300, 40), long_list(300, 40, search_mode=1), plogp.GridArgs(np.arange(1, 101) * 4096, None, 2, 700, np.arange(4, 100, 4))]
+
+    def f():
+        h = load(lib, 8)
+        kept = long_list(20, 2)
+        ok = lib.plogp_select_best(h, kept.ref, OUT, OUT, OUT, None) == plogp.OK
+        for g in grids:
+            calls = [lambda: lib.plogp_select_best(h, g.ref, OUT, OUT, OUT, None), lambda: lib.plogp_predict(h, g.ref, OUT, None, None),
+                     lambda: lib.plogp_select_best_collective(h, g.ref, 4, OUT, OUT, OUT, None), lambda: lib.plogp_segment_surface(h, g.ref, OUT, None)]
+            for call in calls:
+                lib.fake_refuse_host_from(refuse)
+                ok &= call() in (plogp.OK, plogp.E_NOMEM)
+                if refuse == 1:
+                    ok &= lib.plogp_select_best(h, kept.ref, OUT, OUT, OUT, None) in (plogp.OK, plogp.E_NOMEM)
+                lib.fake_refuse_host_from(-1)
+                ok &= call() == plogp.OK and lib.plogp_select_best(h, kept.ref, OUT, OUT, OUT, None) == plogp.OK
+        lib.plogp_profile_enable(C.c_void_p(h.value), 1)
+        lib.fake_refuse_host_from(refuse)
+        ok &= all(lib.plogp_select_best(h, kept.ref, OUT, OUT, OUT, None) == plogp.OK for _ in range(300))
+        return ok & (lib.plogp_table_free(h) == plogp.OK) & (lib.fake_live_bytes() == 0) & (lib.fake_bad_accesses() == 0)
+
+    assert in_a_child(f) == 0
+
+
+def test_device_memory_that_runs_out_for_a_grid_is_a_status(lib):
+    g, h = long_list(300, 40), load(lib, 8)
+    lib.fake_refuse_from(1)
+    assert lib.plogp_select_best(h, g.ref, OUT, OUT, OUT, None) == plogp.E_NOMEM
+    lib.fake_refuse_from(-1)
+    assert lib.plogp_select_best(h, g.ref, OUT, OUT, OUT, None) == plogp.OK
+    assert lib.plogp_table_free(h) == plogp.OK
