@@ -50,3 +50,37 @@ def test_lower_envelope_of_lines_that_differ_by_rounding(plogp, scale, n_s, n_P,
             assert x[:, 0].equal(y[:, 0])
         a, b = plogp.predict(tabs, w), plogp.predict(tabs, replace(w, search_mode=1))
         assert a.time[:, 5].equal(b.time[:, 5]) and a.best_s[:, 1].equal(b.best_s[:, 1])
+
+
+def off_by_one(x):
+    """A tensor like x (its contents too) one element behind the start of an allocation."""
+    import torch
+    y = torch.empty(x.numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x.shape)
+    y.copy_(x)
+    return y
+
+
+@pytest.mark.parametrize("n_tables,n_m,n_P,n_s,listed", [(1, 20, 40, 7, False), (4, 64, 600, 33, True), (600, 64, 24, 9, False), (40, 128, 512, 20, False), (11500, 46, 16, 3, False),
+                                                         (120, 130, 560, 5, False)])
+def test_outputs_at_odd_addresses(plogp, n_tables, n_m, n_P, n_s, listed):
+    """Outputs and inputs aligned for single elements only: the stores of two and four cells give way to single ones on grids
+    that take them otherwise (even n_m, rows off the sectors, sensitivity planes, boundaries of 8 and 16 bytes), with the
+    same decisions and times (Scatter Chain sums to 1e-12: another order of additions)."""
+    import torch
+    w = wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=n_s, seed_offset=n_P)
+    if listed:
+        w = replace(w, P_list=(2 + 3 * np.arange(n_P)).astype(np.int32))
+    with plogp.Tables.from_workload(w) as tabs:
+        dec, pred = plogp.select_best(tabs, w), plogp.predict(tabs, w)
+        d = plogp.DecisionTable(*(off_by_one(torch.zeros_like(x)) for x in (dec.strategy, dec.s_bytes, dec.time)))
+        plogp.select_best(tabs, w, out=d)
+        assert d.strategy.equal(dec.strategy) and d.s_bytes.equal(dec.s_bytes)
+        assert d.time[:, 0].equal(dec.time[:, 0]) and torch.allclose(d.time[:, 1], dec.time[:, 1], rtol=1e-12, atol=0.0)
+        p = plogp.Prediction(off_by_one(torch.zeros_like(pred.time)), off_by_one(torch.zeros_like(pred.best_s)))
+        plogp.predict(tabs, w, out=p)
+        assert p.best_s.equal(pred.best_s) and p.time[:, :11].equal(pred.time[:, :11]) and p.time[:, 12].equal(pred.time[:, 12])
+        assert torch.allclose(p.time[:, 11], pred.time[:, 11], rtol=1e-12, atol=0.0)
+        (fixed, ratio), (f2, r2) = (plogp.segment_sensitivity(tabs, w, 8192, pred=x) for x in (pred, plogp.Prediction(off_by_one(pred.time), None)))
+        assert f2.equal(fixed) and r2.equal(ratio)
+        a, b = plogp.decision_boundaries(dec), plogp.decision_boundaries(plogp.DecisionTable(off_by_one(dec.strategy), None, None))
+        assert a.equal(b)
