@@ -9,7 +9,7 @@
  * lowest predicted time (Sections 1 and 5).  The network enters through the pLogP parameters
  * of Section 2: the latency L and the gap g(m), measured at a list of message sizes.
  *
- * All arithmetic is IEEE double.  There is no CPU fallback: every call needs a CUDA device of
+ * All results are IEEE double arithmetic (bounds in FP32 only decide what need not be compared).  There is no CPU fallback: every call needs a CUDA device of
  * compute capability 10.0.
  *
  * Strategy ids (Table 1 rows in print order, then Table 2 rows):
@@ -139,8 +139,10 @@ typedef struct {
  * The handle keeps the launch plans of its last eight grids: a call with one of them (and per-kernel
  * timing off) copies nothing and allocates nothing, it only launches kernels on `stream`, so a
  * loop of such calls may be captured into a CUDA graph and replayed.  The first call with a new
- * grid uploads the grid and may allocate scratch: make it outside the capture (and re-capture after it: a graph keeps
- * the scratch of its time).
+ * grid uploads the grid and may allocate scratch: make it outside the capture.  A captured graph holds the plan's
+ * device arrays and the scratch of its time: replay it only while no call on the handle has used a new grid since (that
+ * may overwrite or free the arrays of the plan that was not called for longest, replays not counted, and may move the
+ * scratch), else capture it again.
  */
 int plogp_predict(plogp_tables *tables, const plogp_grid *grid, double *d_time, uint32_t *d_best_s,
                   void *stream);
@@ -272,7 +274,9 @@ int plogp_scatter_chain_static(int n_bp, const uint64_t *d_sizes_bytes, const do
 /*
  * Per-kernel device timing (measurement aid, no counterpart in the paper).  While enabled, every
  * kernel that plogp_predict / plogp_select_best launch on this handle is bracketed by two CUDA
- * events recorded on the caller's stream.  plogp_profile_read waits for the recorded events,
+ * events recorded on the caller's stream.  The kernels of a call then run one after another, where they
+ * overlap otherwise, and a small decision table takes a DECIDE and a SCATTER launch instead of one for both
+ * (which is not timed by itself): the sum is more than the call takes with timing off.  plogp_profile_read waits for the recorded events,
  * adds the elapsed milliseconds and launch counts per kernel kind into ms[PLOGP_N_KERNEL_KINDS] and
  * launches[PLOGP_N_KERNEL_KINDS] (HOST arrays), and forgets them.  Read (or free the handle)
  * regularly: each launch keeps two events alive until then.
@@ -280,9 +284,9 @@ int plogp_scatter_chain_static(int n_bp, const uint64_t *d_sizes_bytes, const do
 enum {
     PLOGP_KERNEL_SWEEP = 0,        /* segment sweep over long candidate lists */
     PLOGP_KERNEL_CHAIN_PREFIX = 1, /* no longer launched: the Scatter Chain sums are taken inside the kernels that use them */
-    PLOGP_KERNEL_FUSED = 2,        /* all strategies, lanes <-> m (predictions, long lists' final pass) */
+    PLOGP_KERNEL_FUSED = 2,        /* predictions but for the segmented minima (whichever kernel writes the planes), long lists' final pass */
     PLOGP_KERNEL_DECIDE = 3,       /* Broadcast decision, lanes <-> P (short candidate lists) */
-    PLOGP_KERNEL_SCATTER = 4,      /* Scatter decision */
+    PLOGP_KERNEL_SCATTER = 4,      /* Scatter decision (scatter_kernel or scatter_rows_kernel) */
     PLOGP_KERNEL_ENVELOPE = 5,     /* segment search by lower envelope (search_mode 1) */
     PLOGP_KERNEL_SEGMIN = 6,       /* segmented minima of plogp_predict, lanes <-> P (short candidate lists) */
     PLOGP_KERNEL_GAPS = 7,         /* g(1), g(s), g(m) once per table, in front of the lanes <-> P kernels on large grids */

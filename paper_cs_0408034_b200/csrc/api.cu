@@ -544,8 +544,10 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
     if (pl.empty) return PLOGP_OK;
     rc = ensure_scratch(h, pl.scratch_bytes);
     if (rc != PLOGP_OK) return rc;
-    // Short candidate lists with segmented strategies: the lane<->P decision kernel; everything else
-    // (predictions, long lists reduced by the sweep kernel, Scatter-only grids) goes through fused_kernel.
+    // Decision tables on short candidate lists with segmented strategies: the lane<->P decision kernel for the Broadcast half
+    // (select_kernel for both halves of a small one).  What is left of a decision table, if only Scatter strategies, goes to
+    // scatter_kernel or scatter_rows_kernel; predictions to segmin_kernel, then planes_kernel, scatter_rows_kernel and
+    // fused_kernel; long lists, reduced by sweep_kernel or envelope_kernel, to fused_kernel.
     const bool use_decide = !predict && pl.inline_sweep && pl.n_seg > 0;
     // the kernel that follows the (optional) Broadcast decision kernel: Scatter strategies only => scatter_kernel
     const bool use_scatter = !predict && ((use_decide ? pl.G.mask & 0x1C00u : pl.G.mask) & 0x3FFu) == 0;
@@ -597,7 +599,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         GridDev Gf = pl.G;
         if (predict && pl.inline_sweep && pl.n_seg > 0) {
             // Predictions on short candidate lists: the segmented minima (planes 2, 5, 9 and the best segment sizes)
-            // come from the lane<->P kernel; fused_kernel then writes the closed-form planes only.
+            // come from the lane<->P kernel; the kernels behind it write the other planes.
             SegminParams sp{};
             sp.T = h->T; sp.G = pl.G;
             sp.n_mgroups = pl.bc_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.bc_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs | 1;
@@ -623,7 +625,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             if (!Gf.mask) continue;
         }
         if (use_decide) {
-            // Broadcast half with lanes <-> P; the Scatter half (no candidate lists) follows in fused_kernel.
+            // Broadcast half with lanes <-> P; the Scatter half (no candidate lists) beside it or in the kernel behind it
             DecideParams dp{};
             dp.T = h->T; dp.G = pl.G;
             dp.G.mask &= 0x3FFu;

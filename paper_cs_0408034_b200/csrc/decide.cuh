@@ -2,10 +2,9 @@
 // candidate lists, with lanes mapped to the process count P.  (The Scatter half has no candidate
 // lists and goes through scatter_kernel.)
 //
-// One CTA owns one table, a group of up to 16 message sizes and a tile of 256 process counts.  All
-// four warps work on the same 256 process counts (lane + 32 r, r = 0..7) and split the message
-// sizes, so a warp runs on its own from the candidate lists to the staged result and only the
-// write-out needs the whole CTA.
+// One CTA owns one table, a group of up to 16 message sizes and one or two tiles of 256 or 128 process counts (lane + 32 r,
+// r = 0..7 or 0..3).  Its four warps split the message sizes, each over all process counts of the CTA, so a warp runs on its own
+// from the candidate lists to the staged result and only the write-out needs the whole CTA.
 //
 // Every model of Table 1 is, for a fixed message size (and segment size), a line in P or a function of
 // floor(log2 P) and ceil(log2 P) alone:
@@ -18,14 +17,15 @@
 // (0, its smallest time)), so that a decision is a slot number and equal times go to the smaller one.
 //
 // Per message size:
-//   1. lanes <-> candidates: the lines' coefficients, in FP64 and rounded down to FP32; the pilot, the line that is
-//      best at the tile's middle process count.
+//   1. lanes <-> candidates: the lines' coefficients, in FP64 and rounded down to FP32; the pilots, the lines that are
+//      best at four of the CTA's process counts.
 //   2. lanes <-> (floor, ceil) pairs: the best of ids 6 to 9 in FP64, one candidate after another.
-//   3. per process count the better of the pilot and its pair: the running minimum's start.
+//   3. per process count the best of the pilots and its pair: the running minimum's start.
 //   4. every cell of every other line as a lower bound: FP32 coefficients, process count and fused multiply-add all
 //      rounded down, two lines per instruction; the smallest bound per process count is compared with the running
 //      minimum rounded up.  All terms are non-negative, so the bound is never above the FP64 time.
-//   5. only rows of 32 process counts in which some bound is not above (1.4 of 8 on average) are searched exactly.
+//   5. only rows of 32 process counts in which some bound is not above (1.4 of 8 on average) are searched exactly.  Where all
+//      times lie outside FP32's range every row is, and a call takes 4 times as long.
 // Results are those of the exhaustive FP64 search, bit for bit.  Staged as slot numbers [m][P] (1 byte); the write-out,
 // rows of consecutive m per process count, evaluates the winner's line again (the same fma, the same double).
 #pragma once
@@ -86,8 +86,6 @@ __host__ __device__ inline size_t dec_layout(int npad, int n_s, int n_pairs, int
     }
     return off;
 }
-
-__device__ __forceinline__ int hi32(double x) { return __double2hiint(x); }
 
 }  // namespace decide
 

@@ -15,7 +15,8 @@ namespace plogp {
 // has called dependents_may_start.  A kernel that reads what the one in front writes waits for its end first.  Each kernel's
 // last CTA waits for the end of the kernel in front before it ends itself, so that the end of a call's last kernel is the
 // end of the call.  Nothing here spins: the waits are the hardware's, and a kernel's CTAs only start when all CTAs of the
-// kernel in front have their place.
+// kernel in front have their place.  A kernel launched with `overlap` must therefore not end thread 0 of its last CTA anywhere but
+// behind last_block_waits; envelope_kernel, which returns early, is only ever the first of a call.
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_kernel_in_front() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void last_block_waits(int tid)  // call at the end; thread 0 of a kernel's last CTA must get here

@@ -28,12 +28,6 @@ inline cudaError_t launch(void (*kernel)(P), unsigned gx, unsigned gy, unsigned 
     return cudaLaunchKernelEx(&cfg, kernel, params);
 }
 
-// Tables as they live in device memory.  Per table: three runs of `npad` doubles
-//   key[npad]   breakpoint sizes usable as interval starts (index <= n_bp-2), +inf beyond
-//   gap[npad]   g at the interval start
-//   slope[npad] (g[i+1]-g[i]) / (size[i+1]-size[i])
-// npad is a power of two >= n_bp, so the interval search needs no bounds checks and an upward
-// walk always meets a +inf key.
 // Where a decision kernel puts its results and how it names the strategies.  plogp_select_best writes two planes
 // per table (Broadcast, Scatter) with the ids of Table 1 / Table 2; the derived collectives (Gather, Reduce) reuse
 // the same kernels with one plane per table and the ids of the mirrored strategies.
@@ -44,6 +38,12 @@ struct OutMap {
     uint8_t id_of[16];  // output id of internal strategy id 0..12 (255 beyond)
 };
 
+// Tables as they live in device memory.  Per table: three runs of `npad` doubles
+//   key[npad]   breakpoint sizes usable as interval starts (index <= n_bp-2), +inf beyond
+//   gap[npad]   g at the interval start
+//   slope[npad] (g[i+1]-g[i]) / (size[i+1]-size[i])
+// npad is a power of two >= n_bp, so the interval search needs no bounds checks and an upward
+// walk always meets a +inf key.
 struct TableDev {
     const double *tab;  // [n_tables][3*npad]
     const double *lat;  // [n_tables]
@@ -143,7 +143,7 @@ constexpr uint32_t kPlanesMask = 0x5DBu;  // ids 0 1 3 4 6 7 8 10
 constexpr int kPlanesMaxM = 4096;         // g(m) of all message sizes in shared memory
 cudaError_t launch_planes(const PlanesParams &p, bool overlap, cudaStream_t st);
 
-// Scatter half of the decision table: see scatter.cu
+// Scatter half of the decision table: see scatter.cuh
 struct ScatterParams {
     TableDev T;
     GridDev G;
@@ -191,7 +191,7 @@ struct GapsParams {
     int stride;
 };
 
-// Decision kernel for short candidate lists (lanes <-> P): see decide.cu
+// Decision kernel for short candidate lists (lanes <-> P): see decide.cuh
 struct DecideParams {
     TableDev T;
     GridDev G;
@@ -204,7 +204,7 @@ struct DecideParams {
     int n_pairs;  // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most, made odd: with an even number of
                   // lines in front, neighbouring message sizes then start in different banks (an even one cost 6 % of a call)
     int ctas_per_sm;  // 4 or 5
-    int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cu)
+    int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cuh)
     int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16 / 8 / 2-byte aligned bases)
     int table0, n_tables_launch;
     int out_table0;  // table whose results sit at the start of the output arrays

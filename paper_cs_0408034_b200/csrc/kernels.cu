@@ -14,8 +14,9 @@
 //                  Scatter Chain sum running along each warp's contiguous run of P, and writes either
 //                  the predicted planes or the decision table.  The general path.
 // Short candidate lists have faster, specialised kernels: decide.cu (Broadcast half of the decision
-// table), scatter.cu (Scatter half), segmin.cu (segmented planes of the predictions); the host routes
-// them there, and fused_kernel writes the closed-form planes only.  Rows off the sectors on large grids go to planes.cu and rows.cu.
+// table), scatter.cu (Scatter half), select.cu (both in one launch), segmin.cu (segmented planes of the predictions); the host
+// routes them there, and fused_kernel writes the other prediction planes.  Rows off the sectors on large grids go to planes.cu
+// and rows.cu.
 #include "device_common.cuh"
 
 namespace plogp {
@@ -43,6 +44,9 @@ namespace plogp {
 // 4.6); with list building, barriers and exact passes (2 %) 2.5.  P = 2..4096, 128 message sizes, 1.25e11 cells of
 // ids 2 and 5: 15.05 -> 8.5 ms.  Scalar multiply-adds, 16 process counts per lane, lanes <-> candidates and packing
 // along P run at the same 2.0 - 2.5 cycles.
+// The exact pass is rare as long as candidates' times differ by more than FP32 rounding where they are best.  Equal gaps over
+// many sizes are no matter (g flat below 64 KB or in stairs: 1.1 to 1.7 times as fast as the FP64 loop).  A latency 1e7 times the
+// gaps or more is (0.7 times), and so are times outside FP32's range, where every cell goes through it (0.2 times).
 //
 // A warp owns 256 consecutive process counts (lane + 32 r).  The CTA's 8 warps cover p.wp such tiles side by side and
 // split the candidates of a sub-chunk 8 / p.wp ways, so that a short range of process counts leaves no warp idle.

@@ -10,7 +10,7 @@
 // the Chain model's sum over j = 1..P-1 of g(j m) into a running sum along the thread: the argument
 // j m grows by m per step, the table interval is kept in registers and only reloaded when the
 // argument crosses a breakpoint.  The sum in front of a warp's run is taken in closed form per table interval
-// (chain_front in device_common.cuh), so a range of process counts can be split over any number of CTAs in one launch.
+// (chain_front_parts and chain_front_sum in device_common.cuh), so a range of process counts can be split over any number of CTAs in one launch.
 #pragma once
 
 #include "device_common.cuh"

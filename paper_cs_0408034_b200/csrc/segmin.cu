@@ -2,7 +2,7 @@
 // mapped to the process count P: for each segmented strategy of Table 1 (ids 2, 5, 9) on its own, the minimum
 // of the model over the candidate segment sizes and the smallest size that attains it.
 //
-// Same building blocks as decide_kernel (decide.cu), with one running minimum per strategy instead of one
+// Same building blocks as decide_kernel (decide.cuh), with one running minimum per strategy instead of one
 // over all of them.  One CTA owns one table, up to 16 consecutive message sizes (32 with eight warps) and one or two tiles
 // of 256 process counts (lane + 32 r, r = 0..7); its four (eight) warps split the message sizes.  For a fixed message size the models are
 //     id 2: fma(P-1, Q, L)      id 9: fma(floor(log2 P), Q, ceil(log2 P) L)      Q = g(s) k
