@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
         __syncthreads();
         // (B) the entries whose time is within (1 + near) of the best at the coarse process counts (a few more where times
         // close in on it in steps as small as that): every eighth and the last over the whole window, then the others
-        auto x_of = [&](int c) { return static_cast<double>(P_at(p.G, min(coarse_index(c, p.coarse_log), n_P - 1)) - 1); };
+        auto x_of = [&](int c) { return P_at(p.G, min(coarse_index(c, p.coarse_log), n_P - 1)) - 1; };
         // between coarse indices a and b: from the first of the best at b to the last at a
         auto bracket = [&](int a, int b, int &lo, int &hi) {
             hi = static_cast<int>(s_near[a] >> 16);
@@ -225,36 +225,42 @@ __global__ void __launch_bounds__(1024) envelope_kernel(const EnvParams p)
             for (int i = warp; i < n; i += n_warps) {
                 const int c = min(level * i, n_c - 1);
                 if (level == 1 && (c & 7) == 0) continue;
-                const double x = x_of(c), r = __fdividef(static_cast<float>(x_of(min(c + level, n_c - 1))), static_cast<float>(x));  // to 1e-6
+                const int xi = x_of(c);
+                const double x = static_cast<double>(xi), r = __fdividef(static_cast<float>(x_of(min(c + level, n_c - 1))), static_cast<float>(xi));  // to 1e-6
                 int lo = 0, hi = n_e - 1;
                 if (level == 1) bracket(c & ~7, min((c & ~7) + 8, n_c - 1), lo, hi);
                 // What is within `near` at an index in between must be inside the bracket as well, so that of every eighth
                 // is wider: twice, and by the ratio of process counts once more.
                 const double near = envelope_near(level == 8 ? 2.0 * r * r : r);
-                // One read of the range, which is what this costs (16 bytes an entry out of shared memory; with the nearest times in
-                // a second read of it the kernel took 45.6 us instead of 41.4): per lane the entries from the first to the last whose
-                // high word is at most one above the smallest.  Those behind hi are the list's as well, then kPad that never win.
-                int h = 0x7FFFFFFE, first = n_e - 1, last = 0;
+                // A long range is read once, which is what this costs (16 bytes an entry out of shared memory; with the nearest
+                // times in a second read of it the kernel took 45.6 us instead of 41.4): per lane the entries from the first to
+                // the last whose high word is at most one above the smallest.  Those behind hi are the list's as well, then
+                // kPad that never win.
+                int first = lo, last = hi;
+                bool on;
+                if (hi - lo >= 128 && near <= 0x1p-21) {  // no more than a high word's last bit
+                    int h = 0x7FFFFFFE;
+                    first = n_e - 1; last = 0;
 #pragma unroll 1
-                for (int e = lo + lane; e <= hi; e += 128) {
+                    for (int e = lo + lane; e <= hi; e += 128) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int v = __double2hiint(fma(x, s_line[e + 32 * u].x, s_line[e + 32 * u].y));
-                        first = v < h - 1 ? e + 32 * u : first;  // so much better than all before that none of them counts
-                        last = v <= h + 1 ? e + 32 * u : last;
-                        h = min(h, v);
+                        for (int u = 0; u < 4; ++u) {
+                            const int v = __double2hiint(fma(x, s_line[e + 32 * u].x, s_line[e + 32 * u].y));
+                            first = v < h - 1 ? e + 32 * u : first;  // so much better than all before that none of them counts
+                            last = v <= h + 1 ? e + 32 * u : last;
+                            h = min(h, v);
+                        }
                     }
+                    on = h <= __reduce_min_sync(kFull, h) + 1;
+                    first = __reduce_min_sync(kFull, on ? first : n_e - 1);
+                    last = __reduce_max_sync(kFull, on ? min(last, n_e - 1) : 0);
                 }
-                bool on = h <= __reduce_min_sync(kFull, h) + 1;
-                first = __reduce_min_sync(kFull, on ? first : n_e - 1);
-                last = __reduce_max_sync(kFull, on ? min(last, n_e - 1) : 0);
-                if (near > 0x1p-21) { first = lo; last = hi; }  // more than a high word's last bit
                 // of these the ones that are within `near`
                 double tb = CUDART_INF, up_to = CUDART_INF;
-                const int begin = first + lane, end = last;
+                const int begin = first, end = last;
                 first = n_e - 1; last = 0;
 #pragma unroll 1
-                for (int e = begin; e <= end; e += 32) {
+                for (int e = begin + lane; e <= end; e += 32) {
                     const double t = fma(x, s_line[e].x, s_line[e].y);
                     if (t <= up_to) {
                         const double t_up = fma(t, near, t);
