@@ -118,9 +118,9 @@ typedef struct {
     uint32_t strategy_mask; /* bit i enables strategy id i */
     int32_t k_mode;         /* 0: k = ceil(m/s); 1: k = floor(m/s) */
     int32_t search_mode;    /* how the minimum over s of Section 3.1 is found; the results are the same:
-                               0: exhaustive (the default): every (P, m, s) cell is bounded from below in FP32 and
-                                  compared in FP64 where the bound does not rule it out (ids 6 to 9 are evaluated
-                                  once per pair of floor(log2 P) and ceil(log2 P), on which alone they depend);
+                               0: exhaustive (the default): on every table; every candidate is bounded from below,
+                                  for single process counts or for a range of them at once, and compared in FP64
+                                  where the bound does not rule it out;
                                1: lower envelope: ids 2 and 9 take the s with the smallest g(s) k once per m, id 5
                                   walks the lower envelope of its lines in P (only for tables whose gaps never
                                   decrease with the size; other tables silently take the exhaustive search) */
@@ -285,11 +285,11 @@ enum {
     PLOGP_KERNEL_SWEEP = 0,        /* segment sweep over long candidate lists */
     PLOGP_KERNEL_CHAIN_PREFIX = 1, /* no longer launched: the Scatter Chain sums are taken inside the kernels that use them */
     PLOGP_KERNEL_FUSED = 2,        /* predictions but for the segmented minima (whichever kernel writes the planes), long lists' final pass */
-    PLOGP_KERNEL_DECIDE = 3,       /* Broadcast decision, lanes <-> P (short candidate lists) */
+    PLOGP_KERNEL_DECIDE = 3,       /* Broadcast decision (short candidate lists) */
     PLOGP_KERNEL_SCATTER = 4,      /* Scatter decision (scatter_kernel or scatter_rows_kernel) */
     PLOGP_KERNEL_ENVELOPE = 5,     /* segment search by lower envelope (search_mode 1) */
-    PLOGP_KERNEL_SEGMIN = 6,       /* segmented minima of plogp_predict, lanes <-> P (short candidate lists) */
-    PLOGP_KERNEL_GAPS = 7,         /* g(1), g(s), g(m) once per table, in front of the lanes <-> P kernels on large grids */
+    PLOGP_KERNEL_SEGMIN = 6,       /* segmented minima of plogp_predict (short candidate lists) */
+    PLOGP_KERNEL_GAPS = 7,         /* g(1), g(s), g(m) once per table, in front of these two on large grids */
     PLOGP_N_KERNEL_KINDS = 8
 };
 int plogp_profile_enable(plogp_tables *tables, int enable);

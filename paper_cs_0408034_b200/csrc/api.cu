@@ -65,7 +65,6 @@ struct Plan {
     int n_seg = 0;
     bool inline_sweep = true;
     bool envelope = false;        // envelope_kernel instead of the sweep kernel (long candidate lists)
-    bool envelope_short = false;  // the decision kernel prunes its candidate lists (short candidate lists)
     int env_threads = 256, env_rep_cap = 0, env_coarse_log = 5, env_max_coarse = 0;
     // fused kernel tiling
     int n_mtiles = 0, n_ptiles = 1, passes_per_tile = 1;
@@ -74,16 +73,17 @@ struct Plan {
     // both halves in one launch, and then the Scatter half's split of P
     bool select = false;
     int sel_ptiles = 1, sel_run = 1;
-    // decision kernel tiling (short candidate lists)
-    int bc_mg = kDecMG, bc_mgroups = 0;  // message sizes per CTA of decide_kernel and segmin_kernel as launched
-    int dec_mgroups = 0, dec_ptiles = 1, dec_mg = kDecMG, dec_rows = 8, dec_tiles = 1, dec_pairs = 1;
+    // tiling of decide_kernel and segmin_kernel (short candidate lists)
+    int ln_width = 32, ln_mgroups = 0, ln_np = 512, ln_ptiles = 1, ln_pairs = 1;
+    int ln_staged = 0;  // threads of a CTA that has all message sizes, or 0
+    size_t off_knots = 0;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
     size_t off_pair_m = 0, off_pair_chunk = 0, off_pair_row = 0, off_pair_base = 0;
     int tables_per_batch = 0;
     size_t scratch_bytes = 0;
-    size_t off_k = 0;          // k table of the lane <-> P kernels inside the grid blob
-    bool use_gaps = false;     // run the gap pre-pass in front of the lane <-> P kernels
+    size_t off_k = 0;          // their k table inside the grid blob
+    bool use_gaps = false;     // run the gap pre-pass in front of them
     int gaps_stride = 0;       // doubles per table in its output
     size_t gaps_bytes_per_table = 0;
 };
@@ -297,11 +297,9 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     pl.n_seg = __builtin_popcount(g->strategy_mask & kSegBits);
     pl.inline_sweep = pl.n_seg == 0 || n_s <= kMaxInlineS;
     // search_mode 1 on tables with non-decreasing gaps.  Long candidate lists: envelope_kernel writes the segmented
-    // minima to the scratch rows that fused_kernel reads.  Short lists: the decision kernel prunes its own lists
-    // (predictions of short lists keep the exhaustive inline search; the results are the same).
+    // minima to the scratch rows that fused_kernel reads.  Short lists: decide_kernel and segmin_kernel, as with search_mode 0.
     const bool env_ok = g->search_mode == 1 && pl.n_seg > 0 && n_s > 0 && h->monotone;
     pl.envelope = env_ok && n_s > kMaxInlineS;
-    pl.envelope_short = env_ok && n_s <= kMaxInlineS;
     if (pl.envelope) pl.inline_sweep = false;
 
     // candidates per message size (grid values s <= m)
@@ -344,55 +342,67 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         pl.sc_ptiles = (n_P + kWarps * pl.sc_run - 1) / (kWarps * pl.sc_run);
     }
 
-    // Tiling of the lane <-> P kernels.  Wide CTAs (16 message sizes: 128-byte output rows; two tiles of process counts: the
-    // candidate lists are built once for both; 8 process counts per lane) against the last wave of CTAs: the choice with the
-    // smallest number of waves times the cost of a CTA, in cycles as measured on the batched workload (a message size's
-    // lists and pairs 5000, each of its tiles 5500 with 8 rows and 3200 with 4, 3500 besides; narrower output rows cost
-    // about a tenth more per halving).  64 tables, P = 2..512, 128 m: 16 x 2 tiles takes 45 us, 16 x 1 70; one table,
-    // P = 2..1024, 256 m, 64 candidates: 4 x 1 tile of 4 rows 14.7 us, of 8 rows 19.
-    {
+    // Tiling of decide_kernel and segmin_kernel: the width and the process counts of a CTA with the smallest number of CTAs (at
+    // least what the GPU holds at once) times the instructions of one of its warps: 1000 for itself, 70 per candidate of a
+    // group, 44 per process count of a group with 32 message sizes side by side, more with the shorter stores of fewer (4096
+    // tables, P = 2..512, 32 candidates, on average; 72 message sizes 473 us with 8 side by side, 100 513 with 16, 50 253 with
+    // 32).  Small grids so get many groups with few candidates each.
+    if (pl.inline_sweep && pl.n_seg > 0) {
         long long best = 0;
-        for (int rows = 8; rows >= 4; rows -= 4) {
-            const int p_tiles = (n_P + 32 * rows - 1) / (32 * rows);
-            for (int tiles = std::min(2, p_tiles); tiles >= 1; --tiles) {
-                for (int mg = kDecMG; mg >= kDecWarps; mg >>= 1) {  // never fewer than one message size per warp
-                    const int groups = (n_m + mg - 1) / mg, p_ctas = (p_tiles + tiles - 1) / tiles;
-                    const long long waves = ((long long)groups * p_ctas * h->T.n_tables + h->sm_count * 4 - 1) / (h->sm_count * 4);
-                    const long long per_m = 5000 + (rows == 8 ? 5500LL : 3200LL) * tiles;
-                    const long long cost = waves * (3500 + (std::min(mg, n_m) + kDecWarps - 1) / kDecWarps * per_m) * (kDecMG / mg + 9);
-                    if (best && cost >= best) continue;
-                    best = cost;
-                    pl.dec_rows = rows; pl.dec_mg = mg; pl.dec_tiles = tiles; pl.dec_mgroups = groups; pl.dec_ptiles = p_ctas;
-                }
+        for (int width = 32; width >= 8; width >>= 1) {
+            const int mgroups = (n_m + width - 1) / width, groups = kDecThreads / width;
+            for (int np = 512; np >= groups * 8; np >>= 1) {
+                if (np > groups * 8 && np / 2 >= n_P) continue;
+                const int tiles = (n_P + np - 1) / np;
+                const long long ctas = (long long)mgroups * tiles * h->T.n_tables;
+                const long long per_cta = 1000 + 70 * ((n_s + groups - 1) / groups) + np / groups * (width == 32 ? 44 : width == 16 ? 53 : 77);
+                const long long cost = std::max(ctas, (long long)h->sm_count * 4) * per_cta;
+                if (best && cost >= best) continue;
+                best = cost;
+                pl.ln_width = width; pl.ln_mgroups = mgroups; pl.ln_np = np; pl.ln_ptiles = tiles;
+            }
+        }
+        // All message sizes in a CTA, where there are two for every SM: threads for as many groups as leave the fewest idle
+        if (n_m <= kLineThreads && (long long)pl.ln_ptiles * h->T.n_tables >= (long long)h->sm_count * 2) {
+            double most = 0.0;
+            for (int t = 128; t <= kLineThreads; t += 32) {
+                const double busy = double(t / n_m * n_m) / t;
+                if (busy >= most) { most = busy; pl.ln_staged = t; }
             }
         }
     }
-    // The lane <-> P kernels' CTAs of 16 message sizes and two tiles are long: with few of them per SM, some SMs have one more than
-    // others and all end together.  Half as many message sizes then: P = 2..511, 128 m, 32 sizes: 64 tables (3.5 per SM) 64 -> 58
-    // us, 100 (5.4) 91 -> 81; 48 tables of 100 m (2.3) 54 -> 42; 200 (10.8) 147 -> 148.
-    // Predictions, which wait for memory besides: 48 tables of 100 m 101 -> 94 us, 140 of 128 238 -> 236.
-    pl.bc_mg = pl.dec_mg;
-    if (pl.dec_mg == kDecMG && pl.dec_rows == 8 && pl.dec_tiles == 2 && n_m > kDecMG / 2) {
-        const long long ctas = (long long)pl.dec_mgroups * pl.dec_ptiles * h->T.n_tables;
-        if (ctas > (long long)h->sm_count * 2 && ctas < (long long)h->sm_count * 8) pl.bc_mg = kDecMG / 2;
-    }
-    pl.bc_mgroups = (n_m + pl.bc_mg - 1) / pl.bc_mg;
     // One launch for both halves where the GPU holds all their CTAs at once (four per SM; its Scatter CTAs have four warps)
     {
-        const long long decide = (long long)pl.bc_mgroups * pl.dec_ptiles * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
+        const long long decide = (long long)pl.ln_mgroups * pl.ln_ptiles * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
         const long long room = (long long)h->sm_count * 4 - decide;
-        pl.select = room >= base && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
+        pl.select = pl.ln_mgroups > 0 && room >= base && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
         if (pl.select) {
             pl.sel_run = int(std::max<long long>(4, (n_P + kDecWarps * (room / base) - 1) / (kDecWarps * (room / base))));
             pl.sel_ptiles = (n_P + kDecWarps * pl.sel_run - 1) / (kDecWarps * pl.sel_run);
         }
     }
-    const int dec_p = pl.dec_tiles * 32 * pl.dec_rows;
-    for (int t = 0; t < pl.dec_ptiles; ++t) {
-        const int first = t * dec_p, last = std::min(n_P, first + dec_p) - 1;
-        const int64_t P0 = g->P ? g->P[first] : int64_t(g->P_lo) + first, P1 = g->P ? g->P[last] : int64_t(g->P_lo) + last;
-        pl.dec_pairs = std::max(pl.dec_pairs, log2_pair(P1) - log2_pair(P0) + 1);
-    }
+    // Knots: the ends of up to kLineSegs segments of a CTA's process counts, by the ratio of process counts, on the last one of
+    // a step of eight
+    std::vector<int32_t> knots;
+    if (pl.ln_mgroups > 0)
+        for (int t = 0; t < pl.ln_ptiles; ++t) {
+            const int first = t * pl.ln_np, n = std::min(n_P, first + pl.ln_np) - first;
+            auto P_at = [&](int i) { return g->P ? int64_t(g->P[first + i]) : int64_t(g->P_lo) + first + i; };
+            pl.ln_pairs = std::max(pl.ln_pairs, log2_pair(P_at(n - 1)) - log2_pair(P_at(0)) + 1);
+            const size_t at = knots.size();
+            knots.resize(at + kLineSegs + 2, n - 1);
+            int n_segs = 0, end = 0;
+            knots[at] = 0;
+            while (end < n - 1) {
+                const int left = kLineSegs - n_segs;
+                const double ratio = std::max(2.0, std::pow(double(P_at(n - 1)) / double(P_at(end)), 1.0 / left));
+                int next = std::min(n - 1, end == 0 ? 7 : end + 8);
+                while (next < n - 1 && (left == 1 || double(P_at(std::min(n - 1, next + 8))) <= ratio * double(P_at(end)))) next = std::min(n - 1, next + 8);
+                knots[at + ++n_segs] = end = next;
+            }
+            if (n_segs == 0) n_segs = 1;  // one process count
+            knots[at + kLineSegs + 1] = n_segs;
+        }
 
     // ---- device arrays ----
     std::vector<unsigned char> blob;
@@ -408,16 +418,17 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         off_s = append_aligned(blob, s32);
     }
 
-    // Short candidate lists (lane <-> P kernels): Section 2's k for every (m, candidate), as the doubles the kernels multiply with
+    if (!knots.empty()) pl.off_knots = append_aligned(blob, knots);
+    // Short candidate lists: Section 2's k for every (candidate, m), as the doubles the kernels multiply with
     const bool short_lists = pl.inline_sweep && pl.n_seg > 0 && n_s > 0;
     if (short_lists) {
-        std::vector<double> kt(size_t(n_m) * n_s, 1.0);
+        std::vector<double> kt(size_t(n_s) * n_m, 1.0);
         for (int i = 0; i < n_m; ++i) {
             const uint64_t m = g->m[i];
             for (int c = 0; c < ns_of_m[i]; ++c) {
                 const uint64_t sv = g->s ? g->s[c] : g->s_lo + uint64_t(c) * g->s_step;
                 const uint64_t q = m / sv;
-                kt[size_t(i) * n_s + c] = double(q + ((g->k_mode == 0 && q * sv != m) ? 1 : 0));
+                kt[size_t(c) * n_m + i] = double(q + ((g->k_mode == 0 && q * sv != m) ? 1 : 0));
             }
         }
         pl.off_k = append_aligned(blob, kt);
@@ -494,9 +505,10 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     // ---- scratch: sweep partials (per table batch), gap rows ----
     size_t per_table = 0;
     if (!pl.inline_sweep) per_table += size_t(pl.n_seg) * pl.n_pairs * n_P * (sizeof(double) + sizeof(uint32_t)) + 512;
-    // The gap pre-pass costs a launch: taken where the lane <-> P kernels run many CTAs per table and fill the GPU several times over
+    // The gap pre-pass costs a launch: taken where decide_kernel and segmin_kernel run many CTAs per table and fill the GPU several times over
+    // (4096 tables, P = 2..512, 128 m, 32 sizes: 1290 -> 1280 us)
     if (pl.inline_sweep && pl.n_seg > 0) {
-        const long long ctas_per_table = (long long)pl.dec_mgroups * pl.dec_ptiles;
+        const long long ctas_per_table = (long long)pl.ln_mgroups * pl.ln_ptiles;
         pl.use_gaps = ctas_per_table >= 4 && ctas_per_table * h->T.n_tables >= (long long)h->sm_count * 16;
         if (pl.use_gaps) {
             pl.gaps_stride = (1 + n_s + n_m + 1) & ~1;
@@ -544,7 +556,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
     if (pl.empty) return PLOGP_OK;
     rc = ensure_scratch(h, pl.scratch_bytes);
     if (rc != PLOGP_OK) return rc;
-    // Decision tables on short candidate lists with segmented strategies: the lane<->P decision kernel for the Broadcast half
+    // Decision tables on short candidate lists with segmented strategies: decide_kernel for the Broadcast half
     // (select_kernel for both halves of a small one).  What is left of a decision table, if only Scatter strategies, goes to
     // scatter_kernel or scatter_rows_kernel; predictions to segmin_kernel, then planes_kernel, scatter_rows_kernel and
     // fused_kernel; long lists, reduced by sweep_kernel or envelope_kernel, to fused_kernel.
@@ -597,27 +609,23 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             g_launches += unsigned(n_launches);
         }
         GridDev Gf = pl.G;
+        auto lines = [&]() {
+            LinesParams lp{};
+            lp.T = h->T; lp.G = pl.G;
+            lp.width = pl.ln_width; lp.threads = kDecThreads; lp.n_mgroups = pl.ln_mgroups; lp.n_p = pl.ln_np; lp.n_ptiles = pl.ln_ptiles; lp.n_pairs = pl.ln_pairs;
+            lp.knots = reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_knots);
+            lp.gaps = gaps; lp.gaps_stride = pl.gaps_stride;
+            lp.table0 = t0; lp.n_tables_launch = nt; lp.out_table0 = out.out_table0; lp.om = out.om;
+            return lp;
+        };
+        auto stage = [&](LinesParams &lp) { lp.staged = 1; lp.width = pl.G.n_m; lp.n_mgroups = 1; lp.threads = pl.ln_staged; };
         if (predict && pl.inline_sweep && pl.n_seg > 0) {
             // Predictions on short candidate lists: the segmented minima (planes 2, 5, 9 and the best segment sizes)
-            // come from the lane<->P kernel; the kernels behind it write the other planes.
-            SegminParams sp{};
-            sp.T = h->T; sp.G = pl.G;
-            sp.n_mgroups = pl.bc_mgroups; sp.n_ptiles = pl.dec_ptiles; sp.mg = pl.bc_mg; sp.rows = pl.dec_rows; sp.tiles = pl.dec_tiles; sp.n_pairs = pl.dec_pairs | 1;
-            sp.warps = kDecWarps;
-            // Eight warps and 32 message sizes per CTA instead of four and 16 where rows are no multiple of a 32-byte sector, on
-            // grids of many CTAs: a row segment of 16 message sizes then is two write requests instead of one, a segment of 32
-            // three instead of two, each with part of a sector at either end (1024 tables, P = 2..513, 32 sizes, 16 -> 32: n_m =
-            // 127 1.70 -> 1.36 ms, 130 1.65 -> 1.33, 145 1.96 -> 1.51).  Whole sectors gain nothing (132: 1.17 -> 1.19 ms).
-            if (pl.G.n_m % 4 != 0 && pl.bc_mg == kDecMG && pl.dec_rows == 8 &&
-                (long long)pl.dec_mgroups * pl.dec_ptiles * nt >= (long long)h->sm_count * 16) {
-                sp.warps = 2 * kDecWarps; sp.mg = 2 * kDecMG;
-                sp.n_mgroups = (pl.G.n_m + sp.mg - 1) / sp.mg;
-            }
-            sp.table0 = t0; sp.n_tables_launch = nt; sp.out_table0 = out.out_table0;
+            // come from segmin_kernel; the kernels behind it write the other planes.
+            LinesParams sp = lines();
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
-            sp.gaps = gaps; sp.gaps_stride = pl.gaps_stride;
-            sp.vec_out = (pl.G.n_m % 2 == 0) && pl.bc_mg >= 2 && reinterpret_cast<uintptr_t>(out.p_time) % 16 == 0 &&
-                         (!out.p_best_s || reinterpret_cast<uintptr_t>(out.p_best_s) % 8 == 0);
+            // rows off the sectors of the sizes, or of times and sizes; up to 16 message sizes few warps have many lines (lines.cuh)
+            if (pl.ln_staged && pl.G.n_m % 8 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.p_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.p_best_s) % 16 == 0) stage(sp);
             { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= ~kSegBits;
@@ -625,17 +633,10 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             if (!Gf.mask) continue;
         }
         if (use_decide) {
-            // Broadcast half with lanes <-> P; the Scatter half (no candidate lists) beside it or in the kernel behind it
-            DecideParams dp{};
-            dp.T = h->T; dp.G = pl.G;
+            // Broadcast half; the Scatter half (no candidate lists) beside it or in the kernel behind it
+            LinesParams dp = lines();
             dp.G.mask &= 0x3FFu;
-            dp.n_mgroups = pl.bc_mgroups; dp.n_ptiles = pl.dec_ptiles; dp.mg = pl.bc_mg; dp.rows = pl.dec_rows; dp.tiles = pl.dec_tiles; dp.n_pairs = pl.dec_pairs | 1;
-            dp.table0 = t0; dp.n_tables_launch = nt; dp.out_table0 = out.out_table0; dp.om = out.om;
             dp.d_strategy = out.d_strategy; dp.d_sbytes = out.d_sbytes; dp.d_time = out.d_time;
-            dp.envelope = pl.envelope_short ? 1 : 0;
-            dp.gaps = gaps; dp.gaps_stride = pl.gaps_stride;
-            dp.vec_out = (pl.G.n_m % 2 == 0) && pl.bc_mg >= 2 && reinterpret_cast<uintptr_t>(out.d_time) % 16 == 0 &&
-                         reinterpret_cast<uintptr_t>(out.d_sbytes) % 8 == 0 && reinterpret_cast<uintptr_t>(out.d_strategy) % 2 == 0;
             if (pl.select && !gaps && overlap) {
                 SelectParams sl{};
                 sl.decide = dp;
@@ -648,19 +649,9 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
                 g_launches += 1;
                 continue;
             }
-            // Long lists: three CTAs of 16 message sizes are less than four or five of 8 (2048 tables, P = 2..513, 128 m: 64 sizes
-            // 2.08 -> 1.89 ms; 45 sizes, of which four fit, 1.56 either way).
-            if (dp.mg == kDecMG && 4 * (decide_smem_bytes(dp) + 1024) > 228 * 1024) {
-                dp.mg = kDecMG / 2;
-                dp.n_mgroups = (pl.G.n_m + dp.mg - 1) / dp.mg;
-            }
-            // Five CTAs per SM instead of four where their shared memory fits (228 KB with 1 KB per CTA besides; 32 candidates
-            // over two tiles just do) and the grid has many of them: 4096 tables, P = 2..512, 128 m, 32 sizes 2.65 -> 2.53 ms,
-            // 2048 tables and 8 sizes 0.93 -> 0.90, 300 tables 224 -> 215 us.  Shorter grids wait for the last CTAs, which five
-            // on an SM make later (200 tables 150 -> 153 us, 64 tables 62 -> 65), and 96 registers alone are 1.5 % slower
-            // (64 sizes, which do not fit).  CTAs of fewer message sizes are short enough from 4 per SM on (100 tables 83 -> 81 us).
-            dp.ctas_per_sm = pl.dec_rows == 8 && 5 * (decide_smem_bytes(dp) + 1024) <= 228 * 1024 &&
-                             (long long)dp.n_mgroups * dp.n_ptiles * nt >= (long long)h->sm_count * (dp.mg == kDecMG ? 16 : 4) ? 5 : 4;
+            // odd rows only: with half the bytes of a plane the waits weigh more (lines.cuh has both sides)
+            if (pl.ln_staged && pl.G.n_m % 2 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.d_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 16 == 0 &&
+                reinterpret_cast<uintptr_t>(out.d_strategy) % 4 == 0) stage(dp);
             { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= 0x1C00u;

@@ -117,6 +117,13 @@ __device__ __forceinline__ float min_with2(float a, f32x2 t)
     return r;
 }
 
+// Four doubles from shared to global memory, both 32-byte aligned
+__device__ __forceinline__ void store4(double *out, const double *s)
+{
+    const double2 a = *reinterpret_cast<const double2 *>(s), b = *reinterpret_cast<const double2 *>(s + 2);
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(out), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
+}
+
 // Interval search alone: largest i with key[i] <= x (0 when x is below the table).
 __device__ __forceinline__ int interval_of(const double *s_tab, int npad, double x)
 {

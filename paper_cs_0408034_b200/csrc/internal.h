@@ -59,7 +59,7 @@ struct GridDev {
     int n_s;
     uint32_t s_lo, s_step;
     const int32_t *ns_of_m;  // device [n_m]: number of candidates s <= m (0 => unsegmented fallback)
-    const double *k_list;    // device [n_m][n_s]: Section 2's k for every (m, candidate s <= m), short candidate lists only
+    const double *k_list;    // device [n_s][n_m]: Section 2's k for every (m, candidate s <= m), short candidate lists only
     uint32_t mask;
     int k_mode;
     int lc_max;  // ceil(log2 P_hi)
@@ -181,7 +181,7 @@ struct LayoutParams {
 };
 cudaError_t launch_layout(const LayoutParams &p, cudaStream_t st);
 
-// Gap pre-pass (gaps.cu): g at every distinct argument of the lane <-> P kernels, once per table.
+// Gap pre-pass (gaps.cu): g at every distinct argument of decide_kernel and segmin_kernel, once per table.
 // Row of a table: [0] = g(1), [1 .. n_s] = g(s_i), [1 + n_s .. 1 + n_s + n_m) = g(m_j).
 struct GapsParams {
     TableDev T;
@@ -191,47 +191,37 @@ struct GapsParams {
     int stride;
 };
 
-// Decision kernel for short candidate lists (lanes <-> P): see decide.cuh
-struct DecideParams {
+// Broadcast half of the decision table, or the segmented planes of the predictions (ids 2, 5, 9), for short candidate lists:
+// see lines.cuh
+struct LinesParams {
     TableDev T;
     GridDev G;
     const double *gaps;  // rows of the gap pre-pass for this launch's tables, or nullptr: the kernel interpolates itself
     int gaps_stride;
+    int threads;    // per CTA, at most kLineThreads
+    int width;      // message sizes of a CTA, side by side: 32, 16 or 8, or all of them (staged)
+    int staged;     // outputs aligned for four cells per store (times 32, sizes 16, ids 4 bytes), all message sizes in a CTA
+    int n_p;        // process counts per CTA
     int n_mgroups, n_ptiles;
-    int mg;  // message sizes per CTA, 1..kDecMG
-    int rows;     // process counts per lane and tile: 8 or 4
-    int tiles;    // tiles of 32 x rows process counts per CTA
-    int n_pairs;  // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most, made odd: with an even number of
-                  // lines in front, neighbouring message sizes then start in different banks (an even one cost 6 % of a call)
-    int ctas_per_sm;  // 4 or 5
-    int envelope;  // lower-envelope search: the lists keep only the candidates that can win (see decide.cuh)
-    int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16 / 8 / 2-byte aligned bases)
+    int n_pairs;    // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most
+    const int32_t *knots;  // device [n_ptiles][kLineSegs + 2]: indices inside the CTA's process counts, number of segments
     int table0, n_tables_launch;
     int out_table0;  // table whose results sit at the start of the output arrays
     OutMap om;
-    uint8_t *d_strategy;
+    uint8_t *d_strategy;  // decision
     uint32_t *d_sbytes;
     double *d_time;
+    double *p_time;      // predictions: [n_tables][13][n_P][n_m]
+    uint32_t *p_best_s;  // [n_tables][3][n_P][n_m], or nullptr
 };
+constexpr int kLineThreads = 256;
+constexpr int kLineSegs = 4;  // segments of a CTA's process counts, at most
+using DecideParams = LinesParams;
+using SegminParams = LinesParams;
+size_t decide_smem_bytes(const DecideParams &p);
 
 constexpr int kDecThreads = 128;
 constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kDecMG = 16;                             // message sizes per CTA (at most), split over the warps
-
-// segmin_kernel (segmented minima of plogp_predict on short candidate lists, lanes <-> P): see segmin.cu
-struct SegminParams {
-    TableDev T;
-    GridDev G;
-    const double *gaps;  // as in DecideParams
-    int gaps_stride;
-    int vec_out;  // outputs aligned for two message sizes per store (n_m even, 16-byte aligned times, 8-byte aligned sizes)
-    int n_mgroups, n_ptiles;
-    int mg, rows, tiles, n_pairs;  // as in DecideParams (mg up to 4 * warps)
-    int warps;  // per CTA: 4, or 8 (rows = 8)
-    int table0, n_tables_launch, out_table0;
-    double *p_time;      // [n_tables][13][n_P][n_m]: planes 2, 5, 9 are written
-    uint32_t *p_best_s;  // [n_tables][3][n_P][n_m], or nullptr
-};
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kFusedR = 4;   // process counts per thread and pass in the fused kernel
@@ -252,7 +242,6 @@ struct SelectParams {
     ScatterParams scatter;
     int n_decide;
 };
-size_t decide_smem_bytes(const DecideParams &p);
 size_t scatter_smem_bytes(const ScatterParams &p, int warps);
 cudaError_t launch_select(SelectParams &p, cudaStream_t st);
 cudaError_t launch_fp64_probe(double *d_sink, int iters, int blocks, cudaStream_t st);

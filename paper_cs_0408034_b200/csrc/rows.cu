@@ -20,11 +20,6 @@ __host__ __device__ inline int rows_per_flush(int n_m) { return n_m >= kRowsCell
 
 // A piece of n cells starts `shift` cells behind a group of four that is aligned in the plane; it is staged with the same
 // shift, so that a group is one 32-byte load and store.  The cells of the groups at either end go one by one.
-__device__ __forceinline__ void store4(double *out, const double *s)
-{
-    const double2 a = *reinterpret_cast<const double2 *>(s), b = *reinterpret_cast<const double2 *>(s + 2);
-    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(out), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y) : "memory");
-}
 
 // PREDICT: times of ids 11 and 12 instead of the decision.  ALL: all ids that the kernel writes are enabled.
 template <bool PREDICT, bool ALL>

@@ -1,19 +1,18 @@
 // select_kernel: both halves of a decision table in one launch, for grids that the GPU holds in one go.  There a call is
-// mostly launches: the first CTAs take the Broadcast half (decide.cuh), the others the Scatter half (scatter.cuh, with the
+// mostly launches: the first CTAs take the Broadcast half (lines.cuh), the others the Scatter half (scatter.cuh, with the
 // Broadcast half's four warps per CTA).  One table, P = 2..50, 19 message sizes, 7 candidates: one launch less is 3 us of
 // host time a call and 8.2 -> 6.2 us between calls on the GPU.
-#include "decide.cuh"
+#include "lines.cuh"
 #include "scatter.cuh"
 
 namespace plogp {
 
-template <bool ENV, bool CONTIG>
+template <bool CONTIG>
 __global__ void __launch_bounds__(kDecThreads, 4) select_kernel(const SelectParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (blockIdx.x < static_cast<unsigned>(p.n_decide)) {
-        if (p.decide.rows == 8) decide_block<ENV, 8>(p.decide, blockIdx.x, smem_raw);
-        else decide_block<ENV, 4>(p.decide, blockIdx.x, smem_raw);
+        lines_block<false, false>(p.decide, blockIdx.x, smem_raw);
     } else {
         scatter_block<CONTIG ? kChainRun : kChainRange, false, 1, kDecWarps>(p.scatter, blockIdx.x - p.n_decide, smem_raw);
     }
@@ -27,8 +26,7 @@ cudaError_t launch_select(SelectParams &p, cudaStream_t st)
     p.n_decide = static_cast<int>(nd);
     const size_t a = decide_smem_bytes(p.decide), b = scatter_smem_bytes(p.scatter, kDecWarps);
     const bool contig = p.scatter.G.P_list == nullptr;
-    const auto kernel = p.decide.envelope ? (contig ? select_kernel<true, true> : select_kernel<true, false>)
-                                          : (contig ? select_kernel<false, true> : select_kernel<false, false>);
+    const auto kernel = contig ? select_kernel<true> : select_kernel<false>;
     return launch(kernel, static_cast<unsigned>(nd + ns), 1, kDecThreads, a > b ? a : b, st, false, p);
 }
 

@@ -1,0 +1,88 @@
+"""GPU parity of the Broadcast half and the segmented planes on short candidate lists: lines ruled out for ranges of process
+counts, message sizes side by side in 8, 16 or 32 threads or all of a table's in a CTA."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+from paper_cs_0408034_b200 import workloads as wl
+from parity import check_decision, check_prediction, oracle_tables
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def plogp():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_cs_0408034_b200 import plogp as mod
+    return mod
+
+
+def both(plogp, w, tables=None):
+    """Decision table and predictions against the oracle (times to 1e-12, picks exact: tests/parity.py)."""
+    import torch
+    ot = oracle_tables(w)
+    with plogp.Tables.from_workload(w) as tabs:
+        dec = plogp.select_best(tabs, w)
+        pred = plogp.predict(tabs, w)
+        torch.cuda.synchronize()
+        assert check_decision(w, ot, dec, tables=tables) + check_prediction(w, ot, pred, tables=tables) > 0
+
+
+@pytest.mark.parametrize("n_m", [1, 8, 9, 16, 17, 32, 33])
+@pytest.mark.parametrize("n_s,n_P,k_mode", [(1, 1, 0), (31, 7, 1), (32, 65, 0), (33, 130, 0), (64, 513, 1)])
+def test_widths_and_steps(plogp, n_m, n_s, n_P, k_mode):
+    both(plogp, wl_grid(n_tables=2, n_P=n_P, n_m=n_m, n_s=n_s, k_mode=k_mode))
+
+
+def wl_grid(n_tables, n_P, n_m, n_s, k_mode=0, P_lo=2):
+    w = wl.config4(n_tables=n_tables, P_hi=P_lo + n_P - 1, n_m=n_m, n_s=n_s, seed_offset=n_P + n_m)
+    return replace(w, P_lo=P_lo, k_mode=k_mode)
+
+
+@pytest.mark.parametrize("ids", [(0,), (1, 2), (2,), (3, 5), (4, 5), (5,), (9,), (2, 9), (1, 4, 8), (0, 3, 6), (2, 5, 7), range(10)])
+def test_strategies_alone_and_together(plogp, ids):
+    """Lines without pairs, pairs without lines, rendezvous variants with and without their siblings, whole messages."""
+    w = wl_grid(n_tables=2, n_P=90, n_m=20, n_s=20)
+    m = np.unique(np.concatenate([w.m, w.s_list[3:6]]))  # a candidate of the whole message's size
+    both(plogp, replace(w, m=m, s_list=w.s_list[2:], strategy_mask=sum(1 << i for i in ids)))
+
+
+@pytest.mark.parametrize("kind", ["flat", "stairs", "falls", "latency"])
+@pytest.mark.parametrize("n_s", [20, 64])
+def test_lines_close_to_one_another(plogp, kind, n_s):
+    """Equal gaps over many sizes, gaps that fall, a latency far above the gaps: many candidates within rounding."""
+    w = wl_grid(n_tables=3, n_P=300, n_m=12, n_s=n_s)
+    g = w.gaps.copy()
+    if kind == "flat":
+        g[:, :] = g[:, :1]
+    elif kind == "stairs":
+        g = np.repeat(g[:, ::8], 8, axis=1)
+    elif kind == "falls":
+        g[:, 5:40:3] *= 0.5
+    both(plogp, replace(w, gaps=np.ascontiguousarray(g), latency=w.latency * (1e9 if kind == "latency" else 1.0)))
+
+
+@pytest.mark.parametrize("n_m,n_P,n_s,listed", [(17, 21, 9, False), (33, 520, 33, False), (50, 16, 8, False), (127, 40, 20, True), (129, 9, 64, False), (255, 33, 5, False), (256, 8, 3, False)])
+def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed):
+    """Many tables: the cells of a step put together in shared memory.  The same as with outputs aligned for single elements,
+    which are stored one by one, and as the oracle's for some tables."""
+    import torch
+    w = wl_grid(n_tables=300, n_P=n_P, n_m=n_m, n_s=n_s)
+    if listed:
+        w = replace(w, P_list=(2 + 3 * np.arange(n_P)).astype(np.int32))
+    both(plogp, w, tables=[0, 151, 299])
+
+    def off_by_one(x):
+        return torch.zeros(x.numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x.shape)
+
+    with plogp.Tables.from_workload(w) as tabs:
+        dec, pred = plogp.select_best(tabs, w), plogp.predict(tabs, w)
+        d = plogp.DecisionTable(*(off_by_one(x) for x in (dec.strategy, dec.s_bytes, dec.time)))
+        plogp.select_best(tabs, w, out=d)
+        p = plogp.Prediction(off_by_one(pred.time), off_by_one(pred.best_s))
+        plogp.predict(tabs, w, out=p)
+        for a, b in ((d.strategy, dec.strategy), (d.s_bytes, dec.s_bytes), (d.time, dec.time)):
+            assert a[:, 0].equal(b[:, 0])
+        assert p.best_s.equal(pred.best_s) and all(p.time[:, i].equal(pred.time[:, i]) for i in (2, 5, 9))
