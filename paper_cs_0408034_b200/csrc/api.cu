@@ -448,13 +448,22 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         while ((2 << pl.env_coarse_log) < (n_P + 1023) / 1024) ++pl.env_coarse_log;
         pl.env_max_coarse = envelope_coarse_of(n_P - 1, pl.env_coarse_log) + 2;
     } else if (!pl.inline_sweep) {
-        pl.chunk_len = std::max(2048, ((ns_max + 31) / 32 + kSweepSub - 1) / kSweepSub * kSweepSub);
+        const int p_tiles = (n_P + 32 * kSweepR - 1) / (32 * kSweepR);
+        pl.sweep_wp = kWarps;
+        while (pl.sweep_wp > 1 && pl.sweep_wp / 2 >= p_tiles - 1) pl.sweep_wp >>= 1;
+        pl.sweep_ptiles = 1 + (p_tiles - 1 + pl.sweep_wp - 1) / pl.sweep_wp;
+        // Chunks: about six CTAs per SM, a CTA's upper bounds cost as much as 25 sub-chunks
+        long long cands = 0;
+        for (int i = 0; i < n_m; ++i) cands += ns_of_m[i];
+        const long long share = cands * pl.sweep_ptiles * h->T.n_tables / ((long long)h->sm_count * 6);
+        pl.chunk_len = int(std::min<long long>(std::max<long long>(2048, (share + kSweepSub - 1) / kSweepSub * kSweepSub), (ns_max + kSweepSub - 1) / kSweepSub * kSweepSub));
+        pl.chunk_len = std::min(std::max(pl.chunk_len, kSweepSub), 1 << 20);
         std::vector<int32_t> pair_base(n_m + 1, 0);
         struct Pair { int32_t m, chunk, row, len; };
         std::vector<Pair> pairs;
         for (int i = 0; i < n_m; ++i) {
             pair_base[i] = int32_t(pairs.size());
-            for (int c = 0; c * pl.chunk_len < ns_of_m[i]; ++c)
+            for (int c = 0; (long long)c * pl.chunk_len < ns_of_m[i]; ++c)
                 pairs.push_back({i, c, int32_t(pairs.size()), std::min(pl.chunk_len, ns_of_m[i] - c * pl.chunk_len)});
         }
         pair_base[n_m] = int32_t(pairs.size());
@@ -466,10 +475,6 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         pl.off_pair_chunk = append_aligned(blob, pc);
         pl.off_pair_row = append_aligned(blob, pr);
         pl.off_pair_base = append_aligned(blob, pair_base);
-        const int p_tiles = (n_P + 32 * kSweepR - 1) / (32 * kSweepR);
-        pl.sweep_wp = kWarps;
-        while (pl.sweep_wp > 1 && pl.sweep_wp / 2 >= p_tiles) pl.sweep_wp >>= 1;
-        pl.sweep_ptiles = (p_tiles + pl.sweep_wp - 1) / pl.sweep_wp;
     }
 
     if (blob.size() > slot.grid_cap) {

@@ -74,7 +74,7 @@ struct SweepParams {
     const int32_t *pair_chunk;  // device [n_pairs]
     const int32_t *pair_row;    // device [n_pairs]: row id of the pair (= pair_base[m] + chunk)
     int n_pairs, n_ptiles, chunk_len;
-    int wp;  // tiles of 256 process counts per CTA (1, 2, 4 or 8); its 8 warps split the candidates 8 / wp ways
+    int wp;  // tiles of 256 process counts per CTA behind the first tile (1, 2, 4 or 8); its 8 warps split the candidates 8 / wp ways
     double *part_time;   // [n_tables_batch][n_seg][n_pairs][n_P]
     uint32_t *part_idx;  // same shape: index of s in the candidate list
     int n_seg;           // enabled segmented strategies (slots in id order)
@@ -227,8 +227,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kFusedR = 4;   // process counts per thread and pass in the fused kernel
 constexpr int kSweepR = 8;   // process counts per thread in the sweep kernel
 constexpr int kSweepSub = 256;  // candidates staged per sub-chunk
-constexpr int kSweepU = 8;      // candidates per iteration of the sweep kernel's inner loop
-constexpr int kSweepBatch = 128; // candidates per comparison of the bounds with the best times
+constexpr int kSweepGroups = kSweepSub / 32;  // groups of a sub-chunk
 constexpr int kSweepSeeds = 128;  // log-spaced candidates that the upper bounds start from
 constexpr int kMaxInlineS = 64;
 

@@ -4,10 +4,9 @@
 //
 // This file:
 //   sweep_kernel   lane <-> process count P.  One CTA owns one message size m, a tile of P values
-//                  and a chunk of the candidate segment sizes; the per-(m, s) line coefficients are
-//                  computed once per CTA into shared memory and broadcast to all lanes, so a model
-//                  cell costs half a packed FP32 multiply-add and half a minimum; what the FP32 bounds leave
-//                  open is decided in FP64.  Used when the candidate list is long.
+//                  and a chunk of the candidate segment sizes, whose lines are bounded from below for many
+//                  candidates at a time; what the FP32 bounds leave open is decided in FP64.  Used when the
+//                  candidate list is long.
 //   fused_kernel   lane <-> message size m (32 consecutive m per warp, so every output row is
 //                  written as full, aligned segments).  Evaluates all enabled strategies, reduces the sweep
 //                  kernel's partial minima where segmented ones are among them, keeps the
@@ -29,24 +28,23 @@ namespace plogp {
 //   id 5: (P-1) (g(s)+L) + g(s)(k-1)          = fma(P-1, B, C)   B = g(s)+L, C = g(s)(k-1)
 //   id 2: (P-1) (g(s) k) + L                  = fma(P-1, Q, L)   Q = g(s) k
 //   id 9: floor(log2 P) g(s) k + ceil(log2 P) L = fma(lf, Q, lc L)
-// so the CTA computes (B, C, Q) once per candidate and every lane spends one multiply-add per cell.
+// so the CTA computes (B, C, Q) once per candidate, and a line of the smallest B and C (or Q) of some candidates is below all of
+// theirs at every process count.
 //
-// Every cell is first evaluated as a lower bound: coefficients and process count rounded down to FP32, the packed
-// fused multiply-add rounded down as well.  All terms are non-negative, so the bound is never above the FP64 time.
-// The smallest bound of a batch of candidates, per process count, is compared with an upper bound of the best time
-// known there; only where it is not above does the batch come back, group by group, to the exact FP64 comparison.
-// The results are those of the exhaustive FP64 search, bit for bit.  The upper bounds start from a few log-spaced
-// candidates of the whole list (rounded up in FP32), so a chunk far from the optimum never leaves the fast loop.
-// The best times themselves are touched by the exact pass alone and live in shared memory.
+// All terms are non-negative, and coefficients, process count and multiply-add are rounded down to FP32, so a bound is never above
+// the FP64 time.  It is taken three times, each time for the process counts (lanes) in which the one before is not above the best
+// time known there:
+//   * for a sub-chunk of 256 candidates from its first and last size alone (the smallest g between them, the last one's number
+//     of segments), before any candidate is looked at;
+//   * for its groups of 32, from the smallest coefficients;
+//   * for the group's candidates one by one.
+// Four at a time, what is left is compared in FP64.  The results are those of the exhaustive FP64 search, bit for bit.  The upper
+// bounds of the best times start from log-spaced candidates of the whole list (rounded up in FP32), so a chunk far from the
+// optimum never leaves the first step.  The best times themselves are touched by the exact pass alone and live in shared memory.
 //
-// What bounds it: issue.  Two cells cost one packed multiply-add and one three-input minimum, 2.1 cycles of a scheduler
-// per 32 cells by themselves (an FP64 multiply-add with an integer compare of the high words, as the loop had it before:
-// 4.6); with list building, barriers and exact passes (2 %) 2.5.  P = 2..4096, 128 message sizes, 1.25e11 cells of
-// ids 2 and 5: 15.05 -> 8.5 ms.  Scalar multiply-adds, 16 process counts per lane, lanes <-> candidates and packing
-// along P run at the same 2.0 - 2.5 cycles.
-// The exact pass is rare as long as candidates' times differ by more than FP32 rounding where they are best.  Equal gaps over
-// many sizes are no matter (g flat below 64 KB or in stairs: 1.1 to 1.7 times as fast as the FP64 loop).  A latency 1e7 times the
-// gaps or more is (0.7 times), and so are times outside FP32's range, where every cell goes through it (0.2 times).
+// What bounds it: the exact passes of the CTAs that have the best sizes, one vote after another, while the others are done.  P =
+// 2..4096, 128 message sizes, every 4 B up to 1 MB, ids 2 and 5: 8.4 ms with a bound of every cell, 1.33 with groups of 32, 1.23 with
+// the first 256 process counts in CTAs of their own, 0.64 with sub-chunks passed over.
 //
 // A warp owns 256 consecutive process counts (lane + 32 r).  The CTA's 8 warps cover p.wp such tiles side by side and
 // split the candidates of a sub-chunk 8 / p.wp ways, so that a short range of process counts leaves no warp idle.
@@ -66,7 +64,10 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     double *s_best = s_q + 2 * kSweepSub;                               // [kNid][kWarps][R][32]
     float *s_bf = reinterpret_cast<float *>(s_best + kNid * kWarps * R * 32);  // [2][kSweepSub]
     float *s_cf = s_bf + 2 * kSweepSub, *s_qf = s_cf + 2 * kSweepSub;
-    uint32_t *s_idx = reinterpret_cast<uint32_t *>(s_qf + 2 * kSweepSub);      // [kNid][kWarps][R][32]
+    float *s_gb = s_qf + 2 * kSweepSub, *s_gc = s_gb + 2 * kSweepGroups, *s_gq = s_gc + 2 * kSweepGroups;  // [2][kSweepGroups]: smallest of a group's
+    float *s_lb = s_gq + 2 * kSweepGroups, *s_lc = s_lb + kThreads, *s_lq = s_lc + kThreads;  // [kThreads]: bounds of a sub-chunk's
+    int *s_need = reinterpret_cast<int *>(s_lq + kThreads);                                   // [kThreads]: it has to be looked at
+    uint32_t *s_idx = reinterpret_cast<uint32_t *>(s_need + kThreads);                        // [kNid][kWarps][R][32]
 
     const int tid = threadIdx.x;
     const int pi = blockIdx.x / p.n_ptiles;
@@ -87,25 +88,28 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     const double L = p.T.lat[table];
 
     const int lane = tid & 31, warp = tid >> 5;
-    const int wp = p.wp, wc = kWarps / wp, my_p = warp & (wp - 1), my_c = warp / wp;
-    const int c_len = kSweepSub / wc, batch = min(c_len, kSweepBatch);  // this warp's candidates of a sub-chunk
-    const int p_first = (ptile * wp + my_p) * (32 * R) + lane;
+    // The first 256 process counts have CTAs of their own, whose warps split the candidates: where P is small the best size
+    // moves fast, and most of the groups that have to be looked at are there.
+    const int wp = ptile == 0 ? 1 : p.wp, wc = kWarps / wp, my_p = warp & (wp - 1), my_c = warp / wp;
+    const int tile0 = ptile == 0 ? 0 : 32 * R * (1 + (ptile - 1) * wp);
+    const int g_len = kSweepGroups / wc;  // this warp's groups of a sub-chunk
+    const int p_first = tile0 + my_p * (32 * R) + lane;
     // a process count past the last one repeats the last one
     auto P_of = [&](int r) { return P_at(p.G, min(p_first + 32 * r, p.G.n_P - 1)); };
     auto x_exact = [&](int P) { return IS9 ? static_cast<double>(31 - __clz(P)) : static_cast<double>(P - 1); };
     auto c_exact = [&](int P) { return IS9 ? static_cast<double>(32 - __clz(P - 1)) * L : L; };
 
-    f32x2 x2[R], c2[IS9 ? R : 1];  // multiplier and, where the offset is not a candidate's, offset, rounded down, twice each
-    float T2[HAS2 || IS9 ? R : 1], T5[HAS5 ? R : 1];  // upper bounds of the best times
+    float xf[R], cf[IS9 ? R : 1];  // multiplier and, where the offset is not a candidate's, offset, rounded down
+    float T2[QL ? R : 1], T5[HAS5 ? R : 1];  // upper bounds of the best times
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int P = P_of(r);
-        x2[r] = splat2(IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_rd(P - 1));
-        if (IS9) c2[r] = splat2(__double2float_rd(c_exact(P)));
+        xf[r] = IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_rd(P - 1);
+        if (IS9) cf[r] = __double2float_rd(c_exact(P));
         if (QL) T2[r] = CUDART_INF_F;
         if (HAS5) T5[r] = CUDART_INF_F;
     }
-    if (!IS9) c2[0] = splat2(__double2float_rd(L));
+    if (!IS9) cf[0] = __double2float_rd(L);
     double *best = s_best + warp * R * 32 + lane;  // + id slot * kWarps * R * 32 + r * 32
     uint32_t *bidx = s_idx + warp * R * 32 + lane;
     constexpr int kIdStep = kWarps * R * 32;
@@ -125,16 +129,23 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     };
     auto fill = [&](int sub, int buf) {
         const int si = s_begin + sub * kSweepSub + tid, o = buf * kSweepSub + tid;
-        double B = 0.0, C = CUDART_INF, Q = CUDART_INF;  // padding: the bound is +inf
+        double B = CUDART_INF, C = CUDART_INF, Q = CUDART_INF;  // padding: the bound is +inf
         if (si < s_end) coefficients(si, B, C, Q);
+        // a warp's candidates are a group; non-negative floats are ordered as whole numbers
         if (HAS5) {
+            const float b = __double2float_rd(B), c = __double2float_rd(C);
             s_bc[o] = make_double2(B, C);
-            s_bf[o] = __double2float_rd(B);
-            s_cf[o] = __double2float_rd(C);
+            s_bf[o] = b;
+            s_cf[o] = c;
+            const unsigned b_min = __reduce_min_sync(kFull, __float_as_uint(b)), c_min = __reduce_min_sync(kFull, __float_as_uint(c));
+            if (lane == 0) { s_gb[o >> 5] = __uint_as_float(b_min); s_gc[o >> 5] = __uint_as_float(c_min); }
         }
         if (QL) {
+            const float q = __double2float_rd(Q);
             s_q[o] = Q;
-            s_qf[o] = __double2float_rd(Q);
+            s_qf[o] = q;
+            const unsigned q_min = __reduce_min_sync(kFull, __float_as_uint(q));
+            if (lane == 0) s_gq[o >> 5] = __uint_as_float(q_min);
         }
     };
 
@@ -177,99 +188,139 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     }
     __syncthreads();
 
-    fill(0, 0);
-    __syncthreads();
-    for (int sub = 0; sub < n_sub; ++sub) {
-        const int buf = sub & 1;
-        if (sub + 1 < n_sub) fill(sub + 1, buf ^ 1);
-        const uint32_t base = static_cast<uint32_t>(s_begin + sub * kSweepSub);
-#pragma unroll 1
-        for (int j0 = my_c * c_len; j0 < (my_c + 1) * c_len; j0 += batch) {
-            const float *bf = s_bf + buf * kSweepSub + j0, *cf = s_cf + buf * kSweepSub + j0, *qf = s_qf + buf * kSweepSub + j0;
-            float mn5[HAS5 ? R : 1], mn2[QL ? R : 1];
+    // rows in which the line of these coefficients is not above the best time known: bit r: id 2 or 9, bit 16 + r: id 5
+    auto rows_of = [&](float b, float c, float q) {
+        unsigned hit = 0;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (HAS5) mn5[r] = CUDART_INF_F;
-                if (QL) mn2[r] = CUDART_INF_F;
+        for (int r = 0; r < R; ++r) {
+            if (QL && __fmaf_rd(xf[r], q, cf[IS9 ? r : 0]) <= T2[r]) hit |= 1u << r;
+            if (HAS5 && __fmaf_rd(xf[r], b, c) <= T5[r]) hit |= 0x10000u << r;
+        }
+        return hit;
+    };
+    for (int block0 = 0; block0 < n_sub; block0 += kThreads) {
+        // ---- bounds of whole sub-chunks, a thread each: the smallest g between the first and the last size (at them, or at a
+        // breakpoint between them), the last one's number of segments ----
+        const int n_block = min(kThreads, n_sub - block0);
+        __syncthreads();
+        if (tid < n_block) {
+            const int first = s_begin + (block0 + tid) * kSweepSub, last = min(first + kSweepSub, s_end) - 1;
+            const uint32_t s_last = s_at(p.G, last);
+            const double sa = static_cast<double>(s_at(p.G, first)), sb = static_cast<double>(s_last);
+            const int npad = p.T.npad, ia = interval_of(s_tab, npad, sa), ib = interval_of(s_tab, npad, sb);
+            const double ga = gap_at(s_tab, npad, sa), gz = gap_at(s_tab, npad, sb);
+            double g_min = fmin(ga, gz), g_max = fmax(fmax(ga, gz), s_tab[npad + ia]);
+            for (int i = ia + 1; i <= ib; ++i) {
+                g_min = fmin(g_min, s_tab[npad + i]);
+                g_max = fmax(g_max, s_tab[npad + i]);
             }
-#pragma unroll 1
-            for (int i = 0; i < batch; i += kSweepU) {
-#pragma unroll
-                for (int u = 0; u < kSweepU; u += 4) {
-                    if (HAS5) {
-                        const f32x2x2 bb = *reinterpret_cast<const f32x2x2 *>(bf + i + u), cc = *reinterpret_cast<const f32x2x2 *>(cf + i + u);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) mn5[r] = min_with2(mn5[r], fma2_down(x2[r], bb.x, cc.x));
-#pragma unroll
-                        for (int r = 0; r < R; ++r) mn5[r] = min_with2(mn5[r], fma2_down(x2[r], bb.y, cc.y));
-                    }
-                    if (QL) {
-                        const f32x2x2 qq = *reinterpret_cast<const f32x2x2 *>(qf + i + u);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) mn2[r] = min_with2(mn2[r], fma2_down(x2[r], qq.x, c2[IS9 ? r : 0]));
-#pragma unroll
-                        for (int r = 0; r < R; ++r) mn2[r] = min_with2(mn2[r], fma2_down(x2[r], qq.y, c2[IS9 ? r : 0]));
-                    }
-                }
-            }
-            unsigned hit = 0;  // bit r: id 2 or 9, bit 16 + r: id 5
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (QL && mn2[r] <= T2[r]) hit |= 1u << r;
-                if (HAS5 && mn5[r] <= T5[r]) hit |= 0x10000u << r;
-            }
-            if (__any_sync(kFull, hit != 0)) {
-                // Exact pass over the batch for the flagged rows: candidates in ascending order, strict '<' (smallest s on
-                // ties).  The bounds in T only ever shrink towards the best time, so nothing that could win is passed over.
-#pragma unroll 1
-                for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
-                    const int bit = __ffs(rows) - 1, r = bit & 15;
-                    const bool five = HAS5 && (bit >> 4);
-                    const int P = P_of(r);
-                    const double x = x_exact(P), c = c_exact(P);
-                    const float xf = IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_rd(P - 1), cfl = __double2float_rd(c);
-                    const int o = (five && HAS2 ? kIdStep : 0) + r * 32;
-                    double bt = best[o];
-                    uint32_t bi = bidx[o];
-                    float T = CUDART_INF_F;
-#pragma unroll
-                    for (int q = 0; q < R; ++q) {
-                        if (HAS5 && five && q == r) T = T5[q];
-                        if (QL && !five && q == r) T = T2[q];
-                    }
-#pragma unroll 1
-                    for (int i = 0; i < batch; i += 4) {
-                        float t[4];
-                        if (HAS5 && five) {
-                            const float4 b4 = *reinterpret_cast<const float4 *>(bf + i), c4 = *reinterpret_cast<const float4 *>(cf + i);
-                            t[0] = __fmaf_rd(xf, b4.x, c4.x); t[1] = __fmaf_rd(xf, b4.y, c4.y);
-                            t[2] = __fmaf_rd(xf, b4.z, c4.z); t[3] = __fmaf_rd(xf, b4.w, c4.w);
-                        } else {
-                            const float4 q4 = *reinterpret_cast<const float4 *>(qf + i);
-                            t[0] = __fmaf_rd(xf, q4.x, cfl); t[1] = __fmaf_rd(xf, q4.y, cfl);
-                            t[2] = __fmaf_rd(xf, q4.z, cfl); t[3] = __fmaf_rd(xf, q4.w, cfl);
-                        }
-                        if (__any_sync(kFull, fminf(fminf(t[0], t[1]), fminf(t[2], t[3])) <= T)) {
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const int e = buf * kSweepSub + j0 + i + u;
-                                const double tt = five ? fma(x, s_bc[e].x, s_bc[e].y) : fma(x, s_q[e], c);
-                                if (tt < bt) { bt = tt; bi = base + j0 + i + u; }
-                            }
-                            T = fminf(T, __double2float_ru(bt));
-                        }
-                    }
-                    best[o] = bt;
-                    bidx[o] = bi;
-#pragma unroll
-                    for (int q = 0; q < R; ++q) {
-                        if (HAS5 && five && q == r) T5[q] = T;
-                        if (QL && !five && q == r) T2[q] = T;
-                    }
-                }
-            }
+            // an interpolated g is off by the rounding of the larger of its interval's ends
+            const double g = fmax(fma(g_max, -0x1p-48, g_min), 0.0), k = static_cast<double>(segments(m_u, s_last, p.G.k_mode));
+            s_lb[tid] = __double2float_rd(g + L);
+            s_lc[tid] = __double2float_rd(fmin(g * (k - 1.0), 1.7e308));
+            s_lq[tid] = __double2float_rd(fmin(g * k, 1.7e308));
+            s_need[tid] = 0;
         }
         __syncthreads();
+#pragma unroll 2
+        for (int i = 0; i < n_block; ++i)
+            if (__any_sync(kFull, rows_of(s_lb[i], s_lc[i], s_lq[i]) != 0) && lane == 0) s_need[i] = 1;
+        __syncthreads();
+        auto next = [&](int i) {
+            while (i < n_block && !s_need[i]) ++i;
+            return i;
+        };
+        int sub = next(0);
+        if (sub < n_block) fill(block0 + sub, 0);
+        __syncthreads();
+        for (int buf = 0; sub < n_block; buf ^= 1) {
+            const int then = next(sub + 1);
+            if (then < n_block) fill(block0 + then, buf ^ 1);
+            const uint32_t base = static_cast<uint32_t>(s_begin + (block0 + sub) * kSweepSub);
+            const float *const gb = s_gb + buf * kSweepGroups + my_c * g_len, *const gc = s_gc + buf * kSweepGroups + my_c * g_len,
+                        *const gq = s_gq + buf * kSweepGroups + my_c * g_len;
+            float b_all = CUDART_INF_F, c_all = CUDART_INF_F, q_all = CUDART_INF_F;
+            for (int g = 0; g < g_len; ++g) {
+                if (HAS5) { b_all = fminf(b_all, gb[g]); c_all = fminf(c_all, gc[g]); }
+                if (QL) q_all = fminf(q_all, gq[g]);
+            }
+            if (__any_sync(kFull, rows_of(b_all, c_all, q_all) != 0))
+#pragma unroll 1
+            for (int g = 0; g < g_len; ++g) {
+                const unsigned hit = rows_of(HAS5 ? gb[g] : 0.f, HAS5 ? gc[g] : 0.f, QL ? gq[g] : 0.f);
+                const int j0 = 32 * (my_c * g_len + g);
+                const float *bf = s_bf + buf * kSweepSub + j0, *cf4 = s_cf + buf * kSweepSub + j0, *qf = s_qf + buf * kSweepSub + j0;
+                if (__any_sync(kFull, hit != 0)) {
+                    // Exact pass over the group for the flagged rows: candidates in ascending order, strict '<' (smallest s on
+                    // ties).  The bounds in T only ever shrink towards the best time, so nothing that could win is passed over.
+#pragma unroll 1
+                    for (unsigned rows = __reduce_or_sync(kFull, hit); rows; rows &= rows - 1) {
+                        const int bit = __ffs(rows) - 1, r = bit & 15;
+                        const bool five = HAS5 && (bit >> 4);
+                        const int P = P_of(r);
+                        const double x = x_exact(P), c = c_exact(P);
+                        const float xr = IS9 ? static_cast<float>(31 - __clz(P)) : __int2float_rd(P - 1), cfl = __double2float_rd(c);
+                        const int o = (five && HAS2 ? kIdStep : 0) + r * 32;
+                        double bt = best[o];
+                        uint32_t bi = bidx[o];
+                        float T = CUDART_INF_F;
+#pragma unroll
+                        for (int q = 0; q < R; ++q) {
+                            if (HAS5 && five && q == r) T = T5[q];
+                            if (QL && !five && q == r) T = T2[q];
+                        }
+                        // the group's candidates one by one, in FP32 first and all at once: mostly none is not above
+                        {
+                            const f32x2 x2 = splat2(xr), c2 = splat2(cfl);
+                            float low = CUDART_INF_F;
+#pragma unroll
+                            for (int i = 0; i < 32; i += 4) {
+                                f32x2x2 a, c{c2, c2};
+                                if (HAS5 && five) {
+                                    a = *reinterpret_cast<const f32x2x2 *>(bf + i);
+                                    c = *reinterpret_cast<const f32x2x2 *>(cf4 + i);
+                                } else {
+                                    a = *reinterpret_cast<const f32x2x2 *>(qf + i);
+                                }
+                                low = min_with2(min_with2(low, fma2_down(x2, a.x, c.x)), fma2_down(x2, a.y, c.y));
+                            }
+                            if (!__any_sync(kFull, low <= T)) continue;
+                        }
+#pragma unroll 1
+                        for (int i = 0; i < 32; i += 4) {
+                            float t[4];
+                            if (HAS5 && five) {
+                                const float4 b4 = *reinterpret_cast<const float4 *>(bf + i), c4 = *reinterpret_cast<const float4 *>(cf4 + i);
+                                t[0] = __fmaf_rd(xr, b4.x, c4.x); t[1] = __fmaf_rd(xr, b4.y, c4.y);
+                                t[2] = __fmaf_rd(xr, b4.z, c4.z); t[3] = __fmaf_rd(xr, b4.w, c4.w);
+                            } else {
+                                const float4 q4 = *reinterpret_cast<const float4 *>(qf + i);
+                                t[0] = __fmaf_rd(xr, q4.x, cfl); t[1] = __fmaf_rd(xr, q4.y, cfl);
+                                t[2] = __fmaf_rd(xr, q4.z, cfl); t[3] = __fmaf_rd(xr, q4.w, cfl);
+                            }
+                            if (__any_sync(kFull, fminf(fminf(t[0], t[1]), fminf(t[2], t[3])) <= T)) {
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    const int e = buf * kSweepSub + j0 + i + u;
+                                    const double tt = five ? fma(x, s_bc[e].x, s_bc[e].y) : fma(x, s_q[e], c);
+                                    if (tt < bt) { bt = tt; bi = base + j0 + i + u; }
+                                }
+                                T = fminf(T, __double2float_ru(bt));
+                            }
+                        }
+                        best[o] = bt;
+                        bidx[o] = bi;
+#pragma unroll
+                        for (int q = 0; q < R; ++q) {
+                            if (HAS5 && five && q == r) T5[q] = T;
+                            if (QL && !five && q == r) T2[q] = T;
+                        }
+                    }
+                }
+            }
+            sub = then;
+            __syncthreads();
+        }
     }
 
     // partial results, one row per (table, strategy slot, (m, chunk) pair), P contiguous; the warps that shared a tile of
@@ -279,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
         const int slot = IS9 ? p.n_seg - 1 : q;
         const size_t rbase = (static_cast<size_t>(trel) * p.n_seg + slot) * p.n_pairs + row;
         for (int i = tid; i < wp * 32 * R; i += kThreads) {
-            const int pidx = ptile * wp * 32 * R + i;
+            const int pidx = tile0 + i;
             if (pidx >= p.G.n_P) break;
             double bt = s_best[q * kIdStep + i];
             uint32_t bi = s_idx[q * kIdStep + i];
@@ -607,7 +658,7 @@ static cudaError_t launch_sweep_t(const SweepParams &p, int n_tables_launch, boo
 {
     constexpr int n_id = (HAS2 ? 1 : 0) + (HAS5 ? 1 : 0) + (IS9 ? 1 : 0);
     const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double) +
-                        2 * kSweepSub * (sizeof(double2) + sizeof(double) + 3 * sizeof(float)) +
+                        2 * kSweepSub * (sizeof(double2) + sizeof(double) + 3 * sizeof(float)) + (2 * kSweepGroups + kThreads) * 3 * sizeof(float) + kThreads * sizeof(int) +
                         static_cast<size_t>(n_id) * kWarps * kSweepR * 32 * (sizeof(double) + sizeof(uint32_t));
     const long long bx = static_cast<long long>(p.n_pairs) * p.n_ptiles;
     if (bx <= 0 || bx > 0x7FFFFFFFLL || n_tables_launch > 65535) return cudaErrorInvalidConfiguration;

@@ -86,3 +86,20 @@ def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed):
         for a, b in ((d.strategy, dec.strategy), (d.s_bytes, dec.s_bytes), (d.time, dec.time)):
             assert a[:, 0].equal(b[:, 0])
         assert p.best_s.equal(pred.best_s) and all(p.time[:, i].equal(pred.time[:, i]) for i in (2, 5, 9))
+
+
+@pytest.mark.parametrize("kind", ["as drawn", "flat", "stairs", "falls"])
+@pytest.mark.parametrize("n_s,s_step,n_P,k_mode", [(255, 4, 40, 0), (257, 8, 256, 1), (2600, 4, 257, 0), (700, 400, 530, 0)])
+def test_long_lists_bounded_by_their_ends(plogp, kind, n_s, s_step, n_P, k_mode):
+    """Sub-chunks of 256 candidates passed over by the smallest gap between their first and last size: breakpoints inside one,
+    several sub-chunks between two breakpoints, gaps that fall; process counts in the first 256 and behind them."""
+    w = wl_grid(n_tables=2, n_P=n_P, n_m=4, n_s=1, k_mode=k_mode)
+    g = w.gaps.copy()
+    if kind == "flat":
+        g[:, :] = g[:, :1]
+    elif kind == "stairs":
+        g = np.repeat(g[:, ::8], 8, axis=1)
+    elif kind == "falls":
+        g[:, 3:60:4] *= 0.3
+    both(plogp, replace(w, gaps=np.ascontiguousarray(g), m=np.array([500, 30000, 1 << 20, 1 << 24], dtype=np.uint64), s_list=None, s_lo=4, s_hi=4 + s_step * (n_s - 1),
+                        s_step=s_step, strategy_mask=0x224))
