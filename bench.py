@@ -38,8 +38,8 @@ NOMINAL_FP64_FMA_RATE = 148 * 64 * 1.965e9  # SMs x FP64 lanes per SM x max SM c
 # under profiles/ (batched workload cut to 1024 tables: 0.87 GB of output per kernel, far beyond the L2,
 # so what is still cached when the kernel ends is a few percent; traffic grows in proportion to the table
 # count).  An entry is None while its kernel has changed since the last capture.
-NCU_TRAFFIC_BYTES_PER_TABLE = {"decide_kernel": 817499904 / 1024, "scatter_kernel": 813760256 / 1024, "sweep_kernel": None}
-NCU_TRAFFIC_NOTE = "bytes per launch = bytes per table of the 1024-table ncu capture in profiles/ x tables"
+NCU_TRAFFIC_BYTES_PER_TABLE = {"decide_kernel": 377000000 / 512, "scatter_kernel": 813760256 / 1024, "sweep_kernel": None}
+NCU_TRAFFIC_NOTE = "bytes per launch = bytes per table of the ncu captures in profiles/ (512 tables decide_kernel, 1024 scatter_kernel) x tables"
 FALLBACK_HBM_GBS = 6650.0
 
 
@@ -65,13 +65,13 @@ def make_workload(name: str, scale: str, rank: int):
 
 def work_counts(w):
     """Cells of one step and the algorithmic work of each kernel, in issue slots of a 64-lane pipe (the FP64 pipe's
-    measured rate is the peak).  The lane <-> P kernels evaluate every cell of a line in P as a lower bound in FP32:
-    half a slot for the packed multiply-add (two cells per instruction, 64 lane pairs) and half a slot for its share of a
-    three-input minimum, one slot together; what the bounds leave open is compared in FP64 and not counted.  Models that
-    depend on floor and ceil of log2 P alone (ids 6 to 9) have the same value for all process counts in between and are
-    searched once for them: not counted as slots there.  Elsewhere an unsegmented cell is one DFMA, a Scatter Chain element
-    one interpolation DFMA, one running-sum DADD and the model's DFMA.  HBM bytes are the decision table written once
-    (13 B per decision cell)."""
+    measured rate is the peak).  Candidates of the segmented strategies are ruled out for ranges of process counts, or many
+    at a time, and cost nothing per cell then; what is counted is one DFMA per cell and strategy with lines in P, its
+    winner's.  Models that depend on floor and ceil of log2 P alone (ids 6 to 9) have the same value for all process counts
+    in between: not counted as slots in decide_kernel and segmin_kernel.  Elsewhere an unsegmented cell is one DFMA, a Scatter Chain
+    element one interpolation DFMA, one running-sum DADD and the model's DFMA.  HBM bytes are the decision table written once
+    (13 B per decision cell).  model_cells stays the number of (strategy, P, m, s) cells that the question has, whose minima are
+    found: it says how fast the question is answered, not what is evaluated."""
     mask = w.strategy_mask
     seg_ids = [b for b in (2, 5, 9) if (mask >> b) & 1]
     unseg_b = [b for b in (0, 1, 3, 4, 6, 7, 8) if (mask >> b) & 1]
@@ -80,14 +80,13 @@ def work_counts(w):
     seg_cells = w.n_tables * w.n_P * len(seg_ids) * int(w.n_candidates().sum())
     bcast_dec = cells_pm if (seg_ids or unseg_b) else 0
     scat_dec = cells_pm if scat else 0
-    n_cand = w.n_tables * w.n_P * int(w.n_candidates().sum())
-    line_slots = n_cand * sum((mask >> b) & 1 for b in (2, 5))
+    line_slots = cells_pm * sum((mask >> b) & 1 for b in (2, 5))
     line_unseg = cells_pm * sum((mask >> b) & 1 for b in (0, 1, 3, 4))
     scat_slots = cells_pm * (((mask >> 10) & 1) + 3 * ((mask >> 11) & 1) + ((mask >> 12) & 1))
     long_lists = bool(seg_ids) and len(w.s_values()) > 64
     per_kernel = {}
     if long_lists:
-        per_kernel["sweep_kernel"] = {"fp64_slots": seg_cells, "hbm_bytes": 0}
+        per_kernel["sweep_kernel"] = {"fp64_slots": cells_pm * len(seg_ids), "hbm_bytes": 0}
         per_kernel["fused_kernel"] = {"fp64_slots": len(unseg_b) * cells_pm + scat_slots, "hbm_bytes": 13 * (bcast_dec + scat_dec)}
     else:
         if seg_ids:
@@ -507,9 +506,6 @@ class Bench:
                  "alu_time_ms": t_alu * 1e3, "hbm_time_ms": t_hbm * 1e3,
                  "peak_source": ("DFMA issue rate measured in this run by plogp_fp64_fma_rate, of measured (nominal %.2f T/s = 148 SMs x 64 lanes x 1.965 GHz)"
                                  % (NOMINAL_FP64_FMA_RATE / 1e12)) if alu else "HBM copy bandwidth, of %s" % self.peak_src}
-            if alu and name in ("sweep_kernel", "decide_kernel", "segmin_kernel"):
-                # stricter: the minima run beside the multiply-adds in another pipe, so only the latter count
-                r["frac_multiply_adds_only"] = max(0.5 * slots / fma_rate, t_hbm) / dur
             return r
 
         kernels = [roof(k, v[0], v[1]) for k, v in m["kernel_ms"].items()]
@@ -533,9 +529,9 @@ class Bench:
                 "P": [w.P_lo, w.P_hi], "n_m": w.n_m, "n_s": int(len(w.s_values())), "strategy_mask": w.strategy_mask,
                 "model_cells_per_gpu": counts["model_cells"], "decision_cells_per_gpu": counts["decision_cells"],
                 "parallelism": "tables sharded, %d rank(s)" % self.world,
-                "evaluation": "every (P, m, s) cell of a line in P as a lower bound in FP32 (operands and multiply-add rounded down), decided in "
-                              "FP64 wherever the bound does not rule it out; ids 6 to 9 once per (floor, ceil) of log2 P; results are "
-                              "those of the exhaustive FP64 search",
+                "evaluation": "candidates ruled out by bounds over ranges of process counts (short lists) or groups of sizes (long ones), the "
+                              "rest evaluated in FP64; ids 6 to 9 once per (floor, ceil) of log2 P; results are those of the exhaustive "
+                              "FP64 search; model cells are those of the question, evaluated or ruled out",
                 "l2": "256 MB written between timed steps to flush L2" if m["flushed"]
                 else "outputs (%.1f GB per step) exceed the 126 MB L2" % (m["out_bytes"] / 1e9)}
 
