@@ -3,6 +3,7 @@
 // kernel launches.  Every step of the evaluation itself runs on the device.
 #include "../../include/plogp.h"
 #include "internal.h"
+#include "lines_layout.h"
 
 #include <algorithm>
 #include <atomic>
@@ -623,7 +624,13 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             lp.table0 = t0; lp.n_tables_launch = nt; lp.out_table0 = out.out_table0; lp.om = out.om;
             return lp;
         };
-        auto stage = [&](LinesParams &lp) { lp.staged = 1; lp.width = pl.G.n_m; lp.n_mgroups = 1; lp.threads = pl.ln_staged; };
+        // All message sizes in a CTA, where two of them fit an SM (228 KB, 1 KB of it each CTA's own): the shared memory grows with
+        // message sizes times candidates and times (floor, ceil) pairs, past what a CTA can have.
+        auto stage = [&](LinesParams &lp) {
+            LinesParams whole = lp;
+            whole.staged = 1; whole.width = pl.G.n_m; whole.n_mgroups = 1; whole.threads = pl.ln_staged;
+            if (2 * (lines_smem_bytes(whole) + 1024) <= size_t(228) * 1024) lp = whole;
+        };
         if (predict && pl.inline_sweep && pl.n_seg > 0) {
             // Predictions on short candidate lists: the segmented minima (planes 2, 5, 9 and the best segment sizes)
             // come from segmin_kernel; the kernels behind it write the other planes.

@@ -11,13 +11,11 @@ __global__ void __launch_bounds__(STAGED ? kLineThreads : kDecThreads, STAGED ? 
     last_block_waits(threadIdx.x);
 }
 
-size_t decide_smem_bytes(const DecideParams &p) { return lines::layout(p.gaps ? 0 : p.T.npad, p.G.n_s, p.n_pairs, p.n_p, p.width, p.threads, p.staged, nullptr, nullptr); }
-
 cudaError_t launch_decide(const DecideParams &p, bool overlap, cudaStream_t st)
 {
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    return launch(p.staged ? decide_kernel<true> : decide_kernel<false>, static_cast<unsigned>(blocks), 1, static_cast<unsigned>(p.threads), decide_smem_bytes(p), st, overlap, p);
+    return launch(p.staged ? decide_kernel<true> : decide_kernel<false>, static_cast<unsigned>(blocks), 1, static_cast<unsigned>(p.threads), lines_smem_bytes(p), st, overlap, p);
 }
 
 }  // namespace plogp

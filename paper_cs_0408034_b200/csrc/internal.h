@@ -216,9 +216,8 @@ struct LinesParams {
 };
 constexpr int kLineThreads = 256;
 constexpr int kLineSegs = 4;  // segments of a CTA's process counts, at most
-using DecideParams = LinesParams;
-using SegminParams = LinesParams;
-size_t decide_smem_bytes(const DecideParams &p);
+using DecideParams = LinesParams;  // as decide_kernel takes them,
+using SegminParams = LinesParams;  // and segmin_kernel
 
 constexpr int kDecThreads = 128;
 constexpr int kDecWarps = kDecThreads / 32;

@@ -17,7 +17,7 @@ cudaError_t launch_segmin(const SegminParams &p, bool overlap, cudaStream_t st)
 {
     const long long blocks = static_cast<long long>(p.n_mgroups) * p.n_ptiles * p.n_tables_launch;
     if (blocks <= 0 || blocks > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
-    return launch(p.staged ? segmin_kernel<true> : segmin_kernel<false>, static_cast<unsigned>(blocks), 1, static_cast<unsigned>(p.threads), decide_smem_bytes(p), st, overlap, p);
+    return launch(p.staged ? segmin_kernel<true> : segmin_kernel<false>, static_cast<unsigned>(blocks), 1, static_cast<unsigned>(p.threads), lines_smem_bytes(p), st, overlap, p);
 }
 
 }  // namespace plogp

@@ -24,7 +24,7 @@ cudaError_t launch_select(SelectParams &p, cudaStream_t st)
     const long long ns = static_cast<long long>(p.scatter.n_mtiles) * p.scatter.n_ptiles * p.scatter.n_tables_launch;
     if (nd <= 0 || ns <= 0 || nd + ns > 0x7FFFFFFFLL) return cudaErrorInvalidConfiguration;
     p.n_decide = static_cast<int>(nd);
-    const size_t a = decide_smem_bytes(p.decide), b = scatter_smem_bytes(p.scatter, kDecWarps);
+    const size_t a = lines_smem_bytes(p.decide), b = scatter_smem_bytes(p.scatter, kDecWarps);
     const bool contig = p.scatter.G.P_list == nullptr;
     const auto kernel = contig ? select_kernel<true> : select_kernel<false>;
     return launch(kernel, static_cast<unsigned>(nd + ns), 1, kDecThreads, a > b ? a : b, st, false, p);

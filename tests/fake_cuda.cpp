@@ -6,6 +6,7 @@ template <typename F>  // as nvcc has it
 static cudaError_t cudaFuncSetAttribute(F *f, cudaFuncAttribute a, int v) { return cudaFuncSetAttribute(reinterpret_cast<const void *>(f), a, v); }
 
 #include "../paper_cs_0408034_b200/csrc/internal.h"
+#include "../paper_cs_0408034_b200/csrc/lines_layout.h"
 
 #include <cstdlib>
 #include <cstring>
@@ -15,6 +16,7 @@ static cudaError_t cudaFuncSetAttribute(F *f, cudaFuncAttribute a, int v) { retu
 namespace {
 std::map<const unsigned char *, size_t> live;
 long long refuse_at = -1, bad = 0, launches = 0;  // refuse_at: allocations from that size on fail (-1: none)
+long long too_large = 0, staged = 0;  // launches with more shared memory than an SM has; with all message sizes in a CTA
 
 void inside(const void *p, size_t bytes)
 {
@@ -41,6 +43,8 @@ void fake_refuse_host_from(long long bytes) { refuse_host_at = bytes; }
 void fake_refuse_from(long long bytes) { refuse_at = bytes; }
 long long fake_bad_accesses() { return bad; }
 long long fake_launches() { return launches; }
+long long fake_too_large() { return too_large; }
+long long fake_staged() { return staged; }
 long long fake_live_bytes() { long long n = 0; for (auto &a : live) n += static_cast<long long>(a.second); return n; }
 
 cudaError_t cudaMalloc(void **p, size_t n)
@@ -142,10 +146,17 @@ cudaError_t launch_fused(const FusedParams &p, bool, bool, cudaStream_t)
     if (p.part_time) check_parts(p.part_time, p.part_idx, size_t(p.n_tables_launch) * p.n_seg * p.n_pairs, p.G.n_P);
     return launched();
 }
-cudaError_t launch_decide(const DecideParams &p, bool, cudaStream_t) { check_gaps(p.gaps, p.gaps_stride, p.n_tables_launch); return launched(); }
-cudaError_t launch_segmin(const SegminParams &p, bool, cudaStream_t) { check_gaps(p.gaps, p.gaps_stride, p.n_tables_launch); return launched(); }
+static cudaError_t check_lines(const LinesParams &p)
+{
+    check_gaps(p.gaps, p.gaps_stride, p.n_tables_launch);
+    staged += p.staged != 0;
+    if (lines_smem_bytes(p) > size_t(kMaxSmem)) { ++too_large; return cudaErrorInvalidValue; }
+    return launched();
+}
+cudaError_t launch_decide(const LinesParams &p, bool, cudaStream_t) { return check_lines(p); }
+cudaError_t launch_segmin(const LinesParams &p, bool, cudaStream_t) { return check_lines(p); }
 cudaError_t launch_scatter(const ScatterParams &, bool, cudaStream_t) { return launched(); }
-cudaError_t launch_select(SelectParams &, cudaStream_t) { return launched(); }
+cudaError_t launch_select(SelectParams &p, cudaStream_t) { return check_lines(p.decide); }
 cudaError_t launch_planes(const PlanesParams &, bool, cudaStream_t) { return launched(); }
 cudaError_t launch_rows(const RowsParams &, bool, bool, cudaStream_t) { return launched(); }
 cudaError_t launch_layout(const LayoutParams &p, cudaStream_t)
@@ -158,7 +169,6 @@ cudaError_t launch_surface(const SensParams &, cudaStream_t) { return launched()
 cudaError_t launch_fixed(const SensParams &, cudaStream_t) { return launched(); }
 cudaError_t launch_boundaries(const uint8_t *, uint8_t *, long long, int, int, int, cudaStream_t) { return launched(); }
 cudaError_t launch_fp64_probe(double *, int, int, cudaStream_t) { return launched(); }
-size_t decide_smem_bytes(const DecideParams &) { return 32 * 1024; }
 int envelope_coarse_of(int pidx, int) { return pidx; }
 
 }  // namespace plogp

@@ -88,6 +88,17 @@ def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed):
         assert p.best_s.equal(pred.best_s) and all(p.time[:, i].equal(pred.time[:, i]) for i in (2, 5, 9))
 
 
+@pytest.mark.parametrize("n_m,n_s,octaves", [(255, 64, 0), (253, 48, 0), (201, 32, 0), (250, 64, 0), (229, 8, 29), (255, 27, 29), (255, 64, 29), (157, 20, 29)])
+def test_more_than_a_cta_has_room_for(plogp, n_m, n_s, octaves):
+    """Many tables, odd rows, long lists and process counts over many (floor, ceil) pairs of log2 P: all message sizes together
+    would take more shared memory than a CTA, or than half of an SM, has."""
+    w = wl_grid(n_tables=300, n_P=511, n_m=n_m, n_s=n_s)
+    if octaves:  # P m < 2^53; the oracle would add up the Scatter Chain's terms one by one
+        P = sorted({1 << i for i in range(1, octaves)} | {3 << i for i in range(octaves - 1)})
+        w = replace(w, P_list=np.array(P, dtype=np.int32), m=256 * np.arange(1, n_m + 1, dtype=np.uint64), strategy_mask=0x17FF)
+    both(plogp, w, tables=[0, 299])
+
+
 @pytest.mark.parametrize("kind", ["as drawn", "flat", "stairs", "falls"])
 @pytest.mark.parametrize("n_s,s_step,n_P,k_mode", [(255, 4, 40, 0), (257, 8, 256, 1), (2600, 4, 257, 0), (700, 400, 530, 0)])
 def test_long_lists_bounded_by_their_ends(plogp, kind, n_s, s_step, n_P, k_mode):

@@ -29,17 +29,17 @@ def lib(tmp_path_factory):
     lib.plogp_segment_surface.argtypes = [C.c_void_p] * 4
     lib.plogp_profile_read.argtypes = [C.c_void_p] * 3
     lib.fake_refuse_from.argtypes = lib.fake_refuse_host_from.argtypes = [C.c_longlong]
-    for f in ("fake_bad_accesses", "fake_launches", "fake_live_bytes"):
+    for f in ("fake_bad_accesses", "fake_launches", "fake_live_bytes", "fake_too_large", "fake_staged"):
         getattr(lib, f).restype = C.c_longlong
     return lib
 
 
-def load(lib, n_tables):
-    sizes = np.array([4, 1024, 1 << 20], dtype=np.uint64)
-    gaps = np.ascontiguousarray(np.tile([1.0, 2.0, 900.0], (n_tables, 1)))
+def load(lib, n_tables, n_bp=3):
+    sizes = np.array([4, 1024, 1 << 20], dtype=np.uint64) if n_bp == 3 else 4 * np.arange(1, n_bp + 1, dtype=np.uint64)
+    gaps = np.ascontiguousarray(np.tile([1.0, 2.0, 900.0] if n_bp == 3 else np.arange(1.0, n_bp + 1), (n_tables, 1)))
     h = C.c_void_p()
     lat = np.full(n_tables, 5.0)
-    assert lib.plogp_table_load(n_tables, 3, sizes.ctypes.data, 1, gaps.ctypes.data, lat.ctypes.data, C.byref(h)) == plogp.OK
+    assert lib.plogp_table_load(n_tables, n_bp, sizes.ctypes.data, 1, gaps.ctypes.data, lat.ctypes.data, C.byref(h)) == plogp.OK
     return h
 
 
@@ -128,3 +128,27 @@ def test_device_memory_that_runs_out_for_a_grid_is_a_status(lib):
     lib.fake_refuse_from(-1)
     assert lib.plogp_select_best(h, g.ref, OUT, OUT, OUT, None) == plogp.OK
     assert lib.plogp_table_free(h) == plogp.OK
+
+
+def octaves(n):
+    """Listed process counts over n octaves, two (floor, ceil) pairs of log2 P in each."""
+    return np.array(sorted({1 << i for i in range(1, n)} | {3 << i for i in range(n - 1)}), dtype=np.int32)
+
+
+@pytest.mark.parametrize("n_bp", [64, 1024])
+@pytest.mark.parametrize("n_m,P,n_s,n_tables", [
+    (255, 512, 64, 296), (253, 1024, 64, 148), (255, 3000, 60, 400), (250, 512, 64, 300), (252, 512, 64, 300), (255, 512, 61, 300),
+    (255, 29, 27, 300), (229, 29, 8, 300), (193, 29, 32, 300), (157, 29, 64, 300), (256, 29, 64, 300), (127, 512, 32, 300), (33, 29, 64, 300), (19, 29, 7, 1), (1, 29, 64, 1)])
+def test_shared_memory_fits(lib, n_m, P, n_s, n_tables, n_bp):
+    """Every launch on a short candidate list has at most the shared memory of an SM, whatever the message sizes, the candidates
+    and the (floor, ceil) pairs of log2 P are: P = 2..P, or listed over P octaves."""
+    listed = octaves(P) if P < 30 else None
+    grid = plogp.GridArgs(np.arange(1, n_m + 1) * 64, listed, 2, P, np.arange(1, n_s + 1) * 8)
+    h = load(lib, n_tables, n_bp)
+    try:
+        for call in (lambda: lib.plogp_select_best(h, grid.ref, OUT, OUT, OUT, None), lambda: lib.plogp_predict(h, grid.ref, OUT, OUT, None),
+                     lambda: lib.plogp_select_best_collective(h, grid.ref, 3, OUT, OUT, OUT, None)):
+            n = lib.fake_too_large()
+            assert call() == plogp.OK and lib.fake_too_large() == n and lib.fake_bad_accesses() == 0
+    finally:
+        lib.plogp_table_free(h)
