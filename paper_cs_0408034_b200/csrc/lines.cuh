@@ -128,8 +128,9 @@ __device__ __forceinline__ void lines_block(const LinesParams &p, int block, uns
                has78 = mask & 0x180u, has9 = (mask >> 9) & 1u;
     const bool any_log = mask & 0x3C0u;
     // the Flat Tree (P-1) g(m) + L or its rendezvous form (P-1) g(m) + rdv, the Chain (P-1) (g(m) + L) or its rendezvous form
-    // (P-1) (g(m) + rdv).  Where no candidate fits, id 5 is the chain itself, behind id 4.
-    const bool chain5 = !PREDICT && ns == 0 && has5 && !has3 && !((mask & 0x10u) && rdv <= L);
+    // (P-1) (g(m) + rdv).  Where no candidate fits, id 5 is the chain itself; its rendezvous form, which is never below it, then
+    // wins where the two times are equal.
+    const bool chain5 = !PREDICT && ns == 0 && has5 && !has3;
     const bool flat_on = !PREDICT && (mask & 3u), chain_on = !PREDICT && ((mask & 0x18u) || chain5);
     const double flat_c = has0 ? L : rdv, chain_a = gm + (has3 || chain5 ? L : rdv);
     const int n_seg = knot[kKnots];
@@ -440,7 +441,10 @@ __device__ __forceinline__ void lines_block(const LinesParams &p, int block, uns
                             candidate(c, Q, B, C);
                             line(B, C, sm.sval[c], id5);
                         });
-                    if (f & 4u) line(chain_a, 0.0, chain5 ? m_u : 0u, id_chain);
+                    if (f & 4u) {
+                        line(chain_a, 0.0, chain5 ? m_u : 0u, id_chain);
+                        if (chain5 && (mask & 0x10u)) line(gm + rdv, 0.0, 0u, p.om.id_of[4]);
+                    }
                     if (has2) {
                         if (near0 | near1) {
 #pragma unroll 1

@@ -5,8 +5,9 @@ from dataclasses import replace
 import numpy as np
 import pytest
 
+from oracle import plogp_oracle as po
 from paper_cs_0408034_b200 import workloads as wl
-from parity import check_decision, check_prediction, oracle_tables
+from parity import check_decision, check_prediction, oracle_sgrid, oracle_tables
 
 pytestmark = pytest.mark.gpu
 
@@ -114,3 +115,48 @@ def test_long_lists_bounded_by_their_ends(plogp, kind, n_s, s_step, n_P, k_mode)
         g[:, 3:60:4] *= 0.3
     both(plogp, replace(w, gaps=np.ascontiguousarray(g), m=np.array([500, 30000, 1 << 20, 1 << 24], dtype=np.uint64), s_list=None, s_lo=4, s_hi=4 + s_step * (n_s - 1),
                         s_step=s_step, strategy_mask=0x224))
+
+
+def picks_as_the_oracle(plogp, w, tables):
+    """Strategies and segment sizes of Broadcast equal to the oracle's everywhere, on ties too, and times bit for bit."""
+    import torch
+    ot, sg = oracle_tables(w), oracle_sgrid(w)
+    with plogp.Tables.from_workload(w) as tabs:
+        dec, pred = plogp.select_best(tabs, w), plogp.predict(tabs, w)
+        torch.cuda.synchronize()
+    for t in tables:
+        o = po.predict_grid(ot[t], w.strategy_mask, w.P_values(), w.m, sg, w.k_mode)
+        d = po.select_grid(w.strategy_mask, o)
+        np.testing.assert_array_equal(dec.strategy[t, 0].cpu().numpy(), d.strategy[0])
+        np.testing.assert_array_equal(dec.s_bytes[t, 0].cpu().numpy().view(np.uint32), d.s[0])
+        np.testing.assert_array_equal(dec.time[t, 0].cpu().numpy(), d.time[0])
+        for q, sid in enumerate(po.SEGMENTED_IDS):
+            if (w.strategy_mask >> sid) & 1:
+                np.testing.assert_array_equal(pred.best_s[t, q].cpu().numpy().view(np.uint32), o.best_s[q])
+                np.testing.assert_array_equal(pred.time[t, sid].cpu().numpy(), o.time[sid])
+
+
+@pytest.mark.parametrize("ids", [range(10), (2, 5, 9), (4, 5), (1, 2, 4, 5, 8, 9), (0, 2), (3, 5), (8, 9), (1, 2, 5)])
+@pytest.mark.parametrize("n_tables,n_m,n_P,k_mode", [(40, 19, 70, 0), (300, 33, 70, 1)])
+def test_ties_go_to_the_lowest_id_and_size(plogp, ids, n_tables, n_m, n_P, k_mode):
+    """Whole gaps at powers of two: every product and sum of the models is exact, however it is rounded on the way, and many
+    are equal."""
+    rng = np.random.default_rng(n_m)
+    gaps = np.cumsum(rng.integers(0, 2, (n_tables, 21)) * rng.integers(0, 2, (n_tables, 1)), axis=1).astype(np.float64)
+    w = replace(wl_grid(n_tables=n_tables, n_P=n_P, n_m=n_m, n_s=8, k_mode=k_mode), sizes=(1 << np.arange(21)).astype(np.uint64), gaps=gaps,
+                latency=rng.integers(0, 3, n_tables).astype(np.float64), strategy_mask=sum(1 << i for i in ids),
+                s_list=np.array([64, 128, 192, 256, 1024, 4096, 4100, 65536], dtype=np.uint64))
+    m = np.unique(np.concatenate([w.s_list, [4, 16, 8192, 1 << 20], np.arange(1, n_m) * 516]).astype(np.uint64))[:n_m]
+    picks_as_the_oracle(plogp, replace(w, m=m), range(0, n_tables, 7))
+
+
+def test_rendezvous_times_that_round_to_the_others(plogp):
+    """Handshakes of less than a rounding of the gap: where no candidate fits, ids 4 and 5 cost the same at some process counts
+    and differ by their last bit at others."""
+    rng = np.random.default_rng(4)
+    c = 1.0 + rng.random(64)
+    gaps = np.stack([np.zeros(64), c, c, c], axis=1)
+    w = replace(wl_grid(n_tables=64, n_P=63, n_m=1, n_s=1), sizes=np.array([1, 1024, 1 << 20, 1 << 21], dtype=np.uint64), gaps=gaps,
+                latency=np.where(np.arange(64) < 60, rng.uniform(0.34, 0.49, 64) * 2.0**-52, 1e-25), s_list=np.array([1 << 16, 1 << 18], dtype=np.uint64),
+                m=np.array([1024, 4096, 32768], dtype=np.uint64), strategy_mask=0x30)
+    picks_as_the_oracle(plogp, w, range(64))
