@@ -457,8 +457,17 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         long long cands = 0;
         for (int i = 0; i < n_m; ++i) cands += ns_of_m[i];
         const long long share = cands * pl.sweep_ptiles * h->T.n_tables / ((long long)h->sm_count * 6);
-        pl.chunk_len = int(std::min<long long>(std::max<long long>(2048, (share + kSweepSub - 1) / kSweepSub * kSweepSub), (ns_max + kSweepSub - 1) / kSweepSub * kSweepSub));
-        pl.chunk_len = std::min(std::max(pl.chunk_len, kSweepSub), 1 << 20);
+        const auto whole_subs = [](long long n) { return (n + kSweepSub - 1) / kSweepSub * kSweepSub; };
+        long long chunk = std::min<long long>(std::max(std::min(std::max<long long>(2048, whole_subs(share)), whole_subs(ns_max)), (long long)kSweepSub), 1 << 20);
+        // but no more of them than 32 per message size where a table's partial minima would not fit the scratch of a launch
+        const long long longest = whole_subs((ns_max + 31LL) / 32);
+        const auto partials = [&]() {
+            long long n = 0;
+            for (int i = 0; i < n_m; ++i) n += (ns_of_m[i] + chunk - 1) / chunk;
+            return double(n) * pl.n_seg * n_P * (sizeof(double) + sizeof(uint32_t));
+        };
+        while (chunk < longest && partials() > double(kSweepScratchLimit)) chunk = std::min(2 * chunk, longest);
+        pl.chunk_len = int(chunk);
         std::vector<int32_t> pair_base(n_m + 1, 0);
         struct Pair { int32_t m, chunk, row, len; };
         std::vector<Pair> pairs;

@@ -152,3 +152,17 @@ def test_shared_memory_fits(lib, n_m, P, n_s, n_tables, n_bp):
             assert call() == plogp.OK and lib.fake_too_large() == n and lib.fake_bad_accesses() == 0
     finally:
         lib.plogp_table_free(h)
+
+
+def test_scratch_of_very_long_lists(lib):
+    """Two thousand million candidates, 65535 process counts: partial minima of 32 chunks per message size, 3.2 GB, and not of
+    chunks as short as they are elsewhere."""
+    n_m = 64
+    grid = plogp.GridArgs((1 << 31) + np.arange(n_m), None, 2, 65536, None, s_lo=1, s_hi=(1 << 31) - 1, s_step=1, dtype_bytes=1, strategy_mask=0x24)
+    h = load(lib, 1)
+    try:
+        lib.fake_refuse_from(n_m * 33 * 2 * 65535 * 12)
+        assert lib.plogp_select_best(h, grid.ref, OUT, OUT, OUT, None) == plogp.OK and lib.fake_bad_accesses() == 0
+    finally:
+        lib.fake_refuse_from(-1)
+        lib.plogp_table_free(h)
