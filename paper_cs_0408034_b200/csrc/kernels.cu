@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     const uint32_t m_u = p.G.m_list[m_idx];
     const int ns = p.G.ns_of_m[m_idx];
     const int s_begin = chunk * p.chunk_len;
-    const int s_end = min(ns, s_begin + p.chunk_len);
+    const int s_end = s_begin + min(p.chunk_len, ns - s_begin);  // (indices up to 2^31 - 1: differences only, no sums past the end)
     const int n_sub = (s_end - s_begin + kSweepSub - 1) / kSweepSub;
 
     dependents_may_start();
@@ -128,9 +128,9 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
         Q = gs * k;
     };
     auto fill = [&](int sub, int buf) {
-        const int si = s_begin + sub * kSweepSub + tid, o = buf * kSweepSub + tid;
+        const int first = s_begin + sub * kSweepSub, o = buf * kSweepSub + tid;
         double B = CUDART_INF, C = CUDART_INF, Q = CUDART_INF;  // padding: the bound is +inf
-        if (si < s_end) coefficients(si, B, C, Q);
+        if (tid < s_end - first) coefficients(first + tid, B, C, Q);
         // a warp's candidates are a group; non-negative floats are ordered as whole numbers
         if (HAS5) {
             const float b = __double2float_rd(B), c = __double2float_rd(C);
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
         const int n_block = min(kThreads, n_sub - block0);
         __syncthreads();
         if (tid < n_block) {
-            const int first = s_begin + (block0 + tid) * kSweepSub, last = min(first + kSweepSub, s_end) - 1;
+            const int first = s_begin + (block0 + tid) * kSweepSub, last = first + min(kSweepSub, s_end - first) - 1;
             const uint32_t s_last = s_at(p.G, last);
             const double sa = static_cast<double>(s_at(p.G, first)), sb = static_cast<double>(s_last);
             const int npad = p.T.npad, ia = interval_of(s_tab, npad, sa), ib = interval_of(s_tab, npad, sb);

@@ -160,3 +160,19 @@ def test_rendezvous_times_that_round_to_the_others(plogp):
                 latency=np.where(np.arange(64) < 60, rng.uniform(0.34, 0.49, 64) * 2.0**-52, 1e-25), s_list=np.array([1 << 16, 1 << 18], dtype=np.uint64),
                 m=np.array([1024, 4096, 32768], dtype=np.uint64), strategy_mask=0x30)
     picks_as_the_oracle(plogp, w, range(64))
+
+
+@pytest.mark.parametrize("n_s", [(1 << 31) - 1, (1 << 31) - 200, (1 << 31) - (1 << 20) - 1])
+def test_candidate_indices_up_to_the_last(plogp, n_s):
+    """Every size up to n_s is a candidate and the gap is the same for all: fewer segments are better, and the best size is the
+    message's own, the last candidate for the longest message."""
+    import torch
+    m = np.array([4096, 1 << 30, n_s], dtype=np.uint64)
+    grid = plogp.GridArgs(m, np.array([2, 3, 40, 300], dtype=np.int32), 2, 2, None, s_lo=1, s_hi=n_s, s_step=1, dtype_bytes=1, strategy_mask=0x224)
+    with plogp.Tables(np.array([1, 1 << 20], dtype=np.uint64), np.array([[3.0, 3.0]]), np.array([0.5])) as tabs:
+        dec, pred = plogp.select_best(tabs, grid), plogp.predict(tabs, grid)
+        torch.cuda.synchronize()
+    for x in (dec.s_bytes[0, 0], *pred.best_s[0]):
+        np.testing.assert_array_equal(x.cpu().numpy().view(np.uint32), np.broadcast_to(m, (4, 3)))
+    # the Segmented Binomial Tree of one segment: floor(log2 P) 3 + ceil(log2 P) 0.5
+    np.testing.assert_array_equal(dec.time[0, 0].cpu().numpy(), np.broadcast_to([[3.5], [4.0], [18.0], [28.5]], (4, 3)))
