@@ -78,6 +78,8 @@ struct Plan {
     int ln_width = 32, ln_mgroups = 0, ln_np = 512, ln_ptiles = 1, ln_pairs = 1;
     int ln_staged = 0;  // threads of a CTA that has all message sizes, or 0
     size_t off_knots = 0;
+    bool dr_decide = false, dr_predict = false;  // small grids: a cell per thread
+    int dr_ptiles = 1;
     // sweep kernel
     int n_pairs = 0, sweep_ptiles = 0, sweep_wp = 8, chunk_len = 0;
     size_t off_pair_m = 0, off_pair_chunk = 0, off_pair_row = 0, off_pair_base = 0;
@@ -363,6 +365,17 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
                 pl.ln_width = width; pl.ln_mgroups = mgroups; pl.ln_np = np; pl.ln_ptiles = tiles;
             }
         }
+        // A cell per thread (direct.cuh), 250 instructions and 30 per candidate: where that is half as many as a line for a range of
+        // process counts, or no more and the GPU is nearly empty, so that only the length of a CTA counts.  Calls from a graph, lines ->
+        // cells, us: one table, 49 process counts, 19 message sizes, 7 candidates 6.8 -> 4.6; 18 x 101, 48 candidates 8.7 -> 5.8; 3
+        // tables of 74 x 8, 43 candidates 10.0 -> 6.8; 500 tables of 29 x 8, 5 candidates 13.0 -> 10.1, 2000 of 19 x 6, 4 candidates
+        // 38.4 -> 24.6.  Past the line: 16 tables of 100 x 30, 20 candidates 8.0 -> 9.3, 128 of 63 x 16, 8 candidates 9.0 -> 10.3.
+        // Predictions write more and gain a little longer: the latter 13.3 -> 11.9, but one table of 511 x 64, 32 candidates 8.1 -> 8.8.
+        const long long ctas = ((long long)n_P * n_m + kDecThreads - 1) / kDecThreads * h->T.n_tables;
+        const long long cost = std::max(ctas, (long long)h->sm_count * 4) * (250 + 30 * n_s);
+        pl.dr_decide = 2 * cost < best || (cost < best && ctas <= (long long)h->sm_count * 2);
+        pl.dr_predict = 5 * cost < 3 * best || (cost < best && ctas <= (long long)h->sm_count);
+        pl.dr_ptiles = int(ctas / h->T.n_tables);
         // All message sizes in a CTA, where there are two for every SM: threads for as many groups as leave the fewest idle
         if (n_m <= kLineThreads && (long long)pl.ln_ptiles * h->T.n_tables >= (long long)h->sm_count * 2) {
             double most = 0.0;
@@ -372,10 +385,11 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
             }
         }
     }
-    // One launch for both halves where the GPU holds all their CTAs at once (four per SM; its Scatter CTAs have four warps)
+    // One launch for both halves where the GPU holds all their CTAs at once (four per SM, six with a cell per thread; its Scatter CTAs
+    // have four warps)
     {
-        const long long decide = (long long)pl.ln_mgroups * pl.ln_ptiles * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
-        const long long room = (long long)h->sm_count * 4 - decide;
+        const long long decide = (pl.dr_decide ? (long long)pl.dr_ptiles : (long long)pl.ln_mgroups * pl.ln_ptiles) * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
+        const long long room = (long long)h->sm_count * (pl.dr_decide ? 6 : 4) - decide;
         pl.select = pl.ln_mgroups > 0 && room >= base && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
         if (pl.select) {
             pl.sel_run = int(std::max<long long>(4, (n_P + kDecWarps * (room / base) - 1) / (kDecWarps * (room / base))));
@@ -594,7 +608,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             ws += align_up(cells * sizeof(uint32_t), 256);
         }
         double *gaps = nullptr;
-        if (pl.use_gaps && pl.inline_sweep && pl.n_seg > 0 && (predict || use_decide)) {
+        if (pl.use_gaps && pl.inline_sweep && pl.n_seg > 0 && (predict ? !pl.dr_predict : use_decide && !pl.dr_decide)) {
             gaps = reinterpret_cast<double *>(ws);
             GapsParams gp{};
             gp.T = h->T; gp.G = pl.G;
@@ -631,6 +645,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             lp.knots = reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_knots);
             lp.gaps = gaps; lp.gaps_stride = pl.gaps_stride;
             lp.table0 = t0; lp.n_tables_launch = nt; lp.out_table0 = out.out_table0; lp.om = out.om;
+            if (predict ? pl.dr_predict : pl.dr_decide) { lp.direct = 1; lp.n_mgroups = 1; lp.n_ptiles = pl.dr_ptiles; }
             return lp;
         };
         // All message sizes in a CTA, where two of them fit an SM (228 KB, 1 KB of it each CTA's own): the shared memory grows with
@@ -646,7 +661,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             LinesParams sp = lines();
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
             // rows off the sectors of the sizes, or of times and sizes; up to 16 message sizes few warps have many lines (lines.cuh)
-            if (pl.ln_staged && pl.G.n_m % 8 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.p_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.p_best_s) % 16 == 0) stage(sp);
+            if (!sp.direct && pl.ln_staged && pl.G.n_m % 8 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.p_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.p_best_s) % 16 == 0) stage(sp);
             { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= ~kSegBits;
@@ -671,7 +686,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
                 continue;
             }
             // odd rows only: with half the bytes of a plane the waits weigh more (lines.cuh has both sides)
-            if (pl.ln_staged && pl.G.n_m % 2 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.d_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 16 == 0 &&
+            if (!dp.direct && pl.ln_staged && pl.G.n_m % 2 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.d_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 16 == 0 &&
                 reinterpret_cast<uintptr_t>(out.d_strategy) % 4 == 0) stage(dp);
             { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, overlap && gaps, st)); }
             g_launches += 1;

@@ -202,6 +202,7 @@ struct LinesParams {
     int width;      // message sizes of a CTA, side by side: 32, 16 or 8, or all of them (staged)
     int staged;     // outputs aligned for four cells per store (times 32, sizes 16, ids 4 bytes), all message sizes in a CTA
     int n_p;        // process counts per CTA
+    int direct;     // a cell per thread (direct.cuh): only gaps, outputs and n_ptiles, CTAs of kDecThreads cells per table, count
     int n_mgroups, n_ptiles;
     int n_pairs;    // (floor, ceil) pairs of log2 P in a CTA's range of process counts, at most
     const int32_t *knots;  // device [n_ptiles][kLineSegs + 2]: indices inside the CTA's process counts, number of segments

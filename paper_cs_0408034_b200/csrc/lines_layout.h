@@ -65,6 +65,7 @@ __host__ __device__ inline size_t layout(int npad, int n_s, int n_pairs, int n_p
 
 inline size_t lines_smem_bytes(const LinesParams &p)
 {
+    if (p.direct) return (3 * static_cast<size_t>(p.T.npad) + 3 * static_cast<size_t>(p.G.n_s)) * sizeof(double);
     return lines::layout(p.gaps ? 0 : p.T.npad, p.G.n_s, p.n_pairs, p.n_p, p.width, p.threads, p.staged, nullptr, nullptr);
 }
 

@@ -16,7 +16,7 @@ static cudaError_t cudaFuncSetAttribute(F *f, cudaFuncAttribute a, int v) { retu
 namespace {
 std::map<const unsigned char *, size_t> live;
 long long refuse_at = -1, bad = 0, launches = 0;  // refuse_at: allocations from that size on fail (-1: none)
-long long too_large = 0, staged = 0;  // launches with more shared memory than an SM has; with all message sizes in a CTA
+long long too_large = 0, staged = 0, direct = 0;  // launches with more shared memory than an SM has; with all message sizes in a CTA; a cell per thread
 
 void inside(const void *p, size_t bytes)
 {
@@ -45,6 +45,7 @@ long long fake_bad_accesses() { return bad; }
 long long fake_launches() { return launches; }
 long long fake_too_large() { return too_large; }
 long long fake_staged() { return staged; }
+long long fake_direct() { return direct; }
 long long fake_live_bytes() { long long n = 0; for (auto &a : live) n += static_cast<long long>(a.second); return n; }
 
 cudaError_t cudaMalloc(void **p, size_t n)
@@ -150,6 +151,7 @@ static cudaError_t check_lines(const LinesParams &p)
 {
     check_gaps(p.gaps, p.gaps_stride, p.n_tables_launch);
     staged += p.staged != 0;
+    direct += p.direct != 0;
     if (lines_smem_bytes(p) > size_t(kMaxSmem)) { ++too_large; return cudaErrorInvalidValue; }
     return launched();
 }

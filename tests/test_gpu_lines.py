@@ -176,3 +176,31 @@ def test_candidate_indices_up_to_the_last(plogp, n_s):
         np.testing.assert_array_equal(x.cpu().numpy().view(np.uint32), np.broadcast_to(m, (4, 3)))
     # the Segmented Binomial Tree of one segment: floor(log2 P) 3 + ceil(log2 P) 0.5
     np.testing.assert_array_equal(dec.time[0, 0].cpu().numpy(), np.broadcast_to([[3.5], [4.0], [18.0], [28.5]], (4, 3)))
+
+
+@pytest.mark.parametrize("n_P,n_m,n_s,k_mode,listed,ids", [
+    (1, 1, 1, 0, False, range(13)), (127, 1, 3, 1, False, range(13)), (16, 8, 64, 0, False, range(13)), (43, 3, 33, 0, True, range(13)), (70, 19, 8, 1, False, range(10)),
+    (70, 19, 8, 0, True, (2, 9)), (30, 33, 20, 0, False, (0, 3, 5, 6, 7, 10, 11, 12)), (20, 40, 16, 1, False, (1, 4, 5, 8)), (9, 7, 64, 0, False, (5,)), (64, 2, 12, 0, False, (1, 2, 9, 12))])
+def test_a_cell_per_thread_as_lines(plogp, n_P, n_m, n_s, k_mode, listed, ids):
+    """The same tables once and 300 times: small grids have a cell per thread, large ones lines for ranges of process counts.
+    Times and picks are the same, bit for bit, and the oracle's."""
+    import torch
+    w = wl_grid(n_tables=3, n_P=n_P, n_m=n_m, n_s=n_s, k_mode=k_mode, P_lo=3 if k_mode else 2)
+    if listed:
+        w = replace(w, P_list=(2 + 5 * np.arange(n_P)).astype(np.int32))
+    w = replace(w, strategy_mask=sum(1 << i for i in ids), m=np.unique(np.concatenate([w.m[: max(1, n_m - 2)], w.s_list[-1:]])))
+    both(plogp, w)
+    many = replace(w, gaps=np.tile(w.gaps, (300, 1)), latency=np.tile(w.latency, 300))
+    with plogp.Tables.from_workload(w) as a, plogp.Tables.from_workload(many) as b:
+        x, y = plogp.select_best(a, w), plogp.select_best(b, w)
+        p, q = plogp.predict(a, w), plogp.predict(b, w)
+        r, s = plogp.select_best_collective(a, w, plogp.REDUCE), plogp.select_best_collective(b, w, plogp.REDUCE)
+        torch.cuda.synchronize()
+    for first in (0, 3 * 299):
+        for u, v in ((x.strategy, y.strategy), (x.s_bytes, y.s_bytes), (x.time, y.time)):
+            assert u[:, 0].equal(v[first:first + 3, 0])
+        for u, v in ((r.strategy, s.strategy), (r.s_bytes, s.s_bytes), (r.time, s.time)):
+            assert u.equal(v[first:first + 3])
+        for j, i in enumerate(po.SEGMENTED_IDS):
+            if i in ids:
+                assert p.time[:, i].equal(q.time[first:first + 3, i]) and p.best_s[:, j].equal(q.best_s[first:first + 3, j])

@@ -29,7 +29,7 @@ def lib(tmp_path_factory):
     lib.plogp_segment_surface.argtypes = [C.c_void_p] * 4
     lib.plogp_profile_read.argtypes = [C.c_void_p] * 3
     lib.fake_refuse_from.argtypes = lib.fake_refuse_host_from.argtypes = [C.c_longlong]
-    for f in ("fake_bad_accesses", "fake_launches", "fake_live_bytes", "fake_too_large", "fake_staged"):
+    for f in ("fake_bad_accesses", "fake_launches", "fake_live_bytes", "fake_too_large", "fake_staged", "fake_direct"):
         getattr(lib, f).restype = C.c_longlong
     return lib
 
@@ -165,4 +165,17 @@ def test_scratch_of_very_long_lists(lib):
         assert lib.plogp_select_best(h, grid.ref, OUT, OUT, OUT, None) == plogp.OK and lib.fake_bad_accesses() == 0
     finally:
         lib.fake_refuse_from(-1)
+        lib.plogp_table_free(h)
+
+
+@pytest.mark.parametrize("n_tables,n_P,n_m,n_s,cells", [(1, 49, 19, 7, True), (3, 74, 8, 43, True), (500, 29, 8, 5, True), (1, 1023, 256, 64, False), (64, 511, 128, 32, False),
+                                                        (2, 70, 19, 8, True), (900, 70, 19, 8, False), (900, 30, 33, 64, False)])
+def test_which_grids_have_a_cell_per_thread(lib, n_tables, n_P, n_m, n_s, cells):
+    grid = plogp.GridArgs(np.arange(1, n_m + 1) * 4096, None, 2, n_P + 1, np.arange(1, n_s + 1) * 64)
+    h = load(lib, n_tables)
+    try:
+        for call in (lambda: lib.plogp_select_best(h, grid.ref, OUT, OUT, OUT, None), lambda: lib.plogp_predict(h, grid.ref, OUT, OUT, None)):
+            n = lib.fake_direct()
+            assert call() == plogp.OK and lib.fake_direct() - n == cells and lib.fake_bad_accesses() == 0
+    finally:
         lib.plogp_table_free(h)
