@@ -75,9 +75,13 @@ struct Plan {
     bool select = false;
     int sel_ptiles = 1, sel_run = 1;
     // tiling of decide_kernel and segmin_kernel (short candidate lists)
-    int ln_width = 32, ln_mgroups = 0, ln_np = 512, ln_ptiles = 1, ln_pairs = 1;
+    struct Tiling {
+        int width = 32, mgroups = 0, np = 512, ptiles = 1, pairs = 1;
+        size_t off_knots = 0;
+        bool gaps = false;  // run the gap pre-pass in front
+    };
+    Tiling ln, lp;      // of the decision and of the predictions
     int ln_staged = 0;  // threads of a CTA that has all message sizes, or 0
-    size_t off_knots = 0;
     bool dr_decide = false, dr_predict = false;  // small grids: a cell per thread
     int dr_ptiles = 1;
     // sweep kernel
@@ -86,7 +90,6 @@ struct Plan {
     int tables_per_batch = 0;
     size_t scratch_bytes = 0;
     size_t off_k = 0;          // their k table inside the grid blob
-    bool use_gaps = false;     // run the gap pre-pass in front of them
     int gaps_stride = 0;       // doubles per table in its output
     size_t gaps_bytes_per_table = 0;
 };
@@ -351,20 +354,40 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     // tables, P = 2..512, 32 candidates, on average; 72 message sizes 473 us with 8 side by side, 100 513 with 16, 50 253 with
     // 32).  Small grids so get many groups with few candidates each.
     if (pl.inline_sweep && pl.n_seg > 0) {
-        long long best = 0;
-        for (int width = 32; width >= 8; width >>= 1) {
-            const int mgroups = (n_m + width - 1) / width, groups = kDecThreads / width;
-            for (int np = 512; np >= groups * 8; np >>= 1) {
-                if (np > groups * 8 && np / 2 >= n_P) continue;
-                const int tiles = (n_P + np - 1) / np;
-                const long long ctas = (long long)mgroups * tiles * h->T.n_tables;
-                const long long per_cta = 1000 + 70 * ((n_s + groups - 1) / groups) + np / groups * (width == 32 ? 44 : width == 16 ? 53 : 77);
-                const long long cost = std::max(ctas, (long long)h->sm_count * 4) * per_cta;
-                if (best && cost >= best) continue;
-                best = cost;
-                pl.ln_width = width; pl.ln_mgroups = mgroups; pl.ln_np = np; pl.ln_ptiles = tiles;
+        const long long hold = (long long)h->sm_count * 4;
+        auto choose = [&](Plan::Tiling &best_tiling, long long floor, long long most) {  // with at most `most` CTAs; its cost, 0 if there is none
+            long long best = 0;
+            for (int width = 32; width >= 8; width >>= 1) {
+                const int groups = kDecThreads / width;
+                for (int np = 512; np >= groups * 8; np >>= 1) {
+                    if (np > groups * 8 && np / 2 >= n_P) continue;
+                    Plan::Tiling t;
+                    t.width = width; t.np = np; t.mgroups = (n_m + width - 1) / width; t.ptiles = (n_P + np - 1) / np;
+                    const long long ctas = (long long)t.mgroups * t.ptiles * h->T.n_tables;
+                    const long long per_cta = 1000 + 70 * ((n_s + groups - 1) / groups) + np / groups * (width == 32 ? 44 : width == 16 ? 53 : 77);
+                    const long long cost = std::max(ctas, floor) * per_cta;
+                    if (ctas > most || (best && cost >= best)) continue;
+                    best = cost;
+                    best_tiling = t;
+                }
             }
+            return best;
+        };
+        const long long any = std::numeric_limits<long long>::max(), best = choose(pl.ln, hold, any);
+        pl.lp = pl.ln;
+        // Fewer and larger CTAs where the Scatter half then has room beside them in one launch (below) for runs of at most 64 process
+        // counts, for up to 1.45 of the instructions: 200 tables of 99 x 9, 10 candidates 15.8 -> 11.0 us a call, 16 of 1023 x 64, 32
+        // candidates 30.2 -> 16.7; with runs of 128 (64 of 511 x 37, 16 candidates) 24.2 -> 31.4, at 1.64 (64 of 511 x 128, 32 candidates)
+        // 33.8 -> 38.4, with 40 candidates, of which a group then has more (108 of 32 x 61) 11.6 -> 12.7.
+        const long long scatter_ctas = (long long)((n_m + 31) / 32) * h->T.n_tables;
+        if (n_s <= 32 && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u) && (long long)pl.ln.mgroups * pl.ln.ptiles * h->T.n_tables + scatter_ctas > hold) {
+            Plan::Tiling beside;
+            const long long cost = choose(beside, hold, hold - scatter_ctas * ((n_P + 255) / 256));
+            if (cost && 20 * cost <= 29 * best) pl.ln = beside;
         }
+        // Predictions of few candidates, whose other planes' kernel takes what is left of the GPU: fewer and larger CTAs, which are
+        // mostly set-up (72 tables of 713 x 25, 4 candidates 40.8 -> 38.0 us; one of 999 x 255, 63 candidates 14.8 -> 16.1).
+        if (n_s <= 8) choose(pl.lp, h->sm_count, any);
         // A cell per thread (direct.cuh), 250 instructions and 30 per candidate: where that is half as many as a line for a range of
         // process counts, or no more and the GPU is nearly empty, so that only the length of a CTA counts.  Calls from a graph, lines ->
         // cells, us: one table, 49 process counts, 19 message sizes, 7 candidates 6.8 -> 4.6; 18 x 101, 48 candidates 8.7 -> 5.8; 3
@@ -377,7 +400,7 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         pl.dr_predict = 5 * cost < 3 * best || (cost < best && ctas <= (long long)h->sm_count);
         pl.dr_ptiles = int(ctas / h->T.n_tables);
         // All message sizes in a CTA, where there are two for every SM: threads for as many groups as leave the fewest idle
-        if (n_m <= kLineThreads && (long long)pl.ln_ptiles * h->T.n_tables >= (long long)h->sm_count * 2) {
+        if (n_m <= kLineThreads && (long long)pl.ln.ptiles * h->T.n_tables >= (long long)h->sm_count * 2) {
             double most = 0.0;
             for (int t = 128; t <= kLineThreads; t += 32) {
                 const double busy = double(t / n_m * n_m) / t;
@@ -387,10 +410,10 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     }
     // One launch for both halves where the GPU holds all their CTAs at once (four per SM, six with a cell per thread; its Scatter CTAs
     // have four warps)
-    {
-        const long long decide = (pl.dr_decide ? (long long)pl.dr_ptiles : (long long)pl.ln_mgroups * pl.ln_ptiles) * h->T.n_tables, base = (long long)pl.n_mtiles * h->T.n_tables;
-        const long long room = (long long)h->sm_count * (pl.dr_decide ? 6 : 4) - decide;
-        pl.select = pl.ln_mgroups > 0 && room >= base && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
+    if (pl.ln.mgroups > 0 && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u)) {
+        const long long base = (long long)pl.n_mtiles * h->T.n_tables, hold = (long long)h->sm_count * (pl.dr_decide ? 6 : 4);
+        const long long decide = (pl.dr_decide ? (long long)pl.dr_ptiles : (long long)pl.ln.mgroups * pl.ln.ptiles) * h->T.n_tables, room = hold - decide;
+        pl.select = room >= base;
         if (pl.select) {
             pl.sel_run = int(std::max<long long>(4, (n_P + kDecWarps * (room / base) - 1) / (kDecWarps * (room / base))));
             pl.sel_ptiles = (n_P + kDecWarps * pl.sel_run - 1) / (kDecWarps * pl.sel_run);
@@ -398,12 +421,12 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     }
     // Knots: the ends of up to kLineSegs segments of a CTA's process counts, by the ratio of process counts, on the last one of
     // a step of eight
-    std::vector<int32_t> knots;
-    if (pl.ln_mgroups > 0)
-        for (int t = 0; t < pl.ln_ptiles; ++t) {
-            const int first = t * pl.ln_np, n = std::min(n_P, first + pl.ln_np) - first;
+    auto knots_of = [&](Plan::Tiling &tiling) {
+        std::vector<int32_t> knots;
+        for (int t = 0; t < tiling.ptiles; ++t) {
+            const int first = t * tiling.np, n = std::min(n_P, first + tiling.np) - first;
             auto P_at = [&](int i) { return g->P ? int64_t(g->P[first + i]) : int64_t(g->P_lo) + first + i; };
-            pl.ln_pairs = std::max(pl.ln_pairs, log2_pair(P_at(n - 1)) - log2_pair(P_at(0)) + 1);
+            tiling.pairs = std::max(tiling.pairs, log2_pair(P_at(n - 1)) - log2_pair(P_at(0)) + 1);
             const size_t at = knots.size();
             knots.resize(at + kLineSegs + 2, n - 1);
             int n_segs = 0, end = 0;
@@ -418,6 +441,8 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
             if (n_segs == 0) n_segs = 1;  // one process count
             knots[at + kLineSegs + 1] = n_segs;
         }
+        return knots;
+    };
 
     // ---- device arrays ----
     std::vector<unsigned char> blob;
@@ -433,7 +458,10 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         off_s = append_aligned(blob, s32);
     }
 
-    if (!knots.empty()) pl.off_knots = append_aligned(blob, knots);
+    if (pl.ln.mgroups > 0) {
+        pl.ln.off_knots = append_aligned(blob, knots_of(pl.ln));
+        pl.lp.off_knots = append_aligned(blob, knots_of(pl.lp));
+    }
     // Short candidate lists: Section 2's k for every (candidate, m), as the doubles the kernels multiply with
     const bool short_lists = pl.inline_sweep && pl.n_seg > 0 && n_s > 0;
     if (short_lists) {
@@ -537,9 +565,13 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     // The gap pre-pass costs a launch: taken where decide_kernel and segmin_kernel run many CTAs per table and fill the GPU several times over
     // (4096 tables, P = 2..512, 128 m, 32 sizes: 1290 -> 1280 us)
     if (pl.inline_sweep && pl.n_seg > 0) {
-        const long long ctas_per_table = (long long)pl.ln_mgroups * pl.ln_ptiles;
-        pl.use_gaps = ctas_per_table >= 4 && ctas_per_table * h->T.n_tables >= (long long)h->sm_count * 16;
-        if (pl.use_gaps) {
+        for (Plan::Tiling *tiling : {&pl.ln, &pl.lp}) {
+            const long long ctas_per_table = (long long)tiling->mgroups * tiling->ptiles;
+            tiling->gaps = ctas_per_table >= 4 && ctas_per_table * h->T.n_tables >= (long long)h->sm_count * 16;
+        }
+        pl.ln.gaps &= !pl.dr_decide;
+        pl.lp.gaps &= !pl.dr_predict;
+        if (pl.ln.gaps || pl.lp.gaps) {
             pl.gaps_stride = (1 + n_s + n_m + 1) & ~1;
             pl.gaps_bytes_per_table = size_t(pl.gaps_stride) * sizeof(double);
             per_table += pl.gaps_bytes_per_table;
@@ -608,7 +640,7 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             ws += align_up(cells * sizeof(uint32_t), 256);
         }
         double *gaps = nullptr;
-        if (pl.use_gaps && pl.inline_sweep && pl.n_seg > 0 && (predict ? !pl.dr_predict : use_decide && !pl.dr_decide)) {
+        if (predict ? pl.lp.gaps : use_decide && pl.ln.gaps) {
             gaps = reinterpret_cast<double *>(ws);
             GapsParams gp{};
             gp.T = h->T; gp.G = pl.G;
@@ -641,8 +673,9 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
         auto lines = [&]() {
             LinesParams lp{};
             lp.T = h->T; lp.G = pl.G;
-            lp.width = pl.ln_width; lp.threads = kDecThreads; lp.n_mgroups = pl.ln_mgroups; lp.n_p = pl.ln_np; lp.n_ptiles = pl.ln_ptiles; lp.n_pairs = pl.ln_pairs;
-            lp.knots = reinterpret_cast<const int32_t *>(pl.d_grid + pl.off_knots);
+            const Plan::Tiling &t = predict ? pl.lp : pl.ln;
+            lp.width = t.width; lp.threads = kDecThreads; lp.n_mgroups = t.mgroups; lp.n_p = t.np; lp.n_ptiles = t.ptiles; lp.n_pairs = t.pairs;
+            lp.knots = reinterpret_cast<const int32_t *>(pl.d_grid + t.off_knots);
             lp.gaps = gaps; lp.gaps_stride = pl.gaps_stride;
             lp.table0 = t0; lp.n_tables_launch = nt; lp.out_table0 = out.out_table0; lp.om = out.om;
             if (predict ? pl.dr_predict : pl.dr_decide) { lp.direct = 1; lp.n_mgroups = 1; lp.n_ptiles = pl.dr_ptiles; }
