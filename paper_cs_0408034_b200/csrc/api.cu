@@ -81,7 +81,9 @@ struct Plan {
         bool gaps = false;  // run the gap pre-pass in front
     };
     Tiling ln, lp;      // of the decision and of the predictions
-    int ln_staged = 0;  // threads of a CTA that has all message sizes, or 0
+    int all_threads = 0;        // threads of a CTA that has all message sizes, or 0
+    bool all_decide = false, all_predict = false;  // where such CTAs are taken, if two of them fit an SM
+    bool all_alone = false;     // (predictions) or if one does
     bool dr_decide = false, dr_predict = false;  // small grids: a cell per thread
     int dr_ptiles = 1;
     // sweep kernel
@@ -399,13 +401,33 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         pl.dr_decide = 2 * cost < best || (cost < best && ctas <= (long long)h->sm_count * 2);
         pl.dr_predict = 5 * cost < 3 * best || (cost < best && ctas <= (long long)h->sm_count);
         pl.dr_ptiles = int(ctas / h->T.n_tables);
-        // All message sizes in a CTA, where there are two for every SM: threads for as many groups as leave the fewest idle
-        if (n_m <= kLineThreads && (long long)pl.ln.ptiles * h->T.n_tables >= (long long)h->sm_count * 2) {
-            double most = 0.0;
+        // All message sizes in a CTA (STAGED, lines.cuh), for rows off the sectors: threads for as many groups as leave the fewest
+        // idle.  Worth it where a CTA's process counts make up for its set-up, on grids of several CTAs per SM.
+        if (n_m > 32 && n_m <= kLineThreads) {
+            double busy = 0.0;
             for (int t = 128; t <= kLineThreads; t += 32) {
-                const double busy = double(t / n_m * n_m) / t;
-                if (busy >= most) { most = busy; pl.ln_staged = t; }
+                const double b = double(t / n_m * n_m) / t;
+                if (b >= busy) { busy = b; pl.all_threads = t; }
             }
+            const double busy_lines = double(n_m) / (pl.ln.mgroups * pl.ln.width);
+            const long long d_ctas = (long long)pl.ln.ptiles * h->T.n_tables, p_ctas = (long long)pl.lp.ptiles * h->T.n_tables;
+            // Decision, odd rows only: with half the bytes of a plane the waits weigh more.  Time with row segments = 1: 511 process
+            // counts, 8 / 20 / 32 candidates: 1200 tables of 33 message sizes 0.89 0.96 1.07, 65 1.04 1.17 1.31, 99 0.87 0.99 1.12, 127 0.83
+            // 0.93 1.03, 173 0.84 0.96, 201 0.80 0.90; 148 of 2999 process counts 33 0.80 0.84 0.88, 127 0.76 0.82 0.87; 600 tables of 127
+            // 0.97 1.04 1.14; 320 of 199 process counts and 127 1.58 1.55 1.53.  Fewer process counts: only where lines would leave more
+            // lanes idle (2048 tables of 100, 33 message sizes 0.93 0.89 0.84; 47 1.14 1.13 1.12, 127 1.04 1.05 1.06) or candidates are few
+            // and rows long (1095 of 31, 145 message sizes, 9 candidates 0.87; 4000 of 59, 8 candidates, 127 / 173 / 201 / 255 1.06
+            // 0.99 0.93 0.89).
+            pl.all_decide = n_m % 2 != 0 && d_ctas >= (long long)h->sm_count * 6 &&
+                            ((n_P >= 256 ? n_s <= (n_P >= 1024 ? 32 : 24) && busy >= 0.88 : n_P >= 96 && busy >= 1.1 * busy_lines) || (n_m >= 140 && n_s <= 16));
+            // Predictions, rows off the sectors of the sizes, or of times and sizes.  The same at 511 process counts: 1200 tables of 33 0.56
+            // 0.59 0.63, 65 0.61 0.66 0.72, 127 0.56 0.60 0.64, 201 0.56 0.61, 100 (whole sectors of times) 0.70 0.77 0.85; 2048 tables of
+            // 200 process counts: 33 0.82 0.88 0.96, 127 0.56 0.62 0.67, 100 0.95 1.07 1.33; of 100: 33 1.07 1.04 1.00, 65 0.91 1.07 1.14, 99
+            // 0.76 0.87 0.98, 201 0.70 0.81 0.91; 4000 of 59: 99 1.11 1.14 1.22; 320 of 199: 99 1.01 1.02 1.15.
+            pl.all_predict = n_m % 8 != 0 && p_ctas >= (long long)h->sm_count * 4 && (n_m % 4 == 0 ? n_P >= 256 && n_s <= 32 : n_P >= (n_m >= 96 ? 96 : 192));
+            // One CTA per SM: 1200 tables of 511 process counts, 20 / 32 / 48 candidates: 255 0.79 0.87 0.99, 250 0.83 0.94 1.07, 201 at 32
+            // 0.96, at 48 1.13; 173 at 32 1.10, 127 at 48 1.05; 148 of 2999, 48 candidates 255 0.89, 250 0.98; 2048 of 200, 255 0.80 0.92 1.09.
+            pl.all_alone = n_m % 4 != 0 && n_m > 192 && n_s <= (n_P >= 1024 ? 48 : 32) && n_P >= 192;
         }
     }
     // One launch for both halves where the GPU holds all their CTAs at once (four per SM, six with a cell per thread; its Scatter CTAs
@@ -682,19 +704,21 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
             return lp;
         };
         // All message sizes in a CTA, where two of them fit an SM (228 KB, 1 KB of it each CTA's own): the shared memory grows with
-        // message sizes times candidates and times (floor, ceil) pairs, past what a CTA can have.
-        auto stage = [&](LinesParams &lp) {
+        // message sizes times candidates and times (floor, ceil) pairs, past what a CTA can have.  With one per SM (1200 tables of 511
+        // process counts, 48 candidates, 127 / 173 / 255 message sizes) the decision takes 1.80 / 2.02 / 1.56 times as long as row segments.
+        auto stage = [&](LinesParams &lp, size_t most) {
             LinesParams whole = lp;
-            whole.staged = 1; whole.width = pl.G.n_m; whole.n_mgroups = 1; whole.threads = pl.ln_staged;
-            if (2 * (lines_smem_bytes(whole) + 1024) <= size_t(228) * 1024) lp = whole;
+            whole.staged = 1; whole.width = pl.G.n_m; whole.n_mgroups = 1; whole.threads = pl.all_threads;
+            if (lines_smem_bytes(whole) <= most) lp = whole;
         };
+        constexpr size_t kHalf = 113 * 1024;
         if (predict && pl.inline_sweep && pl.n_seg > 0) {
             // Predictions on short candidate lists: the segmented minima (planes 2, 5, 9 and the best segment sizes)
             // come from segmin_kernel; the kernels behind it write the other planes.
             LinesParams sp = lines();
             sp.p_time = out.p_time; sp.p_best_s = out.p_best_s;
-            // rows off the sectors of the sizes, or of times and sizes; up to 16 message sizes few warps have many lines (lines.cuh)
-            if (!sp.direct && pl.ln_staged && pl.G.n_m % 8 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.p_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.p_best_s) % 16 == 0) stage(sp);
+            if (!sp.direct && pl.all_predict && reinterpret_cast<uintptr_t>(out.p_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.p_best_s) % 16 == 0)
+                stage(sp, pl.all_alone ? size_t(kMaxSmem) : kHalf);
             { LaunchTimer lt(h, PLOGP_KERNEL_SEGMIN, st); CK(launch_segmin(sp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= ~kSegBits;
@@ -718,9 +742,8 @@ int run(plogp_tables *h, const plogp_grid *g, bool predict, FusedParams out, cud
                 g_launches += 1;
                 continue;
             }
-            // odd rows only: with half the bytes of a plane the waits weigh more (lines.cuh has both sides)
-            if (!dp.direct && pl.ln_staged && pl.G.n_m % 2 != 0 && pl.G.n_m > 16 && reinterpret_cast<uintptr_t>(out.d_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 16 == 0 &&
-                reinterpret_cast<uintptr_t>(out.d_strategy) % 4 == 0) stage(dp);
+            if (!dp.direct && pl.all_decide && reinterpret_cast<uintptr_t>(out.d_time) % 32 == 0 && reinterpret_cast<uintptr_t>(out.d_sbytes) % 16 == 0 &&
+                reinterpret_cast<uintptr_t>(out.d_strategy) % 4 == 0) stage(dp, kHalf);
             { LaunchTimer lt(h, PLOGP_KERNEL_DECIDE, st); CK(launch_decide(dp, overlap && gaps, st)); }
             g_launches += 1;
             Gf.mask &= 0x1C00u;

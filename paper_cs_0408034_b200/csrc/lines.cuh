@@ -36,9 +36,8 @@
 // 0.91 ms), and so do loads of k from global memory (0.95).
 //
 // STAGED: rows off the sectors cost twice (parts of sectors at both ends of every row segment); put together first they go out whole,
-// but the CTA's warps wait for the one with the most lines.  2048 tables, direct -> staged, decision half: 127 message sizes 724 -> 676
-// us, 33 296 -> 258, but 100 513 -> 575, 50 253 -> 319; planes (4096): 127 2.01 -> 1.17 ms, 100 1.18 -> 0.97, 50 0.77 -> 0.49,
-// 72 (whole sectors) 0.51 -> 0.69, 9 0.10 -> 0.15.
+// but the CTA's warps wait for the one with the most lines, and its set-up and shared memory are those of all message sizes (up to
+// 256).  api.cu says where, with both sides measured.
 #pragma once
 
 #include "device_common.cuh"

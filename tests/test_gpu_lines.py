@@ -65,15 +65,19 @@ def test_lines_close_to_one_another(plogp, kind, n_s):
     both(plogp, replace(w, gaps=np.ascontiguousarray(g), latency=w.latency * (1e9 if kind == "latency" else 1.0)))
 
 
-@pytest.mark.parametrize("n_m,n_P,n_s,listed", [(17, 21, 9, False), (33, 520, 33, False), (50, 16, 8, False), (127, 40, 20, True), (129, 9, 64, False), (255, 33, 5, False), (256, 8, 3, False)])
-def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed):
-    """Many tables: the cells of a step put together in shared memory.  The same as with outputs aligned for single elements,
-    which are stored one by one, and as the oracle's for some tables."""
+@pytest.mark.parametrize("n_m,n_P,n_s,listed,n_tables", [
+    (17, 21, 9, False, 300), (33, 520, 33, False, 300), (50, 16, 8, False, 300), (127, 40, 20, True, 300), (129, 9, 64, False, 300), (255, 33, 5, False, 300), (256, 8, 3, False, 300),
+    (33, 97, 33, False, 900), (33, 511, 24, True, 900), (127, 257, 24, False, 900), (201, 256, 3, True, 900), (173, 300, 1, False, 900), (99, 520, 9, False, 450),
+    (145, 31, 9, False, 900), (35, 1100, 32, False, 300), (34, 193, 20, False, 600), (52, 257, 32, False, 600), (250, 260, 32, True, 600), (255, 256, 20, False, 600)])
+def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed, n_tables):
+    """Many tables, rows off the sectors: the cells of a step put together in shared memory, for the predictions and the decision
+    (600 tables: the predictions alone; 300 of few process counts: neither).  The same as with outputs aligned for single
+    elements, which are stored one by one, and as the oracle's for some tables."""
     import torch
-    w = wl_grid(n_tables=300, n_P=n_P, n_m=n_m, n_s=n_s)
+    w = wl_grid(n_tables=n_tables, n_P=n_P, n_m=n_m, n_s=n_s)
     if listed:
         w = replace(w, P_list=(2 + 3 * np.arange(n_P)).astype(np.int32))
-    both(plogp, w, tables=[0, 151, 299])
+    both(plogp, w, tables=[0, n_tables // 2 + 1, n_tables - 1])
 
     def off_by_one(x):
         return torch.zeros(x.numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x.shape)
@@ -89,15 +93,15 @@ def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed):
         assert p.best_s.equal(pred.best_s) and all(p.time[:, i].equal(pred.time[:, i]) for i in (2, 5, 9))
 
 
-@pytest.mark.parametrize("n_m,n_s,octaves", [(255, 64, 0), (253, 48, 0), (201, 32, 0), (250, 64, 0), (229, 8, 29), (255, 27, 29), (255, 64, 29), (157, 20, 29)])
+@pytest.mark.parametrize("n_m,n_s,octaves", [(255, 64, 0), (253, 24, 0), (201, 32, 0), (250, 32, 0), (229, 8, 29), (255, 24, 29), (255, 32, 29), (157, 20, 29)])
 def test_more_than_a_cta_has_room_for(plogp, n_m, n_s, octaves):
-    """Many tables, odd rows, long lists and process counts over many (floor, ceil) pairs of log2 P: all message sizes together
-    would take more shared memory than a CTA, or than half of an SM, has."""
-    w = wl_grid(n_tables=300, n_P=511, n_m=n_m, n_s=n_s)
+    """Many tables, rows off the sectors, long lists and process counts over many (floor, ceil) pairs of log2 P: all message sizes
+    together would take more shared memory than a CTA, or than half of an SM, has."""
+    w = wl_grid(n_tables=900, n_P=300, n_m=n_m, n_s=n_s)
     if octaves:  # P m < 2^53; the oracle would add up the Scatter Chain's terms one by one
-        P = sorted({1 << i for i in range(1, octaves)} | {3 << i for i in range(octaves - 1)})
-        w = replace(w, P_list=np.array(P, dtype=np.int32), m=256 * np.arange(1, n_m + 1, dtype=np.uint64), strategy_mask=0x17FF)
-    both(plogp, w, tables=[0, 299])
+        P = np.unique(np.concatenate([1 << np.arange(1, octaves), np.rint(2.0 ** np.linspace(1.5, octaves - 0.5, 256))]))
+        w = replace(w, P_list=P.astype(np.int32), m=256 * np.arange(1, n_m + 1, dtype=np.uint64), strategy_mask=0x17FF)
+    both(plogp, w, tables=[0, 899])
 
 
 @pytest.mark.parametrize("kind", ["as drawn", "flat", "stairs", "falls"])
@@ -204,3 +208,9 @@ def test_a_cell_per_thread_as_lines(plogp, n_P, n_m, n_s, k_mode, listed, ids):
         for j, i in enumerate(po.SEGMENTED_IDS):
             if i in ids:
                 assert p.time[:, i].equal(q.time[first:first + 3, i]) and p.best_s[:, j].equal(q.best_s[first:first + 3, j])
+
+
+@pytest.mark.parametrize("n_tables,n_P,n_m,n_s", [(72, 200, 25, 4), (72, 713, 25, 8), (200, 99, 9, 10), (16, 600, 64, 32), (64, 511, 37, 16)])
+def test_tilings_of_medium_grids(plogp, n_tables, n_P, n_m, n_s):
+    """Fewer and larger CTAs: both halves in one launch, predictions of few candidates."""
+    both(plogp, wl_grid(n_tables=n_tables, n_P=n_P, n_m=n_m, n_s=n_s), tables=[0, n_tables - 1])

@@ -131,14 +131,14 @@ def test_device_memory_that_runs_out_for_a_grid_is_a_status(lib):
 
 
 def octaves(n):
-    """Listed process counts over n octaves, two (floor, ceil) pairs of log2 P in each."""
-    return np.array(sorted({1 << i for i in range(1, n)} | {3 << i for i in range(n - 1)}), dtype=np.int32)
+    """256 and more listed process counts over n octaves, two (floor, ceil) pairs of log2 P in each."""
+    return np.unique(np.concatenate([1 << np.arange(1, n), np.rint(2.0 ** np.linspace(1.5, n - 0.5, 256))])).astype(np.int32)
 
 
 @pytest.mark.parametrize("n_bp", [64, 1024])
 @pytest.mark.parametrize("n_m,P,n_s,n_tables", [
-    (255, 512, 64, 296), (253, 1024, 64, 148), (255, 3000, 60, 400), (250, 512, 64, 300), (252, 512, 64, 300), (255, 512, 61, 300),
-    (255, 29, 27, 300), (229, 29, 8, 300), (193, 29, 32, 300), (157, 29, 64, 300), (256, 29, 64, 300), (127, 512, 32, 300), (33, 29, 64, 300), (19, 29, 7, 1), (1, 29, 64, 1)])
+    (255, 512, 64, 1200), (253, 1024, 24, 900), (255, 3000, 32, 900), (250, 512, 32, 900), (255, 512, 24, 900), (255, 29, 24, 900), (255, 29, 32, 600), (229, 29, 8, 900),
+    (201, 29, 32, 900), (173, 29, 20, 900), (157, 29, 64, 900), (256, 29, 64, 900), (127, 512, 32, 900), (33, 29, 64, 900), (19, 29, 7, 1), (1, 29, 64, 1)])
 def test_shared_memory_fits(lib, n_m, P, n_s, n_tables, n_bp):
     """Every launch on a short candidate list has at most the shared memory of an SM, whatever the message sizes, the candidates
     and the (floor, ceil) pairs of log2 P are: P = 2..P, or listed over P octaves."""
@@ -177,5 +177,21 @@ def test_which_grids_have_a_cell_per_thread(lib, n_tables, n_P, n_m, n_s, cells)
         for call in (lambda: lib.plogp_select_best(h, grid.ref, OUT, OUT, OUT, None), lambda: lib.plogp_predict(h, grid.ref, OUT, OUT, None)):
             n = lib.fake_direct()
             assert call() == plogp.OK and lib.fake_direct() - n == cells and lib.fake_bad_accesses() == 0
+    finally:
+        lib.plogp_table_free(h)
+
+
+@pytest.mark.parametrize("n_tables,n_P,n_m,n_s,decide,predict", [
+    (900, 257, 127, 24, 1, 1), (900, 97, 33, 33, 1, 0), (900, 256, 201, 3, 1, 1), (450, 520, 99, 9, 1, 1), (600, 193, 34, 20, 0, 1), (600, 257, 52, 32, 0, 1),
+    (600, 260, 250, 32, 0, 1), (600, 256, 255, 20, 0, 1), (900, 257, 65, 24, 0, 1), (900, 97, 127, 24, 0, 1), (900, 95, 33, 33, 0, 0), (900, 31, 145, 9, 1, 0),
+    (900, 1100, 127, 32, 1, 1), (900, 257, 127, 64, 0, 0), (300, 257, 127, 24, 0, 0), (900, 257, 128, 24, 0, 0), (900, 257, 31, 8, 0, 0), (900, 257, 257, 8, 0, 0)])
+def test_which_grids_have_all_message_sizes_in_a_cta(lib, n_tables, n_P, n_m, n_s, decide, predict):
+    grid = plogp.GridArgs(np.arange(1, n_m + 1) * 4096, None, 2, n_P + 1, np.arange(1, n_s + 1) * 64)
+    h = load(lib, n_tables, 64)
+    try:
+        for out, want in ((OUT, (decide, predict)), (C.c_void_p(OUT.value + 8), (0, 0))):
+            for call, n in zip((lambda: lib.plogp_select_best(h, grid.ref, out, out, out, None), lambda: lib.plogp_predict(h, grid.ref, out, out, None)), want):
+                before = lib.fake_staged()
+                assert call() == plogp.OK and lib.fake_staged() - before == n and lib.fake_too_large() == 0
     finally:
         lib.plogp_table_free(h)
