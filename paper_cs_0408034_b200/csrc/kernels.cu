@@ -38,13 +38,19 @@ namespace plogp {
 //     of segments), before any candidate is looked at;
 //   * for its groups of 32, from the smallest coefficients;
 //   * for the group's candidates one by one.
-// Four at a time, what is left is compared in FP64.  The results are those of the exhaustive FP64 search, bit for bit.  The upper
-// bounds of the best times start from log-spaced candidates of the whole list (rounded up in FP32), so a chunk far from the
-// optimum never leaves the first step.  The best times themselves are touched by the exact pass alone and live in shared memory.
+// Four at a time, what is left is compared in FP64, unless the group's smallest coefficients in FP64 show that none is better than
+// what the warp has (a rounded fused multiply-add is monotone in them): where gaps are equal over many sizes, times are
+// equal and no bound in FP32 tells them apart, nor where times lie outside its range.  The results are those of the exhaustive FP64
+// search, bit for bit.  The upper bounds of the best times start from log-spaced candidates of the whole list (rounded up in FP32), so a
+// chunk far from the optimum never leaves the first step.  The best times themselves are touched by the exact pass alone and live in
+// shared memory.
 //
 // What bounds it: the exact passes of the CTAs that have the best sizes, one vote after another, while the others are done.  P =
 // 2..4096, 128 message sizes, every 4 B up to 1 MB, ids 2 and 5: 8.4 ms with a bound of every cell, 1.33 with groups of 32, 1.23 with
-// the first 256 process counts in CTAs of their own, 0.64 with sub-chunks passed over.
+// the first 256 process counts in CTAs of their own, 0.64 with sub-chunks passed over.  Tables that defeat the bounds, ms for ids 2
+// and 5 (id 9), with a bound of every cell -> groups compared in FP32 alone -> in FP64 as well: equal gaps 25.7 (12.1) -> 49.4 (19.5) ->
+// 11.4 (4.5), in stairs 11.5 (6.7) -> 4.4 (3.7) -> 1.1 (0.88), a latency 1e9 times the gaps 26.3 (27.1) -> 28.6 (35.1) -> 7.7 (8.9),
+// times outside FP32's range 86.8 (37.0) -> 108.9 (43.4) -> 30.3 (14.6).  Small sweeps pay 1 to 3 % for the groups' minima.
 //
 // A warp owns 256 consecutive process counts (lane + 32 r).  The CTA's 8 warps cover p.wp such tiles side by side and
 // split the candidates of a sub-chunk 8 / p.wp ways, so that a short range of process counts leaves no warp idle.
@@ -62,7 +68,8 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
     double2 *s_bc = reinterpret_cast<double2 *>(s_tab + 3 * p.T.npad);  // [2][kSweepSub]
     double *s_q = reinterpret_cast<double *>(s_bc + 2 * kSweepSub);     // [2][kSweepSub]
     double *s_best = s_q + 2 * kSweepSub;                               // [kNid][kWarps][R][32]
-    float *s_bf = reinterpret_cast<float *>(s_best + kNid * kWarps * R * 32);  // [2][kSweepSub]
+    double *s_db = s_best + kNid * kWarps * R * 32, *s_dc = s_db + 2 * kSweepGroups, *s_dq = s_dc + 2 * kSweepGroups;  // [2][kSweepGroups]: smallest of a group's
+    float *s_bf = reinterpret_cast<float *>(s_dq + 2 * kSweepGroups);  // [2][kSweepSub]
     float *s_cf = s_bf + 2 * kSweepSub, *s_qf = s_cf + 2 * kSweepSub;
     float *s_gb = s_qf + 2 * kSweepSub, *s_gc = s_gb + 2 * kSweepGroups, *s_gq = s_gc + 2 * kSweepGroups;  // [2][kSweepGroups]: smallest of a group's
     float *s_lb = s_gq + 2 * kSweepGroups, *s_lc = s_lb + kThreads, *s_lq = s_lc + kThreads;  // [kThreads]: bounds of a sub-chunk's
@@ -131,21 +138,24 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
         const int first = s_begin + sub * kSweepSub, o = buf * kSweepSub + tid;
         double B = CUDART_INF, C = CUDART_INF, Q = CUDART_INF;  // padding: the bound is +inf
         if (tid < s_end - first) coefficients(first + tid, B, C, Q);
-        // a warp's candidates are a group; non-negative floats are ordered as whole numbers
+        // a warp's candidates are a group
         if (HAS5) {
             const float b = __double2float_rd(B), c = __double2float_rd(C);
             s_bc[o] = make_double2(B, C);
             s_bf[o] = b;
             s_cf[o] = c;
-            const unsigned b_min = __reduce_min_sync(kFull, __float_as_uint(b)), c_min = __reduce_min_sync(kFull, __float_as_uint(c));
-            if (lane == 0) { s_gb[o >> 5] = __uint_as_float(b_min); s_gc[o >> 5] = __uint_as_float(c_min); }
+            const double b_min = warp_min(B), c_min = warp_min(fmin(C, CUDART_INF));  // inf * 0 as inf
+            if (lane == 0) {
+                s_db[o >> 5] = b_min; s_gb[o >> 5] = __double2float_rd(b_min);
+                s_dc[o >> 5] = c_min; s_gc[o >> 5] = __double2float_rd(c_min);
+            }
         }
         if (QL) {
             const float q = __double2float_rd(Q);
             s_q[o] = Q;
             s_qf[o] = q;
-            const unsigned q_min = __reduce_min_sync(kFull, __float_as_uint(q));
-            if (lane == 0) s_gq[o >> 5] = __uint_as_float(q_min);
+            const double q_min = warp_min(Q);
+            if (lane == 0) { s_dq[o >> 5] = q_min; s_gq[o >> 5] = __double2float_rd(q_min); }
         }
     };
 
@@ -248,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
 #pragma unroll 1
             for (int g = 0; g < g_len; ++g) {
                 const unsigned hit = rows_of(HAS5 ? gb[g] : 0.f, HAS5 ? gc[g] : 0.f, QL ? gq[g] : 0.f);
-                const int j0 = 32 * (my_c * g_len + g);
+                const int j0 = 32 * (my_c * g_len + g), gd = buf * kSweepGroups + my_c * g_len + g;
                 const float *bf = s_bf + buf * kSweepSub + j0, *cf4 = s_cf + buf * kSweepSub + j0, *qf = s_qf + buf * kSweepSub + j0;
                 if (__any_sync(kFull, hit != 0)) {
                     // Exact pass over the group for the flagged rows: candidates in ascending order, strict '<' (smallest s on
@@ -269,7 +279,8 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
                             if (HAS5 && five && q == r) T = T5[q];
                             if (QL && !five && q == r) T = T2[q];
                         }
-                        // the group's candidates one by one, in FP32 first and all at once: mostly none is not above
+                        // The group's candidates one by one, in FP32 and all at once: mostly none is not above.  And none is better than what
+                        // this warp has, which is of a smaller size, if the FP64 line of the group's smallest coefficients is not.
                         {
                             const f32x2 x2 = splat2(xr), c2 = splat2(cfl);
                             float low = CUDART_INF_F;
@@ -284,7 +295,8 @@ __global__ void __launch_bounds__(kThreads, 2) sweep_kernel(const SweepParams p)
                                 }
                                 low = min_with2(min_with2(low, fma2_down(x2, a.x, c.x)), fma2_down(x2, a.y, c.y));
                             }
-                            if (!__any_sync(kFull, low <= T)) continue;
+                            const double t_least = five ? fma(x, s_db[gd], s_dc[gd]) : fma(x, s_dq[gd], c);
+                            if (!__any_sync(kFull, low <= T && t_least < bt)) continue;
                         }
 #pragma unroll 1
                         for (int i = 0; i < 32; i += 4) {
@@ -658,7 +670,7 @@ static cudaError_t launch_sweep_t(const SweepParams &p, int n_tables_launch, boo
 {
     constexpr int n_id = (HAS2 ? 1 : 0) + (HAS5 ? 1 : 0) + (IS9 ? 1 : 0);
     const size_t smem = 3 * static_cast<size_t>(p.T.npad) * sizeof(double) +
-                        2 * kSweepSub * (sizeof(double2) + sizeof(double) + 3 * sizeof(float)) + (2 * kSweepGroups + kThreads) * 3 * sizeof(float) + kThreads * sizeof(int) +
+                        2 * kSweepSub * (sizeof(double2) + sizeof(double) + 3 * sizeof(float)) + 2 * kSweepGroups * 3 * (sizeof(double) + sizeof(float)) + kThreads * 3 * sizeof(float) + kThreads * sizeof(int) +
                         static_cast<size_t>(n_id) * kWarps * kSweepR * 32 * (sizeof(double) + sizeof(uint32_t));
     const long long bx = static_cast<long long>(p.n_pairs) * p.n_ptiles;
     if (bx <= 0 || bx > 0x7FFFFFFFLL || n_tables_launch > 65535) return cudaErrorInvalidConfiguration;

@@ -214,3 +214,16 @@ def test_a_cell_per_thread_as_lines(plogp, n_P, n_m, n_s, k_mode, listed, ids):
 def test_tilings_of_medium_grids(plogp, n_tables, n_P, n_m, n_s):
     """Fewer and larger CTAs: both halves in one launch, predictions of few candidates."""
     both(plogp, wl_grid(n_tables=n_tables, n_P=n_P, n_m=n_m, n_s=n_s), tables=[0, n_tables - 1])
+
+
+@pytest.mark.parametrize("ids", [(2, 5), (9,), (2, 5, 9), range(10)])
+@pytest.mark.parametrize("n_s,s_step,k_mode,P_lo", [(65, 4, 0, 2), (600, 4, 1, 2), (3000, 64, 0, 250), (2049, 4, 0, 2)])
+def test_ties_in_long_lists(plogp, ids, n_s, s_step, k_mode, P_lo):
+    """Whole gaps at powers of two, equal over many of them, and long lists of candidates: exact products, many equal times.
+    Sub-chunks and groups that are passed over hold none that is better, nor a smaller size as good."""
+    rng = np.random.default_rng(n_s)
+    gaps = np.cumsum(rng.integers(0, 2, (8, 21)) * rng.integers(0, 2, (8, 21)) * rng.integers(0, 2, (8, 1)), axis=1).astype(np.float64) + 1.0
+    w = replace(wl_grid(n_tables=8, n_P=280, n_m=1, n_s=1, k_mode=k_mode, P_lo=P_lo), sizes=(1 << np.arange(21)).astype(np.uint64), gaps=gaps,
+                latency=rng.integers(0, 3, 8).astype(np.float64), strategy_mask=sum(1 << i for i in ids), s_list=None, s_lo=4, s_hi=4 + s_step * (n_s - 1), s_step=s_step,
+                m=np.array([4, 512, 1024, 6000, 65536, 100000, 1 << 20], dtype=np.uint64))
+    picks_as_the_oracle(plogp, w, range(8))
