@@ -441,8 +441,9 @@ __device__ __forceinline__ void lines_block(const LinesParams &p, int block, uns
                             line(B, C, sm.sval[c], id5);
                         });
                     if (f & 4u) {
-                        line(chain_a, 0.0, chain5 ? m_u : 0u, id_chain);
-                        if (chain5 && (mask & 0x10u)) line(gm + rdv, 0.0, 0u, p.om.id_of[4]);
+#pragma unroll 1
+                        for (int again = chain5 && (mask & 0x10u) ? 1 : 0, i = 0; i <= again; ++i)
+                            line(i ? gm + rdv : chain_a, 0.0, chain5 && !i ? m_u : 0u, i ? static_cast<uint32_t>(p.om.id_of[4]) : id_chain);
                     }
                     if (has2) {
                         if (near0 | near1) {
