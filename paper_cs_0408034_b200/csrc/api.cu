@@ -355,6 +355,11 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
     // group, 44 per process count of a group with 32 message sizes side by side, more with the shorter stores of fewer (4096
     // tables, P = 2..512, 32 candidates, on average; 72 message sizes 473 us with 8 side by side, 100 513 with 16, 50 253 with
     // 32).  Small grids so get many groups with few candidates each.
+    // CTAs of the Scatter half, four warps each, for runs of at most 64 process counts: with longer ones its chains are what a launch of
+    // both halves waits for (48 tables of 1384 x 24, 10 candidates 48.6 us, in two launches 18.9; 4 of 2696 x 33 16.8, where there had been
+    // more room 11.5)
+    const bool both = (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u);
+    const long long scatter_ctas = (long long)pl.n_mtiles * h->T.n_tables * ((n_P + 255) / 256);
     if (pl.inline_sweep && pl.n_seg > 0) {
         const long long hold = (long long)h->sm_count * 4;
         auto choose = [&](Plan::Tiling &best_tiling, long long floor, long long most) {  // with at most `most` CTAs; its cost, 0 if there is none
@@ -377,29 +382,42 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
         };
         const long long any = std::numeric_limits<long long>::max(), best = choose(pl.ln, hold, any);
         pl.lp = pl.ln;
-        // Fewer and larger CTAs where the Scatter half then has room beside them in one launch (below) for runs of at most 64 process
-        // counts, for up to 1.45 of the instructions: 200 tables of 99 x 9, 10 candidates 15.8 -> 11.0 us a call, 16 of 1023 x 64, 32
-        // candidates 30.2 -> 16.7; with runs of 128 (64 of 511 x 37, 16 candidates) 24.2 -> 31.4, at 1.64 (64 of 511 x 128, 32 candidates)
-        // 33.8 -> 38.4, with 40 candidates, of which a group then has more (108 of 32 x 61) 11.6 -> 12.7.
-        const long long scatter_ctas = (long long)((n_m + 31) / 32) * h->T.n_tables;
-        if (n_s <= 32 && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u) && (long long)pl.ln.mgroups * pl.ln.ptiles * h->T.n_tables + scatter_ctas > hold) {
+        // Fewer and larger CTAs where the Scatter half then has room beside them in one launch (below) for runs of at most 32 process
+        // counts (17 tables of 201 x 185, 8 candidates, with runs of 51 17.7 -> 22.0 us a call), for up to 1.45 of the instructions: 200 tables
+        // of 99 x 9, 10 candidates 15.8 -> 11.0, 16 of 1023 x 64, 32 candidates 30.2 -> 16.7; at 1.64 (64 of 511 x 128, 32 candidates) 33.8 ->
+        // 38.4, with 40 candidates, of which a group then has more (108 of 32 x 61) 11.6 -> 12.7.
+        auto fits = [&](const Plan::Tiling &t) { return (long long)t.mgroups * t.ptiles * h->T.n_tables + scatter_ctas <= hold; };
+        const long long lines_ctas = (long long)pl.ln.mgroups * pl.ln.ptiles * h->T.n_tables;
+        if (n_s <= 32 && both && !fits(pl.ln)) {
             Plan::Tiling beside;
-            const long long cost = choose(beside, hold, hold - scatter_ctas * ((n_P + 255) / 256));
+            const long long cost = choose(beside, hold, hold - (long long)pl.n_mtiles * h->T.n_tables * ((n_P + 127) / 128));
             if (cost && 20 * cost <= 29 * best) pl.ln = beside;
         }
-        // Predictions of few candidates, whose other planes' kernel takes what is left of the GPU: fewer and larger CTAs, which are
-        // mostly set-up (72 tables of 713 x 25, 4 candidates 40.8 -> 38.0 us; one of 999 x 255, 63 candidates 14.8 -> 16.1).
-        if (n_s <= 8) choose(pl.lp, h->sm_count, any);
+        // Where another kernel of the call takes what is left of the GPU, the total counts more than a CTA's length: 27 tables of 83 x 168, 34
+        // candidates 15.1 -> 11.2, 200 of 299 x 50, 30 candidates 39.3 -> 34.2, 159 of 594 x 9, 5 candidates 31.2 -> 26.0; long lists, of which a
+        // group then has more, 64 of 511 x 128, 32 candidates 33.8 -> 35.7, 99 of 957 x 24, 62 candidates 73.9 -> 88.1 (two decisions).
+        if (n_s <= 30 && both && !fits(pl.ln)) choose(pl.ln, hold / 2, any);
+        // (predictions: 5 tables of 503 x 150, 20 candidates 16.6 -> 13.6, 22 of 31 x 163, 48 candidates 13.8 -> 10.7, 200 of 299 x 50, 30
+        // candidates 95.7 -> 100.0; of few candidates, CTAs mostly set-up: 72 tables of 713 x 25, 4 candidates 40.8 -> 38.0 us; not where there are few CTAs: 11
+        // tables of 91 x 119, 8 candidates 8.1 -> 9.7)
+        if (lines_ctas >= (long long)h->sm_count * 2) choose(pl.lp, n_s <= 8 ? hold / 4 : hold / 2, any);
         // A cell per thread (direct.cuh), 250 instructions and 30 per candidate: where that is half as many as a line for a range of
         // process counts, or no more and the GPU is nearly empty, so that only the length of a CTA counts.  Calls from a graph, lines ->
         // cells, us: one table, 49 process counts, 19 message sizes, 7 candidates 6.8 -> 4.6; 18 x 101, 48 candidates 8.7 -> 5.8; 3
         // tables of 74 x 8, 43 candidates 10.0 -> 6.8; 500 tables of 29 x 8, 5 candidates 13.0 -> 10.1, 2000 of 19 x 6, 4 candidates
-        // 38.4 -> 24.6.  Past the line: 16 tables of 100 x 30, 20 candidates 8.0 -> 9.3, 128 of 63 x 16, 8 candidates 9.0 -> 10.3.
-        // Predictions write more and gain a little longer: the latter 13.3 -> 11.9, but one table of 511 x 64, 32 candidates 8.1 -> 8.8.
+        // 38.4 -> 24.6.  Past the line: 16 tables of 100 x 30, 20 candidates 8.0 -> 9.3, 128 of 63 x 16, 8 candidates 9.0 -> 10.3.  Tables of
+        // more than 64 sizes, which each CTA stages and searches, only where there are many tables or hardly any CTAs: 21 of 51 x 43, 13
+        // candidates, 16 / 64 / 128 / 200 sizes 7.3 7.7 8.7 10.5 -> 5.5 7.3 9.2 11.2, 500 of 29 x 8 12.0 13.1 14.4 15.5 -> 9.0 10.3 11.5 12.6.
+        // And not where the launch of both halves would be lost.
+        // Predictions, beside whose other planes' CTAs those of few tables are too many (21 of 51 x 43 7.1 -> 8.0, 100 of 60 x 12, 6
+        // candidates 10.7 -> 8.5, 128 of 63 x 16 13.3 -> 11.9; 12 of 44 x 30, 41 candidates 7.9 -> 7.2; 511 x 64, 32 candidates 8.1 -> 9.0).
         const long long ctas = ((long long)n_P * n_m + kDecThreads - 1) / kDecThreads * h->T.n_tables;
         const long long cost = std::max(ctas, (long long)h->sm_count * 4) * (250 + 30 * n_s);
-        pl.dr_decide = 2 * cost < best || (cost < best && ctas <= (long long)h->sm_count * 2);
-        pl.dr_predict = 5 * cost < 3 * best || (cost < best && ctas <= (long long)h->sm_count);
+        const int npad = h->T.npad, sms = h->sm_count;
+        const bool launch_more = both && fits(pl.ln) && ctas + scatter_ctas > sms * 6;  // 9 tables of 668 x 19, 7 candidates 8.0 -> 10.8
+        pl.dr_decide = ((!launch_more && (npad <= 64 || h->T.n_tables >= 256)) && (npad <= 32 ? 5 * cost < 3 * best : 2 * cost < best)) ||
+                       (npad <= 128 && cost < best && 2 * ctas <= sms * (npad <= 64 ? 4 : 3));
+        pl.dr_predict = (h->T.n_tables >= 64 && 5 * cost < 3 * best) || (npad <= 128 && cost < best && ctas * (npad <= 64 ? 1 : 2) <= sms);
         pl.dr_ptiles = int(ctas / h->T.n_tables);
         // All message sizes in a CTA (STAGED, lines.cuh), for rows off the sectors: threads for as many groups as leave the fewest
         // idle.  Worth it where a CTA's process counts make up for its set-up, on grids of several CTAs per SM.
@@ -411,31 +429,43 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
             }
             const double busy_lines = double(n_m) / (pl.ln.mgroups * pl.ln.width);
             const long long d_ctas = (long long)pl.ln.ptiles * h->T.n_tables, p_ctas = (long long)pl.lp.ptiles * h->T.n_tables;
-            // Decision, odd rows only: with half the bytes of a plane the waits weigh more.  Time with row segments = 1: 511 process
-            // counts, 8 / 20 / 32 candidates: 1200 tables of 33 message sizes 0.89 0.96 1.07, 65 1.04 1.17 1.31, 99 0.87 0.99 1.12, 127 0.83
-            // 0.93 1.03, 173 0.84 0.96, 201 0.80 0.90; 148 of 2999 process counts 33 0.80 0.84 0.88, 127 0.76 0.82 0.87; 600 tables of 127
-            // 0.97 1.04 1.14; 320 of 199 process counts and 127 1.58 1.55 1.53.  Fewer process counts: only where lines would leave more
-            // lanes idle (2048 tables of 100, 33 message sizes 0.93 0.89 0.84; 47 1.14 1.13 1.12, 127 1.04 1.05 1.06) or candidates are few
-            // and rows long (1095 of 31, 145 message sizes, 9 candidates 0.87; 4000 of 59, 8 candidates, 127 / 173 / 201 / 255 1.06
-            // 0.99 0.93 0.89).
-            pl.all_decide = n_m % 2 != 0 && d_ctas >= (long long)h->sm_count * 6 &&
-                            ((n_P >= 256 ? n_s <= (n_P >= 1024 ? 32 : 24) && busy >= 0.88 : n_P >= 96 && busy >= 1.1 * busy_lines) || (n_m >= 140 && n_s <= 16));
-            // Predictions, rows off the sectors of the sizes, or of times and sizes.  The same at 511 process counts: 1200 tables of 33 0.56
-            // 0.59 0.63, 65 0.61 0.66 0.72, 127 0.56 0.60 0.64, 201 0.56 0.61, 100 (whole sectors of times) 0.70 0.77 0.85; 2048 tables of
-            // 200 process counts: 33 0.82 0.88 0.96, 127 0.56 0.62 0.67, 100 0.95 1.07 1.33; of 100: 33 1.07 1.04 1.00, 65 0.91 1.07 1.14, 99
-            // 0.76 0.87 0.98, 201 0.70 0.81 0.91; 4000 of 59: 99 1.11 1.14 1.22; 320 of 199: 99 1.01 1.02 1.15.
-            pl.all_predict = n_m % 8 != 0 && p_ctas >= (long long)h->sm_count * 4 && (n_m % 4 == 0 ? n_P >= 256 && n_s <= 32 : n_P >= (n_m >= 96 ? 96 : 192));
+            // Decision, odd rows only: with half the bytes of a plane the waits weigh more.  Time with row segments = 1, 8 / 16 / 29 candidates:
+            //   223 tables of 1832 process counts, 33 message sizes 0.82 0.85 0.92, 65 0.93 0.98 1.11, 99 0.79 0.83 0.94, 137 0.74 0.95 1.09
+            //   1200 of 511                         33 0.90 0.92 1.04, 65 1.05 1.08 1.27, 99 0.88 0.93 1.08, 161 0.91 0.96 1.10
+            //   1200 of 172                         33 1.04 1.01 0.98, 65 1.14 1.15 1.15, 99 1.14 1.15 1.19, 195 1.14 1.18 1.23
+            //   2048 of 100 (8 / 20 / 32)           33 0.93 0.89 0.84, 65 0.97 0.97 0.96, 99 0.95 0.96 0.98, 201 0.92 0.95 0.97, 127 1.04 1.05 1.06
+            //   2048 of 28                          33 1.07 1.00 0.91, 65 0.95 0.95 0.91, 99 0.84 0.85 0.85, 161 0.81 0.85 0.88, 47 1.08 1.04 1.03
+            //   2048 of 14                          33 1.14 1.04 0.95, 65 0.83 0.83 0.82, 99 0.75 0.76 0.78, 161 0.68 0.73 0.78
+            // and 600 tables of 511, 127 message sizes 0.97 1.01 1.12, 320 of 199 1.58 1.57 1.53; fewer CTAs for the longest and the shortest
+            // ranges only (100 of 2097, 109 message sizes, 16 candidates 0.92; 303 of 31, 189 message sizes, 4 candidates 0.91).
+            const int d_least = n_P >= 1024 && n_s <= 16 ? 3 : n_P <= 48 && n_m >= 128 ? 2 : 6;
+            pl.all_decide = n_m % 2 != 0 && d_ctas >= (long long)h->sm_count * d_least &&
+                            (n_P <= 48   ? n_m >= 64
+                             : n_P < 256 ? (n_P >= 96 && busy >= 1.1 * busy_lines) || (n_P <= 128 && n_m >= 192 && n_s <= 16)
+                                         : n_s <= (n_P >= 700 ? 32 : 24) && (n_m >= 72 || busy >= 0.88));
+            // Predictions, rows off the sectors of the sizes, or of times and sizes.  The same:
+            //   1200 tables of 511                  33 0.57 0.58 0.63, 65 0.62 0.65 0.72, 99 0.57 0.60 0.66, 161 0.64 0.66 0.74, 100 (whole sectors of
+            //                                       times; 8 / 20 / 32) 0.70 0.77 0.85
+            //   1200 of 172                         33 0.99 1.03 1.13, 47 0.83 0.86 0.97, 99 0.67 0.71 0.81, 161 0.72 0.76 0.87
+            //   2048 of 100 (8 / 20 / 32)           33 1.07 1.04 1.00, 65 0.91 1.07 1.14, 99 0.76 0.87 0.98, 201 0.70 0.81 0.91, 100 1.21 1.26 1.27
+            //   2048 of 28                          65 1.08 1.10 1.09, 99 1.01 1.01 1.03, 137 0.89 0.95 1.00, 255 0.87 0.91
+            //   2048 of 14                          33 1.30 1.18 1.10, 65 0.99 0.98 0.96, 99 0.86 0.86 0.88, 161 0.82 0.86 0.90
+            // and 4000 of 59, 99 1.11 1.14 1.22, 255 0.86 0.93; 320 of 199, 99 1.01 1.02 1.15; 112 of 1776, 117 message sizes, 31 candidates 0.91.
+            const bool rows_long = n_m % 4 == 0 ? n_P >= 256 && n_s <= 32 : n_P >= (n_m >= 96 ? 96 : n_m >= 44 ? 160 : 192);
+            const bool rows_few = n_m % 4 != 0 && ((n_P <= 20 && n_m >= 64) || (n_s <= 16 && n_m >= (n_P <= 48 ? 128 : 192)));
+            pl.all_predict = n_m % 8 != 0 && p_ctas >= (long long)h->sm_count * (n_P >= 1024 ? 2 : 4) && (rows_long || rows_few);
             // One CTA per SM: 1200 tables of 511 process counts, 20 / 32 / 48 candidates: 255 0.79 0.87 0.99, 250 0.83 0.94 1.07, 201 at 32
-            // 0.96, at 48 1.13; 173 at 32 1.10, 127 at 48 1.05; 148 of 2999, 48 candidates 255 0.89, 250 0.98; 2048 of 200, 255 0.80 0.92 1.09.
-            pl.all_alone = n_m % 4 != 0 && n_m > 192 && n_s <= (n_P >= 1024 ? 48 : 32) && n_P >= 192;
+            // 0.96, at 48 1.13; 173 at 32 1.10, 127 at 48 1.05; 148 of 2999, 48 candidates 255 0.89, 250 0.98; 2048 of 200, 255 0.80 0.92 1.09;
+            // 1200 of 172, 255 at 16 0.90, at 29 1.06.
+            pl.all_alone = n_m % 4 != 0 && n_m > 192 && n_s <= (n_P >= 1024 ? 48 : n_P >= 192 ? 32 : 16) && n_P >= 160;
         }
     }
     // One launch for both halves where the GPU holds all their CTAs at once (four per SM, six with a cell per thread; its Scatter CTAs
     // have four warps)
-    if (pl.ln.mgroups > 0 && (g->strategy_mask & 0x3FFu) && (g->strategy_mask & 0x1C00u)) {
+    if (pl.ln.mgroups > 0 && both) {
         const long long base = (long long)pl.n_mtiles * h->T.n_tables, hold = (long long)h->sm_count * (pl.dr_decide ? 6 : 4);
         const long long decide = (pl.dr_decide ? (long long)pl.dr_ptiles : (long long)pl.ln.mgroups * pl.ln.ptiles) * h->T.n_tables, room = hold - decide;
-        pl.select = room >= base;
+        pl.select = room >= scatter_ctas;
         if (pl.select) {
             pl.sel_run = int(std::max<long long>(4, (n_P + kDecWarps * (room / base) - 1) / (kDecWarps * (room / base))));
             pl.sel_ptiles = (n_P + kDecWarps * pl.sel_run - 1) / (kDecWarps * pl.sel_run);

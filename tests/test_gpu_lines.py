@@ -68,7 +68,7 @@ def test_lines_close_to_one_another(plogp, kind, n_s):
 @pytest.mark.parametrize("n_m,n_P,n_s,listed,n_tables", [
     (17, 21, 9, False, 300), (33, 520, 33, False, 300), (50, 16, 8, False, 300), (127, 40, 20, True, 300), (129, 9, 64, False, 300), (255, 33, 5, False, 300), (256, 8, 3, False, 300),
     (33, 97, 33, False, 900), (33, 511, 24, True, 900), (127, 257, 24, False, 900), (201, 256, 3, True, 900), (173, 300, 1, False, 900), (99, 520, 9, False, 450),
-    (145, 31, 9, False, 900), (35, 1100, 32, False, 300), (34, 193, 20, False, 600), (52, 257, 32, False, 600), (250, 260, 32, True, 600), (255, 256, 20, False, 600)])
+    (145, 31, 9, False, 900), (65, 14, 40, True, 900), (195, 172, 8, False, 900), (35, 1100, 32, False, 300), (34, 193, 20, False, 600), (52, 257, 32, False, 600), (250, 260, 32, True, 600), (255, 256, 20, False, 600)])
 def test_all_message_sizes_in_a_cta(plogp, n_m, n_P, n_s, listed, n_tables):
     """Many tables, rows off the sectors: the cells of a step put together in shared memory, for the predictions and the decision
     (600 tables: the predictions alone; 300 of few process counts: neither).  The same as with outputs aligned for single
@@ -210,7 +210,7 @@ def test_a_cell_per_thread_as_lines(plogp, n_P, n_m, n_s, k_mode, listed, ids):
                 assert p.time[:, i].equal(q.time[first:first + 3, i]) and p.best_s[:, j].equal(q.best_s[first:first + 3, j])
 
 
-@pytest.mark.parametrize("n_tables,n_P,n_m,n_s", [(72, 200, 25, 4), (72, 713, 25, 8), (200, 99, 9, 10), (16, 600, 64, 32), (64, 511, 37, 16)])
+@pytest.mark.parametrize("n_tables,n_P,n_m,n_s", [(72, 200, 25, 4), (72, 713, 25, 8), (200, 99, 9, 10), (16, 600, 64, 32), (64, 511, 37, 16), (48, 1384, 24, 10), (4, 2696, 33, 14)])
 def test_tilings_of_medium_grids(plogp, n_tables, n_P, n_m, n_s):
     """Fewer and larger CTAs: both halves in one launch, predictions of few candidates."""
     both(plogp, wl_grid(n_tables=n_tables, n_P=n_P, n_m=n_m, n_s=n_s), tables=[0, n_tables - 1])

@@ -183,7 +183,8 @@ def test_which_grids_have_a_cell_per_thread(lib, n_tables, n_P, n_m, n_s, cells)
 
 @pytest.mark.parametrize("n_tables,n_P,n_m,n_s,decide,predict", [
     (900, 257, 127, 24, 1, 1), (900, 97, 33, 33, 1, 0), (900, 256, 201, 3, 1, 1), (450, 520, 99, 9, 1, 1), (600, 193, 34, 20, 0, 1), (600, 257, 52, 32, 0, 1),
-    (600, 260, 250, 32, 0, 1), (600, 256, 255, 20, 0, 1), (900, 257, 65, 24, 0, 1), (900, 97, 127, 24, 0, 1), (900, 95, 33, 33, 0, 0), (900, 31, 145, 9, 1, 0),
+    (600, 260, 250, 32, 0, 1), (600, 256, 255, 20, 0, 1), (900, 257, 65, 24, 0, 1), (900, 97, 127, 24, 0, 1), (900, 95, 33, 33, 0, 0), (900, 31, 145, 9, 1, 1), (900, 28, 195, 29, 1, 0),
+    (900, 14, 65, 40, 1, 1), (900, 172, 195, 8, 0, 1), (900, 50, 99, 8, 0, 0),
     (900, 1100, 127, 32, 1, 1), (900, 257, 127, 64, 0, 0), (300, 257, 127, 24, 0, 0), (900, 257, 128, 24, 0, 0), (900, 257, 31, 8, 0, 0), (900, 257, 257, 8, 0, 0)])
 def test_which_grids_have_all_message_sizes_in_a_cta(lib, n_tables, n_P, n_m, n_s, decide, predict):
     grid = plogp.GridArgs(np.arange(1, n_m + 1) * 4096, None, 2, n_P + 1, np.arange(1, n_s + 1) * 64)
