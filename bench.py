@@ -34,12 +34,12 @@ if ROOT not in sys.path:
 from paper_cs_0408034_b200 import workloads as wl  # noqa: E402
 
 NOMINAL_FP64_FMA_RATE = 148 * 64 * 1.965e9  # SMs x FP64 lanes per SM x max SM clock
-# dram__bytes_read.sum + dram__bytes_write.sum per launch and per table from the ncu captures summarised
-# under profiles/ (batched workload cut to 1024 tables: 0.87 GB of output per kernel, far beyond the L2,
-# so what is still cached when the kernel ends is a few percent; traffic grows in proportion to the table
-# count).  An entry is None while its kernel has changed since the last capture.
-NCU_TRAFFIC_BYTES_PER_TABLE = {"decide_kernel": 377000000 / 512, "scatter_kernel": 813760256 / 1024, "sweep_kernel": None}
-NCU_TRAFFIC_NOTE = "bytes per launch = bytes per table of the ncu captures in profiles/ (512 tables decide_kernel, 1024 scatter_kernel) x tables"
+# dram__bytes_read.sum and dram__bytes_write.sum per launch from the ncu captures summarised under profiles/ (batched workload
+# cut to 1024 tables).  Of the 0.87 GB that a kernel writes there, some 60 MB are still in the L2 when it ends, on any number of
+# tables: a larger launch writes 13 B per cell and reads its tables more.  None while a kernel has changed since its last capture.
+NCU_TRAFFIC_TABLES = 1024
+NCU_TRAFFIC = {"decide_kernel": (1456896, 811407872), "scatter_kernel": (1700000, 812060256), "sweep_kernel": None}
+NCU_TRAFFIC_NOTE = "bytes of the ncu captures in profiles/ (1024 tables) and, for each table more, its 13 B per cell and its share of the bytes read"
 FALLBACK_HBM_GBS = 6650.0
 
 
@@ -513,9 +513,12 @@ class Bench:
         for k in kernels:
             k["share"] = k["ms_total"] / tot
         dominant = dict(max(kernels, key=lambda k: k["ms_total"])) if kernels else {}
-        per_table = NCU_TRAFFIC_BYTES_PER_TABLE.get(dominant.get("kernel"))
-        batched = w.name.startswith("cfg4") and not m["predict"]
-        dominant["traffic"] = per_table * w.n_tables if (per_table and batched) else None
+        captured = NCU_TRAFFIC.get(dominant.get("kernel"))
+        dominant["traffic"] = None
+        if captured and w.name.startswith("cfg4") and not m["predict"] and w.n_tables >= NCU_TRAFFIC_TABLES:
+            read, written = captured
+            per_table = read / NCU_TRAFFIC_TABLES + 13.0 * w.n_P * w.n_m
+            dominant["traffic"] = read + written + (w.n_tables - NCU_TRAFFIC_TABLES) * per_table
         dominant["traffic_note"] = NCU_TRAFFIC_NOTE if dominant["traffic"] else None
         t_alu = counts["fp64_slots"] / fma_rate
         t_hbm = counts["hbm_bytes"] / (hbm_gbs * 1e9)

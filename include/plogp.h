@@ -121,9 +121,10 @@ typedef struct {
                                0: exhaustive (the default): on every table; every candidate is bounded from below,
                                   for single process counts or for a range of them at once, and compared in FP64
                                   where the bound does not rule it out;
-                               1: lower envelope: ids 2 and 9 take the s with the smallest g(s) k once per m, id 5
-                                  walks the lower envelope of its lines in P (only for tables whose gaps never
-                                  decrease with the size; other tables silently take the exhaustive search) */
+                               1: lower envelope, on lists of more than PLOGP_MAX_INLINE_S sizes: ids 2 and 9 take the
+                                  s with the smallest g(s) k once per m, id 5 walks the lower envelope of its lines
+                                  in P (only for tables whose gaps never decrease with the size; other tables, and
+                                  shorter lists, silently take the exhaustive search) */
 } plogp_grid;
 
 /*

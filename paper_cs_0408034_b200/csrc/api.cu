@@ -393,13 +393,14 @@ int find_or_build(plogp_tables *h, const plogp_grid *g, cudaStream_t st, const P
             const long long cost = choose(beside, hold, hold - (long long)pl.n_mtiles * h->T.n_tables * ((n_P + 127) / 128));
             if (cost && 20 * cost <= 29 * best) pl.ln = beside;
         }
-        // Where another kernel of the call takes what is left of the GPU, the total counts more than a CTA's length: 27 tables of 83 x 168, 34
-        // candidates 15.1 -> 11.2, 200 of 299 x 50, 30 candidates 39.3 -> 34.2, 159 of 594 x 9, 5 candidates 31.2 -> 26.0; long lists, of which a
-        // group then has more, 64 of 511 x 128, 32 candidates 33.8 -> 35.7, 99 of 957 x 24, 62 candidates 73.9 -> 88.1 (two decisions).
+        // Where another kernel of the call takes what is left of the GPU, the total counts more than a CTA's length: 34 tables of 134 x 126, 10
+        // candidates 16.8 -> 12.0, 200 of 299 x 50, 30 candidates 39.3 -> 34.2, 159 of 594 x 9, 5 candidates 31.2 -> 26.0; with more
+        // candidates, of which a group then has more, either way: 27 of 83 x 168, 34 candidates 15.1 -> 11.2, 64 of 511 x 128, 32 candidates 33.8
+        // -> 35.7, 99 of 957 x 24, 62 candidates 73.9 -> 88.1 (two decisions).
         if (n_s <= 30 && both && !fits(pl.ln)) choose(pl.ln, hold / 2, any);
         // (predictions: 5 tables of 503 x 150, 20 candidates 16.6 -> 13.6, 22 of 31 x 163, 48 candidates 13.8 -> 10.7, 200 of 299 x 50, 30
-        // candidates 95.7 -> 100.0; of few candidates, CTAs mostly set-up: 72 tables of 713 x 25, 4 candidates 40.8 -> 38.0 us; not where there are few CTAs: 11
-        // tables of 91 x 119, 8 candidates 8.1 -> 9.7)
+        // candidates 95.7 -> 100.0; of few candidates, CTAs mostly set-up: 72 tables of 713 x 25, 4 candidates 40.8 -> 38.0; not where there are few
+        // CTAs: 11 tables of 91 x 119, 8 candidates 8.1 -> 9.7)
         if (lines_ctas >= (long long)h->sm_count * 2) choose(pl.lp, n_s <= 8 ? hold / 4 : hold / 2, any);
         // A cell per thread (direct.cuh), 250 instructions and 30 per candidate: where that is half as many as a line for a range of
         // process counts, or no more and the GPU is nearly empty, so that only the length of a CTA counts.  Calls from a graph, lines ->

@@ -1,5 +1,5 @@
-// gaps_kernel: g(x) of Section 2 at every distinct argument of the lane <-> P kernels (decide_kernel,
-// segmin_kernel), once per table: g(1) for the rendezvous handshake, g(s) of every candidate segment size
+// gaps_kernel: g(x) of Section 2 at every distinct argument of decide_kernel and
+// segmin_kernel, once per table: g(1) for the rendezvous handshake, g(s) of every candidate segment size
 // and g(m) of every message size.  The CTAs of those kernels that share a table (one per group of message
 // sizes and tile of process counts) then read the values instead of staging the table and interpolating
 // them again.  One CTA per table; worth its launch only on grids with many CTAs per launch (the host decides).

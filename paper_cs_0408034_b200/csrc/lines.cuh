@@ -2,10 +2,10 @@
 // planes of the predictions, for short candidate lists.  (The Scatter half has no candidate lists and goes through
 // scatter_kernel.)
 //
-// One CTA owns one table, up to 32 consecutive message sizes and up to 512 process counts.  Threads are message sizes: a group
-// of 32 (16, 8) threads holds the CTA's message sizes, and the groups share the candidate segment sizes while lines are ruled
-// out, then the process counts while they are evaluated.  Every store is a row segment of consecutive m, whatever a
-// row's alignment.
+// One CTA owns one table, up to 32 consecutive message sizes (STAGED: all of the table's, up to 256) and up to 512 process counts.
+// Threads are message sizes: a group of 32 (16, 8; STAGED: as many as there are) threads holds the CTA's message sizes, and the groups
+// share the candidate segment sizes while lines are ruled out, then the process counts while they are evaluated.  Every store is a
+// row segment of consecutive m, whatever a row's alignment.
 //
 // Every model of Table 1 is, for a fixed message size (and segment size), a line in P or a function of
 // floor(log2 P) and ceil(log2 P) alone:
@@ -21,7 +21,7 @@
 //     of the double's high word, more than 2^-21 of the time, so rounding cannot bring them together again;
 //   * (decision) a line whose time at the lower end is above the smallest time of ids 6 to 9 at the upper end is above it
 //     everywhere: both grow with P, and a rounded fused multiply-add is monotone.
-// What is left (a mean of 1.2 lines of 67 per warp and process count on the batched workload) is evaluated in FP64 at each process
+// What is left (a mean of 1.5 lines of 67 per warp and process count on the batched workload) is evaluated in FP64 at each process
 // count and compared with the pair's time.
 // Ids 2 and 9 grow with Q = g(s) k at every P, so the candidate with the smallest Q stands for all whose Q + 2 L is two units
 // of the high word above its own (the relative distance of two times is smallest there); the others, hardly ever any, are

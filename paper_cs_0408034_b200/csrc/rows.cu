@@ -19,8 +19,7 @@ __host__ __device__ inline int rows_threads(int n_m) { return (n_m + 31) & ~31; 
 __host__ __device__ inline int rows_per_flush(int n_m) { return n_m >= kRowsCells / 4 ? 4 : (n_m <= kRowsCells / 16 ? 16 : kRowsCells / n_m); }
 
 // A piece of n cells starts `shift` cells behind a group of four that is aligned in the plane; it is staged with the same
-// shift, so that a group is one 32-byte load and store.  The cells of the groups at either end go one by one.
-
+// shift, so that a group is one 32-byte load and store (store4).  The cells of the groups at either end go one by one.
 // PREDICT: times of ids 11 and 12 instead of the decision.  ALL: all ids that the kernel writes are enabled.
 template <bool PREDICT, bool ALL>
 __global__ void __launch_bounds__(kRowsThreads, 4) scatter_rows_kernel(const RowsParams p)

@@ -207,7 +207,7 @@ def test_decisions_on_many_tables(plogp, n_m, n_P, n_s, search):
 
 @pytest.mark.parametrize("n_tables,n_m,n_P,search", [(100, 33, 512, 0), (110, 56, 300, 1), (40, 129, 700, 0)])
 def test_decisions_on_a_few_ctas_per_sm(plogp, n_tables, n_m, n_P, search):
-    """Grids on which the lane <-> P kernels take 8 message sizes per CTA instead of 16, the last group ragged."""
+    """Grids of a few CTAs per SM, the last group of message sizes ragged."""
     w = replace(wl.config4(n_tables=n_tables, P_hi=n_P + 1, n_m=n_m, n_s=24, seed_offset=n_m), search_mode=search)
     with plogp.Tables.from_workload(w) as tabs:
         a, b = plogp.select_best(tabs, w), plogp.predict(tabs, w)

@@ -216,7 +216,7 @@ def test_host_output_entry_point_matches_device_outputs(plogp):
 
 
 def test_many_tables_take_the_gap_prepass(plogp):
-    """Enough tables for the host to run gaps_kernel in front of the lane <-> P kernels (g(1), g(s), g(m) read from
+    """Enough tables for the host to run gaps_kernel in front of decide_kernel and segmin_kernel (g(1), g(s), g(m) read from
     its rows instead of interpolated in every CTA), with a last group of message sizes that is not full, in both
     segment-count modes; three tables are compared with the oracle."""
     from dataclasses import replace

@@ -181,6 +181,19 @@ def test_which_grids_have_a_cell_per_thread(lib, n_tables, n_P, n_m, n_s, cells)
         lib.plogp_table_free(h)
 
 
+@pytest.mark.parametrize("n_tables,n_P,n_m,n_s,launches", [(1, 49, 19, 7, 1), (1, 1023, 256, 64, 1), (4, 2696, 33, 14, 1), (200, 99, 9, 10, 1), (9, 668, 19, 7, 1), (48, 1384, 24, 10, 1), (60, 1805, 8, 33, 2),
+                                                           (17, 201, 185, 8, 1), (64, 511, 128, 32, 2), (4096, 511, 128, 32, 3)])
+def test_launches_of_a_decision(lib, n_tables, n_P, n_m, n_s, launches):
+    """One where both halves have room beside one another; the gap pre-pass on large grids."""
+    grid = plogp.GridArgs(np.arange(1, n_m + 1) * 4096, None, 2, n_P + 1, np.arange(1, n_s + 1) * 64)
+    h = load(lib, n_tables)
+    try:
+        n = lib.fake_launches()
+        assert lib.plogp_select_best(h, grid.ref, OUT, OUT, OUT, None) == plogp.OK and lib.fake_launches() - n == launches
+    finally:
+        lib.plogp_table_free(h)
+
+
 @pytest.mark.parametrize("n_tables,n_P,n_m,n_s,decide,predict", [
     (900, 257, 127, 24, 1, 1), (900, 97, 33, 33, 1, 0), (900, 256, 201, 3, 1, 1), (450, 520, 99, 9, 1, 1), (600, 193, 34, 20, 0, 1), (600, 257, 52, 32, 0, 1),
     (600, 260, 250, 32, 0, 1), (600, 256, 255, 20, 0, 1), (900, 257, 65, 24, 0, 1), (900, 97, 127, 24, 0, 1), (900, 95, 33, 33, 0, 0), (900, 31, 145, 9, 1, 1), (900, 28, 195, 29, 1, 0),
